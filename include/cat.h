@@ -195,7 +195,13 @@ CAT_API int cat_create_ex(int64_t H, int64_t W, const cat_rule_t *rule, int32_t 
 /* Chooses the kernel, operand dtype and storage used by later steps
  * (defaults: CAT_KERNEL_AUTO -> TCGEN05, CAT_DTYPE_AUTO -> FP8_E4M3 for
  * TCGEN05 (FP4_E2M1 on NIB4 storage), FP16 for
- * MMA_SYNC; instances start with CAT_STORE_U8).  A change
+ * MMA_SYNC; instances start with CAT_STORE_U8).  With kernel and dtype both
+ * AUTO, one step per launch and no cat_set_tile (also the state after
+ * cat_create) every option is left to the library: cat_step then advances the
+ * grid by box sums in bit planes on CUDA cores where that is faster (packed
+ * storage, 3 to 16 states, small grids; Moore, r <= 16), with the same next
+ * states, and cat_get_options reports the configuration that serves the other
+ * grids and cat_box_sums.  A change
  * of storage reallocates both buffers and converts the current grid (the
  * device is synchronised; earlier cat_state_ptr addresses become invalid).
  * CAT_STORE_BIT1 needs C = 2, the zero boundary and TCGEN05 with FP8_E4M3 or
@@ -256,7 +262,8 @@ CAT_API int cat_get_options(cat_handle_t h, int32_t *kernel, int32_t *dtype, int
  *   {"key": "H=.. W=.. r=.. C=.. nbhd=.. boundary=.. storage=.. gpu=<name>/<SMs>",
  *    "kernel": k, "dtype": d, "tile": t, "window": w, "steps_per_launch": s,
  *    "cell_updates_per_s": v}
- * and when the file already holds an entry for the instance, that entry is
+ * (with "left": 1 added when leaving every option to the library was the
+ * fastest; the other fields are then what cat_get_options reports) and when the file already holds an entry for the instance, that entry is
  * applied without timing (unless flags has CAT_TUNE_REMEASURE).  With the
  * environment variable CAT_AUTOTUNE_CACHE naming such a file,
  * cat_set_options(CAT_KERNEL_AUTO, ...) takes the cached choice (kernel,

@@ -99,6 +99,8 @@ struct cat_instance {
   uint64_t timeout_ns = 2000000000ull;
   int32_t steps_per_launch = 1;  // > 1: cooperative launches of several steps
   bool owns_buffers = true;      // false after cat_bind: the caller owns buf[0], buf[1]
+  bool auto_choice = true;       // kernel, dtype, steps per launch and tile all left to the library
+  int32_t plane_warps = 0;       // resident warps of the bit-plane kernel (0: not looked up yet)
   uint32_t gbar_count = 0;       // arrivals on the grid-barrier counter (d_err[1]) so far
   // grid cell (0, 0) of buffer b (past the ghost frame when there is one)
   uint8_t *origin(int b) const { return buf[b] + ghost * pitch + ghost; }
@@ -206,11 +208,33 @@ bool short_window(const cat_instance *h) {
          h->window != 160 && !wide_tile(h);
 }
 
+cat::PlanesGrid planes_grid(const cat_instance *h, int in) {
+  return cat::PlanesGrid{h->origin(in), h->origin(1 - in), h->pitch, h->H, h->W, h->storage, h->ghost, h->rd};
+}
+
+// Options left to the library: the bit-plane kernel steps the grids on which
+// it is the faster one (the configuration that cat_get_options reports serves
+// the others, box sums and the bounded-wait test).
+bool use_planes(const cat_instance *h) {
+  return h->auto_choice && h->inject == 0 && cat::planes_preferred(planes_grid(h, 0));
+}
+
+int launch_planes(cat_instance *h, int in, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  const cat::PlanesGrid g = planes_grid(h, in);
+  if (h->plane_warps == 0) e = cat::planes_resident_warps(g, h->dev.sms, &h->plane_warps);
+  if (e == cudaSuccess && h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
+  if (e == cudaSuccess) e = cat::planes_launch(g, h->plane_warps, s);
+  if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+  return CAT_OK;
+}
+
 // n_steps steps of instance h from buffer `in` (into buffer 1 - in after an
 // odd count), or the box sums of buffer `in` into `sums`.  n_steps > 1 is one
 // cooperative launch of the tcgen05 Moore kernel (zero boundary).
 int launch_step(cat_instance *h, int in, int32_t *sums, int64_t sums_ld, cudaStream_t s, int n_steps = 1) {
   cudaError_t e;
+  if (!sums && n_steps == 1 && use_planes(h)) return launch_planes(h, in, s);
   if (h->kernel == CAT_KERNEL_TCGEN05) {
     if (h->ghost) {  // periodic: refresh the input's ghost frame first
       e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
@@ -432,6 +456,7 @@ int host_instance_info(cat_handle_t h, InstanceInfo *f) {
   f->tile = h->tile;
   f->window = h->window;
   f->steps_per_launch = h->steps_per_launch;
+  f->left = h->auto_choice;
   return CAT_OK;
 }
 }  // namespace cat
@@ -621,6 +646,8 @@ int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t stora
   if (steps_per_launch < 1) return fail(CAT_ERR_INVALID_ARG, "steps_per_launch must be >= 1");
   const bool vn = h->rule.nbhd == 'N';
   const bool wide = h->rule.r > 16;
+  bool auto_choice = kernel == CAT_KERNEL_AUTO && dtype == CAT_DTYPE_AUTO && steps_per_launch == 1 &&
+                     h->tile == 0 && h->window == 0;
   // AUTO: the autotuner's cached choice when CAT_AUTOTUNE_CACHE names a file
   // holding one for this instance (with the storage asked for), else a fixed rule
   int32_t tuned_tile = -1, tuned_window = 0;
@@ -630,6 +657,7 @@ int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t stora
     int32_t k = 0, d = 0, t = 0, w = 0, spl = 0;
     if (cat::tune_cache_lookup_env(f, &k, &d, &t, &w, &spl) && k >= CAT_KERNEL_TCGEN05 && k <= CAT_KERNEL_RUNSUM &&
         d >= CAT_DTYPE_AUTO && d <= CAT_DTYPE_FP4_E2M1 && spl >= 1) {
+      auto_choice = false;
       kernel = k;
       dtype = d;
       steps_per_launch = spl;
@@ -716,6 +744,9 @@ int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t stora
     int rc = change_storage(h, storage);
     if (rc) return rc;
   }
+  if (h->auto_choice != auto_choice) drop_plans_with(h);
+  h->auto_choice = auto_choice;
+  h->plane_warps = 0;
   h->kernel = kernel;
   h->dtype = dtype;
   h->steps_per_launch = steps_per_launch;
@@ -764,6 +795,7 @@ int cat_set_tile(cat_handle_t h, int32_t ty, int32_t tx, int32_t window_rows) {
   if (h->tile != (t0 ? 0 : ty) || h->window != window_rows) drop_plans_with(h);
   h->tile = t0 ? 0 : ty;
   h->window = window_rows;
+  if (h->tile || h->window) h->auto_choice = false;
   return CAT_OK;
 }
 

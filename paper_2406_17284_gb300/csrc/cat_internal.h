@@ -115,6 +115,7 @@ struct InstanceInfo {
   int64_t H, W;
   cat_rule_t rule;
   int32_t boundary, storage, kernel, dtype, tile, window, steps_per_launch;
+  bool left;   // options left to the library
 };
 int host_instance_info(cat_handle_t h, InstanceInfo *out);
 // The autotuner's cached choice for an instance from the JSON-lines file named
@@ -166,5 +167,19 @@ cudaError_t swar_launch(const uint8_t *in, uint8_t *out, int64_t pitch, int64_t 
 // after k steps to `out`.
 cudaError_t swar_tb_launch(const uint8_t *in, uint8_t *out, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule,
                            int k, cudaStream_t s);
+
+// Box sums in bit planes on CUDA cores (cat_planes.cuh): one step of a grid.
+struct PlanesGrid {
+  const uint8_t *in;   // grid cell (0, 0) of the input and output buffers
+  uint8_t *out;
+  int64_t pitch, H, W;
+  int32_t storage;
+  int32_t frame;       // ghost frame of a periodic grid (16 cells, filled), else 0
+  RuleDev rule;
+};
+bool planes_preferred(const PlanesGrid &g);
+// Warps of the grid's kernel that the GPU holds at once.
+cudaError_t planes_resident_warps(const PlanesGrid &g, int sms, int *warps);
+cudaError_t planes_launch(const PlanesGrid &g, int resident_warps, cudaStream_t s);
 
 }  // namespace cat

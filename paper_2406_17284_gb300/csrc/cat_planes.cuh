@@ -1,0 +1,565 @@
+// Box sums in bit planes: the step kernel body shared by the translation
+// units cat_planes_*.cu (one storage each, so that they compile in parallel).
+//
+// A thread owns 32 consecutive cells of a row (one word of flags [state == 1])
+// and walks down a strip of rows.  A number per cell is held as bit planes
+// (bit b of all 32 numbers in one word), so one three-input logic operation
+// adds one bit of 32 cells:
+//
+//   horizontal  h(x) = sum_{d = 0..2r} cell(x - r + d), by halving: a window
+//               of 2m (+ 1) cells is two windows of m cells, the second
+//               shifted by m, (plus one cell as the carry-in).  The planes of
+//               the cells to the right come from the next lane by shuffle, so
+//               the cost is about 5 log2(2r) operations for any r;
+//   vertical    S(y) = S(y - 1) + h(y + r) - h(y - r - 1): the last 2r + 1
+//               horizontal sums of each thread stay in a ring in shared
+//               memory, so the cost does not grow with r either;
+//   rule        S >= K for the four bounds of the reduced rule, each the carry
+//               chain of a bit-sliced subtraction; the centre cell picks the
+//               survival or the birth range.
+//
+// All additions are exact, so the next states are those of every other kernel
+// (Sec. IV, Eqs. 1-2 define the same count as two band products).
+//
+// What bounds it: the integer pipe (ncu, one bit per cell, 32768^2, r = 16: ALU
+// 82%, DRAM 9%; four bits, r = 10: ALU 69%).  32768^2 one-bit steps: r = 2
+// 224 -> 148 us, r = 16 594 -> 320 us; 24576^2, C = 16, r = 10: four bits 436
+// -> 297 us, one byte 398 -> 355 us (before: the tensor-core kernels, and at
+// r <= 5 a bit-sliced kernel that added the 2r + 1 cells and rows one by one).
+//
+// Lanes are laid over a virtual row of words: the row strips of the grid side
+// by side, each followed by one zero word (the dead cells beyond its right
+// edge, which are also the dead cells left of the next strip).  A warp takes
+// 32 consecutive virtual words and writes all but the first and the last,
+// whose neighbours it does not hold; narrow grids thus fill warps as well as
+// wide ones.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+#include <type_traits>
+
+#include "cat_internal.h"
+
+namespace cat {
+namespace planes {
+
+// Bits needed for a value up to n.
+__host__ __device__ constexpr int bits_for(int n) { return n < 2 ? 1 : 1 + bits_for(n / 2); }
+
+template <int R>
+struct Dim {
+  static constexpr int kH = bits_for(2 * R + 1);                  // planes of a horizontal sum
+  static constexpr int kS = bits_for((2 * R + 1) * (2 * R + 1));  // planes of a box count
+  static constexpr int kWin = 2 * R + 1;
+  static constexpr int kThreadBytes = 4 * (kH * kWin + R);   // rings of horizontal sums and of centre words
+};
+
+constexpr uint32_t kFull = 0xffffffffu;
+constexpr int kMaxR = 16;   // a window reaches one word to either side
+constexpr int kOut = 30;    // words a warp writes: all but the first and the last
+
+// 32 cells of a row as loaded.
+template <int ST>
+struct Raw {
+  static constexpr int kBytes = ST == CAT_STORE_U8 ? 32 : ST == CAT_STORE_NIB4 ? 16 : 4;
+  static constexpr int kWords = kBytes / 4;
+  uint32_t v[kWords];
+};
+
+// Ordinary loads: a programmatically dependent launch starts before the grid
+// it reads is written, so the read-only path must not be used.
+__device__ __forceinline__ void ld16(uint32_t *v, const uint8_t *p) {
+  const uint4 a = *reinterpret_cast<const uint4 *>(p);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+
+// State-1 flags of 32 loaded cells: bit x = [cell x is 1].
+// uint8, two states: four cells' 0/1 bytes are combined pairwise (w | w' << 4)
+// and the eight flags gathered into the top byte by one multiplication whose
+// partial products never meet (all on the multiply pipe; three byte permutes
+// join the four bytes).
+template <int ST, bool MS>
+__device__ __forceinline__ uint32_t flags(const Raw<ST> &r) {
+  if constexpr (ST == CAT_STORE_BIT1) {
+    return r.v[0];
+  } else {
+    uint32_t q[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if constexpr (ST == CAT_STORE_U8 && !MS) {
+        const uint32_t t = r.v[2 * j + 1] * 16u + r.v[2 * j];
+        q[j] = t * 0x01020408u;
+      } else {
+        const uint32_t t = ST == CAT_STORE_U8 ? r.v[(2 * j + 1) & 7] * 16u + r.v[(2 * j) & 7] : r.v[j & 3];
+        // bit 3 of a nibble of f: the state is 1 (t ^ 1 is zero; no nibble carries)
+        const uint32_t x = t ^ 0x11111111u;
+        const uint32_t f = ~(((x & 0x77777777u) + 0x77777777u) | x) & 0x88888888u;
+        if constexpr (ST == CAT_STORE_U8) q[j] = f * 0x00204081u;              // nibble order: cells 0,4,1,5,2,6,3,7
+        else q[j] = ((f | (f >> 3)) & 0x18181818u) * 0x00208208u;             // nibble order: cells 0..7
+      }
+    }
+    return __byte_perm(__byte_perm(q[0], q[1], 0x0073), __byte_perm(q[2], q[3], 0x0073), 0x5410);
+  }
+}
+
+// b(x + D) of a plane for the cell x at bit x, D in 1..32 (next: the plane in
+// the next lane).
+template <int D>
+__device__ __forceinline__ uint32_t shift_right(uint32_t own, uint32_t next) {
+  if constexpr (D < 32) return __funnelshift_r(own, next, D);
+  else return next;
+}
+
+// Window sums of M cells to the right of each cell (M cells starting at it):
+// planes h[0 .. bits_for(M)).
+template <int M, int NH>
+__device__ __forceinline__ void window_sum(uint32_t b, uint32_t next, uint32_t (&h)[NH]) {
+  if constexpr (M == 1) {
+    h[0] = b;
+  } else {
+    constexpr int HM = M / 2, NB = bits_for(HM), NO = bits_for(M);
+    window_sum<HM, NH>(b, next, h);
+    uint32_t c = 0u;
+    if constexpr (M & 1) c = shift_right<2 * HM>(b, next);
+    uint32_t o[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      if constexpr (HM == 1) o[i] = shift_right<1>(b, next);
+      else o[i] = shift_right<HM>(h[i], __shfl_down_sync(kFull, h[i], 1));
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const uint32_t a = h[i];
+      h[i] = a ^ o[i] ^ c;
+      c = (a & o[i]) | (c & (a ^ o[i]));
+    }
+    if constexpr (NO > NB) h[NB] = c;
+  }
+}
+
+// S >= K for every cell: the carry out of S + ~K + 1, one majority function
+// per plane; k[i] is bit i of ~K over a whole word (kernel parameters, so the
+// words are constant operands).
+template <int NS>
+__device__ __forceinline__ uint32_t at_least(const uint32_t (&S)[NS], const uint32_t *k) {
+  uint32_t c = S[0] | k[0];
+#pragma unroll
+  for (int i = 1; i < NS; ++i) c = (S[i] & k[i]) | (c & (S[i] | k[i]));
+  return c;
+}
+
+// Byte j of x in a word of its own.
+template <int J>
+__device__ __forceinline__ uint32_t byte_of(uint32_t x) { return __byte_perm(x, 0u, 0x4440 + J); }
+
+// 16 flags (bytes 2 T and 2 T + 1 of a word whose low and high nibbles are the
+// bytes of lo and hi) -> four words of four 0/1 bytes: a nibble times 2^0 +
+// 2^7 + 2^14 + 2^21 has bit i at bit 8 i (the copies do not overlap).
+template <int T>
+__device__ __forceinline__ void spread_bytes(uint32_t lo, uint32_t hi, uint32_t (&o)[4]) {
+  o[0] = (byte_of<2 * T>(lo) * 0x00204081u) & 0x01010101u;
+  o[1] = (byte_of<2 * T>(hi) * 0x00204081u) & 0x01010101u;
+  o[2] = (byte_of<2 * T + 1>(lo) * 0x00204081u) & 0x01010101u;
+  o[3] = (byte_of<2 * T + 1>(hi) * 0x00204081u) & 0x01010101u;
+}
+
+// Eight flags (a byte) -> eight nibbles 0/1, flag i in nibble i.
+__device__ __forceinline__ uint32_t spread_nibbles(uint32_t b) {
+  uint32_t x = (b * 0x1001u) & 0x000F000Fu;
+  x = (x * 0x41u) & 0x03030303u;
+  return (x * 9u) & 0x11111111u;
+}
+
+// Next states of eight cells in nibbles: t their states (below C <= 16), f the
+// flags (bit 0) of the cells whose count is in range.  State 0 -> f; 1 -> 1 or
+// 2 (0 when C = 2, via two = 0); c >= 2 -> c + 1, 0 past C - 1.
+__device__ __forceinline__ uint32_t age_nibbles(uint32_t t, uint32_t f, uint32_t last, uint32_t two) {
+  const uint32_t u = (t & 0x77777777u) + 0x66666666u;
+  const uint32_t g = (u | t) & 0x88888888u;                        // state >= 2
+  const uint32_t x = t ^ last;                                     // zero for state C - 1
+  const uint32_t k1 = (g & (((x & 0x77777777u) + 0x77777777u) | x)) >> 3;   // 2 <= state < C - 1
+  const uint32_t older = (t + k1) & (k1 * 15u);
+  const uint32_t g1 = g >> 3;
+  const uint32_t lost = (t & two & ~g1) & ~f;                      // state 1, not kept
+  return older | (lost * 2u + (f & ~g1));
+}
+
+// The ring of horizontal sums, per slot, groups of four planes as 16-byte
+// words per thread, then two, then one (conflict-free, few instructions).
+template <int NH, int NT>
+__device__ __forceinline__ void ring_load(const uint8_t *s, int tid, uint32_t (&h)[NH]) {
+  constexpr int G = NH / 4;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const uint4 a = *reinterpret_cast<const uint4 *>(s + NT * 16 * g + tid * 16);
+    h[4 * g] = a.x; h[4 * g + 1] = a.y; h[4 * g + 2] = a.z; h[4 * g + 3] = a.w;
+  }
+  if constexpr (NH & 2) {
+    const uint2 a = *reinterpret_cast<const uint2 *>(s + NT * 16 * G + tid * 8);
+    h[4 * G] = a.x; h[4 * G + 1] = a.y;
+  }
+  if constexpr (NH & 1) h[NH - 1] = *reinterpret_cast<const uint32_t *>(s + NT * 4 * (NH - 1) + tid * 4);
+}
+template <int NH, int NT>
+__device__ __forceinline__ void ring_store(uint8_t *s, int tid, const uint32_t (&h)[NH]) {
+  constexpr int G = NH / 4;
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+    *reinterpret_cast<uint4 *>(s + NT * 16 * g + tid * 16) =
+        make_uint4(h[4 * g], h[4 * g + 1], h[4 * g + 2], h[4 * g + 3]);
+  if constexpr (NH & 2) *reinterpret_cast<uint2 *>(s + NT * 16 * G + tid * 8) = make_uint2(h[4 * G], h[4 * G + 1]);
+  if constexpr (NH & 1) *reinterpret_cast<uint32_t *>(s + NT * 4 * (NH - 1) + tid * 4) = h[NH - 1];
+}
+
+constexpr int kMaxS = bits_for((2 * kMaxR + 1) * (2 * kMaxR + 1));
+enum { kSurviveLo, kSurviveHi, kBirthLo, kBirthHi };   // in range: >= lo and not >= hi
+
+struct Params {
+  const uint8_t *in;   // grid cell (0, 0)
+  uint8_t *out;
+  int64_t pitch;
+  int32_t H, W;
+  int32_t seg;         // words of a strip in the virtual row (the last one is the zero word)
+  int32_t rows;        // rows per strip (a multiple of the rows loaded ahead)
+  int32_t strips;
+  int32_t frame;       // readable cells around the grid (a periodic grid's ghost frame), else 0
+  uint32_t last;       // C - 1 in every nibble
+  uint32_t two;        // 1 in every nibble when a state-1 cell that fails survival becomes 2, else 0
+  uint32_t bound[4][kMaxS];
+};
+
+// What a warp holds and how far ahead it loads.
+template <int R, int ST, bool MS>
+struct Cfg {
+  static constexpr int kSmem = 32 * Dim<R>::kThreadBytes;
+  static constexpr int kBySmem = 232448 / (kSmem + 1024);
+  static constexpr int kWarps = kBySmem < 16 ? kBySmem : 16;   // resident warps aimed at
+  static constexpr int kAhead = MS ? 2 : 4;   // (the loop body is unrolled as far: larger ones miss the instruction cache)
+};
+
+__device__ __forceinline__ const uint8_t *row_ptr(const uint8_t *base, uint32_t row, uint32_t pitch) {
+  uint64_t r;   // one multiply-add, off the integer pipe that the adders use
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(row), "r"(pitch), "l"(base));
+  return reinterpret_cast<const uint8_t *>(r);
+}
+
+// What a lane reads and writes in memory, a 16-cell half of a word (uint8) or a word.
+template <int ST>
+struct Access {
+  const uint8_t *src;   // row 0 of its strip's rows
+  uint8_t *dst;         // output row 0
+  int lo, hi;           // rows of src that exist
+  int rows;             // output rows written
+  int cells, out;       // uint8: cells of the 16 that are readable, that are the grid's
+};
+
+template <int R, int ST, bool MS>
+__global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(const __grid_constant__ Params p) {
+  using D = Dim<R>;
+  constexpr int NH = D::kH, NS = D::kS, NT = 32;
+  constexpr int B = Raw<ST>::kBytes, kParts = ST == CAT_STORE_U8 ? 2 : 1, A = Cfg<R, ST, MS>::kAhead;
+  constexpr int kSlot = NT * 4 * NH, kRing = D::kWin * kSlot, kCentre = NT * 4 * R;
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint8_t *const cring = smem + kRing;
+  const int lane = threadIdx.x;
+
+  // this lane's strip and word column (word w holds cells x0 .. x0 + 31); a
+  // lane without a word reads along with a neighbour and masks its flags
+  const int v = (int)blockIdx.x * kOut + lane - 1;
+  int strip = v < 0 ? 0 : v / p.seg;
+  int w = v < 0 ? p.seg - 1 : v - strip * p.seg;
+  const bool held = w < p.seg - 1 && strip < p.strips;
+  w = w < p.seg - 1 ? w : p.seg - 2;
+  strip = strip < p.strips ? strip : p.strips - 1;
+  const int64_t y0 = (int64_t)strip * p.rows;
+  const int64_t x0 = (int64_t)w * 32 - p.frame;
+  const int64_t left = p.W + p.frame - x0;   // readable cells from x0 on
+  const uint32_t mask = !held ? 0u : left >= 32 ? ~0u : (1u << (int)left) - 1u;
+  const bool writes = held && lane >= 1 && lane <= kOut;
+  const int my_rows = !writes ? 0 : p.H - y0 < p.rows ? (int)(p.H - y0) : p.rows;
+  const int64_t col = (int64_t)w * B - p.frame;   // (a frame comes with one byte per cell)
+  // the strip's rows y0 - R + i, i in [0, 2 R + rows); those in [lo, hi) exist
+  const int64_t ys = y0 - R;
+  const int lo = ys < -p.frame ? (int)(-p.frame - ys) : 0;
+  const int hi = (int)(p.H + p.frame - ys < (1 << 30) ? p.H + p.frame - ys : (1 << 30));
+  const bool inside = __all_sync(kFull, lo == 0 && hi >= 2 * R + p.rows + A && p.H - y0 >= p.rows);
+  const uint32_t pitch = (uint32_t)p.pitch;
+  // Memory accesses: one word per lane, or with one byte per cell two 16-cell
+  // halves of words, so that a warp's access is contiguous: lane l takes half
+  // l & 1 of the words of lanes l / 2 and 16 + l / 2.
+  Access<ST> acc[kParts];
+#pragma unroll
+  for (int t = 0; t < kParts; ++t) {
+    const int from = kParts == 1 ? lane : 16 * t + (lane >> 1), half = kParts == 1 ? 0 : lane & 1;
+    const int64_t x = __shfl_sync(kFull, x0, from) + 16 * half;
+    const int64_t y = __shfl_sync(kFull, y0, from), c = __shfl_sync(kFull, col, from) + 16 * half;
+    const int64_t readable = p.W + p.frame - x;
+    acc[t].cells = readable >= 16 ? 16 : readable <= 0 ? 0 : (int)readable;
+    // (a half without a cell reads the other half, and clears it)
+    acc[t].src = p.in + (y - R) * p.pitch + c - (ST == CAT_STORE_U8 && readable <= 0 ? 16 : 0);
+    acc[t].dst = p.out + y * p.pitch + c;
+    acc[t].lo = __shfl_sync(kFull, lo, from);
+    acc[t].hi = __shfl_sync(kFull, hi, from);
+    acc[t].rows = __shfl_sync(kFull, my_rows, from);
+    acc[t].out = p.W - x >= 16 ? 16 : (int)(p.W - x);
+    if (ST == CAT_STORE_U8 && (x < 0 || x >= p.W)) acc[t].rows = 0;
+  }
+  bool odd_end = false;   // some access of the warp ends within its 16 cells
+  if (ST == CAT_STORE_U8)
+    odd_end = __any_sync(kFull, acc[0].cells < 16 || acc[kParts - 1].cells < 16 || acc[0].out < 16 || acc[kParts - 1].out < 16);
+
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  // uint8: bytes past the last readable cell belong to whoever owns the buffer
+  auto clear_past = [&](Raw<ST> &r) {
+#pragma unroll
+    for (int i = 0; i < Raw<ST>::kWords; ++i) {
+      const int cells = acc[i / 4 % kParts].cells - 4 * (i % 4);
+      r.v[i] &= cells >= 4 ? ~0u : cells <= 0 ? 0u : (1u << (8 * cells)) - 1u;
+    }
+  };
+  // flags of a loaded row: uint8, the halves of a lane's word come from lanes
+  // 2 l and 2 l + 1, their first accesses for lanes below 16, else their second
+  const uint32_t halves = lane < 16 ? 0x5410u : 0x7632u;
+  auto flags_of = [&](Raw<ST> r, uint32_t valid) {
+    if (ST == CAT_STORE_U8 && odd_end) clear_past(r);
+    uint32_t f = flags<ST, MS>(r);
+    if constexpr (ST == CAT_STORE_U8)
+      f = __byte_perm(__shfl_sync(kFull, f, 2 * lane), __shfl_sync(kFull, f, 2 * lane + 1), halves);
+    return f & valid;
+  };
+  auto hsum = [&](uint32_t c, uint32_t (&h)[NH]) {
+    const uint32_t b = __funnelshift_l(__shfl_up_sync(kFull, c, 1), c, R);   // bit x: cell x - R
+    window_sum<D::kWin, NH>(b, __shfl_down_sync(kFull, b, 1), h);
+  };
+  auto next_slot = [&](int &q) {
+    const int now = q;
+    q = q + kSlot == kRing ? 0 : q + kSlot;
+    return now;
+  };
+  auto next_cslot = [&](int &q) {
+    const int now = q;
+    q = q + 4 * NT == kCentre ? 0 : q + 4 * NT;
+    return now;
+  };
+  // S += h
+  auto add_rows = [&](uint32_t (&S)[NS], const uint32_t (&h)[NH]) {
+    uint32_t cy = 0u;
+#pragma unroll
+    for (int b = 0; b < NS; ++b) {
+      const uint32_t a = S[b], x = b < NH ? h[b] : 0u;
+      S[b] = a ^ x ^ cy;
+      cy = (a & x) | (cy & (a ^ x));
+    }
+  };
+  // S += h - o: the difference (two's complement, its sign in br), then the sum
+  auto slide = [&](uint32_t (&S)[NS], uint32_t (&h)[NH], const uint32_t (&o)[NH]) {
+    uint32_t br = 0u, cy = 0u;
+#pragma unroll
+    for (int b = 0; b < NH; ++b) {
+      const uint32_t d = h[b] ^ o[b] ^ br;
+      br = (~h[b] & o[b]) | (br & ~(h[b] ^ o[b]));
+      h[b] = d;
+    }
+#pragma unroll
+    for (int b = 0; b < NS; ++b) {
+      const uint32_t a = S[b], x = b < NH ? h[b] : br;
+      S[b] = a ^ x ^ cy;
+      cy = (a & x) | (cy & (a ^ x));
+    }
+  };
+  auto rule = [&](const uint32_t (&S)[NS], uint32_t centre) {
+    const uint32_t keep = at_least<NS>(S, p.bound[kSurviveLo]) & ~at_least<NS>(S, p.bound[kSurviveHi]);
+    const uint32_t born = at_least<NS>(S, p.bound[kBirthLo]) & ~at_least<NS>(S, p.bound[kBirthHi]);
+    return (centre & keep) | (~centre & born);
+  };
+  // uint8: flags of the two halves of words that this lane writes
+  const uint32_t mine = lane & 1 ? 0x7632u : 0x5410u;
+  auto split = [&](uint32_t in) {
+    return __byte_perm(__shfl_sync(kFull, in, lane >> 1), __shfl_sync(kFull, in, 16 + (lane >> 1)), mine);
+  };
+  auto store_part = [&](uint8_t *q, uint32_t (&a)[4], int cells) {   // cells of 16: the bytes past W are not the grid's
+    if (cells & 8) {
+      *reinterpret_cast<uint2 *>(q) = make_uint2(a[0], a[1]);
+      q += 8;
+      a[0] = a[2]; a[1] = a[3];
+    }
+    if (cells & 4) {
+      *reinterpret_cast<uint32_t *>(q) = a[0];
+      q += 4;
+      a[0] = a[1];
+    }
+    if (cells & 2) {
+      *reinterpret_cast<uint16_t *>(q) = (uint16_t)a[0];
+      q += 2;
+      a[0] >>= 16;
+    }
+    if (cells & 1) *q = (uint8_t)a[0];
+  };
+  auto put = [&](int j, uint32_t in, const Raw<ST> &cs) {   // output row j of the strip
+    uint32_t lo4 = 0u, hi4 = 0u;
+    if constexpr (ST == CAT_STORE_U8) {
+      in = split(in);
+      lo4 = in & 0x0F0F0F0Fu;
+      hi4 = (in >> 4) & 0x0F0F0F0Fu;
+    }
+#pragma unroll
+    for (int t = 0; t < kParts; ++t) {
+      if (j >= acc[t].rows) continue;
+      uint8_t *const q = const_cast<uint8_t *>(row_ptr(acc[t].dst, (uint32_t)j, pitch));
+      if constexpr (ST == CAT_STORE_BIT1) {
+        *reinterpret_cast<uint32_t *>(q) = in & mask;
+      } else if constexpr (ST == CAT_STORE_NIB4) {
+        const uint32_t f = in & mask;
+        uint4 a;
+        a.x = age_nibbles(cs.v[0], spread_nibbles(byte_of<0>(f)), p.last, p.two);
+        a.y = age_nibbles(cs.v[1], spread_nibbles(byte_of<1>(f)), p.last, p.two);
+        a.z = age_nibbles(cs.v[2], spread_nibbles(byte_of<2>(f)), p.last, p.two);
+        a.w = age_nibbles(cs.v[3], spread_nibbles(byte_of<3>(f)), p.last, p.two);
+        *reinterpret_cast<uint4 *>(q) = a;
+      } else {
+        uint32_t a[4];
+        if (t == 0) spread_bytes<0>(lo4, hi4, a);
+        else spread_bytes<1>(lo4, hi4, a);
+        if constexpr (MS) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {   // nibble pairs: even words in the low nibbles
+            const uint32_t u = cs.v[4 * t + 2 * i + 1] * 16u + cs.v[4 * t + 2 * i];
+            const uint32_t r = age_nibbles(u, a[2 * i + 1] * 16u + a[2 * i], p.last, p.two);
+            a[2 * i] = r & 0x0F0F0F0Fu;
+            a[2 * i + 1] = (r >> 4) & 0x0F0F0F0Fu;
+          }
+        }
+        if (!odd_end || acc[t].out == 16) *reinterpret_cast<uint4 *>(q) = make_uint4(a[0], a[1], a[2], a[3]);
+        else store_part(q, a, acc[t].out);
+      }
+    }
+  };
+
+  // EDGE: a strip at the top or bottom of the grid, whose rows outside it are
+  // zero (the loads stay on rows that exist)
+  auto walk = [&](auto edge) {
+    constexpr bool EDGE = decltype(edge)::value;
+    auto valid_of = [&](int i) { return EDGE && (i < lo || i >= hi) ? 0u : mask; };
+    auto load = [&](Raw<ST> &r, int i) {   // row i of the strip's rows
+#pragma unroll
+      for (int t = 0; t < kParts; ++t) {
+        const int row = !EDGE ? i : i < acc[t].lo ? acc[t].lo : i >= acc[t].hi ? acc[t].hi - 1 : i;
+        const uint8_t *q = row_ptr(acc[t].src, (uint32_t)row, pitch);
+        if constexpr (ST == CAT_STORE_BIT1) r.v[0] = *reinterpret_cast<const uint32_t *>(q);
+        else ld16(r.v + 4 * t, q);
+      }
+    };
+    Raw<ST> raw[A], ctr[2];
+#pragma unroll
+    for (int k = 0; k < A; ++k) load(raw[k], k);
+    if constexpr (MS) {   // centre rows, for their states
+      load(ctr[0], R);
+      load(ctr[1], R + 1);
+    }
+    uint32_t S[NS];
+#pragma unroll
+    for (int b = 0; b < NS; ++b) S[b] = 0u;
+    int slot = 0, cslot = 0;
+
+    // Rows go in pairs, whose chains of dependent operations overlap.
+    auto take = [&](int i, int k) {   // flags of row i from raw[k], which then takes row i + A
+      const uint32_t c = flags_of(raw[k], valid_of(i));
+      load(raw[k], i + A);
+      return c;
+    };
+    auto first_rows = [&](int i, int k) {   // rows i, i + 1 < 2 R: into the sum only
+      uint32_t h0[NH], h1[NH];
+      const uint32_t c0 = take(i, k), c1 = take(i + 1, k + 1);
+      hsum(c0, h0);
+      hsum(c1, h1);
+      ring_store<NH, NT>(smem + next_slot(slot), lane, h0);
+      ring_store<NH, NT>(smem + next_slot(slot), lane, h1);
+      *reinterpret_cast<uint32_t *>(cring + next_cslot(cslot) + 4 * lane) = c0;
+      *reinterpret_cast<uint32_t *>(cring + next_cslot(cslot) + 4 * lane) = c1;
+      add_rows(S, h0);
+      add_rows(S, h1);
+    };
+    constexpr int kRest = (2 * R) % A;
+    for (int i = 0; i < 2 * R - kRest; i += A) {
+#pragma unroll
+      for (int k = 0; k < A; k += 2) first_rows(i + k, k);
+    }
+#pragma unroll
+    for (int k = 0; k < kRest; k += 2) first_rows(2 * R - kRest + k, k);
+    {   // no row leaves the window of the first output row
+      uint32_t z[NH];
+#pragma unroll
+      for (int b = 0; b < NH; ++b) z[b] = 0u;
+      ring_store<NH, NT>(smem + slot, lane, z);
+    }
+
+    for (int j = 0; j < p.rows; j += A) {
+#pragma unroll
+      for (int k = 0; k < A; k += 2) {
+        constexpr int kOdd = kRest;
+        uint32_t h0[NH], h1[NH], o0[NH], o1[NH], m0, m1;
+        const int i = 2 * R + j + k;
+        const uint32_t c0 = take(i, (k + kOdd) % A), c1 = take(i + 1, (k + 1 + kOdd) % A);
+        hsum(c0, h0);
+        hsum(c1, h1);
+        uint8_t *const s0 = smem + next_slot(slot), *const s1 = smem + next_slot(slot);
+        ring_load<NH, NT>(s0, lane, o0);
+        ring_load<NH, NT>(s1, lane, o1);
+        ring_store<NH, NT>(s0, lane, h0);
+        ring_store<NH, NT>(s1, lane, h1);
+        uint32_t *const q0 = reinterpret_cast<uint32_t *>(cring + next_cslot(cslot) + 4 * lane);
+        uint32_t *const q1 = reinterpret_cast<uint32_t *>(cring + next_cslot(cslot) + 4 * lane);
+        m0 = *q0;
+        *q0 = c0;
+        m1 = *q1;   // (the same word as q0 when R = 1)
+        *q1 = c1;
+        if (MS && ST == CAT_STORE_U8 && odd_end) {
+          clear_past(ctr[0]);
+          clear_past(ctr[1]);
+        }
+        slide(S, h0, o0);
+        const uint32_t in0 = rule(S, m0);
+        slide(S, h1, o1);
+        const uint32_t in1 = rule(S, m1);
+        put(j + k, in0, ctr[0]);
+        put(j + k + 1, in1, ctr[1]);
+        if constexpr (MS) {
+          load(ctr[0], R + j + k + 2);
+          load(ctr[1], R + j + k + 3);
+        }
+      }
+    }
+  };
+  if (inside) walk(std::false_type{});
+  else walk(std::true_type{});
+}
+
+// Kernel of radius r for one storage, with the bytes of shared memory a warp
+// takes; nullptr when it is not built.
+struct Kernel {
+  void (*fn)(Params) = nullptr;
+  int smem = 0, out_words = 0, ahead = 0, planes = 0;
+};
+// r <= 16; uint8 with two states, and with 3 .. 16
+Kernel kernel_u8(int r);
+Kernel kernel_u8_ms(int r);
+Kernel kernel_bit1(int r);
+Kernel kernel_nib4(int r);
+
+template <int ST, bool MS, int LO, int HI>
+Kernel find_kernel(int r) {
+  if constexpr (LO > HI) {
+    return Kernel{};
+  } else {
+    if (r == LO)
+      return Kernel{planes_kernel<LO, ST, MS>, Cfg<LO, ST, MS>::kSmem, kOut, Cfg<LO, ST, MS>::kAhead,
+                    Dim<LO>::kS};
+    return find_kernel<ST, MS, LO + 1, HI>(r);
+  }
+}
+
+}  // namespace planes
+}  // namespace cat

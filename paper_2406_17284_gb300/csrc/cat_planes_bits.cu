@@ -1,0 +1,10 @@
+// The bit-plane box-sum kernels (cat_planes.cuh), one bit per cell.
+#include "cat_planes.cuh"
+
+namespace cat {
+namespace planes {
+
+Kernel kernel_bit1(int r) { return find_kernel<CAT_STORE_BIT1, false, 1, 16>(r); }
+
+}  // namespace planes
+}  // namespace cat

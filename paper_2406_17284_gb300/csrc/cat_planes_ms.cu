@@ -1,0 +1,10 @@
+// The bit-plane box-sum kernels (cat_planes.cuh), one byte per cell, three to sixteen states.
+#include "cat_planes.cuh"
+
+namespace cat {
+namespace planes {
+
+Kernel kernel_u8_ms(int r) { return find_kernel<CAT_STORE_U8, true, 1, 16>(r); }
+
+}  // namespace planes
+}  // namespace cat

@@ -26,6 +26,7 @@ namespace {
 
 struct Cand {
   int32_t kernel, dtype, tile, window, spl;
+  bool left = false;   // every option left to the library (CAT_KERNEL_AUTO); the others are then what it reports
 };
 
 std::string cache_key(const InstanceInfo &f) {
@@ -58,6 +59,7 @@ bool cache_read(const char *path, const std::string &key, Cand *out, double *rat
     if (o && sscanf(o, "\"kernel\": %d, \"dtype\": %d, \"tile\": %d, \"window\": %d, \"steps_per_launch\": %d, "
                        "\"cell_updates_per_s\": %lf",
                     &c.kernel, &c.dtype, &c.tile, &c.window, &c.spl, &v) == 6) {
+      c.left = strstr(o, "\"left\": 1") != nullptr;
       *out = c;
       if (rate) *rate = v;
       found = true;
@@ -72,8 +74,8 @@ void cache_write(const char *path, const std::string &key, const Cand &c, double
   if (!fp) return;
   fprintf(fp,
           "{\"key\": \"%s\", \"kernel\": %d, \"dtype\": %d, \"tile\": %d, \"window\": %d, \"steps_per_launch\": %d, "
-          "\"cell_updates_per_s\": %.6e}\n",
-          key.c_str(), c.kernel, c.dtype, c.tile, c.window, c.spl, rate);
+          "\"cell_updates_per_s\": %.6e%s}\n",
+          key.c_str(), c.kernel, c.dtype, c.tile, c.window, c.spl, rate, c.left ? ", \"left\": 1" : "");
   fclose(fp);
 }
 
@@ -81,12 +83,14 @@ void cache_write(const char *path, const std::string &key, const Cand &c, double
 // when the instance cannot run it.
 bool apply(cat_handle_t h, const InstanceInfo &f, const Cand &c) {
   if (cat_set_tile(h, 0, 0, 0) != CAT_OK) return false;
+  if (c.left) return cat_set_options(h, CAT_KERNEL_AUTO, CAT_DTYPE_AUTO, f.storage, 1) == CAT_OK;
   if (cat_set_options(h, c.kernel, c.dtype, f.storage, c.spl) != CAT_OK) return false;
   return cat_set_tile(h, c.tile, c.tile, c.window) == CAT_OK;
 }
 
 std::vector<Cand> candidates(const InstanceInfo &f) {
   std::vector<Cand> out;
+  out.push_back({CAT_KERNEL_AUTO, CAT_DTYPE_AUTO, 0, 0, 1, true});
   for (int spl : {1, 4, 16}) {
     for (int dt : {CAT_DTYPE_FP8_E4M3, CAT_DTYPE_FP16}) {
       out.push_back({CAT_KERNEL_TCGEN05, dt, 128, 160, spl});
@@ -116,7 +120,7 @@ bool tune_cache_lookup_env(const InstanceInfo &info, int32_t *kernel, int32_t *d
                            int32_t *spl) {
   const char *path = getenv("CAT_AUTOTUNE_CACHE");
   Cand c{};
-  if (!path || !*path || !cache_read(path, cache_key(info), &c, nullptr)) return false;
+  if (!path || !*path || !cache_read(path, cache_key(info), &c, nullptr) || c.left) return false;
   *kernel = c.kernel;
   *dtype = c.dtype;
   *tile = c.tile;
@@ -142,7 +146,7 @@ extern "C" CAT_API int cat_autotune(cat_handle_t h, int32_t n_steps, const char 
   if (!(flags & CAT_TUNE_REMEASURE) && cat::cache_read(cache_path, key, &best, &best_rate) &&
       cat::apply(h, f, best))
     return CAT_OK;
-  const Cand before{f.kernel, f.dtype, f.tile, f.window, f.steps_per_launch};
+  const Cand before{f.kernel, f.dtype, f.tile, f.window, f.steps_per_launch, f.left};
   cudaStream_t s = (cudaStream_t)stream;
   // the state is saved once and restored before every candidate and at the end
   uint8_t *saved = nullptr;
@@ -179,6 +183,7 @@ extern "C" CAT_API int cat_autotune(cat_handle_t h, int32_t n_steps, const char 
   cudaFree(saved);
   if (rs) return rs;
   if (e != cudaSuccess) return cat::cuda_err(e, "cat_autotune");
+  if (best.left) cat_get_options(h, &best.kernel, &best.dtype, nullptr, &best.spl, &best.tile, &best.window);
   if (rc == CAT_OK && !(flags & CAT_TUNE_NO_WRITE)) cat::cache_write(cache_path, key, best, best_rate);
   return rc;
 }

@@ -1,0 +1,93 @@
+"""The bit-plane box-sum kernel (options left to the library) vs the CPU
+oracle: radii at the edges of its plane counts, widths around 32-cell words
+and the words a warp writes, strips shorter and longer than the grid, every
+storage, both boundaries, and buffers whose bytes past W belong to the caller.
+All values are whole numbers, so every comparison is exact.
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2406_17284_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(1, 1), (9, 16), (40, 33), (33, 961), (70, 1031), (700, 95)]
+
+
+@pytest.fixture(scope="module")
+def cat():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2406_17284_gb300 import build
+    build.build()
+    from paper_2406_17284_gb300 import cat as catmod
+    catmod.load()
+    return catmod
+
+
+def board(H, W, C, seed):
+    g = inputs.bernoulli(H, W, 0.5, seed)
+    if C > 2:
+        u = inputs.uniform_states(H, W, C, seed + 1)
+        g = np.where((u >= 2) & (inputs.bernoulli(H, W, 0.3, seed + 2) == 1), u, g)
+    return g.astype(np.uint8)
+
+
+def check(cat, H, W, rule, storage, boundary=0, steps=3):
+    grid = board(H, W, rule["C"], 7 * H + W + rule["r"])
+    g = cat.Grid(H, W, rule, kernel="auto", dtype="auto", storage=storage, boundary=boundary)
+    try:
+        g.set_state(grid)
+        g.step(steps)
+        got = g.get_state()
+        assert g.status() == cat.CAT_OK
+    finally:
+        g.close()
+    want = oracle.step(grid, oracle.Rule(**rule), boundary=boundary, n_steps=steps)
+    assert np.array_equal(got, want), (H, W, rule, storage, boundary, int((got != want).sum()))
+
+
+def rules(r, C):
+    s = inputs.scaled_rule(r, M=r & 1, C=C)
+    top = (2 * r + 1) ** 2
+    # empty survival range, birth of everything; survival of full boxes only
+    return [s, dict(s, s1=3, s2=2, b1=0, b2=top), dict(s, M=1, s1=top, s2=1 << 30, b1=1, b2=top // 2)]
+
+
+@pytest.mark.parametrize("storage,C,radii", [(0, 2, (1, 2, 3, 7, 8, 9)), (1, 2, (1, 2, 3, 5, 7, 8, 15, 16)),
+                                             (2, 2, (1, 9)), (2, 16, (1, 10, 16)), (0, 3, (1, 15)), (0, 16, (2, 10))])
+def test_planes_match_the_oracle(cat, storage, C, radii):
+    for r in radii:
+        for H, W in SHAPES:
+            for rule in rules(r, C):
+                check(cat, H, W, rule, storage)
+
+
+@pytest.mark.parametrize("C", [2, 5])
+def test_planes_on_a_torus(cat, C):
+    for r in (1, 6, 9):
+        for H, W in [(20, 17), (33, 64), (70, 1031)]:
+            check(cat, H, W, inputs.scaled_rule(r, C=C), 0, boundary=1)
+
+
+@pytest.mark.parametrize("C", [2, 16])
+def test_bytes_past_the_grid_are_not_read_or_written(cat, C):
+    """Bound buffers with a pitch above W, the gap full of other data."""
+    import torch
+    for H, W, pitch in [(50, 37, 48), (50, 1000, 1024), (9, 97, 112)]:
+        rule = inputs.scaled_rule(4, C=C)
+        grid = board(H, W, C, W)
+        a = torch.full((H, pitch), 255, dtype=torch.uint8, device="cuda")
+        b = torch.full((H, pitch), 254, dtype=torch.uint8, device="cuda")
+        a[:, :W] = torch.from_numpy(grid).cuda()
+        g = cat.Grid(H, W, rule, kernel="auto", dtype="auto")
+        try:
+            cat.cat_bind(g.handle, a.data_ptr(), b.data_ptr(), pitch)
+            g.step(3)
+            torch.cuda.synchronize()
+        finally:
+            g.close()
+        assert np.array_equal(b[:, :W].cpu().numpy(), oracle.step(grid, oracle.Rule(**rule), n_steps=3))
+        assert bool((a[:, W:] == 255).all()) and bool((b[:, W:] == 254).all())
