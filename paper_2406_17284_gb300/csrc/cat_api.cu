@@ -100,7 +100,6 @@ struct cat_instance {
   int32_t steps_per_launch = 1;  // > 1: cooperative launches of several steps
   bool owns_buffers = true;      // false after cat_bind: the caller owns buf[0], buf[1]
   bool auto_choice = true;       // kernel, dtype, steps per launch and tile all left to the library
-  int32_t plane_warps = 0;       // resident warps of the bit-plane kernel (0: not looked up yet)
   uint32_t gbar_count = 0;       // arrivals on the grid-barrier counter (d_err[1]) so far
   // grid cell (0, 0) of buffer b (past the ghost frame when there is one)
   uint8_t *origin(int b) const { return buf[b] + ghost * pitch + ghost; }
@@ -209,7 +208,8 @@ bool short_window(const cat_instance *h) {
 }
 
 cat::PlanesGrid planes_grid(const cat_instance *h, int in) {
-  return cat::PlanesGrid{h->origin(in), h->origin(1 - in), h->pitch, h->H, h->W, h->storage, h->ghost, h->rd};
+  return cat::PlanesGrid{h->origin(in), h->origin(1 - in), h->pitch, h->H, h->W, h->storage, h->storage, h->ghost, h->rd,
+                         h->dev.id, h->dev.sms};
 }
 
 // Options left to the library: the bit-plane kernel steps the grids on which
@@ -221,11 +221,45 @@ bool use_planes(const cat_instance *h) {
 
 int launch_planes(cat_instance *h, int in, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  const cat::PlanesGrid g = planes_grid(h, in);
-  if (h->plane_warps == 0) e = cat::planes_resident_warps(g, h->dev.sms, &h->plane_warps);
-  if (e == cudaSuccess && h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
-  if (e == cudaSuccess) e = cat::planes_launch(g, h->plane_warps, s);
+  if (h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
+  if (e == cudaSuccess) e = cat::planes_launch(planes_grid(h, in), s);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+  return CAT_OK;
+}
+
+// Several steps of a two-state uint8 grid in one call: the states between the
+// first and the last step are kept one bit per cell, within the rows of
+// whichever of the two buffers holds no state that is still needed (a row of
+// bits takes an eighth of a row of cells, so two fit beside each other; bytes
+// outside the grid's rows are not touched).
+bool use_packed_steps(const cat_instance *h, int64_t n_steps) {
+  return n_steps >= 2 && h->auto_choice && h->inject == 0 && h->storage == CAT_STORE_U8 && h->rule.C == 2 &&
+         h->rule.nbhd == 'M' && h->rule.r <= 16 && h->ghost == 0 && h->W >= 64;
+}
+
+int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
+  const int64_t second = round_up((h->W + 31) / 32 * 4, 16);   // byte offset of a row's second row of bits
+  const int last = h->cur ^ (int)(n_steps & 1);                // the buffer the final states go to
+  cat::PlanesGrid g = planes_grid(h, h->cur);                  // first step: bits into the other buffer
+  g.storage_out = CAT_STORE_BIT1;
+  int at = 1 - h->cur;
+  int64_t off = 0;
+  for (int64_t t = 0; t < n_steps; ++t) {
+    if (t > 0) {
+      g.in = h->buf[at] + off;
+      g.storage_in = CAT_STORE_BIT1;
+      if (t == n_steps - 1) {
+        g.out = h->buf[last];
+        g.storage_out = CAT_STORE_U8;
+      } else {   // stay out of the final states' buffer once the first states have been read
+        off = at == last ? 0 : off ? 0 : second;
+        at = 1 - last;
+        g.out = h->buf[at] + off;
+      }
+    }
+    const cudaError_t e = cat::planes_launch(g, s);
+    if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+  }
   return CAT_OK;
 }
 
@@ -746,7 +780,6 @@ int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t stora
   }
   if (h->auto_choice != auto_choice) drop_plans_with(h);
   h->auto_choice = auto_choice;
-  h->plane_warps = 0;
   h->kernel = kernel;
   h->dtype = dtype;
   h->steps_per_launch = steps_per_launch;
@@ -834,6 +867,11 @@ int cat_state_ptr(cat_handle_t h, void **dptr, int64_t *pitch) {
 int cat_step(cat_handle_t h, int64_t n_steps, void *stream) {
   if (!h) return fail(CAT_ERR_INVALID_ARG, "handle is NULL");
   if (n_steps < 0) return fail(CAT_ERR_INVALID_ARG, "n_steps < 0");
+  if (use_packed_steps(h, n_steps)) {
+    const int rc = launch_packed_steps(h, n_steps, (cudaStream_t)stream);
+    if (rc == CAT_OK) h->cur ^= (int)(n_steps & 1);
+    return rc;
+  }
   for (int64_t t = 0; t < n_steps;) {
     const int m = (int)std::min<int64_t>(h->steps_per_launch, n_steps - t);
     int rc = launch_step(h, h->cur, nullptr, 0, (cudaStream_t)stream, m);

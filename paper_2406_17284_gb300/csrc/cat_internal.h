@@ -172,14 +172,14 @@ cudaError_t swar_tb_launch(const uint8_t *in, uint8_t *out, int64_t pitch, int64
 struct PlanesGrid {
   const uint8_t *in;   // grid cell (0, 0) of the input and output buffers
   uint8_t *out;
-  int64_t pitch, H, W;
-  int32_t storage;
+  int64_t pitch, H, W; // (one pitch for both)
+  int32_t storage_in, storage_out;   // the same, or uint8 and one bit (C = 2, no frame)
   int32_t frame;       // ghost frame of a periodic grid (16 cells, filled), else 0
   RuleDev rule;
+  int32_t device, sms;
 };
+// Whether a step from and to storage_in is faster this way.
 bool planes_preferred(const PlanesGrid &g);
-// Warps of the grid's kernel that the GPU holds at once.
-cudaError_t planes_resident_warps(const PlanesGrid &g, int sms, int *warps);
-cudaError_t planes_launch(const PlanesGrid &g, int resident_warps, cudaStream_t s);
+cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s);
 
 }  // namespace cat

@@ -1,16 +1,46 @@
 // Host side of the bit-plane box-sum kernels (cat_planes.cuh): the kernel for
 // a storage and radius, and the split of a grid into strips.
+#include <atomic>
+
 #include "cat_planes.cuh"
 
 namespace cat {
 namespace {
 
-planes::Kernel find(const PlanesGrid &g) {
+// The kernel for a grid's storages, and which of them it is (kinds x radii).
+constexpr int kKinds = 6;
+planes::Kernel find(const PlanesGrid &g, int *kind) {
   const int r = g.rule.r;
-  if (g.rule.nbhd != 0 || r < 1 || r > 16 || g.rule.C > 16) return planes::Kernel{};
-  if (g.storage == CAT_STORE_BIT1) return g.rule.C == 2 ? planes::kernel_bit1(r) : planes::Kernel{};
-  if (g.storage == CAT_STORE_NIB4) return planes::kernel_nib4(r);
-  return g.rule.C > 2 ? planes::kernel_u8_ms(r) : planes::kernel_u8(r);
+  const bool from_u8 = g.storage_in == CAT_STORE_U8, to_u8 = g.storage_out == CAT_STORE_U8;
+  *kind = from_u8 && to_u8 ? (g.rule.C > 2 ? 1 : 0) : from_u8 ? 2 : to_u8 ? 3 : g.storage_in == CAT_STORE_BIT1 ? 4 : 5;
+  if (g.rule.nbhd != 0 || r < 1 || r > planes::kMaxR || g.rule.C > 16) return planes::Kernel{};
+  if (*kind >= 2 && *kind <= 4 && g.rule.C != 2) return planes::Kernel{};
+  switch (*kind) {
+    case 0: return planes::kernel_u8(r);
+    case 1: return planes::kernel_u8_ms(r);
+    case 2: return planes::kernel_u8_to_bit1(r);
+    case 3: return planes::kernel_bit1_to_u8(r);
+    case 4: return planes::kernel_bit1(r);
+    default: return planes::kernel_nib4(r);
+  }
+}
+
+// Warps of a kernel that the current device holds at once (looked up once per
+// device, kind and radius; the value is a property of the device, so threads
+// that race write the same).
+cudaError_t resident_warps(const planes::Kernel &k, int kind, int r, const PlanesGrid &g, int *warps) {
+  static std::atomic<int> seen[16][kKinds][planes::kMaxR + 1];
+  std::atomic<int> *slot = g.device >= 0 && g.device < 16 ? &seen[g.device][kind][r] : nullptr;
+  if (slot && (*warps = slot->load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  int per_sm = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, 32, k.smem);
+  if (e != cudaSuccess) return e;
+  *warps = per_sm * g.sms;
+  if (slot) slot->store(*warps, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 // A bound K of the rule as the words of a carry chain (planes::at_least), K
@@ -35,27 +65,19 @@ void set_bound(uint32_t *k, int64_t K, int planes) {
 //                         18.4 against 11.6 / 14.8 / 14.8; 16384^2, r = 4:
 //                         111 against 97
 bool planes_preferred(const PlanesGrid &g) {
-  if (!find(g).fn) return false;
-  if (g.storage != CAT_STORE_U8) return true;
+  int kind;
+  if (!find(g, &kind).fn) return false;
+  if (g.storage_in != CAT_STORE_U8) return true;
   if (g.rule.C > 2) return g.rule.r <= 15;
   return g.rule.r <= 9 && g.H * g.W <= (1 << 24);
 }
 
-cudaError_t planes_resident_warps(const PlanesGrid &g, int sms, int *warps) {
-  const planes::Kernel k = find(g);
+cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
+  int kind, resident;
+  const planes::Kernel k = find(g, &kind);
   if (!k.fn) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, 32, k.smem);
-  if (e == cudaSuccess) *warps = per_sm * sms;
-  return e;
-}
-
-cudaError_t planes_launch(const PlanesGrid &g, int resident_warps, cudaStream_t s) {
-  const planes::Kernel k = find(g);
-  if (!k.fn) return cudaErrorInvalidValue;
+  cudaError_t e = resident_warps(k, kind, g.rule.r, g, &resident);
+  if (e != cudaSuccess) return e;
   planes::Params p;
   p.in = g.in;
   p.out = g.out;
@@ -71,14 +93,14 @@ cudaError_t planes_launch(const PlanesGrid &g, int resident_warps, cudaStream_t 
   set_bound(p.bound[planes::kBirthLo], g.rule.b_lo, k.planes);
   set_bound(p.bound[planes::kBirthHi], (int64_t)g.rule.b_lo + g.rule.b_w + 1, k.planes);
   // as many strips as fill the GPU once
-  int64_t strips = (int64_t)resident_warps * k.out_words / p.seg;
+  int64_t strips = (int64_t)resident * planes::kOut / p.seg;
   if (strips < 1) strips = 1;
   int64_t rows = (g.H + strips - 1) / strips;
   rows = (rows + k.ahead - 1) / k.ahead * k.ahead;
   strips = (g.H + rows - 1) / rows;
   p.rows = (int32_t)rows;
   p.strips = (int32_t)strips;
-  const int64_t warps = (strips * p.seg + k.out_words - 1) / k.out_words;
+  const int64_t warps = (strips * p.seg + planes::kOut - 1) / planes::kOut;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -230,7 +230,7 @@ struct Params {
 };
 
 // What a warp holds and how far ahead it loads.
-template <int R, int ST, bool MS>
+template <int R, bool MS>
 struct Cfg {
   static constexpr int kSmem = 32 * Dim<R>::kThreadBytes;
   static constexpr int kBySmem = 232448 / (kSmem + 1024);
@@ -244,21 +244,26 @@ __device__ __forceinline__ const uint8_t *row_ptr(const uint8_t *base, uint32_t 
   return reinterpret_cast<const uint8_t *>(r);
 }
 
-// What a lane reads and writes in memory, a 16-cell half of a word (uint8) or a word.
-template <int ST>
-struct Access {
-  const uint8_t *src;   // row 0 of its strip's rows
-  uint8_t *dst;         // output row 0
-  int lo, hi;           // rows of src that exist
-  int rows;             // output rows written
-  int cells, out;       // uint8: cells of the 16 that are readable, that are the grid's
+// What a lane reads and writes in memory: a 16-cell half of a word (uint8) or a word.
+struct Source {
+  const uint8_t *base;   // row 0 of its strip's rows
+  int lo, hi;            // rows that exist
+  int cells;             // uint8: readable cells of the 16
+};
+struct Target {
+  const uint8_t *base;   // output row 0
+  int rows;              // rows written
+  int cells;             // uint8: cells of the 16 that are the grid's
 };
 
-template <int R, int ST, bool MS>
-__global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(const __grid_constant__ Params p) {
+// One step from storage SI to storage SO (the same one, or between uint8 and
+// one bit for two states).
+template <int R, int SI, int SO, bool MS>
+__global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __grid_constant__ Params p) {
   using D = Dim<R>;
   constexpr int NH = D::kH, NS = D::kS, NT = 32;
-  constexpr int B = Raw<ST>::kBytes, kParts = ST == CAT_STORE_U8 ? 2 : 1, A = Cfg<R, ST, MS>::kAhead;
+  constexpr int A = Cfg<R, MS>::kAhead;
+  constexpr int kParts = SI == CAT_STORE_U8 ? 2 : 1, kOutParts = SO == CAT_STORE_U8 ? 2 : 1;
   constexpr int kSlot = NT * 4 * NH, kRing = D::kWin * kSlot, kCentre = NT * 4 * R;
   extern __shared__ __align__(16) uint8_t smem[];
   uint8_t *const cring = smem + kRing;
@@ -278,7 +283,8 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
   const uint32_t mask = !held ? 0u : left >= 32 ? ~0u : (1u << (int)left) - 1u;
   const bool writes = held && lane >= 1 && lane <= kOut;
   const int my_rows = !writes ? 0 : p.H - y0 < p.rows ? (int)(p.H - y0) : p.rows;
-  const int64_t col = (int64_t)w * B - p.frame;   // (a frame comes with one byte per cell)
+  // bytes from cell 0 of a row (a frame comes with one byte per cell)
+  const int64_t col_in = (int64_t)w * Raw<SI>::kBytes - p.frame, col_out = (int64_t)w * Raw<SO>::kBytes - p.frame;
   // the strip's rows y0 - R + i, i in [0, 2 R + rows); those in [lo, hi) exist
   const int64_t ys = y0 - R;
   const int lo = ys < -p.frame ? (int)(-p.frame - ys) : 0;
@@ -288,45 +294,51 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
   // Memory accesses: one word per lane, or with one byte per cell two 16-cell
   // halves of words, so that a warp's access is contiguous: lane l takes half
   // l & 1 of the words of lanes l / 2 and 16 + l / 2.
-  Access<ST> acc[kParts];
+  Source from[kParts];
+  Target to[kOutParts];
 #pragma unroll
-  for (int t = 0; t < kParts; ++t) {
-    const int from = kParts == 1 ? lane : 16 * t + (lane >> 1), half = kParts == 1 ? 0 : lane & 1;
-    const int64_t x = __shfl_sync(kFull, x0, from) + 16 * half;
-    const int64_t y = __shfl_sync(kFull, y0, from), c = __shfl_sync(kFull, col, from) + 16 * half;
-    const int64_t readable = p.W + p.frame - x;
-    acc[t].cells = readable >= 16 ? 16 : readable <= 0 ? 0 : (int)readable;
-    // (a half without a cell reads the other half, and clears it)
-    acc[t].src = p.in + (y - R) * p.pitch + c - (ST == CAT_STORE_U8 && readable <= 0 ? 16 : 0);
-    acc[t].dst = p.out + y * p.pitch + c;
-    acc[t].lo = __shfl_sync(kFull, lo, from);
-    acc[t].hi = __shfl_sync(kFull, hi, from);
-    acc[t].rows = __shfl_sync(kFull, my_rows, from);
-    acc[t].out = p.W - x >= 16 ? 16 : (int)(p.W - x);
-    if (ST == CAT_STORE_U8 && (x < 0 || x >= p.W)) acc[t].rows = 0;
+  for (int t = 0; t < 2; ++t) {
+    if (t < kParts) {
+      const int of = kParts == 1 ? lane : 16 * t + (lane >> 1), half = kParts == 1 ? 0 : 16 * (lane & 1);
+      const int64_t y = __shfl_sync(kFull, y0, of), c = __shfl_sync(kFull, col_in, of) + half;
+      const int64_t readable = __shfl_sync(kFull, left, of) - half;
+      from[t].cells = readable >= 16 ? 16 : readable <= 0 ? 0 : (int)readable;
+      // (a half without a cell reads the other half, and clears it)
+      from[t].base = p.in + (y - R) * p.pitch + c - (readable <= 0 ? 16 : 0);
+      from[t].lo = __shfl_sync(kFull, lo, of);
+      from[t].hi = __shfl_sync(kFull, hi, of);
+    }
+    if (t < kOutParts) {
+      const int of = kOutParts == 1 ? lane : 16 * t + (lane >> 1), half = kOutParts == 1 ? 0 : 16 * (lane & 1);
+      const int64_t x = __shfl_sync(kFull, x0, of) + half, y = __shfl_sync(kFull, y0, of);
+      to[t].base = p.out + y * p.pitch + __shfl_sync(kFull, col_out, of) + half;
+      to[t].cells = p.W - x >= 16 ? 16 : (int)(p.W - x);
+      to[t].rows = __shfl_sync(kFull, my_rows, of);
+      if (SO == CAT_STORE_U8 && (x < 0 || x >= p.W)) to[t].rows = 0;
+    }
   }
-  bool odd_end = false;   // some access of the warp ends within its 16 cells
-  if (ST == CAT_STORE_U8)
-    odd_end = __any_sync(kFull, acc[0].cells < 16 || acc[kParts - 1].cells < 16 || acc[0].out < 16 || acc[kParts - 1].out < 16);
+  // some access of the warp ends within its 16 cells
+  const bool odd_in = SI == CAT_STORE_U8 && __any_sync(kFull, from[0].cells < 16 || from[kParts - 1].cells < 16);
+  const bool odd_out = SO == CAT_STORE_U8 && __any_sync(kFull, to[0].cells < 16 || to[kOutParts - 1].cells < 16);
 
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // uint8: bytes past the last readable cell belong to whoever owns the buffer
-  auto clear_past = [&](Raw<ST> &r) {
+  auto clear_past = [&](Raw<SI> &r) {
 #pragma unroll
-    for (int i = 0; i < Raw<ST>::kWords; ++i) {
-      const int cells = acc[i / 4 % kParts].cells - 4 * (i % 4);
+    for (int i = 0; i < Raw<SI>::kWords; ++i) {
+      const int cells = from[i / 4 % kParts].cells - 4 * (i % 4);
       r.v[i] &= cells >= 4 ? ~0u : cells <= 0 ? 0u : (1u << (8 * cells)) - 1u;
     }
   };
   // flags of a loaded row: uint8, the halves of a lane's word come from lanes
   // 2 l and 2 l + 1, their first accesses for lanes below 16, else their second
   const uint32_t halves = lane < 16 ? 0x5410u : 0x7632u;
-  auto flags_of = [&](Raw<ST> r, uint32_t valid) {
-    if (ST == CAT_STORE_U8 && odd_end) clear_past(r);
-    uint32_t f = flags<ST, MS>(r);
-    if constexpr (ST == CAT_STORE_U8)
+  auto flags_of = [&](Raw<SI> r, uint32_t valid) {
+    if (odd_in) clear_past(r);
+    uint32_t f = flags<SI, MS>(r);
+    if constexpr (SI == CAT_STORE_U8)
       f = __byte_perm(__shfl_sync(kFull, f, 2 * lane), __shfl_sync(kFull, f, 2 * lane + 1), halves);
     return f & valid;
   };
@@ -398,20 +410,20 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
     }
     if (cells & 1) *q = (uint8_t)a[0];
   };
-  auto put = [&](int j, uint32_t in, const Raw<ST> &cs) {   // output row j of the strip
+  auto put = [&](int j, uint32_t in, const Raw<SI> &cs) {   // output row j of the strip
     uint32_t lo4 = 0u, hi4 = 0u;
-    if constexpr (ST == CAT_STORE_U8) {
+    if constexpr (SO == CAT_STORE_U8) {
       in = split(in);
       lo4 = in & 0x0F0F0F0Fu;
       hi4 = (in >> 4) & 0x0F0F0F0Fu;
     }
 #pragma unroll
-    for (int t = 0; t < kParts; ++t) {
-      if (j >= acc[t].rows) continue;
-      uint8_t *const q = const_cast<uint8_t *>(row_ptr(acc[t].dst, (uint32_t)j, pitch));
-      if constexpr (ST == CAT_STORE_BIT1) {
+    for (int t = 0; t < kOutParts; ++t) {
+      if (j >= to[t].rows) continue;
+      uint8_t *const q = const_cast<uint8_t *>(row_ptr(to[t].base, (uint32_t)j, pitch));
+      if constexpr (SO == CAT_STORE_BIT1) {
         *reinterpret_cast<uint32_t *>(q) = in & mask;
-      } else if constexpr (ST == CAT_STORE_NIB4) {
+      } else if constexpr (SO == CAT_STORE_NIB4) {
         const uint32_t f = in & mask;
         uint4 a;
         a.x = age_nibbles(cs.v[0], spread_nibbles(byte_of<0>(f)), p.last, p.two);
@@ -432,8 +444,8 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
             a[2 * i + 1] = (r >> 4) & 0x0F0F0F0Fu;
           }
         }
-        if (!odd_end || acc[t].out == 16) *reinterpret_cast<uint4 *>(q) = make_uint4(a[0], a[1], a[2], a[3]);
-        else store_part(q, a, acc[t].out);
+        if (!odd_out || to[t].cells == 16) *reinterpret_cast<uint4 *>(q) = make_uint4(a[0], a[1], a[2], a[3]);
+        else store_part(q, a, to[t].cells);
       }
     }
   };
@@ -443,16 +455,16 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
   auto walk = [&](auto edge) {
     constexpr bool EDGE = decltype(edge)::value;
     auto valid_of = [&](int i) { return EDGE && (i < lo || i >= hi) ? 0u : mask; };
-    auto load = [&](Raw<ST> &r, int i) {   // row i of the strip's rows
+    auto load = [&](Raw<SI> &r, int i) {   // row i of the strip's rows
 #pragma unroll
       for (int t = 0; t < kParts; ++t) {
-        const int row = !EDGE ? i : i < acc[t].lo ? acc[t].lo : i >= acc[t].hi ? acc[t].hi - 1 : i;
-        const uint8_t *q = row_ptr(acc[t].src, (uint32_t)row, pitch);
-        if constexpr (ST == CAT_STORE_BIT1) r.v[0] = *reinterpret_cast<const uint32_t *>(q);
+        const int row = !EDGE ? i : i < from[t].lo ? from[t].lo : i >= from[t].hi ? from[t].hi - 1 : i;
+        const uint8_t *q = row_ptr(from[t].base, (uint32_t)row, pitch);
+        if constexpr (SI == CAT_STORE_BIT1) r.v[0] = *reinterpret_cast<const uint32_t *>(q);
         else ld16(r.v + 4 * t, q);
       }
     };
-    Raw<ST> raw[A], ctr[2];
+    Raw<SI> raw[A], ctr[2];
 #pragma unroll
     for (int k = 0; k < A; ++k) load(raw[k], k);
     if constexpr (MS) {   // centre rows, for their states
@@ -516,7 +528,7 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
         *q0 = c0;
         m1 = *q1;   // (the same word as q0 when R = 1)
         *q1 = c1;
-        if (MS && ST == CAT_STORE_U8 && odd_end) {
+        if (MS && odd_in) {
           clear_past(ctr[0]);
           clear_past(ctr[1]);
         }
@@ -541,23 +553,24 @@ __global__ void __launch_bounds__(32, Cfg<R, ST, MS>::kWarps) planes_kernel(cons
 // takes; nullptr when it is not built.
 struct Kernel {
   void (*fn)(Params) = nullptr;
-  int smem = 0, out_words = 0, ahead = 0, planes = 0;
+  int smem = 0, ahead = 0, planes = 0;
 };
-// r <= 16; uint8 with two states, and with 3 .. 16
+// r <= kMaxR; uint8 with two states and with 3 .. 16, from uint8 to one bit per
+// cell and back
 Kernel kernel_u8(int r);
 Kernel kernel_u8_ms(int r);
+Kernel kernel_u8_to_bit1(int r);
+Kernel kernel_bit1_to_u8(int r);
 Kernel kernel_bit1(int r);
 Kernel kernel_nib4(int r);
 
-template <int ST, bool MS, int LO, int HI>
+template <int SI, int SO, bool MS, int LO = 1>
 Kernel find_kernel(int r) {
-  if constexpr (LO > HI) {
+  if constexpr (LO > kMaxR) {
     return Kernel{};
   } else {
-    if (r == LO)
-      return Kernel{planes_kernel<LO, ST, MS>, Cfg<LO, ST, MS>::kSmem, kOut, Cfg<LO, ST, MS>::kAhead,
-                    Dim<LO>::kS};
-    return find_kernel<ST, MS, LO + 1, HI>(r);
+    if (r == LO) return Kernel{planes_kernel<LO, SI, SO, MS>, Cfg<LO, MS>::kSmem, Cfg<LO, MS>::kAhead, Dim<LO>::kS};
+    return find_kernel<SI, SO, MS, LO + 1>(r);
   }
 }
 

@@ -4,7 +4,7 @@
 namespace cat {
 namespace planes {
 
-Kernel kernel_bit1(int r) { return find_kernel<CAT_STORE_BIT1, false, 1, 16>(r); }
+Kernel kernel_bit1(int r) { return find_kernel<CAT_STORE_BIT1, CAT_STORE_BIT1, false>(r); }
 
 }  // namespace planes
 }  // namespace cat

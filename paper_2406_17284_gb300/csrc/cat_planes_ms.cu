@@ -4,7 +4,7 @@
 namespace cat {
 namespace planes {
 
-Kernel kernel_u8_ms(int r) { return find_kernel<CAT_STORE_U8, true, 1, 16>(r); }
+Kernel kernel_u8_ms(int r) { return find_kernel<CAT_STORE_U8, CAT_STORE_U8, true>(r); }
 
 }  // namespace planes
 }  // namespace cat

@@ -4,7 +4,7 @@
 namespace cat {
 namespace planes {
 
-Kernel kernel_nib4(int r) { return find_kernel<CAT_STORE_NIB4, true, 1, 16>(r); }
+Kernel kernel_nib4(int r) { return find_kernel<CAT_STORE_NIB4, CAT_STORE_NIB4, true>(r); }
 
 }  // namespace planes
 }  // namespace cat

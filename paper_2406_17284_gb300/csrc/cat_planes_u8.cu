@@ -4,7 +4,7 @@
 namespace cat {
 namespace planes {
 
-Kernel kernel_u8(int r) { return find_kernel<CAT_STORE_U8, false, 1, 16>(r); }
+Kernel kernel_u8(int r) { return find_kernel<CAT_STORE_U8, CAT_STORE_U8, false>(r); }
 
 }  // namespace planes
 }  // namespace cat

@@ -91,3 +91,29 @@ def test_bytes_past_the_grid_are_not_read_or_written(cat, C):
             g.close()
         assert np.array_equal(b[:, :W].cpu().numpy(), oracle.step(grid, oracle.Rule(**rule), n_steps=3))
         assert bool((a[:, W:] == 255).all()) and bool((b[:, W:] == 254).all())
+
+
+@pytest.mark.parametrize("r", [1, 4, 16])
+def test_packed_steps_between_uint8_states(cat, r):
+    """Several steps in one call keep the states between packed, inside the
+    grid's own rows: any number of steps, the state where the parity puts it,
+    no byte past W touched."""
+    import torch
+    rule = inputs.scaled_rule(r, M=1)
+    for H, W, pitch in [(40, 64, 64), (33, 97, 112), (130, 1031, 1056)]:
+        grid = board(H, W, 2, W + r)
+        for n in (2, 3, 4, 5, 9):
+            a = torch.full((H, pitch), 255, dtype=torch.uint8, device="cuda")
+            b = torch.full((H, pitch), 254, dtype=torch.uint8, device="cuda")
+            a[:, :W] = torch.from_numpy(grid).cuda()
+            g = cat.Grid(H, W, rule, kernel="auto", dtype="auto")
+            try:
+                cat.cat_bind(g.handle, a.data_ptr(), b.data_ptr(), pitch)
+                g.step(n)
+                torch.cuda.synchronize()
+                got = (b if n & 1 else a)[:, :W].cpu().numpy()
+                assert cat.cat_state_ptr(g.handle)[0] == (b if n & 1 else a).data_ptr()
+            finally:
+                g.close()
+            assert np.array_equal(got, oracle.step(grid, oracle.Rule(**rule), n_steps=n)), (H, W, r, n)
+            assert bool((a[:, W:] == 255).all()) and bool((b[:, W:] == 254).all())
