@@ -219,10 +219,14 @@ bool use_planes(const cat_instance *h) {
   return h->auto_choice && h->inject == 0 && cat::planes_preferred(planes_grid(h, 0));
 }
 
-int launch_planes(cat_instance *h, int in, cudaStream_t s) {
+// The first steps of n_steps from buffer `in` into the other one; *taken: how many.
+int launch_planes(cat_instance *h, int in, int64_t n_steps, int64_t *taken, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
+  const cat::PlanesGrid g = planes_grid(h, in);
+  const cat::TilePlan plan = cat::planes_tile_plan(g, n_steps);
+  *taken = plan.steps > 0 ? plan.steps : 1;
   if (h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
-  if (e == cudaSuccess) e = cat::planes_launch(planes_grid(h, in), s);
+  if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return CAT_OK;
 }
@@ -244,21 +248,31 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
   g.storage_out = CAT_STORE_BIT1;
   int at = 1 - h->cur;
   int64_t off = 0;
-  for (int64_t t = 0; t < n_steps; ++t) {
+  for (int64_t t = 0; t < n_steps;) {
     if (t > 0) {
       g.in = h->buf[at] + off;
       g.storage_in = CAT_STORE_BIT1;
-      if (t == n_steps - 1) {
-        g.out = h->buf[last];
-        g.storage_out = CAT_STORE_U8;
-      } else {   // stay out of the final states' buffer once the first states have been read
-        off = at == last ? 0 : off ? 0 : second;
-        at = 1 - last;
-        g.out = h->buf[at] + off;
-      }
     }
-    const cudaError_t e = cat::planes_launch(g, s);
+    // no launch writes the final states into the buffer that it reads: bits
+    // that lie there move over by one launch first
+    const bool here = last == (t == 0 ? h->cur : at);
+    cat::TilePlan plan = cat::planes_tile_plan(g, n_steps - t - (here ? 1 : 0));
+    int64_t k = plan.steps > 0 ? plan.steps : 1;
+    if (t == 0 && !here && t + k == n_steps - 1) {   // (which takes two more steps)
+      plan = cat::planes_tile_plan(g, k - 1);
+      k = plan.steps > 0 ? plan.steps : 1;
+    }
+    if (t + k == n_steps) {
+      g.out = h->buf[last];
+      g.storage_out = CAT_STORE_U8;
+    } else if (t > 0) {   // stay out of the final states' buffer once the first states have been read
+      off = at == last ? 0 : off ? 0 : second;
+      at = 1 - last;
+      g.out = h->buf[at] + off;
+    }
+    const cudaError_t e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+    t += k;
   }
   return CAT_OK;
 }
@@ -268,7 +282,10 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
 // cooperative launch of the tcgen05 Moore kernel (zero boundary).
 int launch_step(cat_instance *h, int in, int32_t *sums, int64_t sums_ld, cudaStream_t s, int n_steps = 1) {
   cudaError_t e;
-  if (!sums && n_steps == 1 && use_planes(h)) return launch_planes(h, in, s);
+  if (!sums && n_steps == 1 && use_planes(h)) {
+    int64_t taken;
+    return launch_planes(h, in, 1, &taken, s);
+  }
   if (h->kernel == CAT_KERNEL_TCGEN05) {
     if (h->ghost) {  // periodic: refresh the input's ghost frame first
       e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
@@ -332,10 +349,12 @@ int launch_step(cat_instance *h, int in, int32_t *sums, int64_t sums_ld, cudaStr
     p.rule = h->rd;
     p.sums = sums;
     p.sums_ld = sums_ld;
-    if (h->kernel == CAT_KERNEL_BITSLICE && n_steps > 1)   // temporal blocking: n_steps in one launch
-      e = cat::swar_tb_launch(h->buf[in], h->buf[1 - in], h->pitch, h->H, h->W, h->rd, n_steps, s);
+    if (h->kernel == CAT_KERNEL_BITSLICE && sums)
+      e = cat::swar_sums_launch(h->buf[in], h->pitch, h->H, h->W, h->rd, sums, sums_ld, s);
+    else if (h->kernel == CAT_KERNEL_BITSLICE && n_steps > 1)   // temporal blocking: n_steps in one launch
+      e = cat::planes_tile_launch(planes_grid(h, in), cat::planes_tile_fixed(planes_grid(h, in), n_steps), s);
     else if (h->kernel == CAT_KERNEL_BITSLICE)
-      e = cat::swar_launch(h->buf[in], h->buf[1 - in], h->pitch, h->H, h->W, h->rd, sums, sums_ld, s);
+      e = cat::planes_launch(planes_grid(h, in), s);
     else if (h->kernel == CAT_KERNEL_RUNSUM)
       e = cat::runsum_launch(p, s);
     else
@@ -873,6 +892,14 @@ int cat_step(cat_handle_t h, int64_t n_steps, void *stream) {
     return rc;
   }
   for (int64_t t = 0; t < n_steps;) {
+    if (h->storage == CAT_STORE_BIT1 && use_planes(h)) {   // library-owned buffers: the state moves with every launch
+      int64_t taken;
+      const int rc = launch_planes(h, h->cur, n_steps - t, &taken, (cudaStream_t)stream);
+      if (rc) return rc;
+      h->cur ^= 1;
+      t += taken;
+      continue;
+    }
     const int m = (int)std::min<int64_t>(h->steps_per_launch, n_steps - t);
     int rc = launch_step(h, h->cur, nullptr, 0, (cudaStream_t)stream, m);
     if (rc) return rc;

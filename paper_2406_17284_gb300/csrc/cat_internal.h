@@ -158,16 +158,10 @@ cudaError_t mma_launch(const SimpleParams &p, int dt, cudaStream_t s);
 // (cat_stencil.cu).
 cudaError_t stencil_launch(const SimpleParams &p, cudaStream_t s);
 cudaError_t runsum_launch(const SimpleParams &p, cudaStream_t s);
-// Bit-sliced CUDA-core step on one-bit storage, r <= 5 (cat_swar.cu): in/out
-// are packed rows at `pitch` bytes (a multiple of 4); sums: counts instead.
-cudaError_t swar_launch(const uint8_t *in, uint8_t *out, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule,
-                        int32_t *sums, int64_t sums_ld, cudaStream_t s);
-// The same rule, k steps per launch on tiles held in shared memory (temporal
-// blocking, a k r-cell stale halo; k r <= 8); reads `in`, writes the state
-// after k steps to `out`.
-cudaError_t swar_tb_launch(const uint8_t *in, uint8_t *out, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule,
-                           int k, cudaStream_t s);
-
+// Box counts of a one-bit grid, r <= 5, by bitwise adders (cat_swar.cu): `in`
+// holds packed rows at `pitch` bytes (a multiple of 4).
+cudaError_t swar_sums_launch(const uint8_t *in, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule, int32_t *sums,
+                             int64_t sums_ld, cudaStream_t s);
 // Box sums in bit planes on CUDA cores (cat_planes.cuh): one step of a grid.
 struct PlanesGrid {
   const uint8_t *in;   // grid cell (0, 0) of the input and output buffers
@@ -181,5 +175,14 @@ struct PlanesGrid {
 // Whether a step from and to storage_in is faster this way.
 bool planes_preferred(const PlanesGrid &g);
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s);
+// Several steps per launch on tiles in shared memory (cat_planes_tile.cuh; two
+// states): the split for a launch with n_left steps to go; steps = 0 where
+// planes_launch, step by step, is faster.
+struct TilePlan {
+  int32_t steps, rows;   // steps per launch, output rows per strip
+};
+TilePlan planes_tile_plan(const PlanesGrid &g, int64_t n_left);
+TilePlan planes_tile_fixed(const PlanesGrid &g, int steps);
+cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaStream_t s);
 
 }  // namespace cat

@@ -164,6 +164,26 @@ __device__ __forceinline__ void spread_bytes(uint32_t lo, uint32_t hi, uint32_t 
   o[3] = (byte_of<2 * T + 1>(hi) * 0x00204081u) & 0x01010101u;
 }
 
+// The first `cells` (< 16) of 16 bytes: those past W are not the grid's.
+__device__ __forceinline__ void store_part(uint8_t *q, uint32_t (&a)[4], int cells) {
+  if (cells & 8) {
+    *reinterpret_cast<uint2 *>(q) = make_uint2(a[0], a[1]);
+    q += 8;
+    a[0] = a[2]; a[1] = a[3];
+  }
+  if (cells & 4) {
+    *reinterpret_cast<uint32_t *>(q) = a[0];
+    q += 4;
+    a[0] = a[1];
+  }
+  if (cells & 2) {
+    *reinterpret_cast<uint16_t *>(q) = (uint16_t)a[0];
+    q += 2;
+    a[0] >>= 16;
+  }
+  if (cells & 1) *q = (uint8_t)a[0];
+}
+
 // Eight flags (a byte) -> eight nibbles 0/1, flag i in nibble i.
 __device__ __forceinline__ uint32_t spread_nibbles(uint32_t b) {
   uint32_t x = (b * 0x1001u) & 0x000F000Fu;
@@ -391,24 +411,6 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
   const uint32_t mine = lane & 1 ? 0x7632u : 0x5410u;
   auto split = [&](uint32_t in) {
     return __byte_perm(__shfl_sync(kFull, in, lane >> 1), __shfl_sync(kFull, in, 16 + (lane >> 1)), mine);
-  };
-  auto store_part = [&](uint8_t *q, uint32_t (&a)[4], int cells) {   // cells of 16: the bytes past W are not the grid's
-    if (cells & 8) {
-      *reinterpret_cast<uint2 *>(q) = make_uint2(a[0], a[1]);
-      q += 8;
-      a[0] = a[2]; a[1] = a[3];
-    }
-    if (cells & 4) {
-      *reinterpret_cast<uint32_t *>(q) = a[0];
-      q += 4;
-      a[0] = a[1];
-    }
-    if (cells & 2) {
-      *reinterpret_cast<uint16_t *>(q) = (uint16_t)a[0];
-      q += 2;
-      a[0] >>= 16;
-    }
-    if (cells & 1) *q = (uint8_t)a[0];
   };
   auto put = [&](int j, uint32_t in, const Raw<SI> &cs) {   // output row j of the strip
     uint32_t lo4 = 0u, hi4 = 0u;
