@@ -238,19 +238,23 @@ int launch_planes(cat_instance *h, int in, int64_t n_steps, int64_t *taken, cuda
 // outside the grid's rows are not touched).
 bool use_packed_steps(const cat_instance *h, int64_t n_steps) {
   return n_steps >= 2 && h->auto_choice && h->inject == 0 && h->storage == CAT_STORE_U8 && h->rule.C == 2 &&
-         h->rule.nbhd == 'M' && h->rule.r <= 16 && h->ghost == 0 && h->W >= 64;
+         h->rule.nbhd == 'M' && h->rule.r <= 16 && h->W >= 64;
 }
 
 int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
-  const int64_t second = round_up((h->W + 31) / 32 * 4, 16);   // byte offset of a row's second row of bits
+  // byte offset of a row's second row of bits
+  const int64_t second = round_up((h->W + 2 * h->ghost + 31) / 32 * 4, 16);
+  // row 0 of a buffer's bits (on a torus they start at the frame's first cell)
+  auto bits = [&](int b, int64_t off) { return h->buf[b] + h->ghost * h->pitch + off; };
   const int last = h->cur ^ (int)(n_steps & 1);                // the buffer the final states go to
   cat::PlanesGrid g = planes_grid(h, h->cur);                  // first step: bits into the other buffer
   g.storage_out = CAT_STORE_BIT1;
+  g.out = bits(1 - h->cur, 0);
   int at = 1 - h->cur;
   int64_t off = 0;
   for (int64_t t = 0; t < n_steps;) {
     if (t > 0) {
-      g.in = h->buf[at] + off;
+      g.in = bits(at, off);
       g.storage_in = CAT_STORE_BIT1;
     }
     // no launch writes the final states into the buffer that it reads: bits
@@ -262,15 +266,19 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
       plan = cat::planes_tile_plan(g, k - 1);
       k = plan.steps > 0 ? plan.steps : 1;
     }
+    cudaError_t e = cudaSuccess;
+    if (h->ghost)
+      e = t == 0 ? cat::ghost_fill_launch(h->buf[h->cur], h->pitch, h->H, h->W, h->ghost, s)
+                 : cat::ghost_bits_launch(bits(at, off), h->pitch, h->H, h->W, s);
     if (t + k == n_steps) {
-      g.out = h->buf[last];
+      g.out = h->origin(last);
       g.storage_out = CAT_STORE_U8;
     } else if (t > 0) {   // stay out of the final states' buffer once the first states have been read
       off = at == last ? 0 : off ? 0 : second;
       at = 1 - last;
-      g.out = h->buf[at] + off;
+      g.out = bits(at, off);
     }
-    const cudaError_t e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
+    if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     t += k;
   }

@@ -71,7 +71,55 @@ __global__ void ghost_fill_kernel(uint8_t *base, int64_t pitch, int H, int W, in
   }
 }
 
+// The ghost frame of a one-bit grid (the states between the steps of one call):
+// position p of a row holds cell p - 16, so the grid's cells start in the middle
+// of word 0 and the frame's right cells end the row.  Items: the frame cells
+// beside each grid row (two 16-bit fields, one thread per row), and the words
+// of the 32 frame rows, each made from its source row's grid cells only.
+__global__ void ghost_bits_kernel(uint32_t *base, int64_t pitch_words, int H, int W, int words) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int wl = W / 32, sl = W % 32;                  // cells W - 16 .. W - 1 start here
+  const int wr = (W + 16) / 32, sr = (W + 16) % 32;    // cells W .. W + 15 start here
+  const int64_t n_all = H + 32 * (int64_t)words;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_all; i += (int64_t)gridDim.x * blockDim.x) {
+    const bool beside = i < H;
+    const int k = beside ? 0 : (int)((i - H) / words), w = beside ? 0 : (int)(i - H - (int64_t)k * words);
+    const int row = beside ? (int)i : k < 16 ? k - 16 : H + k - 16;
+    const uint32_t *src = base + (int64_t)wrap32(row, H) * pitch_words;
+    const uint32_t first = src[0];
+    const uint32_t left = __funnelshift_r(src[wl], src[wl + 1], sl) & 0xFFFFu, right = first >> 16;
+    const uint32_t low = (1u << sr) - 1u;              // the grid's cells of word wr
+    const uint32_t w0 = (first & 0xFFFF0000u) | left, w1 = (src[wr] & low) | (right << sr);
+    const uint32_t w2 = sr > 16 ? right >> (32 - sr) : 0u;
+    uint32_t *dst = base + (int64_t)row * pitch_words;
+    if (beside) {
+      dst[0] = w0;
+      dst[wr] = w1;
+      if (wr + 1 < words) dst[wr + 1] = w2;
+    } else {
+      dst[w] = w == 0 ? w0 : w == wr ? w1 : w == wr + 1 ? w2 : src[w];
+    }
+  }
+}
+
 }  // namespace
+
+cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W, cudaStream_t s) {
+  const int words = (int)((W + 32 + 31) / 32), threads = 256;
+  const int64_t want = (H + 32 * (int64_t)words + threads - 1) / threads;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(want < 4096 ? want : 4096));
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, ghost_bits_kernel, reinterpret_cast<uint32_t *>(row0), pitch / 4, (int)H, (int)W,
+                            words);
+}
 
 // Launched programmatically dependent on the previous kernel in the stream
 // (see ghost_fill_kernel); the tcgen05 step launched after it is in turn

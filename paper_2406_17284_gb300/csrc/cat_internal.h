@@ -151,6 +151,9 @@ cudaError_t unpack_nib_launch(const uint8_t *src, int64_t spitch, uint8_t *dst, 
 // H x W grid whose cell (0, 0) is at base + G * pitch + G with the cells the
 // frame wraps to.
 cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, cudaStream_t s);
+// The same for a one-bit grid whose rows start at cell -16 (G = 16; W >= 64);
+// row0: row 0 of the grid.
+cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W, cudaStream_t s);
 
 // Paper-style fragment kernels (cat_mma.cu).  dt: FP16 or INT8.
 cudaError_t mma_launch(const SimpleParams &p, int dt, cudaStream_t s);
@@ -164,10 +167,10 @@ cudaError_t swar_sums_launch(const uint8_t *in, int64_t pitch, int64_t H, int64_
                              int64_t sums_ld, cudaStream_t s);
 // Box sums in bit planes on CUDA cores (cat_planes.cuh): one step of a grid.
 struct PlanesGrid {
-  const uint8_t *in;   // grid cell (0, 0) of the input and output buffers
+  const uint8_t *in;   // row 0 of the input and output: grid cell 0 for uint8, cell -frame for packed rows
   uint8_t *out;
   int64_t pitch, H, W; // (one pitch for both)
-  int32_t storage_in, storage_out;   // the same, or uint8 and one bit (C = 2, no frame)
+  int32_t storage_in, storage_out;   // the same, or uint8 and one bit (C = 2)
   int32_t frame;       // ghost frame of a periodic grid (16 cells, filled), else 0
   RuleDev rule;
   int32_t device, sms;

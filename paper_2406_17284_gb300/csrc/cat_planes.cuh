@@ -236,7 +236,7 @@ constexpr int kMaxS = bits_for((2 * kMaxR + 1) * (2 * kMaxR + 1));
 enum { kSurviveLo, kSurviveHi, kBirthLo, kBirthHi };   // in range: >= lo and not >= hi
 
 struct Params {
-  const uint8_t *in;   // grid cell (0, 0)
+  const uint8_t *in;   // row 0: cell 0 of the grid for uint8, cell -frame for packed rows
   uint8_t *out;
   int64_t pitch;
   int32_t H, W;
@@ -303,8 +303,9 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
   const uint32_t mask = !held ? 0u : left >= 32 ? ~0u : (1u << (int)left) - 1u;
   const bool writes = held && lane >= 1 && lane <= kOut;
   const int my_rows = !writes ? 0 : p.H - y0 < p.rows ? (int)(p.H - y0) : p.rows;
-  // bytes from cell 0 of a row (a frame comes with one byte per cell)
-  const int64_t col_in = (int64_t)w * Raw<SI>::kBytes - p.frame, col_out = (int64_t)w * Raw<SO>::kBytes - p.frame;
+  // bytes from the row's start: cell 0 of the grid for uint8, cell -frame for packed rows
+  const int64_t col_in = (int64_t)w * Raw<SI>::kBytes - (SI == CAT_STORE_U8 ? p.frame : 0);
+  const int64_t col_out = (int64_t)w * Raw<SO>::kBytes - (SO == CAT_STORE_U8 ? p.frame : 0);
   // the strip's rows y0 - R + i, i in [0, 2 R + rows); those in [lo, hi) exist
   const int64_t ys = y0 - R;
   const int lo = ys < -p.frame ? (int)(-p.frame - ys) : 0;

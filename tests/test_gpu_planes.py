@@ -72,6 +72,14 @@ def test_planes_on_a_torus(cat, C):
             check(cat, H, W, inputs.scaled_rule(r, C=C), 0, boundary=1)
 
 
+@pytest.mark.parametrize("r", [1, 7, 16])
+def test_packed_steps_on_a_torus(cat, r):
+    """Several steps in one call: the one-bit ghost frame at every word offset of W."""
+    for H, W in [(5, 64), (20, 79), (33, 80), (40, 81), (64, 95), (70, 96), (33, 1031)]:
+        for n in (2, 3, 6):
+            check(cat, H, W, inputs.scaled_rule(r, M=1), 0, boundary=1, steps=n)
+
+
 @pytest.mark.parametrize("C", [2, 16])
 def test_bytes_past_the_grid_are_not_read_or_written(cat, C):
     """Bound buffers with a pitch above W, the gap full of other data."""
