@@ -199,8 +199,8 @@ CAT_API int cat_create_ex(int64_t H, int64_t W, const cat_rule_t *rule, int32_t 
  * AUTO, one step per launch and no cat_set_tile (also the state after
  * cat_create) every option is left to the library: cat_step then advances the
  * grid by box sums in bit planes on CUDA cores where that is faster (packed
- * storage, 3 to 16 states, small grids; Moore, r <= 16), with the same next
- * states, and cat_get_options reports the configuration that serves the other
+ * storage, 3 to 16 states, small grids, several steps of a two-state grid in
+ * one call; Moore, r <= 16), with the same next states, and cat_get_options reports the configuration that serves the other
  * grids and cat_box_sums.  A change
  * of storage reallocates both buffers and converts the current grid (the
  * device is synchronised; earlier cat_state_ptr addresses become invalid).
@@ -315,8 +315,9 @@ CAT_API int cat_state_ptr(cat_handle_t h, void **dptr, int64_t *pitch);
  * is taken from a as it is (no copy); after a step the state is in b, then a
  * again, as cat_state_ptr reports.  The instance's own buffers are freed; the
  * library never frees bound ones (cat_destroy leaves them to the caller, who
- * must keep them alive while the instance uses them).  Synchronises the
- * device.  Zero boundary and uint8 storage only (UNSUPPORTED otherwise, and
+ * must keep them alive while the instance uses them).  Of the two buffers,
+ * the one that does not hold the state is the library's to work in.
+ * Synchronises the device.  Zero boundary and uint8 storage only (UNSUPPORTED otherwise, and
  * for a later change to one-bit storage).  Errors: INVALID_ARG, UNSUPPORTED,
  * CUDA.                                                                     */
 CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
@@ -324,7 +325,8 @@ CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
 /* Advances the instance by n_steps >= 0 synchronous LTL steps on `stream`:
  * the host loop of Sec. IV-C (Alg. 1), one launch reading buffer A and
  * writing buffer B, then the two swap (with steps_per_launch = k > 1, k steps
- * per launch, the swap inside it).  Each step computes the band products of
+ * per launch, the swap inside it).  The buffer that does not hold the state
+ * afterwards has no defined contents.  Each step computes the band products of
  * Sec. IV (Eqs. 1-2) and the rule of Sec. V-A for every cell.  Errors:
  * INVALID_ARG (NULL, n_steps < 0), CUDA (launch failure); device-side
  * timeouts are reported by cat_status.                                     */
@@ -336,7 +338,9 @@ CAT_API int cat_step(cat_handle_t h, int64_t n_steps, void *stream);
  * boundary and uint8 storage, and share the dtype, each step is ONE
  * persistent launch over a flat tile work-list of all instances, and when
  * `stream` is not capturing the n_steps launches are replayed from a CUDA
- * graph cached for this handle list; otherwise every instance is stepped by
+ * graph cached for this handle list (with every instance's options left to the
+ * library, n_steps >= 4 and 2^25 cells or more, that graph packs the two-state
+ * grids, steps them on bit planes and unpacks them); otherwise every instance is stepped by
  * its own launches, one step at a time.  Errors: INVALID_ARG (NULL or
  * repeated handles, instances on different devices, mixed dtypes in a
  * batched launch), UNSUPPORTED (a batched instance above 4194176 cells per

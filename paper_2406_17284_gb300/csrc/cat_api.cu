@@ -241,9 +241,11 @@ bool use_packed_steps(const cat_instance *h, int64_t n_steps) {
          h->rule.nbhd == 'M' && h->rule.r <= 16 && h->W >= 64;
 }
 
+// Byte offset of a row's second row of bits.
+int64_t packed_second(const cat_instance *h) { return round_up((h->W + 2 * h->ghost + 31) / 32 * 4, 16); }
+
 int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
-  // byte offset of a row's second row of bits
-  const int64_t second = round_up((h->W + 2 * h->ghost + 31) / 32 * 4, 16);
+  const int64_t second = packed_second(h);
   // row 0 of a buffer's bits (on a torus they start at the frame's first cell)
   auto bits = [&](int b, int64_t off) { return h->buf[b] + h->ghost * h->pitch + off; };
   const int last = h->cur ^ (int)(n_steps & 1);                // the buffer the final states go to
@@ -382,11 +384,12 @@ struct BatchPlan {
   int32_t dtype = 0;
   bool encode = false;
   bool sw = false;            // every instance qualifies for the short-window kernel
+  cat::PlanesBatch *packed = nullptr;   // tables for calls on bit planes, made by the first such call
   cat::BatchInst *d_inst = nullptr;
   cat::BatchTile *d_tiles = nullptr;
   int n_tiles = 0, grid = 0;
-  cudaGraphExec_t exec[2] = {nullptr, nullptr};  // by start parity
-  int64_t exec_steps[2] = {0, 0};
+  cudaGraphExec_t exec[4] = {};   // by start parity, the calls on bit planes after the others
+  int64_t exec_steps[4] = {};
   cudaStream_t capture_stream = nullptr;
 };
 
@@ -394,11 +397,12 @@ std::mutex g_plan_mu;
 std::vector<BatchPlan *> g_plans;
 
 void free_plan(BatchPlan *pl) {
-  for (int i = 0; i < 2; ++i)
-    if (pl->exec[i]) cudaGraphExecDestroy(pl->exec[i]);
+  for (cudaGraphExec_t x : pl->exec)
+    if (x) cudaGraphExecDestroy(x);
   if (pl->capture_stream) cudaStreamDestroy(pl->capture_stream);
   cudaFree(pl->d_inst);
   cudaFree(pl->d_tiles);
+  cat::planes_batch_free(pl->packed);
   delete pl;
 }
 
@@ -414,12 +418,30 @@ void drop_plans_with(cat_instance *h) {
   }
 }
 
+std::vector<cat::PlanesBatchItem> batch_items(const BatchPlan *pl) {
+  std::vector<cat::PlanesBatchItem> items;
+  for (size_t i = 0; i < pl->hs.size(); ++i) {
+    const cat_instance *h = pl->hs[i];
+    items.push_back(cat::PlanesBatchItem{{h->buf[0], h->buf[1]}, h->pitch, h->H, h->W, pl->cur0[i],
+                                         (int32_t)packed_second(h), h->rd});
+  }
+  return items;
+}
+
 // (Re)writes the instance table of a plan from the handles' current state.
 int upload_instances(BatchPlan *pl) {
   CAT_CUDA(cudaDeviceSynchronize());  // earlier launches of this plan may still read the table
+  pl->steps_done = 0;
+  for (int i = 0; i < 4; ++i) {
+    if (pl->exec[i]) cudaGraphExecDestroy(pl->exec[i]);
+    pl->exec[i] = nullptr;
+    pl->exec_steps[i] = 0;
+  }
+  pl->cur0.resize(pl->hs.size());
+  for (size_t i = 0; i < pl->hs.size(); ++i) pl->cur0[i] = pl->hs[i]->cur;
+  if (pl->packed) CAT_CUDA(cat::planes_batch_update(pl->packed, batch_items(pl)));
   std::vector<cat::BatchInst> inst(pl->hs.size());
   memset(inst.data(), 0, inst.size() * sizeof(cat::BatchInst));
-  pl->cur0.resize(pl->hs.size());
   for (size_t i = 0; i < pl->hs.size(); ++i) {
     const cat_instance *h = pl->hs[i];
     for (int b = 0; b < 2; ++b) {
@@ -432,15 +454,8 @@ int upload_instances(BatchPlan *pl) {
     inst[i].W = (int32_t)h->W;
     inst[i].cur = h->cur;
     inst[i].err = h->d_err;
-    pl->cur0[i] = h->cur;
   }
   CAT_CUDA(cudaMemcpy(pl->d_inst, inst.data(), inst.size() * sizeof(cat::BatchInst), cudaMemcpyHostToDevice));
-  pl->steps_done = 0;
-  for (int i = 0; i < 2; ++i) {
-    if (pl->exec[i]) cudaGraphExecDestroy(pl->exec[i]);
-    pl->exec[i] = nullptr;
-    pl->exec_steps[i] = 0;
-  }
   return CAT_OK;
 }
 
@@ -919,30 +934,62 @@ int cat_step(cat_handle_t h, int64_t n_steps, void *stream) {
   return CAT_OK;
 }
 
-int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void *stream) {
+int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void *stream) try {
   if (!hs || count < 0 || n_steps < 0) return fail(CAT_ERR_INVALID_ARG, "bad batch arguments");
-  for (int32_t i = 0; i < count; ++i) {
+  for (int32_t i = 0; i < count; ++i)
     if (!hs[i]) return fail(CAT_ERR_INVALID_ARG, "instance %d is NULL", i);
-    for (int32_t k = 0; k < i; ++k)
-      if (hs[k] == hs[i]) return fail(CAT_ERR_INVALID_ARG, "instance %d appears twice", i);
-  }
-  if (count == 0 || n_steps == 0) return CAT_OK;
+  if (count == 0) return CAT_OK;
   cudaStream_t s = (cudaStream_t)stream;
+  // One pass over the instances (thousands, in no order in memory).
   bool all_tc = true;   // Moore, zero boundary, uint8 storage, no FP4: other instances step one by one
+  // Several steps of grids whose options are all left to the library, on bit
+  // planes: from four steps and 2^25 cells on (512 grids with sides up to 512 /
+  // 1024 / 2048, us for 4 steps: tiles 125 / 206 / 432, planes 128 / 199 / 406;
+  // for 16 steps: 475 / 799 / 1698 against 426 / 582 / 1227; 100 grids up to
+  // 1024: 80 against 110).  A captured call keeps to the tiles, one launch per
+  // step, since the planes need the radii side by side.
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CAT_CUDA(cudaStreamIsCapturing(s, &cs));
+  bool packed = n_steps >= 4 && cs == cudaStreamCaptureStatusNone;
+  int64_t cells = 0;
+  bool one_device = true, one_dtype = true, small = true;
   for (int32_t i = 0; i < count; ++i) {
-    all_tc &= hs[i]->kernel == CAT_KERNEL_TCGEN05 && hs[i]->ghost == 0 && hs[i]->storage == CAT_STORE_U8 &&
-              hs[i]->rule.nbhd == 'M' && !wide_tile(hs[i]) && hs[i]->dtype != CAT_DTYPE_FP4_E2M1;
-    if (hs[i]->dev.id != hs[0]->dev.id) return fail(CAT_ERR_INVALID_ARG, "instances of a batch must share the device");
+    const cat_instance *h = hs[i];
+    all_tc &= h->kernel == CAT_KERNEL_TCGEN05 && h->ghost == 0 && h->storage == CAT_STORE_U8 &&
+              h->rule.nbhd == 'M' && !wide_tile(h) && h->dtype != CAT_DTYPE_FP4_E2M1;
+    packed &= use_packed_steps(h, n_steps);
+    cells += h->H * h->W;
+    one_device &= h->dev.id == hs[0]->dev.id;
+    one_dtype &= h->dtype == hs[0]->dtype;
+    small &= h->H <= 128 * 32767 && h->W <= 128 * 32767;
   }
-  if (all_tc) {   // one persistent launch over every instance: one kernel instantiation
-    for (int32_t i = 0; i < count; ++i) {
-      if (hs[i]->dtype != hs[0]->dtype)
-        return fail(CAT_ERR_INVALID_ARG, "instances of a batched tcgen05 launch must share the dtype");
-      if (hs[i]->H > 128 * 32767 || hs[i]->W > 128 * 32767)
-        return fail(CAT_ERR_UNSUPPORTED, "batched instances are limited to 4194176 x 4194176 cells");
+  packed &= cells >= 1 << 25;
+  std::unique_lock<std::mutex> lk(g_plan_mu);
+  BatchPlan *pl = nullptr;
+  for (BatchPlan *c : g_plans)
+    if (all_tc && (int32_t)c->hs.size() == count && std::equal(c->hs.begin(), c->hs.end(), hs) &&
+        c->dtype == hs[0]->dtype) {
+      pl = c;
+      break;
+    }
+  if (!pl) {   // (a plan's handles are distinct)
+    std::vector<cat_handle_t> sorted(hs, hs + count);
+    std::sort(sorted.begin(), sorted.end());
+    const auto twice = std::adjacent_find(sorted.begin(), sorted.end());
+    if (twice != sorted.end()) {
+      const auto first = std::find(hs, hs + count, *twice);
+      return fail(CAT_ERR_INVALID_ARG, "instance %d appears twice", (int)(std::find(first + 1, hs + count, *twice) - hs));
     }
   }
+  if (n_steps == 0) return CAT_OK;
+  if (!one_device) return fail(CAT_ERR_INVALID_ARG, "instances of a batch must share the device");
+  if (all_tc) {   // one persistent launch over every instance: one kernel instantiation
+    if (!one_dtype)
+      return fail(CAT_ERR_INVALID_ARG, "instances of a batched tcgen05 launch must share the dtype");
+    if (!small) return fail(CAT_ERR_UNSUPPORTED, "batched instances are limited to 4194176 x 4194176 cells");
+  }
   if (!all_tc) {  // the comparator kernels have no batched launch: one launch per instance and step
+    lk.unlock();
     for (int64_t t = 0; t < n_steps; ++t)
       for (int32_t i = 0; i < count; ++i) {
         int rc = launch_step(hs[i], hs[i]->cur, nullptr, 0, s);
@@ -951,13 +998,6 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
       }
     return CAT_OK;
   }
-  std::lock_guard<std::mutex> lk(g_plan_mu);
-  BatchPlan *pl = nullptr;
-  for (BatchPlan *c : g_plans)
-    if ((int32_t)c->hs.size() == count && std::equal(c->hs.begin(), c->hs.end(), hs) && c->dtype == hs[0]->dtype) {
-      pl = c;
-      break;
-    }
   int rc;
   if (!pl) {
     if ((rc = build_plan(hs, count, &pl))) return rc;
@@ -966,31 +1006,46 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   bool in_sync = true;
   for (int32_t i = 0; i < count; ++i) in_sync &= hs[i]->cur == (pl->cur0[i] ^ (int)(pl->steps_done & 1));
   if (!in_sync && (rc = upload_instances(pl))) return rc;
-  const int par = (int)(pl->steps_done & 1);
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  CAT_CUDA(cudaStreamIsCapturing(s, &cs));
+  const int par = (int)(pl->steps_done & 1), kind = par + (packed ? 2 : 0);
+  if (packed && !pl->packed) {
+    const cudaError_t e = cat::planes_batch_create(batch_items(pl), hs[0]->dev.sms, &pl->packed);
+    if (e != cudaSuccess) {
+      (void)cudaGetLastError();
+      return e == cudaErrorMemoryAllocation ? fail(CAT_ERR_OOM, "allocation of the batch tables failed")
+                                            : cuda_fail(e, "batch plan");
+    }
+  }
   if (cs != cudaStreamCaptureStatusNone) {
     if ((rc = launch_batch_steps(pl, n_steps, pl->steps_done, s))) return rc;
   } else {
-    if (!pl->exec[par] || pl->exec_steps[par] != n_steps) {
-      if (pl->exec[par]) cudaGraphExecDestroy(pl->exec[par]);
-      pl->exec[par] = nullptr;
+    if (!pl->exec[kind] || pl->exec_steps[kind] != n_steps) {
+      if (pl->exec[kind]) cudaGraphExecDestroy(pl->exec[kind]);
+      pl->exec[kind] = nullptr;
       cudaGraph_t g = nullptr;
-      CAT_CUDA(cudaStreamBeginCapture(pl->capture_stream, cudaStreamCaptureModeThreadLocal));
-      rc = launch_batch_steps(pl, n_steps, pl->steps_done, pl->capture_stream);
-      cudaError_t e = cudaStreamEndCapture(pl->capture_stream, &g);
-      if (rc) { if (g) cudaGraphDestroy(g); return rc; }
-      if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-      e = cudaGraphInstantiate(&pl->exec[par], g, 0);
+      cudaError_t e;
+      if (packed) {
+        CAT_CUDA(cudaGraphCreate(&g, 0));
+        e = cat::planes_batch_add(pl->packed, n_steps, par, g);
+        if (e != cudaSuccess) { cudaGraphDestroy(g); return cuda_fail(e, "cudaGraphAddKernelNode"); }
+      } else {
+        CAT_CUDA(cudaStreamBeginCapture(pl->capture_stream, cudaStreamCaptureModeThreadLocal));
+        rc = launch_batch_steps(pl, n_steps, pl->steps_done, pl->capture_stream);
+        e = cudaStreamEndCapture(pl->capture_stream, &g);
+        if (rc) { if (g) cudaGraphDestroy(g); return rc; }
+        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+      }
+      e = cudaGraphInstantiate(&pl->exec[kind], g, 0);
       cudaGraphDestroy(g);
       if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-      pl->exec_steps[par] = n_steps;
+      pl->exec_steps[kind] = n_steps;
     }
-    CAT_CUDA(cudaGraphLaunch(pl->exec[par], s));
+    CAT_CUDA(cudaGraphLaunch(pl->exec[kind], s));
   }
   pl->steps_done += n_steps;
   for (int32_t i = 0; i < count; ++i) hs[i]->cur ^= (int)(n_steps & 1);
   return CAT_OK;
+} catch (const std::bad_alloc &) {
+  return fail(CAT_ERR_OOM, "host allocation failed");
 }
 
 int cat_box_sums(cat_handle_t h, int32_t *dst, int64_t ld, void *stream) {

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "../../include/cat.h"
 
@@ -187,5 +188,22 @@ struct TilePlan {
 TilePlan planes_tile_plan(const PlanesGrid &g, int64_t n_left);
 TilePlan planes_tile_fixed(const PlanesGrid &g, int steps);
 cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaStream_t s);
+// Two-state uint8 grids of any sizes, radii (<= 16) and rules, advanced several
+// steps per call on states packed to bits.  `buf` holds the states in buf[cur]; after n steps they are in
+// buf[cur ^ (n & 1)].
+struct PlanesBatchItem {
+  uint8_t *buf[2];
+  int64_t pitch, H, W;
+  int32_t cur, second;   // second: byte offset of a row's second row of bits
+  RuleDev rule;
+};
+struct PlanesBatch;   // descriptor tables on the device
+cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int sms, PlanesBatch **out);
+// The current buffers of the items again (the device is idle).
+cudaError_t planes_batch_update(PlanesBatch *b, const std::vector<PlanesBatchItem> &items);
+void planes_batch_free(PlanesBatch *b);
+// n_steps >= 2 steps as nodes of a graph (three ranges of radii side by side);
+// flip: the parity of the steps since the table was made.
+cudaError_t planes_batch_add(const PlanesBatch *b, int64_t n_steps, int flip, cudaGraph_t graph);
 
 }  // namespace cat

@@ -2,6 +2,8 @@
 // a storage and radius, and the split of a grid into strips.
 #include <algorithm>
 #include <atomic>
+#include <new>
+#include <vector>
 
 #include "cat_planes_tile.cuh"
 
@@ -59,7 +61,7 @@ planes::Params make_params(const PlanesGrid &g, int planes) {
   p.out = g.out;
   p.pitch = g.pitch;
   p.H = (int32_t)g.H;
-  p.W = (int32_t)g.W;
+  p.W = p.written = (int32_t)g.W;
   p.frame = g.frame;
   p.seg = (int32_t)((g.W + 2 * g.frame + 31) / 32) + 1;
   p.rows = p.strips = 0;
@@ -191,6 +193,152 @@ cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaSt
   if (e != cudaSuccess) return e;
   const int64_t blocks = ((int64_t)t.p.strips * t.p.seg + planes::kOut - 1) / planes::kOut;
   return launch(k.fn, t, blocks, 32 * planes::kTileWarps, (int)smem, s);
+}
+
+struct PlanesBatch {
+  struct Chain {
+    int range;                            // of radii (planes::kRangeEnd)
+    int smem;                             // of the largest radius
+    unsigned blocks;                      // blocks of one launch (planes::kBatchWarps warps each)
+    const planes::BatchBlock *first;
+  };
+  std::vector<Chain> chains;
+  unsigned pack_blocks = 0;               // blocks that pack or unpack all grids
+  const planes::BatchBlock *pack_first = nullptr;
+  std::vector<planes::BatchGrid> grids;
+  planes::BatchGrid *d_grids = nullptr;
+  planes::BatchBlock *d_blocks = nullptr;
+};
+
+namespace {
+
+// Rows per strip of a batch: about this many warps per SM over all grids, so
+// that the 2r rows before a strip's first output row stay a small part (512
+// uneven grids: 32 / 48 / 64 / 96 rows: 467 / 465 / 466 / 518 us).
+constexpr int kBatchFill = 24;
+
+planes::BatchParams batch_params(const PlanesBatch *b, const planes::BatchBlock *first, int64_t step, int64_t steps,
+                                 int flip) {
+  return planes::BatchParams{b->d_grids, first, flip, (int32_t)step, (int32_t)steps};
+}
+
+}  // namespace
+
+cudaError_t planes_batch_update(PlanesBatch *b, const std::vector<PlanesBatchItem> &items) {
+  for (size_t i = 0; i < items.size(); ++i) {
+    b->grids[i].buf[0] = items[i].buf[0];
+    b->grids[i].buf[1] = items[i].buf[1];
+    b->grids[i].cur = items[i].cur;
+  }
+  return cudaMemcpy(b->d_grids, b->grids.data(), sizeof(planes::BatchGrid) * b->grids.size(), cudaMemcpyHostToDevice);
+}
+
+cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int sms, PlanesBatch **out) {
+  PlanesBatch *b = new (std::nothrow) PlanesBatch();
+  if (!b) return cudaErrorMemoryAllocation;
+  double warp_rows = 0;
+  for (const PlanesBatchItem &q : items) warp_rows += (double)q.H * ((q.W + 31) / 32 + 1) / planes::kOut;
+  const int64_t rows = std::max<int64_t>(32, std::min<int64_t>(512, (int64_t)(warp_rows / (kBatchFill * sms)) / 4 * 4));
+  b->grids.resize(items.size());
+  for (size_t i = 0; i < items.size(); ++i) {
+    const PlanesBatchItem &q = items[i];
+    planes::BatchGrid &g = b->grids[i];
+    g = planes::BatchGrid{};
+    g.pitch = q.pitch;
+    g.H = (int32_t)q.H;
+    g.W = (int32_t)q.W;
+    g.seg = (int32_t)((q.W + 31) / 32) + 1;
+    g.rows = (int32_t)std::min<int64_t>(rows, (q.H + 3) / 4 * 4);
+    g.strips = (int32_t)((q.H + g.rows - 1) / g.rows);
+    g.second = q.second;
+    g.r = q.rule.r;
+    const int planes = planes::kernel_bit1(q.rule.r).planes;
+    set_bound(g.bound[planes::kSurviveLo], q.rule.s_lo, planes);
+    set_bound(g.bound[planes::kSurviveHi], (int64_t)q.rule.s_lo + q.rule.s_w + 1, planes);
+    set_bound(g.bound[planes::kBirthLo], q.rule.b_lo, planes);
+    set_bound(g.bound[planes::kBirthHi], (int64_t)q.rule.b_lo + q.rule.b_w + 1, planes);
+  }
+  std::vector<planes::BatchBlock> blocks;
+  std::vector<size_t> first;
+  for (int r = planes::kMaxR; r >= 1; --r) {   // (the larger radii, whose blocks take longest, first)
+    int range = 0;
+    while (r > planes::kRangeEnd[range]) ++range;
+    const size_t at = blocks.size();
+    for (size_t i = 0; i < items.size(); ++i) {
+      if (items[i].rule.r != r) continue;
+      const int64_t n = ((int64_t)b->grids[i].strips * b->grids[i].seg + planes::kOut - 1) / planes::kOut;
+      for (int64_t k = 0; k < n; ++k) blocks.push_back(planes::BatchBlock{(int32_t)i, (int32_t)k});
+    }
+    if (blocks.size() == at) continue;
+    while (blocks.size() % planes::kBatchWarps) blocks.push_back(planes::BatchBlock{-1, 0});
+    if (b->chains.empty() || b->chains.back().range != range) {
+      b->chains.push_back(PlanesBatch::Chain{range, planes::kBatchWarps * planes::kernel_bit1(r).smem, 0u, nullptr});
+      first.push_back(at);
+    }
+    b->chains.back().blocks += (unsigned)((blocks.size() - at) / planes::kBatchWarps);
+  }
+  const size_t pack_at = blocks.size();
+  for (size_t i = 0; i < items.size(); ++i) {
+    const int64_t words = (int64_t)b->grids[i].H * (b->grids[i].seg - 1);
+    for (int64_t k = 0; k * planes::kPackWords < words; ++k) blocks.push_back(planes::BatchBlock{(int32_t)i, (int32_t)k});
+  }
+  b->pack_blocks = (unsigned)(blocks.size() - pack_at);
+  cudaError_t e = blocks.size() > 0x7fffffffu ? cudaErrorInvalidValue
+                                              : cudaMalloc(&b->d_grids, sizeof(planes::BatchGrid) * b->grids.size());
+  if (e == cudaSuccess) e = cudaMalloc(&b->d_blocks, sizeof(planes::BatchBlock) * blocks.size());
+  if (e == cudaSuccess)
+    e = cudaMemcpy(b->d_blocks, blocks.data(), sizeof(planes::BatchBlock) * blocks.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = planes_batch_update(b, items);
+  b->pack_first = b->d_blocks + pack_at;
+  for (size_t c = 0; c < b->chains.size() && e == cudaSuccess; ++c) {
+    b->chains[c].first = b->d_blocks + first[c];
+    const planes::BatchFn fn = planes::batch_kernel(b->chains[c].range);
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  }
+  if (e != cudaSuccess) {
+    planes_batch_free(b);
+    return e;
+  }
+  *out = b;
+  return cudaSuccess;
+}
+
+void planes_batch_free(PlanesBatch *b) {
+  if (!b) return;
+  cudaFree(b->d_grids);
+  cudaFree(b->d_blocks);
+  delete b;
+}
+
+cudaError_t planes_batch_add(const PlanesBatch *b, int64_t n_steps, int flip, cudaGraph_t graph) {
+  const auto add = [&](planes::BatchFn fn, planes::BatchParams p, unsigned blocks, int threads, int smem,
+                       const std::vector<cudaGraphNode_t> &after, cudaGraphNode_t *node) {
+    void *args[1] = {&p};
+    cudaKernelNodeParams k = {};
+    k.func = reinterpret_cast<void *>(fn);
+    k.gridDim = dim3(blocks);
+    k.blockDim = dim3((unsigned)threads);
+    k.sharedMemBytes = (unsigned)smem;
+    k.kernelParams = args;
+    return cudaGraphAddKernelNode(node, graph, after.data(), after.size(), &k);
+  };
+  cudaGraphNode_t pack{}, unpack{};
+  cudaError_t e = add(planes::batch_pack_kernel(false), batch_params(b, b->pack_first, 0, n_steps, flip), b->pack_blocks,
+                      planes::kPackThreads, 0, {}, &pack);
+  std::vector<cudaGraphNode_t> ends;
+  for (const PlanesBatch::Chain &c : b->chains) {   // the ranges of radii side by side
+    cudaGraphNode_t before = pack;
+    for (int64_t t = 0; t < n_steps && e == cudaSuccess; ++t)
+      e = add(planes::batch_kernel(c.range), batch_params(b, c.first, t, n_steps, flip), c.blocks,
+              32 * planes::kBatchWarps, c.smem, {before}, &before);
+    ends.push_back(before);
+  }
+  if (e == cudaSuccess)
+    e = add(planes::batch_pack_kernel(true), batch_params(b, b->pack_first, n_steps, n_steps, flip), b->pack_blocks,
+            planes::kPackThreads, 0, ends, &unpack);
+  return e;
 }
 
 }  // namespace cat

@@ -240,6 +240,7 @@ struct Params {
   uint8_t *out;
   int64_t pitch;
   int32_t H, W;
+  int32_t written;     // cells written per row (W, or more where what lies past W is not kept)
   int32_t seg;         // words of a strip in the virtual row (the last one is the zero word)
   int32_t rows;        // rows per strip (a multiple of the rows loaded ahead)
   int32_t strips;
@@ -277,21 +278,20 @@ struct Target {
 };
 
 // One step from storage SI to storage SO (the same one, or between uint8 and
-// one bit for two states).
-template <int R, int SI, int SO, bool MS>
-__global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __grid_constant__ Params p) {
+// one bit for two states), by one warp; block: which 30 virtual words, smem:
+// its rings.
+template <int R, int SI, int SO, bool MS, int A = Cfg<R, MS>::kAhead>
+__device__ __forceinline__ void planes_step(const Params &p, int block, uint8_t *smem) {
   using D = Dim<R>;
   constexpr int NH = D::kH, NS = D::kS, NT = 32;
-  constexpr int A = Cfg<R, MS>::kAhead;
   constexpr int kParts = SI == CAT_STORE_U8 ? 2 : 1, kOutParts = SO == CAT_STORE_U8 ? 2 : 1;
   constexpr int kSlot = NT * 4 * NH, kRing = D::kWin * kSlot, kCentre = NT * 4 * R;
-  extern __shared__ __align__(16) uint8_t smem[];
   uint8_t *const cring = smem + kRing;
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31;
 
   // this lane's strip and word column (word w holds cells x0 .. x0 + 31); a
   // lane without a word reads along with a neighbour and masks its flags
-  const int v = (int)blockIdx.x * kOut + lane - 1;
+  const int v = block * kOut + lane - 1;
   int strip = v < 0 ? 0 : v / p.seg;
   int w = v < 0 ? p.seg - 1 : v - strip * p.seg;
   const bool held = w < p.seg - 1 && strip < p.strips;
@@ -301,6 +301,8 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
   const int64_t x0 = (int64_t)w * 32 - p.frame;
   const int64_t left = p.W + p.frame - x0;   // readable cells from x0 on
   const uint32_t mask = !held ? 0u : left >= 32 ? ~0u : (1u << (int)left) - 1u;
+  const int64_t out_left = left + p.written - p.W;   // (packed) cells written from x0 on
+  const uint32_t out_mask = SO == CAT_STORE_U8 || out_left >= 32 ? ~0u : (1u << (int)out_left) - 1u;
   const bool writes = held && lane >= 1 && lane <= kOut;
   const int my_rows = !writes ? 0 : p.H - y0 < p.rows ? (int)(p.H - y0) : p.rows;
   // bytes from the row's start: cell 0 of the grid for uint8, cell -frame for packed rows
@@ -333,9 +335,9 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
       const int of = kOutParts == 1 ? lane : 16 * t + (lane >> 1), half = kOutParts == 1 ? 0 : 16 * (lane & 1);
       const int64_t x = __shfl_sync(kFull, x0, of) + half, y = __shfl_sync(kFull, y0, of);
       to[t].base = p.out + y * p.pitch + __shfl_sync(kFull, col_out, of) + half;
-      to[t].cells = p.W - x >= 16 ? 16 : (int)(p.W - x);
+      to[t].cells = p.written - x >= 16 ? 16 : (int)(p.written - x);
       to[t].rows = __shfl_sync(kFull, my_rows, of);
-      if (SO == CAT_STORE_U8 && (x < 0 || x >= p.W)) to[t].rows = 0;
+      if (SO == CAT_STORE_U8 && (x < 0 || x >= p.written)) to[t].rows = 0;
     }
   }
   // some access of the warp ends within its 16 cells
@@ -346,12 +348,15 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // uint8: bytes past the last readable cell belong to whoever owns the buffer
+  uint32_t past[Raw<SI>::kWords];
+#pragma unroll
+  for (int i = 0; i < Raw<SI>::kWords; ++i) {
+    const int cells = from[i / 4 % kParts].cells - 4 * (i % 4);
+    past[i] = cells >= 4 ? ~0u : cells <= 0 ? 0u : (1u << (8 * cells)) - 1u;
+  }
   auto clear_past = [&](Raw<SI> &r) {
 #pragma unroll
-    for (int i = 0; i < Raw<SI>::kWords; ++i) {
-      const int cells = from[i / 4 % kParts].cells - 4 * (i % 4);
-      r.v[i] &= cells >= 4 ? ~0u : cells <= 0 ? 0u : (1u << (8 * cells)) - 1u;
-    }
+    for (int i = 0; i < Raw<SI>::kWords; ++i) r.v[i] &= past[i];
   };
   // flags of a loaded row: uint8, the halves of a lane's word come from lanes
   // 2 l and 2 l + 1, their first accesses for lanes below 16, else their second
@@ -425,9 +430,9 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
       if (j >= to[t].rows) continue;
       uint8_t *const q = const_cast<uint8_t *>(row_ptr(to[t].base, (uint32_t)j, pitch));
       if constexpr (SO == CAT_STORE_BIT1) {
-        *reinterpret_cast<uint32_t *>(q) = in & mask;
+        *reinterpret_cast<uint32_t *>(q) = in & out_mask;
       } else if constexpr (SO == CAT_STORE_NIB4) {
-        const uint32_t f = in & mask;
+        const uint32_t f = in & out_mask;
         uint4 a;
         a.x = age_nibbles(cs.v[0], spread_nibbles(byte_of<0>(f)), p.last, p.two);
         a.y = age_nibbles(cs.v[1], spread_nibbles(byte_of<1>(f)), p.last, p.two);
@@ -552,6 +557,94 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
   else walk(std::true_type{});
 }
 
+template <int R, int SI, int SO, bool MS>
+__global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __grid_constant__ Params p) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  planes_step<R, SI, SO, MS>(p, (int)blockIdx.x, smem);
+}
+
+// Batches of two-state uint8 grids, several steps per call on states kept one
+// bit per cell, within the rows of whichever of a grid's buffers holds no
+// state that is still needed (as one grid's steps are): the bytes are packed,
+// stepped and unpacked by separate launches, since the small grids' few warps
+// do not keep enough bytes in flight to step from them (512 uneven grids, 4
+// steps: 465 us with the first and last step on bytes, 310 us so).
+struct BatchGrid {
+  uint8_t *buf[2];
+  int64_t pitch;
+  int32_t H, W, seg, rows, strips;
+  int32_t r;
+  int32_t cur;       // the buffer that holds the states when the table is made
+  int32_t second;    // byte offset of a row's second row of bits
+  uint32_t bound[4][kMaxS];
+};
+struct BatchBlock {   // what a warp (a block when packing) does; grid < 0: nothing
+  int32_t grid, block;
+};
+struct BatchParams {
+  const BatchGrid *grids;
+  const BatchBlock *blocks;
+  int32_t flip;          // steps since the table was made, mod 2
+  int32_t step, steps;   // this launch's step of the call's
+};
+
+// Where the packed states after t steps of a call lie: in the buffer that does
+// not take the final states, but for the first ones (t = 0), which must leave
+// the buffer that they are packed from.  (Table reads: nothing writes a table
+// while a launch may read it.)
+__device__ __forceinline__ uint8_t *packed_place(const BatchGrid *g, int cur, int t, int steps) {
+  const bool odd = steps & 1;
+  const int b = t == 0 || !odd ? 1 - cur : cur;
+  const bool second = odd ? t > 0 && !(t & 1) : t & 1;
+  return reinterpret_cast<uint8_t *>(__ldg(reinterpret_cast<const unsigned long long *>(&g->buf[b]))) +
+         (second ? __ldg(&g->second) : 0);
+}
+
+template <int R>
+__device__ __forceinline__ void batch_step(const BatchParams &b, const BatchGrid *g, int block) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int cur = __ldg(&g->cur) ^ b.flip;
+  Params p;
+  p.in = packed_place(g, cur, b.step, b.steps);
+  p.out = packed_place(g, cur, b.step + 1, b.steps);
+  p.pitch = __ldg(reinterpret_cast<const long long *>(&g->pitch));
+  p.H = __ldg(&g->H);
+  p.W = __ldg(&g->W);
+  // the last step's row goes on to the end of its last 16 cells, like the
+  // tensor-core kernel's stores (the first step's input ends at W)
+  p.written = b.step == b.steps - 1 ? (p.W + 15) & ~15 : p.W;
+  p.seg = __ldg(&g->seg);
+  p.rows = __ldg(&g->rows);
+  p.strips = __ldg(&g->strips);
+  p.frame = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int i = 0; i < Dim<R>::kS; ++i) p.bound[k][i] = __ldg(&g->bound[k][i]);
+  planes_step<R, CAT_STORE_BIT1, CAT_STORE_BIT1, false, 2>(p, block, smem + (threadIdx.x >> 5) * Cfg<R, false>::kSmem);
+}
+
+// One launch serves the radii LO .. HI, and the warps of a block serve one
+// radius: an SM then runs the code of one or two radii at a time.  (Radii mixed
+// warp by warp, or sixteen launches side by side, fetch more code than the
+// instruction caches hold: 128 grids of 1024^2, 4 steps, one radius 224 us,
+// eight radii 777 us; for the same reason the loop is unrolled by two rows.)
+constexpr int kBatchWarps = 8;
+template <int LO, int HI, int R = LO>
+__device__ __forceinline__ void batch_pick(const BatchParams &b, const BatchGrid *g, int block) {
+  if constexpr (R <= HI) {
+    if (__ldg(&g->r) == R) batch_step<R>(b, g, block);
+    else batch_pick<LO, HI, R + 1>(b, g, block);
+  }
+}
+template <int LO, int HI>
+__global__ void __launch_bounds__(32 * kBatchWarps, (Cfg<HI, false>::kWarps + kBatchWarps - 1) / kBatchWarps)
+    planes_batch_kernel(const __grid_constant__ BatchParams b) {
+  const int2 at = __ldg(reinterpret_cast<const int2 *>(b.blocks) + blockIdx.x * kBatchWarps + (threadIdx.x >> 5));
+  if (at.x < 0) return;
+  batch_pick<LO, HI>(b, b.grids + at.x, at.y);
+}
+
 // Kernel of radius r for one storage, with the bytes of shared memory a warp
 // takes; nullptr when it is not built.
 struct Kernel {
@@ -576,6 +669,15 @@ Kernel find_kernel(int r) {
     return find_kernel<SI, SO, MS, LO + 1>(r);
   }
 }
+
+// The batch kernels: of three ranges of radii (a launch's blocks take the shared
+// memory of its largest radius), and from bytes (step 0 of the parameters) and
+// back (step = steps).
+constexpr int kRanges = 3, kRangeEnd[kRanges] = {7, 11, kMaxR};
+constexpr int kPackWords = 2048, kPackThreads = 256;   // words per block, threads
+typedef void (*BatchFn)(BatchParams);
+BatchFn batch_kernel(int range);
+BatchFn batch_pack_kernel(bool unpack);
 
 }  // namespace planes
 }  // namespace cat

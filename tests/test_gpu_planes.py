@@ -125,3 +125,52 @@ def test_packed_steps_between_uint8_states(cat, r):
                 g.close()
             assert np.array_equal(got, oracle.step(grid, oracle.Rule(**rule), n_steps=n)), (H, W, r, n)
             assert bool((a[:, W:] == 255).all()) and bool((b[:, W:] == 254).all())
+
+
+def test_packed_batch_of_uneven_grids(cat):
+    """cat_batch_step with the options left to the library: every radius, grids
+    narrower and wider than a warp's words, and one large enough for the batch
+    to step on bit planes; calls of different lengths one after the other (also
+    short and captured ones, which take the tiles)."""
+    import torch
+    specs = [dict(r=r, H=H, W=W, M=r & 1) for r, H, W in
+             [(r, 20 + 7 * r, 64 + 61 * (r % 5)) for r in range(1, 17)] + [(3, 300, 1031), (16, 90, 961), (9, 1, 64)]]
+    grids, hosts = [], []
+    for i, d in enumerate(specs):
+        rule = inputs.scaled_rule(d["r"], M=d["M"])
+        host = board(d["H"], d["W"], 2, 50 + i)
+        g = cat.Grid(d["H"], d["W"], rule, kernel="auto", dtype="auto")
+        g.set_state(host)
+        grids.append(g)
+        hosts.append((host, oracle.Rule(**rule)))
+    rule, large = inputs.scaled_rule(2), board(5801, 5803, 2, 9)
+    big = cat.Grid(5801, 5803, rule, kernel="auto", dtype="auto")
+    ref = cat.Grid(5801, 5803, rule, kernel="tcgen05", dtype="fp8")
+    big.set_state(large)
+    ref.set_state(large)
+    handles = [g.handle for g in grids] + [big.handle]
+
+    def compare(done):
+        for g, (host, rule) in zip(grids, hosts):
+            assert np.array_equal(g.get_state(), oracle.step(host, rule, n_steps=done)), (done, rule, host.shape)
+        assert torch.equal(big.state_tensor(), ref.state_tensor()), done
+    try:
+        done = 0
+        for n in (4, 5, 1, 7, 4):
+            cat.cat_batch_step(handles, n)
+            ref.step(n)
+            done += n
+            compare(done)
+        s = torch.cuda.Stream()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            cat.cat_batch_step(handles, 4, s)
+        graph.replay()
+        torch.cuda.synchronize()
+        ref.step(4)
+        compare(done + 4)
+        with pytest.raises(cat.CatError):
+            cat.cat_batch_step(handles + handles[:1], 4)
+    finally:
+        for g in grids + [big, ref]:
+            g.close()
