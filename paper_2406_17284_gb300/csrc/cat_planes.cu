@@ -2,6 +2,7 @@
 // a storage and radius, and the split of a grid into strips.
 #include <algorithm>
 #include <atomic>
+#include <cstdlib>
 #include <new>
 #include <vector>
 
@@ -9,6 +10,8 @@
 
 namespace cat {
 namespace {
+
+constexpr int kMaxSmem = 232448;   // of one block
 
 // The kernel for a grid's storages, and which of them it is (kinds x radii).
 constexpr int kKinds = 6;
@@ -28,21 +31,35 @@ planes::Kernel find(const PlanesGrid &g, int *kind) {
   }
 }
 
-// Warps of a kernel that the current device holds at once (looked up once per
-// device, kind and radius; the value is a property of the device, so threads
-// that race write the same).
-cudaError_t resident_warps(const planes::Kernel &k, int kind, int r, const PlanesGrid &g, int *warps) {
+// Warps of a kernel that an SM of the current device holds, and the shared
+// memory per warp that makes it so.  All warps have equal work, so an SM that
+// takes one more than the others, or a scheduler of its four, is waited for:
+// the warps per SM are a multiple of four, and a warp asks for as much shared
+// memory as lets just that many in (one bit, 16384^2, r = 10 / 11 / 14: 14, 13
+// and 10 warps 79 / 86 / 84 us a step, 12, 12 and 8 warps 69 / 71 / 71).  Looked
+// up once per device, kind and radius; the values are a property of the
+// device, so threads that race write the same.
+struct Resident {
+  int warps, smem;
+};
+constexpr int kSmSmem = 233472, kBlockReserve = 1024;   // bytes per SM, taken by the system per block
+
+cudaError_t resident_warps(const planes::Kernel &k, int kind, int r, const PlanesGrid &g, Resident *out) {
   static std::atomic<int> seen[16][kKinds][planes::kMaxR + 1];
   std::atomic<int> *slot = g.device >= 0 && g.device < 16 ? &seen[g.device][kind][r] : nullptr;
-  if (slot && (*warps = slot->load(std::memory_order_relaxed)) > 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, 32, k.smem);
-  if (e != cudaSuccess) return e;
-  *warps = per_sm * g.sms;
-  if (slot) slot->store(*warps, std::memory_order_relaxed);
+  int per_sm = slot ? slot->load(std::memory_order_relaxed) : 0;
+  if (per_sm == 0) {
+    cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, 32, k.smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm > 4 && per_sm % 4) per_sm = -(per_sm / 4 * 4);   // negative: only by asking for more
+    if (slot) slot->store(per_sm, std::memory_order_relaxed);
+  }
+  const int n = std::max(1, std::abs(per_sm));
+  out->warps = n * g.sms;
+  out->smem = per_sm < 0 ? std::max(k.smem, (kSmSmem / n - kBlockReserve) / 128 * 128) : k.smem;
   return cudaSuccess;
 }
 
@@ -91,8 +108,6 @@ cudaError_t launch(void (*fn)(P), const P &p, int64_t blocks, int threads, int s
   return cudaLaunchKernelEx(&cfg, fn, p);
 }
 
-constexpr int kMaxSmem = 232448;
-
 // Steps before the words that a tile's warps write need a stale cell: the left
 // neighbour word loses r cells a step; the right one r, and r more because the
 // sums of a word are formed from the next word's shifted copy.
@@ -117,7 +132,11 @@ int64_t tile_smem(const PlanesGrid &g, const TilePlan &t) {
 //   one bit per cell      every radius: 32768^2, r = 2 / 16: 147 / 320 against
 //                         the former bit-sliced kernel's 224 and tcgen05's 594
 //   four bits per cell    every radius: 24576^2, C 16, r = 10: 297 against 435
-//   uint8, C > 2          24576^2, r = 10 / 16: 356 / 418 against 398: r <= 15
+//   uint8, C > 2          16384^2, r = 1 / 10 / 15: 117 / 156 / 175 against 180
+//                         / 182 / 182; 4096^2: 9.0 / 17.7 / 18.9 against 18.9 /
+//                         19.2 / 19.3; 2048^2, r = 8 / 10 / 15: 10.9 / 14 / 14
+//                         against 11: up to r = 15, but not where a strip is
+//                         shorter than the 2r rows before it
 //   uint8, two states     only where a launch's latency counts: 1024^2, r = 1:
 //                         2.9 against 6.5; 4096^2, r = 4 / 9 / 16: 9.5 / 14.8 /
 //                         18.4 against 11.6 / 14.8 / 14.8; 16384^2, r = 4:
@@ -126,19 +145,20 @@ bool planes_preferred(const PlanesGrid &g) {
   int kind;
   if (!find(g, &kind).fn) return false;
   if (g.storage_in != CAT_STORE_U8) return true;
-  if (g.rule.C > 2) return g.rule.r <= 15;
+  if (g.rule.C > 2) return g.rule.r <= 15 && (g.rule.r <= 8 || g.H * g.W <= (1 << 20) || g.H * g.W >= (1 << 24));
   return g.rule.r <= 9 && g.H * g.W <= (1 << 24);
 }
 
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
-  int kind, resident;
+  int kind;
+  Resident resident;
   const planes::Kernel k = find(g, &kind);
   if (!k.fn) return cudaErrorInvalidValue;
   cudaError_t e = resident_warps(k, kind, g.rule.r, g, &resident);
   if (e != cudaSuccess) return e;
   planes::Params p = make_params(g, k.planes);
   // as many strips as fill the GPU once
-  int64_t strips = (int64_t)resident * planes::kOut / p.seg;
+  int64_t strips = (int64_t)resident.warps * planes::kOut / p.seg;
   if (strips < 1) strips = 1;
   int64_t rows = (g.H + strips - 1) / strips;
   rows = (rows + k.ahead - 1) / k.ahead * k.ahead;
@@ -146,7 +166,7 @@ cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
   p.rows = (int32_t)rows;
   p.strips = (int32_t)strips;
   const int64_t warps = (strips * p.seg + planes::kOut - 1) / planes::kOut;
-  return launch(k.fn, p, warps, 32, k.smem, s);
+  return launch(k.fn, p, warps, 32, resident.smem, s);
 }
 
 // One wave of blocks, the strips as short as that allows, and k so that a
