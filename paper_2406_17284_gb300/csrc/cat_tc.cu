@@ -304,12 +304,23 @@ __device__ __forceinline__ void encode_window(const uint8_t *xs, uint8_t *xe, bo
       else reinterpret_cast<uint4 *>(xe)[q] = make_uint4(w[0], w[1], w[2], w[3]);
     }
   } else {
-    // f16 operands take two units per source unit: positions through op_off;
-    // consecutive threads take consecutive rows of one 16-byte column chunk,
-    // so every warp access touches each bank group evenly under both swizzles
-    for (int q = tid; q < kUnits; q += nthr) {
-      const int c = q / kWin, row = q - c * kWin;
-      uint4 v = *reinterpret_cast<const uint4 *>(xs + op_off(kWin, 1, row, 16 * c));
+    // f16 operands take two units per source unit, side by side under either
+    // swizzle (their chunk indices differ in the lowest bit).  A warp takes 32
+    // rows of one 16-byte column chunk at a time, so that a thread's row is the
+    // same in every swizzle and the chunk is a warp's: few integer operations
+    // per unit, and every access touches each bank group evenly.
+    const int lane = tid & 31, l7 = lane & 7;
+    for (int item = tid >> 5; item < 10 * (kWin / 32); item += nthr >> 5) {
+      const int c = item / 5, row = 32 * (item - 5 * c) + lane;   // (warp-uniform but for the lane)
+      uint32_t src, dst;
+      if (c < 8) {
+        src = row * 128 + ((c ^ l7) << 4);
+        dst = (c >> 2) * (kWin * 128) + row * 128 + ((((2 * c) & 7) ^ l7) << 4);
+      } else {   // the last 32 cells: rows of 32 bytes
+        src = kWin * 128 + row * 32 + (((c & 1) ^ ((lane >> 2) & 1)) << 4);
+        dst = 2 * kWin * 128 + (c - 8) * (kWin * 32) + row * 32 + (((lane >> 2) & 1) << 4);
+      }
+      uint4 v = *reinterpret_cast<const uint4 *>(xs + src);
       uint32_t w[4] = {v.x, v.y, v.z, v.w};
       if (multistate) {
 #pragma unroll
@@ -321,8 +332,8 @@ __device__ __forceinline__ void encode_window(const uint8_t *xs, uint8_t *xe, bo
         h[2 * i] = __byte_perm(w[i], 0, 0x4140) * 0x3C00u;
         h[2 * i + 1] = __byte_perm(w[i], 0, 0x4342) * 0x3C00u;
       }
-      *reinterpret_cast<uint4 *>(xe + op_off(kWin, 2, row, 32 * c)) = make_uint4(h[0], h[1], h[2], h[3]);
-      *reinterpret_cast<uint4 *>(xe + op_off(kWin, 2, row, 32 * c + 16)) = make_uint4(h[4], h[5], h[6], h[7]);
+      *reinterpret_cast<uint4 *>(xe + dst) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4 *>(xe + (dst ^ 16u)) = make_uint4(h[4], h[5], h[6], h[7]);
     }
   }
 }
@@ -423,6 +434,13 @@ __device__ __forceinline__ uint32_t bytes_to_nib_pairs(uint32_t w) { return w | 
 // writes lanes 32q .. 32q+31 and every other 8-column chunk from chunk kq.
 // The big window holds the e4m3 band and the band of 16s, 48 columns each
 // (K = 192), with offset 32.
+// v << n, 0 from n = 32 on.
+__device__ __forceinline__ uint32_t shl_clamp(uint32_t v, int n) {
+  uint32_t r;
+  asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
+}
+
 template <int DT, bool SW, bool WIDE = false, bool FP4 = false, bool BITS = false, bool BIG = false>
 __device__ __forceinline__ void store_bands(uint32_t tmem, int r, int q, int kq, int lane) {
   using G = Geo<SW, WIDE, BIG>;
@@ -450,26 +468,17 @@ __device__ __forceinline__ void store_bands(uint32_t tmem, int r, int q, int kq,
                        : SW ? (first ? G::kBand8 : G::kBand8P2) : (first ? G::kBand16 : T::kBand8);
     const uint32_t one8 = third ? 0x08u : (W32 && !first) ? 0x58u : 0x38u;   // e2m1 1.0, e4m3 16.0 or 1.0
     const uint32_t one16 = FP4 ? 0x1C00u : 0x3C00u;                             // f16 2^-8 or 1.0
+    // a word of the band's values, cut to k in [lo, hi1) by two clamped shifts
+    // (256^2, r = 12: 7.8 us a step with a comparison per element and the
+    // bands built after the wait for the previous kernel, 5.2 us so)
+    const int per = f16 ? 2 : 4, bits = 32 / per;
+    const uint32_t ones = f16 ? one16 * 0x00010001u : m >= G::kTS ? 0u : third && !FP4 ? 0x20283038u : one8 * 0x01010101u;
+    const int lo = off - r + m - per * 8 * cc, hi1 = lo + 2 * r + 1;
     uint32_t v[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int k0 = (f16 ? 2 : 4) * (8 * cc + i);
-      uint32_t w = 0;
-      if (f16) {
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          const int d = k0 + b - m;
-          if (d >= off - r && d <= off + r) w |= one16 << (16 * b);
-        }
-      } else if (m < G::kTS) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int d = k0 + b - m;
-          const uint32_t v8 = (third && !FP4) ? 0x38u - 8u * (uint32_t)b : one8;   // 1, 1/2, 1/4, 1/8
-          if (d >= off - r && d <= off + r) w |= v8 << (8 * b);
-        }
-      }
-      v[i] = w;
+      const int a = lo - per * i, b = hi1 - per * i;
+      v[i] = ones & shl_clamp(~0u, bits * (a > 0 ? a : 0)) & ~shl_clamp(~0u, bits * (b > 0 ? b : 0));
     }
     tmem_st8(tmem + la + col + 8 * cc, v);
   }
@@ -841,9 +850,12 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   // start its own set-up, and this one reads and writes global memory only
   // once the previous kernel has completed
   griddep_launch_dependents();
-  griddep_wait();
   const uint32_t tmem = bars->tmem_base;
   const uint32_t s_base = smem_u32(smem);
+  // (the convert warps build the bands for the first tile before they wait:
+  // those depend on its radius only)
+  constexpr bool kEarlyBands = DT == 1;
+  if (!(kEarlyBands && warp >= 4 && warp < 4 + kCvtWarps)) griddep_wait();
 
   // The convert warps encode window j into buffer j % NE once pass 1 of tile
   // j - NE has read that buffer (at the start of the loop iteration of tile
@@ -1098,11 +1110,13 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       off16b[c] = op_off(kTile, 2, row, 32 * cc + 16);
       off8[c] = op_off(kTile, 1, row, 16 * cc);
     }
-    // the bands for the first tile
+    // the bands for the first tile (a batch's table is not written while its
+    // launches run)
     store_bands<DT, SW, WIDE, FP4, BITS, BIG>(tmem, r0, q, kq, lane);
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(&bars->band_ready);
+    if (kEarlyBands) griddep_wait();
     if (ENC && !MS)
       for (int j = 0; ok && j < n_all && j < L::NE; ++j) ok = encode(j, wtid, kCvtThreads);
     int enc_next = 0;   // MS: next window to encode
