@@ -27,7 +27,10 @@
 // centre states and writes 16 contiguous next states per access.
 //
 // Precision (exact in every case, Sec. V-A):
-//   FP16 kernel: X, band and H in f16; D1 = H, D2 = S.
+//   FP16 kernel: X, band and H in f16.  A live cell is the f16 with the code 1,
+//                2^-24 (its byte widened, nothing to multiply), the band 2^8,
+//                so D1 = H * 2^-16 and D2 = S * 2^-8, all exact (f16
+//                subnormals are full operands and results of kind::f16).
 //   FP8 kernel:  pass 1 on e4m3 -- the raw 0/1 state bytes ARE the B operand
 //                (0x01 reads as e4m3 2^-9), so D1 = H * 2^-9 exactly; pass 2
 //                takes H * 2^-9 as e4m3 when 2r+1 <= 15 (all such values are
@@ -275,7 +278,7 @@ __device__ __forceinline__ uint32_t bits8_to_nibbles(uint32_t b) {
 }
 
 // Encodes the 160 x 160 u8 window xs as operand values: alive (state 1) ->
-// 0x01 (e4m3 2^-9, FP8 kernel), f16 1.0 (FP16 kernel) or e2m1 0.5 (FP4
+// 0x01 (e4m3 2^-9, FP8 kernel), f16 2^-24 (FP16 kernel) or e2m1 0.5 (FP4
 // kernel, packed units), anything else -> 0.
 // FP8 and FP4: the encoded window has the raw window's layout unit for unit
 // (a swizzle moves whole 16-byte units, and a unit holds 16 consecutive cells
@@ -308,7 +311,10 @@ __device__ __forceinline__ void encode_window(const uint8_t *xs, uint8_t *xe, bo
     // swizzle (their chunk indices differ in the lowest bit).  A warp takes 32
     // rows of one 16-byte column chunk at a time, so that a thread's row is the
     // same in every swizzle and the chunk is a warp's: few integer operations
-    // per unit, and every access touches each bank group evenly.
+    // per unit, and every access touches each bank group evenly.  The convert
+    // warps' instructions bound this kernel (16384^2: 210.5 us a step with
+    // positions computed per unit and f16 1.0 for a live cell; 178 with the
+    // positions, 162 with 2^-24).
     const int lane = tid & 31, l7 = lane & 7;
     for (int item = tid >> 5; item < 10 * (kWin / 32); item += nthr >> 5) {
       const int c = item / 5, row = 32 * (item - 5 * c) + lane;   // (warp-uniform but for the lane)
@@ -329,8 +335,8 @@ __device__ __forceinline__ void encode_window(const uint8_t *xs, uint8_t *xe, bo
       uint32_t h[8];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        h[2 * i] = __byte_perm(w[i], 0, 0x4140) * 0x3C00u;
-        h[2 * i + 1] = __byte_perm(w[i], 0, 0x4342) * 0x3C00u;
+        h[2 * i] = __byte_perm(w[i], 0, 0x4140);
+        h[2 * i + 1] = __byte_perm(w[i], 0, 0x4342);
       }
       *reinterpret_cast<uint4 *>(xe + dst) = make_uint4(h[0], h[1], h[2], h[3]);
       *reinterpret_cast<uint4 *>(xe + (dst ^ 16u)) = make_uint4(h[4], h[5], h[6], h[7]);
@@ -467,7 +473,7 @@ __device__ __forceinline__ void store_bands(uint32_t tmem, int r, int q, int kq,
                        : W32 ? (first ? T::kBand8 : T::kBand8x16)
                        : SW ? (first ? G::kBand8 : G::kBand8P2) : (first ? G::kBand16 : T::kBand8);
     const uint32_t one8 = third ? 0x08u : (W32 && !first) ? 0x58u : 0x38u;   // e2m1 1.0, e4m3 16.0 or 1.0
-    const uint32_t one16 = FP4 ? 0x1C00u : 0x3C00u;                             // f16 2^-8 or 1.0
+    const uint32_t one16 = FP4 ? 0x1C00u : DT == 0 ? 0x5C00u : 0x3C00u;         // f16 2^-8, 2^8 or 1.0
     // a word of the band's values, cut to k in [lo, hi1) by two clamped shifts
     // (256^2, r = 12: 7.8 us a step with a comparison per element and the
     // bands built after the wait for the previous kernel, 5.2 us so)
@@ -792,7 +798,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   constexpr int NS = L::NS;
   constexpr int NR = L::NR;
   constexpr int NH = L::NH;
-  constexpr float kScale = DT == 1 ? (1.0f / 512.0f) : 1.0f;   // accumulator = count * kScale
+  constexpr float kScale = DT == 1 ? (1.0f / 512.0f) : (1.0f / 256.0f);   // accumulator = count * kScale
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
