@@ -88,8 +88,9 @@ enum { CAT_BOUNDARY_ZERO = 0, CAT_BOUNDARY_PERIODIC = 1 };
  *             horizontal sums H <= 2r+1 are exact, and so is every partial sum.
  *   FP8_E4M3  a state byte 0x01 read as e4m3 is 2^-9, so the raw bytes are the
  *             pass-1 operand; H * 2^-9 is an e4m3 number while H <= 15
- *             (2r+1 <= 15).  Beyond that the TCGEN05 kernel passes H to the
- *             second product as f16 operands in the 160-row window, and with
+ *             (2r+1 <= 15).  Beyond that the TCGEN05 kernel passes H - 16 to
+ *             the second product for 2r+1 <= 31 (C = 2, uint8, one grid) and
+ *             H as f16 operands elsewhere in the 160-row window, and with
  *             a 32-cell halo (H <= 65) as two e4m3 digits, H & 15 against the
  *             band and H >> 4 against a band of 16s (f32 accumulation).
  *   INT8      H <= 65 < 127; served by MMA_SYNC (sm_103a has no tcgen05 kind::i8).

@@ -34,8 +34,10 @@
 //   FP8 kernel:  pass 1 on e4m3 -- the raw 0/1 state bytes ARE the B operand
 //                (0x01 reads as e4m3 2^-9), so D1 = H * 2^-9 exactly; pass 2
 //                takes H * 2^-9 as e4m3 when 2r+1 <= 15 (all such values are
-//                e4m3 numbers) and as f16 otherwise (e4m3 cannot hold the odd
-//                counts above 16); D2 = S * 2^-9.  The wide tile (r <= 32,
+//                e4m3 numbers), H - 16 as e4m3 up to 2r+1 = 31 where no
+//                window is re-encoded (see pass2_offset), and H * 2^-9 as
+//                f16 otherwise (e4m3 cannot hold the odd counts above 16);
+//                D2 = S * 2^-9, less a constant with H - 16.  The wide tile (r <= 32,
 //                H <= 65) splits H into e4m3 digits instead (see Tm).
 // The epilogue compares S (as f16, exact up to 2048) against the rule's
 // ranges two cells at a time in half2 arithmetic.
@@ -117,7 +119,7 @@ constexpr uint32_t kTmemCols = 512;
 // (The same split for the 128 x 128 FP8 kernel -- pass 2 on e4m3 for every r,
 // no f16 band, and separate D1 / D2 regions, 2 + 1 or 1 + 2 -- measured 8%
 // and 3% slower at r >= 8 than the shared regions, 2.05 and 2.15 against
-// 2.22 * 10^12 cell updates/s, so it is not used there.)
+// 2.22 * 10^12 cell updates/s, so it is not used there; pass2_offset is.)
 template <int DT, bool SW, bool WIDE = false, bool BIG = false>
 struct Tm {
   using GB = Geo<SW, false, BIG>;
@@ -205,7 +207,7 @@ __device__ __forceinline__ void band_mma(uint32_t d, uint32_t a_tmem, const OpDe
 // BIG: a window stage is 192 x 192 bytes (a 128-column and two 32-column
 // boxes), an H buffer two 128 x 192 digit halves.
 template <int DT, bool ENC, bool SW = false, bool BITS = false, bool WIDE = false, bool NIB = false,
-          bool BIG = false>
+          bool BIG = false, bool OF = false>
 struct Layout {
   static constexpr int E1 = DT == 0 ? 2 : 1;                  // pass-1 operand bytes
   static constexpr int NS = (SW || BITS || NIB) ? 4 : ((DT == 0 || ENC || BIG) ? 2 : 3);   // TMA window stages
@@ -222,7 +224,7 @@ struct Layout {
   static constexpr uint32_t kXeStride = kWin * kWin * E1;     // one encoded window (25 or 50 KiB)
   static constexpr uint32_t kXeBytes = ENC ? NE * kXeStride : 0;
   static constexpr uint32_t kH = kXe + kXeBytes;              // pass-2 operand (K padded to 160)
-  static constexpr uint32_t kHBytes = kTile * (BIG ? 192 : kWin) * (SW ? 1 : 2);
+  static constexpr uint32_t kHBytes = kTile * (BIG ? 192 : kWin) * (SW || OF ? 1 : 2);
   static constexpr uint32_t kRing = kH + NH * kHBytes;        // centre tiles / output staging
   static constexpr uint32_t kRingBytes = BITS ? 16 * kTile : NIB ? 64 * kTile : Geo<SW, WIDE>::kTS * Geo<SW, WIDE>::kTS;
   static constexpr uint32_t kBars = kRing + NR * kRingBytes;
@@ -440,6 +442,24 @@ __device__ __forceinline__ uint32_t bytes_to_nib_pairs(uint32_t w) { return w | 
 // writes lanes 32q .. 32q+31 and every other 8-column chunk from chunk kq.
 // The big window holds the e4m3 band and the band of 16s, 48 columns each
 // (K = 192), with offset 32.
+// Pass 2 reads f16 in the FP16 kernel and, in the FP8 kernel, whenever H can
+// exceed 15 (e4m3 holds every integer multiple of 2^-9 up to 15 * 2^-9) ...
+__device__ __forceinline__ bool pass2_f16(int DT, int r) { return DT == 0 || 2 * r + 1 > 15; }
+
+// ... but in the offset kernels (OF; r = 8 .. 15): H - 16 is an e4m3 number
+// then (all integers from -16 to 16 are), so pass 2 runs on e4m3 at half the
+// operand bytes and K-steps, against a band of 2^-9, and
+// D2 = (S - 16 (2r + 1)) * 2^-9, every partial sum exact in f16: every row of
+// the band has 2r + 1 ones, so the offset is a constant that the rule's bounds
+// take up.  16384^2, us a step: r = 8 .. 15 106.3 against 116.8 with H in f16
+// (r = 12: 256^2 4.8 against 5.1, 2048^2 6.0 against 6.8, 8192^2 31.0 against
+// 33.7).  Only the one-instance kernel without a re-encoded window has it: a
+// choice by radius inside a kernel cost r = 16 2%, and with a re-encoded
+// window the convert warps are what bounds the kernel and four conversions a
+// word cost more than the shorter pass 2 gives (r = 10, C = 16: 184.0 against
+// 180.7).
+constexpr __host__ __device__ bool pass2_offset(int r) { return r >= 8 && r <= 15; }
+
 // v << n, 0 from n = 32 on.
 __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, int n) {
   uint32_t r;
@@ -447,7 +467,7 @@ __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, int n) {
   return r;
 }
 
-template <int DT, bool SW, bool WIDE = false, bool FP4 = false, bool BITS = false, bool BIG = false>
+template <int DT, bool SW, bool WIDE = false, bool FP4 = false, bool BITS = false, bool BIG = false, bool OF = false>
 __device__ __forceinline__ void store_bands(uint32_t tmem, int r, int q, int kq, int lane) {
   using G = Geo<SW, WIDE, BIG>;
   using T = Tm<DT, SW, WIDE, BIG>;
@@ -459,26 +479,27 @@ __device__ __forceinline__ void store_bands(uint32_t tmem, int r, int q, int kq,
   // 32, rows 96..127 zero), or in the FP4 kernel the f16 band of 2^-8 (pass 2
   // on H / 2), the e4m3 band and the e2m1 band (pass 1, after the e4m3 one);
   // the one-bit kernel's pass-1 band sits there too: e4m3 2^-(k mod 4) at
-  // column k, against window bytes 2^(k mod 4) * 2^-9 for live cells
-  constexpr int n0 = BIG ? 6 : WIDE ? 5 : (SW ? 5 : 10), n1 = BIG ? 12 : WIDE ? 10 : (SW ? 10 : (DT == 1 ? 15 : 10));
+  // column k, against window bytes 2^(k mod 4) * 2^-9 for live cells.  The
+  // offset kernels have the e4m3 band of 2^-9 (pass 2) in the f16 band's place
+  constexpr int n0 = BIG ? 6 : WIDE ? 5 : (SW || OF ? 5 : 10), n1 = BIG ? 12 : WIDE ? 10 : (SW || OF ? 10 : (DT == 1 ? 15 : 10));
   constexpr int n = (FP4 || BITS) ? 20 : n1;
   const int m = 32 * q + lane;
   const uint32_t la = static_cast<uint32_t>(32 * q) << 16;
   for (int c = kq; c < n; c += 2) {                 // warp-uniform
     const bool first = c < n0, third = c >= n1;
-    const bool f16 = !SW && !W32 && first;
+    const bool f16 = !SW && !W32 && !OF && first;
     const int cc = first ? c : third ? c - n1 : c - n0;
     const int off = W32 ? G::kXOff : (SW && !first) ? G::kYOff : 16;
     const uint32_t col = third ? T::kBand8 + 40
                        : W32 ? (first ? T::kBand8 : T::kBand8x16)
                        : SW ? (first ? G::kBand8 : G::kBand8P2) : (first ? G::kBand16 : T::kBand8);
-    const uint32_t one8 = third ? 0x08u : (W32 && !first) ? 0x58u : 0x38u;   // e2m1 1.0, e4m3 16.0 or 1.0
+    const uint32_t one8 = third ? 0x08u : (W32 && !first) ? 0x58u : OF && first ? 0x01u : 0x38u;   // e2m1 1.0, e4m3 16.0, 2^-9 or 1.0
     const uint32_t one16 = FP4 ? 0x1C00u : DT == 0 ? 0x5C00u : 0x3C00u;         // f16 2^-8, 2^8 or 1.0
     // a word of the band's values, cut to k in [lo, hi1) by two clamped shifts
     // (256^2, r = 12: 7.8 us a step with a comparison per element and the
     // bands built after the wait for the previous kernel, 5.2 us so)
     const int per = f16 ? 2 : 4, bits = 32 / per;
-    const uint32_t ones = f16 ? one16 * 0x00010001u : m >= G::kTS ? 0u : third && !FP4 ? 0x20283038u : one8 * 0x01010101u;
+    const uint32_t ones = f16 ? one16 * 0x00010001u : m >= G::kTS ? 0u : BITS && third && !FP4 ? 0x20283038u : one8 * 0x01010101u;
     const int lo = off - r + m - per * 8 * cc, hi1 = lo + 2 * r + 1;
     uint32_t v[8];
 #pragma unroll
@@ -505,9 +526,11 @@ __device__ __forceinline__ uint32_t half_pair(float v) {
   return *reinterpret_cast<uint32_t *>(&h);
 }
 
-__device__ __forceinline__ HalfRule make_half_rule(const RuleDev &R, float scale) {
-  auto lo_of = [](int lo) { return lo > 2048 ? 4096.0f : (float)lo; };
-  auto hi_of = [](int lo, int w) { return lo > 2048 ? 2048.0f : fminf((float)lo + (float)w, 2048.0f); };
+// `offset`: what the accumulator's counts lack (pass2_offset).
+__device__ __forceinline__ HalfRule make_half_rule(const RuleDev &R, float scale, int offset = 0) {
+  const float o = (float)offset;
+  auto lo_of = [o](int lo) { return lo > 2048 ? 4096.0f : (float)lo - o; };
+  auto hi_of = [o](int lo, int w) { return lo > 2048 ? 2048.0f : fminf((float)lo + (float)w, 2048.0f) - o; };
   HalfRule h;
   h.bl2 = half_pair(lo_of(R.b_lo) * scale);
   h.bh2 = half_pair(hi_of(R.b_lo, R.b_w) * scale);
@@ -519,6 +542,14 @@ __device__ __forceinline__ HalfRule make_half_rule(const RuleDev &R, float scale
 __device__ __forceinline__ __half2 as_h2(uint32_t v) { return *reinterpret_cast<const __half2 *>(&v); }
 
 __device__ __forceinline__ uint32_t h2_bits(__half2 h) { return *reinterpret_cast<uint32_t *>(&h); }
+
+// Four f16 values that are e4m3 numbers, as e4m3 bytes.
+__device__ __forceinline__ uint32_t e4m3x4(__half2 a, __half2 b) {
+  uint16_t x, y;
+  asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(x) : "r"(h2_bits(a)));
+  asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(y) : "r"(h2_bits(b)));
+  return (uint32_t)x | ((uint32_t)y << 16);
+}
 
 // As rule4_binary, from counts already packed as f16 pairs (cells 0,1 and 2,3).
 // One multiply builds both byte-permute selectors (low half: cells 0, 1; high
@@ -762,12 +793,8 @@ __device__ __forceinline__ int32_t *tile_err(const TcParams &p, int first, int j
   else return p.err;
 }
 
-// Pass 2 reads f16 in the FP16 kernel and, in the FP8 kernel, whenever H can
-// exceed 15 (e4m3 holds every integer multiple of 2^-9 up to 15 * 2^-9).
-__device__ __forceinline__ bool pass2_f16(int DT, int r) { return DT == 0 || 2 * r + 1 > 15; }
-
 template <int DT, bool ENC, bool BATCH, bool SW, bool BITS, bool MS, bool WIDE = false, bool NIB = false,
-          bool FP4 = false, bool BIG = false, int HB = 0>
+          bool FP4 = false, bool BIG = false, int HB = 0, bool OF = false>
 __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   static_assert(!MS || !BATCH, "several steps per launch serve single instances");
   static_assert(!WIDE || (DT == 1 && !ENC && !BATCH && !SW && !BITS && !MS),
@@ -783,9 +810,11 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   // epilogue tests f16 pairs, converted from the f32 accumulator (1) or
   // accumulated in f16 by pass 2 (2); 0: the f32 integer test
   static_assert(HB == 0 || BIG, "f16 pairs serve the big window");
+  static_assert(!OF || (DT == 1 && !ENC && !BATCH && !SW && !BITS && !WIDE && !NIB && !FP4 && !BIG),
+                "the offset pass 2 serves single two-state instances on FP8 operands in the standard window");
   static_assert(Layout<DT, ENC, SW, BITS>::NS <= kMaxStages && Layout<DT, ENC, SW, BITS>::NR <= kMaxStages &&
                 Layout<DT, ENC, SW, BITS>::NE <= 3, "barrier arrays");
-  using L = Layout<DT, ENC, SW, BITS, WIDE, NIB, BIG>;
+  using L = Layout<DT, ENC, SW, BITS, WIDE, NIB, BIG, OF>;
   // x-coordinate of a tile's centre box in its tensor map (bytes of packed rows)
   auto ctr_x = [](int tx0) { return BITS ? tx0 / 8 : NIB ? tx0 / 2 : tx0; };
   using G = Geo<SW, WIDE, BIG>;
@@ -1079,6 +1108,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             band_mma<1, kTile, 1, true>(d2, band_hi, OpDesc{hop.d128 + kHi, hop.d32 + kHi}, idesc2);
           }
           mma_commit(&bars->h_empty[j % NH]);
+        } else if constexpr (OF) {
+          band_mma<1, kTile, 1>(d2, tmem + T::kBand16, hop, idesc2);
         } else if (pass2_f16(DT, rj)) {
           band_mma<0, kTile, 2>(d2, band16, hop, idesc2);
         } else {
@@ -1118,7 +1149,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     }
     // the bands for the first tile (a batch's table is not written while its
     // launches run)
-    store_bands<DT, SW, WIDE, FP4, BITS, BIG>(tmem, r0, q, kq, lane);
+    store_bands<DT, SW, WIDE, FP4, BITS, BIG, OF>(tmem, r0, q, kq, lane);
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(&bars->band_ready);
@@ -1155,7 +1186,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
           if (!ok) break;
         }
         tc_fence_after();
-        store_bands<DT, SW, WIDE, FP4, BITS, BIG>(tmem, rj, q, kq, lane);
+        store_bands<DT, SW, WIDE, FP4, BITS, BIG, OF>(tmem, rj, q, kq, lane);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->band_ready);
@@ -1233,6 +1264,14 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               for (int i = 0; i < 4; ++i) hi[i] = (e[i] >> 4) & 0x0F0F0F0Fu;
               *reinterpret_cast<uint4 *>(hop + kTile * kWin + off8[c]) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             }
+          } else if constexpr (OF) {
+            // H * 2^-9 * 512 - 16, exact in f16 and in e4m3
+            const __half2 k512 = __float2half2_rn(512.0f), m16 = __float2half2_rn(-16.0f);
+            uint32_t e[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              e[i] = e4m3x4(__hfma2(as_h2(v[c][2 * i]), k512, m16), __hfma2(as_h2(v[c][2 * i + 1]), k512, m16));
+            *reinterpret_cast<uint4 *>(hop + off8[c]) = make_uint4(e[0], e[1], e[2], e[3]);
           } else if (p2f16) {
             *reinterpret_cast<uint4 *>(hop + off16a[c]) = make_uint4(v[c][0], v[c][1], v[c][2], v[c][3]);
             *reinterpret_cast<uint4 *>(hop + off16b[c]) = make_uint4(v[c][4], v[c][5], v[c][6], v[c][7]);
@@ -1356,13 +1395,14 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       off_c[c] = y * 128 + (((cc ^ y) & 7) << 4);
     }
     bool ok = true;
-    HalfRule hr = make_half_rule(BATCH ? RuleDev{} : p.rule, kScale);
+    auto offset_of = [](const RuleDev &R) { return OF ? 16 * (2 * R.r + 1) : 0; };
+    HalfRule hr = make_half_rule(BATCH ? RuleDev{} : p.rule, kScale, BATCH ? 0 : offset_of(p.rule));
     TileSeq<BATCH, MS, G::kTS> seq(p, first, n_my);
     for (int j = 0; ok && j < n_all; ++j, seq.next(p)) {
       const int reg = j % ND2, k = j % NR;
       const Tile t = seq.get(p);
       const RuleDev &R = t.R;
-      if (BATCH) hr = make_half_rule(R, kScale);
+      if (BATCH) hr = make_half_rule(R, kScale, offset_of(R));
       if (!(ok = warp_wait(&bars->d2_full[reg], (j / ND2) & 1, bars, p.timeout_ns))) break;
       tc_fence_after();
       // read S and free the region (the next pass 1, or in DEC the next pass
@@ -1480,7 +1520,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               const uint32_t h2 = v[c][i >> 1];
               const float s = (i & 1) ? half_hi(h2) : half_lo(h2);
               const int gx = t.x0 + 16 * cc + i;
-              if (gy < t.H && gx < t.W) p.sums[(int64_t)gy * p.sums_ld + gx] = __float2int_rn(s * (1.0f / kScale));
+              if (gy < t.H && gx < t.W) p.sums[(int64_t)gy * p.sums_ld + gx] = __float2int_rn(s * (1.0f / kScale)) + offset_of(R);
             }
           }
         }
@@ -1500,9 +1540,9 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   }
 }
 
-template <int DT, bool ENC, bool BATCH, bool SW>
+template <int DT, bool ENC, bool BATCH, bool SW, bool OF>
 __global__ void __launch_bounds__(kThreads, 1) ltl_tc_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<DT, ENC, BATCH, SW, false, false>(p);
+  ltl_tc_body<DT, ENC, BATCH, SW, false, false, false, false, false, false, 0, OF>(p);
 }
 
 // One bit per cell: the same body under its own name, so that a profiler can
@@ -1548,9 +1588,9 @@ __global__ void __launch_bounds__(kThreads, 1) ltl_big16_kernel(const __grid_con
 
 // Several steps of a single instance in one cooperative launch (separate
 // instantiations, so that the one-step kernels carry none of it).
-template <int DT, bool ENC, bool SW, bool BITS>
+template <int DT, bool ENC, bool SW, bool BITS, bool OF>
 __global__ void __launch_bounds__(kThreads, 1) ltl_tc_multi_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<DT, ENC, false, SW, BITS, true>(p);
+  ltl_tc_body<DT, ENC, false, SW, BITS, true, false, false, false, false, 0, OF>(p);
 }
 
 // ---------------------------------------------------------------------------
@@ -1880,13 +1920,13 @@ static cudaError_t launch_pdl(void (*kern)(TcParams), int grid, size_t smem, cud
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-template <int DT, bool ENC, bool BATCH, bool SW = false, bool BITS = false>
+template <int DT, bool ENC, bool BATCH, bool SW = false, bool BITS = false, bool OF = false>
 static cudaError_t launch_one(const TcParams &p, int grid, cudaStream_t s) {
   static bool configured = false;
-  const size_t smem = tc::Layout<DT, ENC, SW, BITS>::kDyn;
+  const size_t smem = tc::Layout<DT, ENC, SW, BITS, false, false, false, OF>::kDyn;
   void (*kern)(TcParams);
   if constexpr (BITS) kern = tc::ltl_bits_kernel;
-  else kern = tc::ltl_tc_kernel<DT, ENC, BATCH, SW>;
+  else kern = tc::ltl_tc_kernel<DT, ENC, BATCH, SW, OF>;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1895,7 +1935,7 @@ static cudaError_t launch_one(const TcParams &p, int grid, cudaStream_t s) {
   if constexpr (!BATCH) {
     if (p.n_steps > 1) {  // CTAs wait on one another: all must be resident at once
       static bool configured_multi = false;
-      void (*multi)(TcParams) = tc::ltl_tc_multi_kernel<DT, ENC, SW, BITS>;
+      void (*multi)(TcParams) = tc::ltl_tc_multi_kernel<DT, ENC, SW, BITS, OF>;
       if (!configured_multi) {
         cudaError_t e = cudaFuncSetAttribute(multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1914,12 +1954,13 @@ static cudaError_t launch_one(const TcParams &p, int grid, cudaStream_t s) {
 // passes the tensor maps whose window boxes are 144 rows high.  bits: the
 // grid is stored one bit per cell (FP8, two-state rules, single instance);
 // the caller passes the 48 x 160 window and 16 x 128 tile maps of the packed
-// buffers.
+// buffers.  Two-state FP8 grids of r = 8 .. 15 take the offset kernel.
 cudaError_t tc_launch(const TcParams &p, int dt, bool encode, bool sw, bool bits, int grid, cudaStream_t s) {
   if (bits) return launch_one<1, true, false, false, true>(p, grid, s);
   if (dt == 1) return launch_one<0, true, false>(p, grid, s);
   if (encode) return launch_one<1, true, false>(p, grid, s);
   if (sw) return launch_one<1, false, false, true>(p, grid, s);
+  if (tc::pass2_offset(p.rule.r)) return launch_one<1, false, false, false, false, true>(p, grid, s);
   return launch_one<1, false, false>(p, grid, s);
 }
 
