@@ -225,7 +225,7 @@ int launch_planes(cat_instance *h, int in, int64_t n_steps, int64_t *taken, cuda
   const cat::PlanesGrid g = planes_grid(h, in);
   const cat::TilePlan plan = cat::planes_tile_plan(g, n_steps);
   *taken = plan.steps > 0 ? plan.steps : 1;
-  if (h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
+  if (h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, false, s);
   if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return CAT_OK;
@@ -270,7 +270,7 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
     }
     cudaError_t e = cudaSuccess;
     if (h->ghost)
-      e = t == 0 ? cat::ghost_fill_launch(h->buf[h->cur], h->pitch, h->H, h->W, h->ghost, s)
+      e = t == 0 ? cat::ghost_fill_launch(h->buf[h->cur], h->pitch, h->H, h->W, h->ghost, false, s)
                  : cat::ghost_bits_launch(bits(at, off), h->pitch, h->H, h->W, s);
     if (t + k == n_steps) {
       g.out = h->origin(last);
@@ -298,7 +298,7 @@ int launch_step(cat_instance *h, int in, int32_t *sums, int64_t sums_ld, cudaStr
   }
   if (h->kernel == CAT_KERNEL_TCGEN05) {
     if (h->ghost) {  // periodic: refresh the input's ghost frame first
-      e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, s);
+      e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, true, s);
       if (e != cudaSuccess) return cuda_fail(e, "ghost-frame launch");
     }
     cat::TcParams p;

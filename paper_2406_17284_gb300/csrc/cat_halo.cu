@@ -71,45 +71,88 @@ __global__ void ghost_fill_kernel(uint8_t *base, int64_t pitch, int H, int W, in
   }
 }
 
+// The same for H, W >= 16, which is nearly every grid, in as few instructions
+// as that takes, a thread per cell: frame position f of 32 (0 .. 15 before the
+// grid, 16 .. 31 after it) is framed coordinate f or N + f and wraps to N + f
+// or f.  The step kernel leaves none of these instructions in an SM's cache,
+// so their number is the kernel's time: loops over a thread's cells and a
+// remainder for each (above) took longer than the step itself where W % 16 is
+// not 0, and whole chunks shifted into place in registers hardly less
+// (4600^2, r = 5, tensor-core steps back to back: 64 and 31 us a step; so
+// 14.8, and 13.1 with no frame to refresh).  Chunks of 16 cells to a thread
+// where W % 16 is 0 are no better (8192^2, r = 5 / 12 / 16: 36.0 / 34.4 / 38.5
+// against 33.1 / 33.5 / 35.4).
+// early: the next kernel may start its set-up beside the previous one's end.
+// The tensor-core step gains by that (256^2: 5.6 against 6.4), the bit-plane
+// steps, whose blocks only wait, lose (2048^2, r = 12, two steps: 10.1 against 9.1).
+__device__ __forceinline__ int frame_at(int f, int n) { return f < 16 ? f : n + f; }
+__device__ __forceinline__ int frame_from(int f, int n) { return f < 16 ? n + f : f; }
+
+__global__ void ghost_frame_kernel(uint8_t *base, int64_t pitch, int H, int W, unsigned row_blocks, bool early) {
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blockIdx.x < row_blocks) {   // the grid's columns of the 32 frame rows: chunks of 16, then single cells
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x, chunks = (unsigned)W / 16, per = chunks + W % 16;
+    const unsigned f = i / per, k = i - f * per;
+    if (f >= 32) return;
+    uint8_t *dst = base + frame_at((int)f, H) * pitch + 16;
+    const uint8_t *src = base + frame_from((int)f, H) * pitch + 16;
+    if (k < chunks) reinterpret_cast<uint4 *>(dst)[k] = reinterpret_cast<const uint4 *>(src)[k];
+    else dst[15 * (int64_t)chunks + k] = src[15 * (int64_t)chunks + k];
+  } else {                         // the frame's cells beside the grid's rows, and the corners
+    const int64_t i = (int64_t)(blockIdx.x - row_blocks) * blockDim.x + threadIdx.x, q = i >> 5;
+    if (q >= H + 32) return;
+    const int f = (int)(i & 31);
+    const int64_t to = q < H ? q + 16 : frame_at((int)(q - H), H), from = q < H ? q + 16 : frame_from((int)(q - H), H);
+    base[to * pitch + frame_at(f, W)] = base[from * pitch + frame_from(f, W)];
+  }
+}
+
 // The ghost frame of a one-bit grid (the states between the steps of one call):
 // position p of a row holds cell p - 16, so the grid's cells start in the middle
-// of word 0 and the frame's right cells end the row.  Items: the frame cells
-// beside each grid row (two 16-bit fields, one thread per row), and the words
-// of the 32 frame rows, each made from its source row's grid cells only.
-__global__ void ghost_bits_kernel(uint32_t *base, int64_t pitch_words, int H, int W, int words) {
+// of word 0 and the frame's right cells end the row.  Items, again in few
+// instructions: the words with cells beside the grid's columns, a thread per
+// row of the frame, and the other words of the 32 frame rows; each made from
+// its source row's grid cells only.
+__global__ void ghost_bits_kernel(uint32_t *base, int64_t pitch_words, int H, int W, int words, unsigned row_blocks) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int wl = W / 32, sl = W % 32;                  // cells W - 16 .. W - 1 start here
-  const int wr = (W + 16) / 32, sr = (W + 16) % 32;    // cells W .. W + 15 start here
-  const int64_t n_all = H + 32 * (int64_t)words;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_all; i += (int64_t)gridDim.x * blockDim.x) {
-    const bool beside = i < H;
-    const int k = beside ? 0 : (int)((i - H) / words), w = beside ? 0 : (int)(i - H - (int64_t)k * words);
-    const int row = beside ? (int)i : k < 16 ? k - 16 : H + k - 16;
-    const uint32_t *src = base + (int64_t)wrap32(row, H) * pitch_words;
-    const uint32_t first = src[0];
-    const uint32_t left = __funnelshift_r(src[wl], src[wl + 1], sl) & 0xFFFFu, right = first >> 16;
-    const uint32_t low = (1u << sr) - 1u;              // the grid's cells of word wr
-    const uint32_t w0 = (first & 0xFFFF0000u) | left, w1 = (src[wr] & low) | (right << sr);
-    const uint32_t w2 = sr > 16 ? right >> (32 - sr) : 0u;
-    uint32_t *dst = base + (int64_t)row * pitch_words;
-    if (beside) {
-      dst[0] = w0;
-      dst[wr] = w1;
-      if (wr + 1 < words) dst[wr + 1] = w2;
-    } else {
-      dst[w] = w == 0 ? w0 : w == wr ? w1 : w == wr + 1 ? w2 : src[w];
-    }
+  const int wr = (W + 16) / 32;                        // cells W .. W + 15 start in this word
+  const bool middle = blockIdx.x < row_blocks;
+  int64_t q = (int64_t)(blockIdx.x - (middle ? 0u : row_blocks)) * blockDim.x + threadIdx.x;
+  int w = 0;
+  if (middle) {
+    const unsigned k = (unsigned)q / (unsigned)words;
+    w = (int)((unsigned)q - k * (unsigned)words);
+    q = H + k;
+    if (w == 0 || w >= wr) return;
   }
+  if (q >= H + 32) return;
+  const int f = (int)(q - H);
+  const int row = f < 0 ? (int)q : f < 16 ? f - 16 : H + f - 16;
+  const uint32_t *src = base + (f < 0 ? row : wrap32(row, H)) * pitch_words;
+  uint32_t *dst = base + row * pitch_words;
+  if (middle) {
+    dst[w] = src[w];
+    return;
+  }
+  const int sl = W % 32, sr = (W + 16) % 32;
+  const uint32_t first = src[0], right = first >> 16;
+  const uint32_t left = __funnelshift_r(src[W / 32], src[W / 32 + 1], sl) & 0xFFFFu;   // cells W - 16 .. W - 1
+  const uint32_t last = (src[wr] & ((1u << sr) - 1u)) | (right << sr);                 // the grid's last cells, then the frame's
+  dst[0] = (first & 0xFFFF0000u) | left;
+  dst[wr] = last;
+  if (wr + 1 < words) dst[wr + 1] = sr > 16 ? right >> (32 - sr) : 0u;
 }
 
 }  // namespace
 
 cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W, cudaStream_t s) {
   const int words = (int)((W + 32 + 31) / 32), threads = 256;
-  const int64_t want = (H + 32 * (int64_t)words + threads - 1) / threads;
+  const int64_t rows = (32 * (int64_t)words + threads - 1) / threads, sides = (H + 32 + threads - 1) / threads;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(want < 4096 ? want : 4096));
+  cfg.gridDim = dim3((unsigned)(rows + sides));
   cfg.blockDim = dim3(threads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -118,18 +161,21 @@ cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, ghost_bits_kernel, reinterpret_cast<uint32_t *>(row0), pitch / 4, (int)H, (int)W,
-                            words);
+                            words, (unsigned)rows);
 }
 
 // Launched programmatically dependent on the previous kernel in the stream
 // (see ghost_fill_kernel); the tcgen05 step launched after it is in turn
 // dependent on it.
-cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, cudaStream_t s) {
-  const int64_t n = 2 * (int64_t)G * ((W + 15) / 16) + 2 * H + 4 * (int64_t)G * G;
+cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, bool early, cudaStream_t s) {
   const int threads = 256;
+  const bool small = H < 16 || W < 16 || G != 16;
+  const int64_t rows = (32 * (W / 16 + W % 16) + threads - 1) / threads;
+  const int64_t sides = ((H + 32) * 32 + threads - 1) / threads;
+  const int64_t n = 2 * (int64_t)G * ((W + 15) / 16) + 2 * H + 4 * (int64_t)G * G;
   const int64_t want = (n + threads - 1) / threads;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(want < 4096 ? want : 4096));
+  cfg.gridDim = dim3((unsigned)(!small ? rows + sides : want < 4096 ? want : 4096));
   cfg.blockDim = dim3(threads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -137,7 +183,9 @@ cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, ghost_fill_kernel, base, pitch, (int)H, (int)W, G);
+  if (small) return cudaLaunchKernelEx(&cfg, ghost_fill_kernel, base, pitch, (int)H, (int)W, G);
+  return cudaLaunchKernelEx(&cfg, ghost_frame_kernel, base, pitch, (int)H, (int)W,
+                            (unsigned)rows, early);
 }
 
 }  // namespace cat

@@ -150,8 +150,9 @@ cudaError_t unpack_nib_launch(const uint8_t *src, int64_t spitch, uint8_t *dst, 
 
 // Periodic boundary (cat_halo.cu): fills the G-cell ghost frame around the
 // H x W grid whose cell (0, 0) is at base + G * pitch + G with the cells the
-// frame wraps to.
-cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, cudaStream_t s);
+// frame wraps to.  early: the next kernel's set-up may begin before the previous
+// kernel's end.
+cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, bool early, cudaStream_t s);
 // The same for a one-bit grid whose rows start at cell -16 (G = 16; W >= 64);
 // row0: row 0 of the grid.
 cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W, cudaStream_t s);
