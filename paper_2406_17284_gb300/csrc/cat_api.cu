@@ -236,9 +236,13 @@ int launch_planes(cat_instance *h, int in, int64_t n_steps, int64_t *taken, cuda
 // whichever of the two buffers holds no state that is still needed (a row of
 // bits takes an eighth of a row of cells, so two fit beside each other; bytes
 // outside the grid's rows are not touched).
-bool use_packed_steps(const cat_instance *h, int64_t n_steps) {
+bool packed_steps_possible(const cat_instance *h, int64_t n_steps) {
   return n_steps >= 2 && h->auto_choice && h->inject == 0 && h->storage == CAT_STORE_U8 && h->rule.C == 2 &&
          h->rule.nbhd == 'M' && h->rule.r <= 16 && h->W >= 64;
+}
+
+bool use_packed_steps(const cat_instance *h, int64_t n_steps) {
+  return packed_steps_possible(h, n_steps) && cat::planes_steps_preferred(planes_grid(h, 0), n_steps);
 }
 
 // Byte offset of a row's second row of bits.
@@ -943,10 +947,11 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   // One pass over the instances (thousands, in no order in memory).
   bool all_tc = true;   // Moore, zero boundary, uint8 storage, no FP4: other instances step one by one
   // Several steps of grids whose options are all left to the library, on bit
-  // planes: from four steps and 2^25 cells on (512 grids with sides up to 512 /
-  // 1024 / 2048, us for 4 steps: tiles 125 / 206 / 432, planes 128 / 199 / 406;
-  // for 16 steps: 475 / 799 / 1698 against 426 / 582 / 1227; 100 grids up to
-  // 1024: 80 against 110).  A captured call keeps to the tiles, one launch per
+  // planes: from six steps and 2^25 cells on, or four and 2^27 (512 grids with
+  // sides up to 900 / 1400 / 2048, 54 / 102 / 179 million cells, us for 4 steps:
+  // tiles 171 / 270 / 423, planes 185 / 274 / 409; for 6: 251 / 401 / 627
+  // against 244 / 364 / 547; for 12: 490 / 788 / 1241 against 420 / 635 / 959).
+  // A captured call keeps to the tiles, one launch per
   // step, since the planes need the radii side by side.
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   CAT_CUDA(cudaStreamIsCapturing(s, &cs));
@@ -957,13 +962,13 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
     const cat_instance *h = hs[i];
     all_tc &= h->kernel == CAT_KERNEL_TCGEN05 && h->ghost == 0 && h->storage == CAT_STORE_U8 &&
               h->rule.nbhd == 'M' && !wide_tile(h) && h->dtype != CAT_DTYPE_FP4_E2M1;
-    packed &= use_packed_steps(h, n_steps);
+    packed &= packed_steps_possible(h, n_steps);
     cells += h->H * h->W;
     one_device &= h->dev.id == hs[0]->dev.id;
     one_dtype &= h->dtype == hs[0]->dtype;
     small &= h->H <= 128 * 32767 && h->W <= 128 * 32767;
   }
-  packed &= cells >= 1 << 25;
+  packed &= cells >= (n_steps >= 6 ? 1 << 25 : 1 << 27);
   std::unique_lock<std::mutex> lk(g_plan_mu);
   BatchPlan *pl = nullptr;
   for (BatchPlan *c : g_plans)
@@ -1006,15 +1011,15 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   bool in_sync = true;
   for (int32_t i = 0; i < count; ++i) in_sync &= hs[i]->cur == (pl->cur0[i] ^ (int)(pl->steps_done & 1));
   if (!in_sync && (rc = upload_instances(pl))) return rc;
-  const int par = (int)(pl->steps_done & 1), kind = par + (packed ? 2 : 0);
   if (packed && !pl->packed) {
     const cudaError_t e = cat::planes_batch_create(batch_items(pl), hs[0]->dev.sms, &pl->packed);
     if (e != cudaSuccess) {
       (void)cudaGetLastError();
-      return e == cudaErrorMemoryAllocation ? fail(CAT_ERR_OOM, "allocation of the batch tables failed")
-                                            : cuda_fail(e, "batch plan");
+      if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "batch plan");
+      packed = false;   // no room for its tables: the tiles serve the call
     }
   }
+  const int par = (int)(pl->steps_done & 1), kind = par + (packed ? 2 : 0);
   if (cs != cudaStreamCaptureStatusNone) {
     if ((rc = launch_batch_steps(pl, n_steps, pl->steps_done, s))) return rc;
   } else {

@@ -179,6 +179,9 @@ struct PlanesGrid {
 };
 // Whether a step from and to storage_in is faster this way.
 bool planes_preferred(const PlanesGrid &g);
+// Whether n_steps >= 2 steps of a two-state uint8 grid are faster this way, the
+// states between them kept as bits.
+bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps);
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s);
 // Several steps per launch on tiles in shared memory (cat_planes_tile.cuh; two
 // states): the split for a launch with n_left steps to go; steps = 0 where

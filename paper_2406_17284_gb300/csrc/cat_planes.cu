@@ -132,21 +132,52 @@ int64_t tile_smem(const PlanesGrid &g, const TilePlan &t) {
 //   one bit per cell      every radius: 32768^2, r = 2 / 16: 147 / 320 against
 //                         the former bit-sliced kernel's 224 and tcgen05's 594
 //   four bits per cell    every radius: 24576^2, C 16, r = 10: 297 against 435
-//   uint8, C > 2          16384^2, r = 1 / 10 / 15: 117 / 156 / 175 against 180
-//                         / 182 / 182; 4096^2: 9.0 / 17.7 / 18.9 against 18.9 /
-//                         19.2 / 19.3; 2048^2, r = 8 / 10 / 15: 10.9 / 14 / 14
-//                         against 11: up to r = 15, but not where a strip is
-//                         shorter than the 2r rows before it
-//   uint8, two states     only where a launch's latency counts: 1024^2, r = 1:
-//                         2.9 against 6.5; 4096^2, r = 4 / 9 / 16: 9.5 / 14.8 /
-//                         18.4 against 11.6 / 14.8 / 14.8; 16384^2, r = 4:
-//                         111 against 97
+//   uint8, C > 2          up to a radius that falls while the strips get too
+//                         short for the 2r rows before them and rises again with
+//                         the size: 1024^2, r = 12 / 13: 5.9 / 6.6 against 6.0;
+//                         2048^2, r = 5 / 6: 7.4 / 8.0 against 7.8; 4096^2, r =
+//                         7 / 8: 14.4 / 17.1 against 15.9 / 16.1; 8192^2, r = 12
+//                         / 13: 47.1 / 49.5 against 49.3; 16384^2, r = 1 / 10 /
+//                         15: 118 / 155 / 174 against 178 / 180 / 180
+//   uint8, two states     only where a launch's latency counts: 1024^2, r = 1 /
+//                         9 / 15: 2.2 / 3.7 / 4.3 against 4.6; 2048^2, r = 9 /
+//                         10: 5.6 / 5.8 against 5.7; 4096^2, r = 4 / 5: 9.2 /
+//                         10.3 against 10.2; 16384^2, r = 4: 111 against 96.
+//                         The frame that a torus refreshes first costs a short
+//                         step more: 1024^2, r = 7 / 9: 5.5 / 5.8 against 5.7;
+//                         2048^2, r = 4 / 6: 6.4 / 7.5 against 7.4
 bool planes_preferred(const PlanesGrid &g) {
   int kind;
   if (!find(g, &kind).fn) return false;
   if (g.storage_in != CAT_STORE_U8) return true;
-  if (g.rule.C > 2) return g.rule.r <= 15 && (g.rule.r <= 8 || g.H * g.W <= (1 << 20) || g.H * g.W >= (1 << 24));
-  return g.rule.r <= 9 && g.H * g.W <= (1 << 24);
+  const int64_t m = (g.H * g.W + (1 << 20) - 1) >> 20;   // 2^20 cells
+  if (g.rule.C > 2) return g.rule.r <= (m <= 1 ? (g.frame ? 9 : 12) : m < 16 ? 5 : m < 30 ? 7 : m < 128 ? 12 : 15);
+  if (g.frame) return g.rule.r <= (m <= 1 ? 7 : m <= 16 ? 4 : 0);
+  return g.rule.r <= (m <= 1 ? 16 : m <= 4 ? 9 : m <= 16 ? 4 : 0);
+}
+
+// Several steps of a two-state uint8 grid (us per step, tensor-core steps
+// last).  Reading and writing bits is worth most on large grids and with many
+// steps between the bytes at both ends; a wave of strips fits grids of 10 to 36
+// 2^20 cells badly, and a torus pays for a frame per launch:
+//   4096^2, n = 2 / 4 / 8   r = 4: 9.4 / 7.3 / 5.8 and 10.2; r = 7: 11.2 / 7.9 /
+//                           7.7 and 10.6; r = 10: 11.7 / 9.6 / 9.4 and 11.1;
+//                           r = 12: 12.0 / 11.5 / 11.3 and 11.1
+//   5792^2, n = 2 / 4 / 8   r = 8: 18.5 / 16.5 / 15.4 and 17.9; r = 16: 22.0 /
+//                           19.9 / 18.7 and 19.5
+//   7000^2, n = 2 / 3       r = 16: 27.8 / 26.0 and 26.1
+//   8192^2, n = 2 / 8       r = 4: 20.1 / 17.3 and 28.3; r = 16: 33.5 / 28.2 and 33.3
+//   16384^2, n = 2 / 8      r = 12: 92.6 / 75.5 and 106.4
+//   torus, n = 8            2048^2, r = 12: 9.0 and 7.5; 4096^2, r = 7 / 12: 10.9
+//                           / 14.6 and 13.0; 5792^2, r = 12: 17.9 and 19.6
+bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps) {
+  const int64_t m = (g.H * g.W + (1 << 20) - 1) >> 20;
+  const int r = g.rule.r;
+  if (g.frame) return r <= 7 || (m >= 30 && n_steps >= (m >= 64 ? 2 : r == 16 ? 8 : 3));
+  if (r <= 7) return m <= 4 || m > 16 || n_steps >= (r == 7 ? 4 : r >= 5 ? 3 : 2);
+  if (m <= 10 || m > 50) return true;
+  if (m <= 24) return r <= 10 && n_steps >= 4;
+  return n_steps >= (m <= 36 ? (r == 16 ? 8 : 4) : (r == 16 ? 3 : 2));
 }
 
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
@@ -226,8 +257,7 @@ struct PlanesBatch {
   unsigned pack_blocks = 0;               // blocks that pack or unpack all grids
   const planes::BatchBlock *pack_first = nullptr;
   std::vector<planes::BatchGrid> grids;
-  planes::BatchGrid *d_grids = nullptr;
-  planes::BatchBlock *d_blocks = nullptr;
+  planes::BatchGrid *d_grids = nullptr;   // the lists of blocks follow in the same allocation
 };
 
 namespace {
@@ -280,6 +310,10 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
   }
   std::vector<planes::BatchBlock> blocks;
   std::vector<size_t> first;
+  size_t most = planes::kMaxR * planes::kBatchWarps;
+  for (const planes::BatchGrid &g : b->grids)
+    most += (size_t)((int64_t)g.strips * g.seg / planes::kOut + (int64_t)g.H * g.seg / planes::kPackWords + 2);
+  blocks.reserve(most);
   for (int r = planes::kMaxR; r >= 1; --r) {   // (the larger radii, whose blocks take longest, first)
     int range = 0;
     while (r > planes::kRangeEnd[range]) ++range;
@@ -303,15 +337,17 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
     for (int64_t k = 0; k * planes::kPackWords < words; ++k) blocks.push_back(planes::BatchBlock{(int32_t)i, (int32_t)k});
   }
   b->pack_blocks = (unsigned)(blocks.size() - pack_at);
+  const size_t grid_bytes = (sizeof(planes::BatchGrid) * b->grids.size() + 255) / 256 * 256;
+  const size_t block_bytes = sizeof(planes::BatchBlock) * blocks.size();
   cudaError_t e = blocks.size() > 0x7fffffffu ? cudaErrorInvalidValue
-                                              : cudaMalloc(&b->d_grids, sizeof(planes::BatchGrid) * b->grids.size());
-  if (e == cudaSuccess) e = cudaMalloc(&b->d_blocks, sizeof(planes::BatchBlock) * blocks.size());
-  if (e == cudaSuccess)
-    e = cudaMemcpy(b->d_blocks, blocks.data(), sizeof(planes::BatchBlock) * blocks.size(), cudaMemcpyHostToDevice);
+                                              : cudaMalloc(&b->d_grids, grid_bytes + block_bytes);
+  planes::BatchBlock *d_blocks =
+      reinterpret_cast<planes::BatchBlock *>(reinterpret_cast<uint8_t *>(b->d_grids) + grid_bytes);
+  if (e == cudaSuccess) e = cudaMemcpy(d_blocks, blocks.data(), block_bytes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = planes_batch_update(b, items);
-  b->pack_first = b->d_blocks + pack_at;
+  b->pack_first = d_blocks + pack_at;
   for (size_t c = 0; c < b->chains.size() && e == cudaSuccess; ++c) {
-    b->chains[c].first = b->d_blocks + first[c];
+    b->chains[c].first = d_blocks + first[c];
     const planes::BatchFn fn = planes::batch_kernel(b->chains[c].range);
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e == cudaSuccess)
@@ -328,7 +364,6 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
 void planes_batch_free(PlanesBatch *b) {
   if (!b) return;
   cudaFree(b->d_grids);
-  cudaFree(b->d_blocks);
   delete b;
 }
 

@@ -72,12 +72,31 @@ def test_planes_on_a_torus(cat, C):
             check(cat, H, W, inputs.scaled_rule(r, C=C), 0, boundary=1)
 
 
-@pytest.mark.parametrize("r", [1, 7, 16])
+@pytest.mark.parametrize("r", [1, 4, 7])
 def test_packed_steps_on_a_torus(cat, r):
     """Several steps in one call: the one-bit ghost frame at every word offset of W."""
     for H, W in [(5, 64), (20, 79), (33, 80), (40, 81), (64, 95), (70, 96), (33, 1031)]:
         for n in (2, 3, 6):
             check(cat, H, W, inputs.scaled_rule(r, M=1), 0, boundary=1, steps=n)
+
+
+@pytest.mark.parametrize("r", [8, 16])
+@pytest.mark.parametrize("H,W", [(5611, 5807), (33, 1048577)])
+def test_packed_steps_on_a_large_torus(cat, r, H, W):
+    """The larger radii take the bits from 30 * 2^20 cells on: against the
+    tensor-core kernel's steps from the same state."""
+    import torch
+    rule, host = inputs.scaled_rule(r), board(H, W, 2, r)
+    a = cat.Grid(H, W, rule, kernel="auto", dtype="auto", boundary=1)
+    b = cat.Grid(H, W, rule, kernel="tcgen05", dtype="fp8", boundary=1)
+    try:
+        for g in (a, b):
+            g.set_state(host)
+            g.step(9)
+        assert torch.equal(a.state_tensor(), b.state_tensor())
+    finally:
+        a.close()
+        b.close()
 
 
 @pytest.mark.parametrize("C", [2, 16])
@@ -156,7 +175,7 @@ def test_packed_batch_of_uneven_grids(cat):
         assert torch.equal(big.state_tensor(), ref.state_tensor()), done
     try:
         done = 0
-        for n in (4, 5, 1, 7, 4):
+        for n in (6, 7, 1, 9, 4):
             cat.cat_batch_step(handles, n)
             ref.step(n)
             done += n
