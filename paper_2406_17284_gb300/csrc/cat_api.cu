@@ -389,12 +389,12 @@ struct BatchPlan {
   bool encode = false;
   bool sw = false;            // every instance qualifies for the short-window kernel
   cat::PlanesBatch *packed = nullptr;   // tables for calls on bit planes, made by the first such call
-  cat::BatchInst *d_inst = nullptr;
+  cat::BatchInst *d_inst = nullptr;     // tables of the tiles, likewise (build_tiles)
   cat::BatchTile *d_tiles = nullptr;
   int n_tiles = 0, grid = 0;
   cudaGraphExec_t exec[4] = {};   // by start parity, the calls on bit planes after the others
   int64_t exec_steps[4] = {};
-  cudaStream_t capture_stream = nullptr;
+  cudaStream_t capture_stream = nullptr;   // with those tables
 };
 
 std::mutex g_plan_mu;
@@ -432,18 +432,8 @@ std::vector<cat::PlanesBatchItem> batch_items(const BatchPlan *pl) {
   return items;
 }
 
-// (Re)writes the instance table of a plan from the handles' current state.
-int upload_instances(BatchPlan *pl) {
-  CAT_CUDA(cudaDeviceSynchronize());  // earlier launches of this plan may still read the table
-  pl->steps_done = 0;
-  for (int i = 0; i < 4; ++i) {
-    if (pl->exec[i]) cudaGraphExecDestroy(pl->exec[i]);
-    pl->exec[i] = nullptr;
-    pl->exec_steps[i] = 0;
-  }
-  pl->cur0.resize(pl->hs.size());
-  for (size_t i = 0; i < pl->hs.size(); ++i) pl->cur0[i] = pl->hs[i]->cur;
-  if (pl->packed) CAT_CUDA(cat::planes_batch_update(pl->packed, batch_items(pl)));
+// The instance table of a plan's tiles, from the handles' state at cur0.
+std::vector<cat::BatchInst> instance_table(const BatchPlan *pl) {
   std::vector<cat::BatchInst> inst(pl->hs.size());
   memset(inst.data(), 0, inst.size() * sizeof(cat::BatchInst));
   for (size_t i = 0; i < pl->hs.size(); ++i) {
@@ -456,10 +446,27 @@ int upload_instances(BatchPlan *pl) {
     inst[i].rule = h->rd;
     inst[i].H = (int32_t)h->H;
     inst[i].W = (int32_t)h->W;
-    inst[i].cur = h->cur;
+    inst[i].cur = pl->cur0[i];
     inst[i].err = h->d_err;
   }
-  CAT_CUDA(cudaMemcpy(pl->d_inst, inst.data(), inst.size() * sizeof(cat::BatchInst), cudaMemcpyHostToDevice));
+  return inst;
+}
+
+// Takes the handles' current state as the plan's start, in the tables that it has.
+int upload_instances(BatchPlan *pl) {
+  CAT_CUDA(cudaDeviceSynchronize());  // earlier launches of this plan may still read the tables
+  pl->steps_done = 0;
+  for (int i = 0; i < 4; ++i) {
+    if (pl->exec[i]) cudaGraphExecDestroy(pl->exec[i]);
+    pl->exec[i] = nullptr;
+    pl->exec_steps[i] = 0;
+  }
+  for (size_t i = 0; i < pl->hs.size(); ++i) pl->cur0[i] = pl->hs[i]->cur;
+  if (pl->packed) CAT_CUDA(cat::planes_batch_update(pl->packed, batch_items(pl)));
+  if (pl->d_inst) {
+    const std::vector<cat::BatchInst> inst = instance_table(pl);
+    CAT_CUDA(cudaMemcpy(pl->d_inst, inst.data(), inst.size() * sizeof(cat::BatchInst), cudaMemcpyHostToDevice));
+  }
   return CAT_OK;
 }
 
@@ -469,12 +476,25 @@ int build_plan(const cat_handle_t *hs, int32_t count, BatchPlan **out) {
   pl->hs.assign(hs, hs + count);
   pl->dtype = hs[0]->dtype;
   pl->encode = false;
-  for (int32_t i = 0; i < count; ++i) pl->encode |= hs[i]->rule.C > 2;
   pl->sw = true;
-  for (int32_t i = 0; i < count; ++i) pl->sw &= short_window(hs[i]);
+  for (int32_t i = 0; i < count; ++i) {
+    pl->encode |= hs[i]->rule.C > 2;
+    pl->sw &= short_window(hs[i]);
+    pl->cur0.push_back(hs[i]->cur);
+  }
+  *out = pl;
+  return CAT_OK;
+}
+
+// The tables of a plan's tiles, made by the first call that takes them: also a
+// captured one after calls on bit planes, so the copies go over a stream of the
+// plan's own, outside the capture.
+int build_tiles(BatchPlan *pl) {
+  if (pl->d_inst) return CAT_OK;
+  const std::vector<cat_instance *> &hs = pl->hs;
   // work-list: instances ordered by radius, tiles row-major within an instance
-  std::vector<int> order(count);
-  for (int32_t i = 0; i < count; ++i) order[i] = i;
+  std::vector<int> order(hs.size());
+  for (size_t i = 0; i < hs.size(); ++i) order[i] = (int)i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hs[a]->rule.r < hs[b]->rule.r; });
   std::vector<cat::BatchTile> tiles;
   for (int i : order) {
@@ -482,19 +502,30 @@ int build_plan(const cat_handle_t *hs, int32_t count, BatchPlan **out) {
     for (int64_t y = 0; y < ty; ++y)
       for (int64_t x = 0; x < tx; ++x) tiles.push_back(cat::BatchTile{i, (int16_t)y, (int16_t)x});
   }
-  if (tiles.size() > (size_t)INT32_MAX) { delete pl; return fail(CAT_ERR_UNSUPPORTED, "batch too large"); }
+  if (tiles.size() > (size_t)INT32_MAX) return fail(CAT_ERR_UNSUPPORTED, "batch too large");
   pl->n_tiles = (int)tiles.size();
   pl->grid = std::min(pl->n_tiles, hs[0]->dev.sms);
-  cudaError_t e = cudaMalloc(&pl->d_inst, sizeof(cat::BatchInst) * count);
+  const std::vector<cat::BatchInst> inst = instance_table(pl);
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CAT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+  cudaError_t e = pl->capture_stream ? cudaSuccess : cudaStreamCreateWithFlags(&pl->capture_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMalloc(&pl->d_tiles, sizeof(cat::BatchTile) * tiles.size());
+  if (e == cudaSuccess) e = cudaMalloc(&pl->d_inst, sizeof(cat::BatchInst) * inst.size());
   if (e == cudaSuccess)
-    e = cudaMemcpy(pl->d_tiles, tiles.data(), sizeof(cat::BatchTile) * tiles.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&pl->capture_stream, cudaStreamNonBlocking);
-  if (e != cudaSuccess) { free_plan(pl); return cuda_fail(e, "batch plan"); }
-  int rc = upload_instances(pl);
-  if (rc) { free_plan(pl); return rc; }
-  *out = pl;
-  return CAT_OK;
+    e = cudaMemcpyAsync(pl->d_tiles, tiles.data(), sizeof(cat::BatchTile) * tiles.size(), cudaMemcpyHostToDevice,
+                        pl->capture_stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(pl->d_inst, inst.data(), sizeof(cat::BatchInst) * inst.size(), cudaMemcpyHostToDevice,
+                        pl->capture_stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(pl->capture_stream);
+  if (e != cudaSuccess) {   // a later call tries again
+    cudaFree(pl->d_tiles);
+    cudaFree(pl->d_inst);
+    pl->d_tiles = nullptr;
+    pl->d_inst = nullptr;
+  }
+  CAT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+  return e == cudaSuccess ? CAT_OK : cuda_fail(e, "batch plan");
 }
 
 int launch_batch_steps(BatchPlan *pl, int64_t n_steps, int64_t start, cudaStream_t s) {
@@ -1019,6 +1050,7 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
       packed = false;   // no room for its tables: the tiles serve the call
     }
   }
+  if (!packed && (rc = build_tiles(pl))) return rc;
   const int par = (int)(pl->steps_done & 1), kind = par + (packed ? 2 : 0);
   if (cs != cudaStreamCaptureStatusNone) {
     if ((rc = launch_batch_steps(pl, n_steps, pl->steps_done, s))) return rc;

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>
+#include <cstring>
 #include <new>
 #include <vector>
 
@@ -274,12 +275,16 @@ planes::BatchParams batch_params(const PlanesBatch *b, const planes::BatchBlock 
 
 }  // namespace
 
-cudaError_t planes_batch_update(PlanesBatch *b, const std::vector<PlanesBatchItem> &items) {
+static void set_buffers(PlanesBatch *b, const std::vector<PlanesBatchItem> &items) {
   for (size_t i = 0; i < items.size(); ++i) {
     b->grids[i].buf[0] = items[i].buf[0];
     b->grids[i].buf[1] = items[i].buf[1];
     b->grids[i].cur = items[i].cur;
   }
+}
+
+cudaError_t planes_batch_update(PlanesBatch *b, const std::vector<PlanesBatchItem> &items) {
+  set_buffers(b, items);
   return cudaMemcpy(b->d_grids, b->grids.data(), sizeof(planes::BatchGrid) * b->grids.size(), cudaMemcpyHostToDevice);
 }
 
@@ -290,6 +295,7 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
   for (const PlanesBatchItem &q : items) warp_rows += (double)q.H * ((q.W + 31) / 32 + 1) / planes::kOut;
   const int64_t rows = std::max<int64_t>(32, std::min<int64_t>(512, (int64_t)(warp_rows / (kBatchFill * sms)) / 4 * 4));
   b->grids.resize(items.size());
+  std::vector<int32_t> of_radius[planes::kMaxR + 1];
   for (size_t i = 0; i < items.size(); ++i) {
     const PlanesBatchItem &q = items[i];
     planes::BatchGrid &g = b->grids[i];
@@ -302,6 +308,7 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
     g.strips = (int32_t)((q.H + g.rows - 1) / g.rows);
     g.second = q.second;
     g.r = q.rule.r;
+    of_radius[g.r].push_back((int32_t)i);
     const int planes = planes::kernel_bit1(q.rule.r).planes;
     set_bound(g.bound[planes::kSurviveLo], q.rule.s_lo, planes);
     set_bound(g.bound[planes::kSurviveHi], (int64_t)q.rule.s_lo + q.rule.s_w + 1, planes);
@@ -318,10 +325,9 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
     int range = 0;
     while (r > planes::kRangeEnd[range]) ++range;
     const size_t at = blocks.size();
-    for (size_t i = 0; i < items.size(); ++i) {
-      if (items[i].rule.r != r) continue;
+    for (const int32_t i : of_radius[r]) {
       const int64_t n = ((int64_t)b->grids[i].strips * b->grids[i].seg + planes::kOut - 1) / planes::kOut;
-      for (int64_t k = 0; k < n; ++k) blocks.push_back(planes::BatchBlock{(int32_t)i, (int32_t)k});
+      for (int64_t k = 0; k < n; ++k) blocks.push_back(planes::BatchBlock{i, (int32_t)k});
     }
     if (blocks.size() == at) continue;
     while (blocks.size() % planes::kBatchWarps) blocks.push_back(planes::BatchBlock{-1, 0});
@@ -343,8 +349,13 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
                                               : cudaMalloc(&b->d_grids, grid_bytes + block_bytes);
   planes::BatchBlock *d_blocks =
       reinterpret_cast<planes::BatchBlock *>(reinterpret_cast<uint8_t *>(b->d_grids) + grid_bytes);
-  if (e == cudaSuccess) e = cudaMemcpy(d_blocks, blocks.data(), block_bytes, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = planes_batch_update(b, items);
+  if (e == cudaSuccess) {   // (one copy: each waits for the device)
+    set_buffers(b, items);
+    std::vector<uint8_t> table(grid_bytes + block_bytes);
+    memcpy(table.data(), b->grids.data(), sizeof(planes::BatchGrid) * b->grids.size());
+    memcpy(table.data() + grid_bytes, blocks.data(), block_bytes);
+    e = cudaMemcpy(b->d_grids, table.data(), table.size(), cudaMemcpyHostToDevice);
+  }
   b->pack_first = d_blocks + pack_at;
   for (size_t c = 0; c < b->chains.size() && e == cudaSuccess; ++c) {
     b->chains[c].first = d_blocks + first[c];

@@ -175,19 +175,19 @@ def test_packed_batch_of_uneven_grids(cat):
         assert torch.equal(big.state_tensor(), ref.state_tensor()), done
     try:
         done = 0
-        for n in (6, 7, 1, 9, 4):
-            cat.cat_batch_step(handles, n)
+        for n, captured in ((6, False), (4, True), (7, False), (1, False), (9, False), (4, False), (2, True)):
+            if captured:   # (the first one comes before any call has taken the tiles)
+                s = torch.cuda.Stream()
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=s):
+                    cat.cat_batch_step(handles, n, s)
+                graph.replay()
+                torch.cuda.synchronize()
+            else:
+                cat.cat_batch_step(handles, n)
             ref.step(n)
             done += n
             compare(done)
-        s = torch.cuda.Stream()
-        graph = torch.cuda.CUDAGraph()
-        with torch.cuda.graph(graph, stream=s):
-            cat.cat_batch_step(handles, 4, s)
-        graph.replay()
-        torch.cuda.synchronize()
-        ref.step(4)
-        compare(done + 4)
         with pytest.raises(cat.CatError):
             cat.cat_batch_step(handles + handles[:1], 4)
     finally:
