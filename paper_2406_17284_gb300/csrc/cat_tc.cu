@@ -526,11 +526,9 @@ __device__ __forceinline__ uint32_t half_pair(float v) {
   return *reinterpret_cast<uint32_t *>(&h);
 }
 
-// `offset`: what the accumulator's counts lack (pass2_offset).
-__device__ __forceinline__ HalfRule make_half_rule(const RuleDev &R, float scale, int offset = 0) {
-  const float o = (float)offset;
-  auto lo_of = [o](int lo) { return lo > 2048 ? 4096.0f : (float)lo - o; };
-  auto hi_of = [o](int lo, int w) { return lo > 2048 ? 2048.0f : fminf((float)lo + (float)w, 2048.0f) - o; };
+__device__ __forceinline__ HalfRule make_half_rule(const RuleDev &R, float scale) {
+  auto lo_of = [](int lo) { return lo > 2048 ? 4096.0f : (float)lo; };
+  auto hi_of = [](int lo, int w) { return lo > 2048 ? 2048.0f : fminf((float)lo + (float)w, 2048.0f); };
   HalfRule h;
   h.bl2 = half_pair(lo_of(R.b_lo) * scale);
   h.bh2 = half_pair(hi_of(R.b_lo, R.b_w) * scale);
@@ -570,6 +568,36 @@ __device__ __forceinline__ uint32_t rule4_binary_h(uint32_t s01, uint32_t s23, u
   uint32_t neg;   // bytes 1, 3 of t01 and 5, 7 of t23 (the sign bytes), sign-replicated
   asm("prmt.b32 %0, %1, %2, 0xFDB9;" : "=r"(neg) : "r"(h2_bits(t01)), "r"(h2_bits(t23)));
   return ~neg & 0x01010101u;
+}
+
+// The same where no count is above 961 (r <= 15): S is in a range iff
+// |S - middle| <= half its width, both exact in f16 as multiples of half the
+// scale below 2^11, and so is every difference (equality gives +0; an empty
+// range has half width -1/2).  Two operations a range and pair instead of
+// three, so both ranges are tested for every cell and one logic operation
+// picks by the cell's byte: RULEFIG
+// (The fields of HalfRule hold middles, bl2 and sl2, and half widths then.)
+__device__ __forceinline__ HalfRule make_range_rule(const RuleDev &R, float scale, int offset) {
+  const float top = (float)((2 * R.r + 1) * (2 * R.r + 1)), o = (float)offset;
+  auto put = [&](int lo, int w, uint32_t &mid, uint32_t &half) {
+    const float l = (float)lo, h = fminf(l + (float)w, top);
+    mid = half_pair(l > h ? 0.0f : ((l + h) * 0.5f - o) * scale);
+    half = half_pair((l > h ? -0.5f : (h - l) * 0.5f) * scale);
+  };
+  HalfRule h;
+  put(R.b_lo, R.b_w, h.bl2, h.bh2);
+  put(R.s_lo, R.s_w, h.sl2, h.sh2);
+  return h;
+}
+
+__device__ __forceinline__ uint32_t rule4_range_h(uint32_t s01, uint32_t s23, uint32_t cw, const HalfRule &h) {
+  auto test = [](uint32_t s, uint32_t mid, uint32_t half) {
+    return h2_bits(__hsub2(as_h2(half), __habs2(__hsub2(as_h2(s), as_h2(mid)))));
+  };
+  uint32_t born, keep;   // 0xFF in the bytes of the cells out of the range
+  asm("prmt.b32 %0, %1, %2, 0xFDB9;" : "=r"(born) : "r"(test(s01, h.bl2, h.bh2)), "r"(test(s23, h.bl2, h.bh2)));
+  asm("prmt.b32 %0, %1, %2, 0xFDB9;" : "=r"(keep) : "r"(test(s01, h.sl2, h.sh2)), "r"(test(s23, h.sl2, h.sh2)));
+  return ~((cw & keep) | (~cw & born)) & 0x01010101u;
 }
 
 // Out-of-range flags (product signs) of four cells as a nibble, cell k in bit
@@ -819,6 +847,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   auto ctr_x = [](int tx0) { return BITS ? tx0 / 8 : NIB ? tx0 / 2 : tx0; };
   using G = Geo<SW, WIDE, BIG>;
   using T = Tm<DT, SW, WIDE, BIG>;
+  constexpr bool kRange = OF || SW;   // r <= 15 and two states: the epilogue's test by middle and half width
   constexpr bool DEC = T::kDec;       // D1 and D2 in separate regions, pass 2 on e4m3 digits
   constexpr int KW = BIG ? 192 : kWin;   // window columns = pass-1 K = pass-2 K
   constexpr int KS = KW / 32;            // K-steps of one e4m3 band product
@@ -1396,13 +1425,17 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     }
     bool ok = true;
     auto offset_of = [](const RuleDev &R) { return OF ? 16 * (2 * R.r + 1) : 0; };
-    HalfRule hr = make_half_rule(BATCH ? RuleDev{} : p.rule, kScale, BATCH ? 0 : offset_of(p.rule));
+    auto make_rule = [&](const RuleDev &R) {
+      if constexpr (kRange) return make_range_rule(R, kScale, offset_of(R));
+      else return make_half_rule(R, kScale);
+    };
+    HalfRule hr = make_rule(BATCH ? RuleDev{} : p.rule);
     TileSeq<BATCH, MS, G::kTS> seq(p, first, n_my);
     for (int j = 0; ok && j < n_all; ++j, seq.next(p)) {
       const int reg = j % ND2, k = j % NR;
       const Tile t = seq.get(p);
       const RuleDev &R = t.R;
-      if (BATCH) hr = make_half_rule(R, kScale, offset_of(R));
+      if (BATCH) hr = make_rule(R);
       if (!(ok = warp_wait(&bars->d2_full[reg], (j / ND2) & 1, bars, p.timeout_ns))) break;
       tc_fence_after();
       // read S and free the region (the next pass 1, or in DEC the next pass
@@ -1464,10 +1497,11 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             uint4 *cell = reinterpret_cast<uint4 *>(ring + off_c[c]);
             const uint4 cv = *cell;
             uint4 ov;
-            ov.x = rule4_binary_h(v[c][0], v[c][1], cv.x, hr);
-            ov.y = rule4_binary_h(v[c][2], v[c][3], cv.y, hr);
-            ov.z = rule4_binary_h(v[c][4], v[c][5], cv.z, hr);
-            ov.w = rule4_binary_h(v[c][6], v[c][7], cv.w, hr);
+            auto next = [&](int i, uint32_t cells) {
+              if constexpr (kRange) return rule4_range_h(v[c][i], v[c][i + 1], cells, hr);
+              else return rule4_binary_h(v[c][i], v[c][i + 1], cells, hr);
+            };
+            ov = make_uint4(next(0, cv.x), next(2, cv.y), next(4, cv.z), next(6, cv.w));
             *cell = ov;
           }
         } else if (!sums_mode) {
