@@ -42,10 +42,10 @@
 // The epilogue compares S (as f16, exact up to 2048) against the rule's
 // ranges two cells at a time in half2 arithmetic.
 //
-// Roles (896 threads): warp 0 = window TMA loads, warp 1 = TMEM allocator and
+// Roles (640 threads; 896 with 16 epilogue warps): warp 0 = window TMA loads, warp 1 = TMEM allocator and
 // pass-1 MMA issuer, warp 2 = centre-tile TMA loads and TMA stores, warp 3 =
 // pass-2 MMA issuer, warps 4..11 = convert warps (D1 -> pass-2 operand,
-// window encoding when needed, bands), warps 12..27 = epilogue warps (fused
+// window encoding when needed, bands), warps 12..19 = epilogue warps (fused
 // transition).  The two worker roles
 // work on different tiles at once; tensor memory holds the accumulator
 // regions and the bands (see Tm below).  Both products
@@ -65,10 +65,18 @@ namespace tc {
 constexpr int kTile = 128;
 constexpr int kWin = 160;
 constexpr int kCvtWarps = 8;                       // two per TMEM lane quarter
-constexpr int kEpiWarps = 16;                      // four per TMEM lane quarter
+// Two epilogue warps per TMEM lane quarter, of four 16-column chunks each: the
+// waits and the tile's place cost a warp as much as a chunk, and the integer
+// pipe is what bounds these kernels.  16384^2, us a step, with four warps of
+// two chunks -> with two of four: FP8 r = 7 / 12 / 16 94.4 / 100.3 / 116.6 ->
+// 92.0 / 99.0 / 112.3, C = 16 180 -> 171, FP16 161.9 -> 150.8 (one warp of
+// eight chunks: r = 7 / 12 96.0 / 100.6).
+// Four of two where that is faster: the big window (8192^2, r = 24: 39.9 against
+// 46.1) and four-bit storage on FP4 operands (16384^2, C = 16: 199 against 203).
+constexpr int kEpiWarps = 8, kEpiWarpsMore = 16;
 constexpr int kCvtThreads = 32 * kCvtWarps;
-constexpr int kEpiThreads = 32 * kEpiWarps;
-constexpr int kThreads = 128 + kCvtThreads + kEpiThreads;
+constexpr __host__ __device__ int threads_with(int epi_warps) { return 128 + kCvtThreads + 32 * epi_warps; }
+constexpr int kThreads = threads_with(kEpiWarps);
 constexpr int kMaxRegions = 3;
 
 // Window geometry and tensor memory, by kernel variant.  The standard window
@@ -575,7 +583,8 @@ __device__ __forceinline__ uint32_t rule4_binary_h(uint32_t s01, uint32_t s23, u
 // scale below 2^11, and so is every difference (equality gives +0; an empty
 // range has half width -1/2).  Two operations a range and pair instead of
 // three, so both ranges are tested for every cell and one logic operation
-// picks by the cell's byte: RULEFIG
+// picks by the cell's byte: 16384^2, r = 7 / 12, 96.2
+// -> 94.2 and 106.6 -> 100.6 us a step.
 // (The fields of HalfRule hold middles, bl2 and sl2, and half widths then.)
 __device__ __forceinline__ HalfRule make_range_rule(const RuleDev &R, float scale, int offset) {
   const float top = (float)((2 * R.r + 1) * (2 * R.r + 1)), o = (float)offset;
@@ -669,7 +678,7 @@ __device__ __forceinline__ uint32_t rule4_multistate_small_h(uint32_t s01, uint3
   return (aged & dm) | (r01 & ~dm);
 }
 
-// The rule's two ranges for the wide tile's integer test: the bounds of each
+// The rule's two ranges for an integer test (the big window above r = 22): the bounds of each
 // range as two 16-bit halves, the upper ones with bit 15 set.  An empty range
 // (or one starting above 4225, the largest count) gets lo = 0x7FFF.
 struct IntRule {
@@ -688,7 +697,7 @@ __host__ __device__ __forceinline__ IntRule make_int_rule(const RuleDev &R) {
 }
 
 // Next states of four cells (bytes of cw, 0/1) of a two-state rule from their
-// counts as the wide tile's f32 accumulators (S * 2^-9, S <= 4225).  Adding
+// counts as f32 accumulators (S * 2^-9, S <= 4225).  Adding
 // 16384 puts S in the low bits of the f32's mantissa (16384 + S * 2^-9 is
 // exact: the ulp at 2^14 is 2^-9), so one byte permute packs the counts of two
 // cells as 16-bit halves; per half, 0x8000 + S - lo and 0x8000 + hi - S stay
@@ -707,6 +716,40 @@ __device__ __forceinline__ uint32_t rule4_binary_i(const uint32_t *f4, uint32_t 
   const uint32_t in01 = ((S01 | 0x80008000u) - lo01) & (hi01 - S01) & 0x80008000u;
   const uint32_t in23 = ((S23 | 0x80008000u) - lo23) & (hi23 - S23) & 0x80008000u;
   return (__byte_perm(in01, in23, 0x7531) >> 7) & 0x01010101u;   // bytes 1 and 3 of each: cells 0..3
+}
+
+// As rule4_range_h from the wide tile's f32 accumulators (S * 2^-9, S <= 4225):
+// every middle, half width and difference is a multiple of 2^-10 and exact in
+// f32.  What is left over of the half width goes to f16 for its sign alone,
+// which rounding keeps (2^-10 is a normal f16).  8192^2, r = 24, with two
+// warps per quarter: 59.5 us a step with the integer test, 53.5 so; but in the
+// big window, with four, 39.9 with the integer test and 43.9 so.
+struct FloatRule {
+  float bm, bw, sm, sw;   // middles and half widths
+};
+
+__device__ __forceinline__ FloatRule make_float_rule(const RuleDev &R, float scale) {
+  const float top = (float)((2 * R.r + 1) * (2 * R.r + 1));
+  auto put = [&](int lo, int w, float &mid, float &half) {
+    const float l = (float)lo, h = fminf(l + (float)w, top);
+    mid = l > h ? 0.0f : (l + h) * 0.5f * scale;
+    half = l > h ? -0.5f * scale : (h - l) * 0.5f * scale;
+  };
+  FloatRule f;
+  put(R.b_lo, R.b_w, f.bm, f.bw);
+  put(R.s_lo, R.s_w, f.sm, f.sw);
+  return f;
+}
+
+__device__ __forceinline__ uint32_t rule4_range_f(const uint32_t *f4, uint32_t cw, const FloatRule &f) {
+  auto test = [&](int i, float mid, float half) {   // cells i, i + 1
+    return h2_bits(__floats2half2_rn(half - fabsf(__uint_as_float(f4[i]) - mid),
+                                     half - fabsf(__uint_as_float(f4[i + 1]) - mid)));
+  };
+  uint32_t born, keep;
+  asm("prmt.b32 %0, %1, %2, 0xFDB9;" : "=r"(born) : "r"(test(0, f.bm, f.bw)), "r"(test(2, f.bm, f.bw)));
+  asm("prmt.b32 %0, %1, %2, 0xFDB9;" : "=r"(keep) : "r"(test(0, f.sm, f.sw)), "r"(test(2, f.sm, f.sw)));
+  return ~((cw & keep) | (~cw & born)) & 0x01010101u;
 }
 
 __device__ __forceinline__ float half_lo(uint32_t h2) { return __low2float(as_h2(h2)); }
@@ -836,7 +879,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
                 "the big window serves single two-state instances on FP8 operands, one step per launch");
   // HB (big window, r <= 22, every count <= 45^2 = 2025 exact in f16): the
   // epilogue tests f16 pairs, converted from the f32 accumulator (1) or
-  // accumulated in f16 by pass 2 (2); 0: the f32 integer test
+  // accumulated in f16 by pass 2 (2); 0: the f32 test
   static_assert(HB == 0 || BIG, "f16 pairs serve the big window");
   static_assert(!OF || (DT == 1 && !ENC && !BATCH && !SW && !BITS && !WIDE && !NIB && !FP4 && !BIG),
                 "the offset pass 2 serves single two-state instances on FP8 operands in the standard window");
@@ -845,6 +888,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   using L = Layout<DT, ENC, SW, BITS, WIDE, NIB, BIG, OF>;
   // x-coordinate of a tile's centre box in its tensor map (bytes of packed rows)
   auto ctr_x = [](int tx0) { return BITS ? tx0 / 8 : NIB ? tx0 / 2 : tx0; };
+  constexpr int EW = BIG || (NIB && FP4) ? kEpiWarpsMore : kEpiWarps;   // epilogue warps
+  constexpr int EK = EW / 4, EC = 8 / EK;   // of a quarter; warp kq takes the 16-column chunks kq, kq + EK, ..
   using G = Geo<SW, WIDE, BIG>;
   using T = Tm<DT, SW, WIDE, BIG>;
   constexpr bool kRange = OF || SW;   // r <= 15 and two states: the epilogue's test by middle and half width
@@ -878,13 +923,13 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       mbar_init(&bars->x_full[i], 1);
       mbar_init(&bars->x_empty[i], ENC ? kCvtWarps : 1);  // encoders, or pass 1's commit
       mbar_init(&bars->c_full[i], 1);
-      mbar_init(&bars->out_full[i], kEpiWarps);
+      mbar_init(&bars->out_full[i], EW);
     }
     for (int i = 0; i < kMaxRegions; ++i) {
       mbar_init(&bars->d1_full[i], 1);
       mbar_init(&bars->d1_empty[i], kCvtWarps);
       mbar_init(&bars->d2_full[i], 1);
-      mbar_init(&bars->tmem_empty[i], kEpiWarps);
+      mbar_init(&bars->tmem_empty[i], EW);
     }
     for (int i = 0; i < 3; ++i) {
       mbar_init(&bars->h_full[i], kCvtWarps);
@@ -903,7 +948,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     tmem_relinquish();
   }
   if constexpr (SW) {  // pass-2 operand columns 144..159 (K padding) stay zero
-    for (int i = threadIdx.x; i < (int)(L::NH * L::kHBytes / 16); i += kThreads)
+    for (int i = threadIdx.x; i < (int)(L::NH * L::kHBytes / 16); i += threads_with(EW))
       reinterpret_cast<uint4 *>(smem + L::kH)[i] = make_uint4(0, 0, 0, 0);
   }
   fence_proxy_async_smem();
@@ -1327,9 +1372,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     }
     if (!ok) set_abort(bars, err0, 8);
   } else if constexpr (WIDE || BIG) {
-    // ------------------------- epilogue warps, wide tile or big window (12 .. 27)
-    // S as f32 (D2, lane y < 96, columns x < 96: six chunks of 16, chunks kq
-    // and kq + 4 per warp) and the centre tile (96-byte rows, no swizzle) ->
+    // ------------------------- epilogue warps, wide tile or big window (12 .. 19)
+    // S as f32 (D2, lane y < 96, columns x < 96: six chunks of 16) and the centre tile (96-byte rows, no swizzle) ->
     // next states in place, stored by TMA.  Warps of lane quarter 3 (rows
     // 96..127, outside the tile) only take part in the barriers.  Big window:
     // all 128 rows and eight chunks, the centre tile in the standard
@@ -1339,9 +1383,13 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     const int y = 32 * q + lane;
     const uint32_t lane_addr = static_cast<uint32_t>(32 * q) << 16;
     const bool rows = BIG || q < 3;
-    const int nch = (BIG || kq + 4 < 6) ? 2 : 1;
+    constexpr int nch = G::kTS / 16 / EK;
+    static_assert(nch * EK * 16 == G::kTS, "the warps of a quarter take the same number of chunks");
     bool ok = true;
-    const IntRule ir = make_int_rule(p.rule);
+    const auto ir = [&] {
+      if constexpr (WIDE) return make_float_rule(p.rule, kScale);
+      else return make_int_rule(p.rule);
+    }();
     const HalfRule hr = make_half_rule(p.rule, kScale);
     TileSeq<false, false, G::kTS> seq(p, first, n_my);
     for (int j = 0; ok && j < n_all; ++j, seq.next(p)) {
@@ -1349,15 +1397,13 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       const Tile t = seq.get(p);
       if (!(ok = warp_wait(&bars->d2_full[reg], (j / ND2) & 1, bars, p.timeout_ns))) break;
       tc_fence_after();
-      uint32_t v[2][HB == 2 ? 8 : 16];                 // S * scale as f32, or f16 pairs (HB 2)
+      uint32_t v[nch][HB == 2 ? 8 : 16];               // S * scale as f32, or f16 pairs (HB 2)
       if (rows) {
         const uint32_t treg = tmem + lane_addr + T::kD2Base + reg * T::kD2Cols;
-        if constexpr (HB == 2) {
-          tmem_ld16_pack16(treg + 16 * kq, v[0]);
-          tmem_ld16_pack16(treg + 16 * (kq + 4), v[1]);
-        } else {
-          tmem_ld16(treg + 16 * kq, v[0]);
-          if (nch == 2) tmem_ld16(treg + 16 * (kq + 4), v[1]);
+#pragma unroll
+        for (int c = 0; c < nch; ++c) {
+          if constexpr (HB == 2) tmem_ld16_pack16(treg + 16 * (kq + EK * c), v[c]);
+          else tmem_ld16(treg + 16 * (kq + EK * c), v[c]);
         }
         tmem_wait_ld();
       }
@@ -1367,17 +1413,19 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       if (!(ok = warp_wait(&bars->c_full[k], (j / NR) & 1, bars, p.timeout_ns))) break;
       if (rows) {
         uint8_t *ring = smem + L::kRing + k * L::kRingBytes;
+#pragma unroll
         for (int c = 0; c < nch; ++c) {
-          const int cc = kq + 4 * c;
+          const int cc = kq + EK * c;
           if (!p.sums) {
             uint4 *cell = reinterpret_cast<uint4 *>(ring + (BIG ? y * 128 + (((cc ^ y) & 7) << 4) : y * G::kTS + 16 * cc));
             const uint4 cv = *cell;
             uint4 ov;
             if constexpr (HB == 0) {
-              ov.x = rule4_binary_i(v[c], cv.x, ir);
-              ov.y = rule4_binary_i(v[c] + 4, cv.y, ir);
-              ov.z = rule4_binary_i(v[c] + 8, cv.z, ir);
-              ov.w = rule4_binary_i(v[c] + 12, cv.w, ir);
+              auto next = [&](int i, uint32_t cells) {
+                if constexpr (WIDE) return rule4_range_f(v[c] + i, cells, ir);
+                else return rule4_binary_i(v[c] + i, cells, ir);
+              };
+              ov = make_uint4(next(0, cv.x), next(4, cv.y), next(8, cv.z), next(12, cv.w));
             } else {
               // f16 pairs of cells (2i, 2i + 1): packed by pass 2, or converted
               // here (exact, S * 2^-9 < 4)
@@ -1410,17 +1458,17 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     }
     if (!ok) set_abort(bars, err0, 8);
   } else {
-    // ------------------------------------------------ epilogue warps (12 .. 27)
+    // ------------------------------------------------ epilogue warps (12 .. 19)
     // S (D2, lane y, columns x) and the centre tile -> next states, written in
     // place over the centre tile and stored from there by TMA.
     const int q = warp & 3;
-    const int kq = (warp - 4 - kCvtWarps) >> 2;        // 0..3: which warp of the quarter
+    const int kq = (warp - 4 - kCvtWarps) >> 2;        // which warp of the quarter
     const int y = 32 * q + lane;                       // TMEM lane = output row y
     const uint32_t lane_addr = static_cast<uint32_t>(32 * q) << 16;
-    uint32_t off_c[2];                                 // D2 column chunks kq and kq + 4
+    uint32_t off_c[EC];                        // D2 column chunks of this warp
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int cc = kq + 4 * c;
+    for (int c = 0; c < EC; ++c) {
+      const int cc = kq + EK * c;
       off_c[c] = y * 128 + (((cc ^ y) & 7) << 4);
     }
     bool ok = true;
@@ -1440,11 +1488,11 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       tc_fence_after();
       // read S and free the region (the next pass 1, or in DEC the next pass
       // 2, waits for it) before waiting for the centre tile
-      uint32_t v[2][8];                                // S * scale as f16 pairs
+      uint32_t v[EC][8];                       // S * scale as f16 pairs
       {
         const uint32_t treg = tmem + lane_addr + T::kD2Base + reg * T::kD2Cols;
-        tmem_ld16_pack16(treg + 16 * kq, v[0]);
-        tmem_ld16_pack16(treg + 16 * (kq + 4), v[1]);
+#pragma unroll
+        for (int c = 0; c < EC; ++c) tmem_ld16_pack16(treg + 16 * (kq + EK * c), v[c]);
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
@@ -1458,8 +1506,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
           // 16 cells of a chunk are 16 bits of the row (lowest x lowest);
           // cells at x >= W, inside the row's last byte, stay dead
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int cc = kq + 4 * c;
+          for (int c = 0; c < EC; ++c) {
+            const int cc = kq + EK * c;
             uint16_t *cellp = reinterpret_cast<uint16_t *>(ring + y * 16 + 2 * cc);
             uint32_t nb = rule16_bits(v[c], *cellp, hr);
             const int lim = t.W - (t.x0 + 16 * cc);
@@ -1472,8 +1520,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
           // unit u of row y at u ^ ((y >> 1) & 3)); cells at x >= W stay 0
           const uint32_t Kc = (uint32_t)((0x80 - R.C) & 0xFF) * 0x01010101u;
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int cc = kq + 4 * c;
+          for (int c = 0; c < EC; ++c) {
+            const int cc = kq + EK * c;
             uint2 *cellp = reinterpret_cast<uint2 *>(ring + y * 64 + ((((cc >> 1) ^ (y >> 1)) & 3) << 4) + 8 * (cc & 1));
             const uint2 cv = *cellp;
             const uint32_t st[4] = {nib4_to_bytes(cv.x, 0x4140), nib4_to_bytes(cv.x, 0x4342),
@@ -1493,7 +1541,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
           }
         } else if (!sums_mode && R.C == 2) {
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
+          for (int c = 0; c < EC; ++c) {
             uint4 *cell = reinterpret_cast<uint4 *>(ring + off_c[c]);
             const uint4 cv = *cell;
             uint4 ov;
@@ -1509,7 +1557,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             const uint32_t Cb = (uint32_t)R.C * 0x01010101u;
             const uint32_t Kc = (uint32_t)((0x80 - R.C) & 0xFF) * 0x01010101u;
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
+            for (int c = 0; c < EC; ++c) {
               uint4 *cell = reinterpret_cast<uint4 *>(ring + off_c[c]);
               const uint4 cv = *cell;
               uint4 ov;
@@ -1533,7 +1581,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             // the surrounding loop), so it stays.
             const uint32_t Cb = (uint32_t)R.C * 0x01010101u;
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
+            for (int c = 0; c < EC; ++c) {
               uint4 *cell = reinterpret_cast<uint4 *>(ring + off_c[c]);
               const uint4 cv = *cell;
               uint4 ov;
@@ -1547,8 +1595,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
         } else {   // box counts
           const int gy = t.y0 + y;
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int cc = kq + 4 * c;
+          for (int c = 0; c < EC; ++c) {
+            const int cc = kq + EK * c;
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const uint32_t h2 = v[c][i >> 1];
@@ -1593,7 +1641,7 @@ __global__ void __launch_bounds__(kThreads, 1) ltl_fp4_kernel(const __grid_const
 __global__ void __launch_bounds__(kThreads, 1) ltl_fp4_bits_kernel(const __grid_constant__ TcParams p) {
   ltl_tc_body<1, true, false, false, true, false, false, false, true>(p);
 }
-__global__ void __launch_bounds__(kThreads, 1) ltl_fp4_nib_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(threads_with(kEpiWarpsMore), 1) ltl_fp4_nib_kernel(const __grid_constant__ TcParams p) {
   ltl_tc_body<1, true, false, false, false, false, false, true, true>(p);
 }
 
@@ -1610,13 +1658,13 @@ __global__ void __launch_bounds__(kThreads, 1) ltl_wide_kernel(const __grid_cons
 
 // Radii up to 32 on the 128 x 128 tile: the 192 x 192 window, single
 // instance, FP8 operands, two-state rules, one step per launch.
-__global__ void __launch_bounds__(kThreads, 1) ltl_big_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(threads_with(kEpiWarpsMore), 1) ltl_big_kernel(const __grid_constant__ TcParams p) {
   ltl_tc_body<1, false, false, false, false, false, false, false, false, true>(p);
 }
 // The same for r <= 22, where every count is exact in f16: pass 2
 // accumulates in f16 and the epilogue tests f16 pairs (measured 7% faster
 // than the f32 test, 2% faster than converting the f32 accumulator).
-__global__ void __launch_bounds__(kThreads, 1) ltl_big16_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(threads_with(kEpiWarpsMore), 1) ltl_big16_kernel(const __grid_constant__ TcParams p) {
   ltl_tc_body<1, false, false, false, false, false, false, false, false, true, 2>(p);
 }
 
@@ -1697,7 +1745,7 @@ __device__ __forceinline__ uint32_t piece_off(int w, int row, int kb) {
 
 // One step (or the counts R) of a single instance, FP8 operands, two-state
 // rules.  Warps: 0 loads, 1 allocates tensor memory and issues the MMAs, 2
-// stores, 4..11 build the two bands, 12..27 evaluate the rule.
+// stores, 4..11 build the two bands, 12..19 evaluate the rule.
 __global__ void __launch_bounds__(kThreads, 1) ltl_vn_kernel(const __grid_constant__ TcParams p) {
   constexpr float kScale = 1.0f / 512.0f;            // accumulator = R * kScale
   extern __shared__ uint8_t smem_raw[];
@@ -1851,30 +1899,31 @@ __global__ void __launch_bounds__(kThreads, 1) ltl_vn_kernel(const __grid_consta
     __syncwarp();
     if (lane == 0) mbar_arrive(&bars->band_ready);
   } else {
-    // ------------------------------------------------ epilogue warps (12 .. 27)
+    // ------------------------------------------------ epilogue warps (12 .. 19)
+    constexpr int kEpiK = kEpiWarps / 4, kEpiChunks = 8 / kEpiK;
     const int q = warp & 3;
-    const int kq = (warp - 4 - kCvtWarps) >> 2;      // 0..3: which warp of the quarter
+    const int kq = (warp - 4 - kCvtWarps) >> 2;      // which warp of the quarter
     const int y = 32 * q + lane;                     // TMEM lane = output row y
     const uint32_t lane_addr = static_cast<uint32_t>(32 * q) << 16;
-    uint32_t off_c[2];                               // column chunks kq and kq + 4 of row y
+    uint32_t off_c[kEpiChunks];                      // this warp's column chunks of row y
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int cc = kq + 4 * c;
+    for (int c = 0; c < kEpiChunks; ++c) {
+      const int cc = kq + kEpiK * c;
       off_c[c] = y * 128 + (((cc ^ y) & 7) << 4);
     }
     bool ok = true;
-    const HalfRule hr = make_half_rule(p.rule, kScale);
+    const HalfRule hr = make_range_rule(p.rule, kScale, 0);
     TileSeq<false> seq(p, first);
     for (int j = 0; ok && j < n_my; ++j, seq.next(p)) {
       const int reg = j % vn::kRegions, s = j % vn::NS;
       const Tile t = seq.get(p);
       if (!(ok = warp_wait(&bars->d2_full[reg], (j / vn::kRegions) & 1, bars, p.timeout_ns))) break;
       tc_fence_after();
-      uint32_t v[2][8];                              // R * scale as f16 pairs
+      uint32_t v[kEpiChunks][8];                     // R * scale as f16 pairs
       {
         const uint32_t treg = tmem + lane_addr + reg * kTile;
-        tmem_ld16_pack16(treg + 16 * kq, v[0]);
-        tmem_ld16_pack16(treg + 16 * (kq + 4), v[1]);
+#pragma unroll
+        for (int c = 0; c < kEpiChunks; ++c) tmem_ld16_pack16(treg + 16 * (kq + kEpiK * c), v[c]);
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
@@ -1887,21 +1936,21 @@ __global__ void __launch_bounds__(kThreads, 1) ltl_vn_kernel(const __grid_consta
       uint8_t *ctr = smem + s * vn::kStage + vn::kCtrOff;
       if (!p.sums) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
+        for (int c = 0; c < kEpiChunks; ++c) {
           uint4 *cell = reinterpret_cast<uint4 *>(ctr + off_c[c]);
           const uint4 cv = *cell;
           uint4 ov;
-          ov.x = rule4_binary_h(v[c][0], v[c][1], cv.x, hr);
-          ov.y = rule4_binary_h(v[c][2], v[c][3], cv.y, hr);
-          ov.z = rule4_binary_h(v[c][4], v[c][5], cv.z, hr);
-          ov.w = rule4_binary_h(v[c][6], v[c][7], cv.w, hr);
+          ov.x = rule4_range_h(v[c][0], v[c][1], cv.x, hr);
+          ov.y = rule4_range_h(v[c][2], v[c][3], cv.y, hr);
+          ov.z = rule4_range_h(v[c][4], v[c][5], cv.z, hr);
+          ov.w = rule4_range_h(v[c][6], v[c][7], cv.w, hr);
           *cell = ov;
         }
       } else {  // the counts R of Eq. 3
         const int gy = t.y0 + y;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int cc = kq + 4 * c;
+        for (int c = 0; c < kEpiChunks; ++c) {
+          const int cc = kq + kEpiK * c;
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const uint32_t h2 = v[c][i >> 1];
@@ -1940,10 +1989,11 @@ size_t tc_smem_bytes(int dt, bool encode, bool sw) {
 // stream drains (its CTAs start on SMs as the previous grid's CTAs leave
 // them), sets up its barriers and tensor memory, and waits for the previous
 // grid's completion (griddepcontrol.wait) before any global memory access.
-static cudaError_t launch_pdl(void (*kern)(TcParams), int grid, size_t smem, cudaStream_t s, const TcParams &p) {
+static cudaError_t launch_pdl(void (*kern)(TcParams), int grid, size_t smem, cudaStream_t s, const TcParams &p,
+                              int threads = tc::kThreads) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(tc::kThreads);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -2025,7 +2075,7 @@ cudaError_t fp4_launch(const TcParams &p, int storage, int grid, cudaStream_t s)
     if (e != cudaSuccess) return e;
     configured[storage] = true;
   }
-  return launch_pdl(kern, grid, smem, s, p);
+  return launch_pdl(kern, grid, smem, s, p, storage == 2 ? tc::threads_with(tc::kEpiWarpsMore) : tc::kThreads);
 }
 
 // The 96 x 96 tile: map_in_a / map_in_b are the 128 x 160 and 32 x 160 window
@@ -2055,7 +2105,7 @@ cudaError_t big_launch(const TcParams &p, int grid, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured[k] = true;
   }
-  return launch_pdl(kern, grid, L::kDyn, s, p);
+  return launch_pdl(kern, grid, L::kDyn, s, p, tc::threads_with(tc::kEpiWarpsMore));
 }
 
 // Simplified von Neumann neighbourhood: FP8, two-state rules, single instance

@@ -44,3 +44,21 @@ def test_offset_pass2(cat, r, shape):
                 finally:
                     g.close()
                 assert np.array_equal(got, oracle.step(grid, oracle.Rule(**rule), n_steps=3)), (rule, per_launch)
+
+
+@pytest.mark.parametrize("r", [16, 32])
+def test_ranges_of_the_wide_tile(cat, r):
+    """Its counts are compared as f32: the same edges of the rule's ranges."""
+    top = (2 * r + 1) ** 2
+    s = inputs.scaled_rule(r)
+    grid = inputs.bernoulli(131, 200, 0.5, r)
+    for g0 in (grid, np.ones_like(grid)):
+        for rule in (s, dict(s, s1=3, s2=2, b1=0, b2=0), dict(s, M=1, s1=top, s2=1 << 30, b1=1, b2=top // 2)):
+            g = cat.Grid(131, 200, rule, kernel="tcgen05", dtype="fp8", tile=96)
+            try:
+                g.set_state(g0)
+                g.step(2)
+                got = g.get_state()
+            finally:
+                g.close()
+            assert np.array_equal(got, oracle.step(g0, oracle.Rule(**rule), n_steps=2)), rule
