@@ -584,7 +584,8 @@ __device__ __forceinline__ uint32_t rule4_binary_h(uint32_t s01, uint32_t s23, u
 // range has half width -1/2).  Two operations a range and pair instead of
 // three, so both ranges are tested for every cell and one logic operation
 // picks by the cell's byte: 16384^2, r = 7 / 12, 96.2
-// -> 94.2 and 106.6 -> 100.6 us a step.
+// -> 94.2 and 106.6 -> 100.6 us a step; C = 16, r = 10, 171.5 -> 160.3; FP16 150.9
+// -> 146.8.
 // (The fields of HalfRule hold middles, bl2 and sl2, and half widths then.)
 __device__ __forceinline__ HalfRule make_range_rule(const RuleDev &R, float scale, int offset) {
   const float top = (float)((2 * R.r + 1) * (2 * R.r + 1)), o = (float)offset;
@@ -647,13 +648,14 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
 // state 1 when its count is in the birth range; an alive cell (1) stays alive
 // in the survival range and otherwise starts dying (state 2); a dying cell
 // (c >= 2) ages to c + 1, and to 0 after state C - 1.  Cb = C in every byte.
+template <bool RANGE>
 __device__ __forceinline__ uint32_t rule4_multistate_h(uint32_t s01, uint32_t s23, uint32_t cw, const HalfRule &h,
                                                        uint32_t Cb) {
   const uint32_t nonzero = nonzero_bytes(cw);                       // c >= 1
   const uint32_t dying = nonzero_bytes((cw >> 1) & 0x7F7F7F7Fu);    // c >= 2
   const uint32_t alive = nonzero ^ dying;                           // c == 1
   const uint32_t dead = nonzero ^ 0x01010101u;                      // c == 0
-  const uint32_t inr = rule4_binary_h(s01, s23, nonzero, h);        // birth range (c = 0) or survival range
+  const uint32_t inr = RANGE ? rule4_range_h(s01, s23, nonzero, h) : rule4_binary_h(s01, s23, nonzero, h);        // birth range (c = 0) or survival range
   const uint32_t inc = cw + 0x01010101u;                            // c + 1 <= C <= 255: no carries
   const uint32_t aged = inc & (nonzero_bytes(inc ^ Cb) * 0xFFu);    // c + 1, or 0 where c + 1 == C
   return (inr & dead) | ((0x02020202u - inr) & (alive * 0xFFu)) | (aged & (dying * 0xFFu));
@@ -665,11 +667,12 @@ __device__ __forceinline__ uint32_t rule4_multistate_h(uint32_t s01, uint32_t s2
 // c + 1 >= C (c + 1 + Kc, Kc = 0x80 - C in every byte).  A cell alive (c = 1)
 // becomes inr ? 1 : 2 = inr + 2 (1 - inr); a dead one inr; a dying one c + 1,
 // or 0 at C.
+template <bool RANGE>
 __device__ __forceinline__ uint32_t rule4_multistate_small_h(uint32_t s01, uint32_t s23, uint32_t cw,
                                                              const HalfRule &h, uint32_t Kc) {
   const uint32_t ge1 = ((cw + 0x7F7F7F7Fu) >> 7) & 0x01010101u;
   const uint32_t ge2 = ((cw + 0x7E7E7E7Eu) >> 7) & 0x01010101u;
-  const uint32_t inr = rule4_binary_h(s01, s23, ge1, h);
+  const uint32_t inr = RANGE ? rule4_range_h(s01, s23, ge1, h) : rule4_binary_h(s01, s23, ge1, h);
   const uint32_t r01 = inr + 2u * (ge1 & ~ge2 & ~inr);
   const uint32_t inc = cw + 0x01010101u;
   const uint32_t wrap = ((inc + Kc) >> 7) & 0x01010101u;
@@ -865,8 +868,9 @@ __device__ __forceinline__ int32_t *tile_err(const TcParams &p, int first, int j
 }
 
 template <int DT, bool ENC, bool BATCH, bool SW, bool BITS, bool MS, bool WIDE = false, bool NIB = false,
-          bool FP4 = false, bool BIG = false, int HB = 0, bool OF = false>
+          bool FP4 = false, bool BIG = false, int HB = 0, bool R15 = false>
 __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
+  constexpr bool OF = R15 && DT == 1 && !ENC;   // the offset pass 2
   static_assert(!MS || !BATCH, "several steps per launch serve single instances");
   static_assert(!WIDE || (DT == 1 && !ENC && !BATCH && !SW && !BITS && !MS),
                 "the wide tile serves single two-state instances on FP8 operands, one step per launch");
@@ -881,8 +885,10 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   // epilogue tests f16 pairs, converted from the f32 accumulator (1) or
   // accumulated in f16 by pass 2 (2); 0: the f32 test
   static_assert(HB == 0 || BIG, "f16 pairs serve the big window");
-  static_assert(!OF || (DT == 1 && !ENC && !BATCH && !SW && !BITS && !WIDE && !NIB && !FP4 && !BIG),
-                "the offset pass 2 serves single two-state instances on FP8 operands in the standard window");
+  // R15 (r <= 15): the epilogue tests ranges by middle and half width, and
+  // without a re-encoded window (r >= 8 then) pass 2 takes H - 16
+  static_assert(!R15 || (!BATCH && !SW && !BITS && !WIDE && !NIB && !FP4 && !BIG),
+                "serves single uint8 instances in the standard window");
   static_assert(Layout<DT, ENC, SW, BITS>::NS <= kMaxStages && Layout<DT, ENC, SW, BITS>::NR <= kMaxStages &&
                 Layout<DT, ENC, SW, BITS>::NE <= 3, "barrier arrays");
   using L = Layout<DT, ENC, SW, BITS, WIDE, NIB, BIG, OF>;
@@ -892,7 +898,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   constexpr int EK = EW / 4, EC = 8 / EK;   // of a quarter; warp kq takes the 16-column chunks kq, kq + EK, ..
   using G = Geo<SW, WIDE, BIG>;
   using T = Tm<DT, SW, WIDE, BIG>;
-  constexpr bool kRange = OF || SW;   // r <= 15 and two states: the epilogue's test by middle and half width
+  constexpr bool kRange = R15 || SW;
   constexpr bool DEC = T::kDec;       // D1 and D2 in separate regions, pass 2 on e4m3 digits
   constexpr int KW = BIG ? 192 : kWin;   // window columns = pass-1 K = pass-2 K
   constexpr int KS = KW / 32;            // K-steps of one e4m3 band product
@@ -1530,7 +1536,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
 #pragma unroll
             for (int i = 0; i < 4; ++i)   // C <= 16 here
               ns[i] = bytes_to_nib_pairs(R.C == 2 ? rule4_binary_h(v[c][2 * i], v[c][2 * i + 1], st[i], hr)
-                                                  : rule4_multistate_small_h(v[c][2 * i], v[c][2 * i + 1], st[i], hr, Kc));
+                                                  : rule4_multistate_small_h<kRange>(v[c][2 * i], v[c][2 * i + 1], st[i], hr, Kc));
             uint2 ov = make_uint2(__byte_perm(ns[0], ns[1], 0x6420), __byte_perm(ns[2], ns[3], 0x6420));
             const int lim = t.W - (t.x0 + 16 * cc);
             if (lim < 16) {
@@ -1562,15 +1568,15 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               const uint4 cv = *cell;
               uint4 ov;
               if (R.C <= 128) {
-                ov.x = rule4_multistate_small_h(v[c][0], v[c][1], cv.x, hr, Kc);
-                ov.y = rule4_multistate_small_h(v[c][2], v[c][3], cv.y, hr, Kc);
-                ov.z = rule4_multistate_small_h(v[c][4], v[c][5], cv.z, hr, Kc);
-                ov.w = rule4_multistate_small_h(v[c][6], v[c][7], cv.w, hr, Kc);
+                ov.x = rule4_multistate_small_h<kRange>(v[c][0], v[c][1], cv.x, hr, Kc);
+                ov.y = rule4_multistate_small_h<kRange>(v[c][2], v[c][3], cv.y, hr, Kc);
+                ov.z = rule4_multistate_small_h<kRange>(v[c][4], v[c][5], cv.z, hr, Kc);
+                ov.w = rule4_multistate_small_h<kRange>(v[c][6], v[c][7], cv.w, hr, Kc);
               } else {
-                ov.x = rule4_multistate_h(v[c][0], v[c][1], cv.x, hr, Cb);
-                ov.y = rule4_multistate_h(v[c][2], v[c][3], cv.y, hr, Cb);
-                ov.z = rule4_multistate_h(v[c][4], v[c][5], cv.z, hr, Cb);
-                ov.w = rule4_multistate_h(v[c][6], v[c][7], cv.w, hr, Cb);
+                ov.x = rule4_multistate_h<kRange>(v[c][0], v[c][1], cv.x, hr, Cb);
+                ov.y = rule4_multistate_h<kRange>(v[c][2], v[c][3], cv.y, hr, Cb);
+                ov.z = rule4_multistate_h<kRange>(v[c][4], v[c][5], cv.z, hr, Cb);
+                ov.w = rule4_multistate_h<kRange>(v[c][6], v[c][7], cv.w, hr, Cb);
               }
               *cell = ov;
             }
@@ -1585,10 +1591,10 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               uint4 *cell = reinterpret_cast<uint4 *>(ring + off_c[c]);
               const uint4 cv = *cell;
               uint4 ov;
-              ov.x = rule4_multistate_h(v[c][0], v[c][1], cv.x, hr, Cb);
-              ov.y = rule4_multistate_h(v[c][2], v[c][3], cv.y, hr, Cb);
-              ov.z = rule4_multistate_h(v[c][4], v[c][5], cv.z, hr, Cb);
-              ov.w = rule4_multistate_h(v[c][6], v[c][7], cv.w, hr, Cb);
+              ov.x = rule4_multistate_h<kRange>(v[c][0], v[c][1], cv.x, hr, Cb);
+              ov.y = rule4_multistate_h<kRange>(v[c][2], v[c][3], cv.y, hr, Cb);
+              ov.z = rule4_multistate_h<kRange>(v[c][4], v[c][5], cv.z, hr, Cb);
+              ov.w = rule4_multistate_h<kRange>(v[c][6], v[c][7], cv.w, hr, Cb);
               *cell = ov;
             }
           }
@@ -1622,9 +1628,9 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   }
 }
 
-template <int DT, bool ENC, bool BATCH, bool SW, bool OF>
+template <int DT, bool ENC, bool BATCH, bool SW, bool R15>
 __global__ void __launch_bounds__(kThreads, 1) ltl_tc_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<DT, ENC, BATCH, SW, false, false, false, false, false, false, 0, OF>(p);
+  ltl_tc_body<DT, ENC, BATCH, SW, false, false, false, false, false, false, 0, R15>(p);
 }
 
 // One bit per cell: the same body under its own name, so that a profiler can
@@ -1670,9 +1676,9 @@ __global__ void __launch_bounds__(threads_with(kEpiWarpsMore), 1) ltl_big16_kern
 
 // Several steps of a single instance in one cooperative launch (separate
 // instantiations, so that the one-step kernels carry none of it).
-template <int DT, bool ENC, bool SW, bool BITS, bool OF>
+template <int DT, bool ENC, bool SW, bool BITS, bool R15>
 __global__ void __launch_bounds__(kThreads, 1) ltl_tc_multi_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<DT, ENC, false, SW, BITS, true, false, false, false, false, 0, OF>(p);
+  ltl_tc_body<DT, ENC, false, SW, BITS, true, false, false, false, false, 0, R15>(p);
 }
 
 // ---------------------------------------------------------------------------
@@ -2004,13 +2010,13 @@ static cudaError_t launch_pdl(void (*kern)(TcParams), int grid, size_t smem, cud
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-template <int DT, bool ENC, bool BATCH, bool SW = false, bool BITS = false, bool OF = false>
+template <int DT, bool ENC, bool BATCH, bool SW = false, bool BITS = false, bool R15 = false>
 static cudaError_t launch_one(const TcParams &p, int grid, cudaStream_t s) {
   static bool configured = false;
-  const size_t smem = tc::Layout<DT, ENC, SW, BITS, false, false, false, OF>::kDyn;
+  const size_t smem = tc::Layout<DT, ENC, SW, BITS, false, false, false, R15 && DT == 1 && !ENC>::kDyn;
   void (*kern)(TcParams);
   if constexpr (BITS) kern = tc::ltl_bits_kernel;
-  else kern = tc::ltl_tc_kernel<DT, ENC, BATCH, SW, OF>;
+  else kern = tc::ltl_tc_kernel<DT, ENC, BATCH, SW, R15>;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -2019,7 +2025,7 @@ static cudaError_t launch_one(const TcParams &p, int grid, cudaStream_t s) {
   if constexpr (!BATCH) {
     if (p.n_steps > 1) {  // CTAs wait on one another: all must be resident at once
       static bool configured_multi = false;
-      void (*multi)(TcParams) = tc::ltl_tc_multi_kernel<DT, ENC, SW, BITS, OF>;
+      void (*multi)(TcParams) = tc::ltl_tc_multi_kernel<DT, ENC, SW, BITS, R15>;
       if (!configured_multi) {
         cudaError_t e = cudaFuncSetAttribute(multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -2041,8 +2047,9 @@ static cudaError_t launch_one(const TcParams &p, int grid, cudaStream_t s) {
 // buffers.  Two-state FP8 grids of r = 8 .. 15 take the offset kernel.
 cudaError_t tc_launch(const TcParams &p, int dt, bool encode, bool sw, bool bits, int grid, cudaStream_t s) {
   if (bits) return launch_one<1, true, false, false, true>(p, grid, s);
-  if (dt == 1) return launch_one<0, true, false>(p, grid, s);
-  if (encode) return launch_one<1, true, false>(p, grid, s);
+  const bool r15 = p.rule.r <= 15;
+  if (dt == 1) return r15 ? launch_one<0, true, false, false, false, true>(p, grid, s) : launch_one<0, true, false>(p, grid, s);
+  if (encode) return r15 ? launch_one<1, true, false, false, false, true>(p, grid, s) : launch_one<1, true, false>(p, grid, s);
   if (sw) return launch_one<1, false, false, true>(p, grid, s);
   if (tc::pass2_offset(p.rule.r)) return launch_one<1, false, false, false, false, true>(p, grid, s);
   return launch_one<1, false, false>(p, grid, s);
