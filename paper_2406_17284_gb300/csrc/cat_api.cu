@@ -980,8 +980,8 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   // Several steps of grids whose options are all left to the library, on bit
   // planes: from six steps and 2^25 cells on, or four and 2^27 (512 grids with
   // sides up to 900 / 1400 / 2048, 54 / 102 / 179 million cells, us for 4 steps:
-  // tiles 171 / 270 / 423, planes 185 / 274 / 409; for 6: 251 / 401 / 627
-  // against 244 / 364 / 547; for 12: 490 / 788 / 1241 against 420 / 635 / 959).
+  // tiles 165 / 260 / 408, planes 185 / 274 / 408; for 6: 242 / 385 / 607
+  // against 243 / 362 / 545; for 12: 472 / 761 / 1201 against 418 / 632 / 956).
   // A captured call keeps to the tiles, one launch per
   // step, since the planes need the radii side by side.
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

@@ -132,53 +132,59 @@ int64_t tile_smem(const PlanesGrid &g, const TilePlan &t) {
 // tensor-core kernel that the options would otherwise name):
 //   one bit per cell      every radius: 32768^2, r = 2 / 16: 147 / 320 against
 //                         the former bit-sliced kernel's 224 and tcgen05's 594
-//   four bits per cell    every radius: 24576^2, C 16, r = 10: 297 against 435
+//   four bits per cell    every radius: 24576^2, C 16, r = 10: 269 against 435
 //   uint8, C > 2          up to a radius that falls while the strips get too
 //                         short for the 2r rows before them and rises again with
 //                         the size: 1024^2, r = 12 / 13: 5.9 / 6.6 against 6.0;
-//                         2048^2, r = 5 / 6: 7.4 / 8.0 against 7.8; 4096^2, r =
-//                         7 / 8: 14.4 / 17.1 against 15.9 / 16.1; 8192^2, r = 12
-//                         / 13: 47.1 / 49.5 against 49.3; 16384^2, r = 1 / 10 /
-//                         15: 118 / 155 / 174 against 178 / 180 / 180
+//                         2048^2, r = 5 / 6: 7.4 / 8.0 against 7.5; 4096^2, r =
+//                         7 / 8: 14.4 / 17.1 against 14.8 / 15.3; 8192^2, r = 9
+//                         / 10: 44.3 / 45.8 against 44.1; 16384^2, r = 1 / 10 /
+//                         12 / 15: 117 / 154 / 157 / 172 against 153 / 159 ..
 //   uint8, two states     only where a launch's latency counts: 1024^2, r = 1 /
-//                         9 / 15: 2.2 / 3.7 / 4.3 against 4.6; 2048^2, r = 9 /
-//                         10: 5.6 / 5.8 against 5.7; 4096^2, r = 4 / 5: 9.2 /
-//                         10.3 against 10.2; 16384^2, r = 4: 111 against 96.
+//                         9 / 15: 2.2 / 3.7 / 4.3 against 4.5; 2048^2, r = 9 /
+//                         10: 5.5 / 5.8 against 5.5; 4096^2, r = 4 / 5: 9.2 /
+//                         10.3 against 9.9; 16384^2, r = 4: 111 against 92.
 //                         The frame that a torus refreshes first costs a short
 //                         step more: 1024^2, r = 7 / 9: 5.5 / 5.8 against 5.7;
-//                         2048^2, r = 4 / 6: 6.4 / 7.5 against 7.4
+//                         2048^2, r = 4 / 6: 6.4 / 7.5 against 7.1
 bool planes_preferred(const PlanesGrid &g) {
   int kind;
   if (!find(g, &kind).fn) return false;
   if (g.storage_in != CAT_STORE_U8) return true;
   const int64_t m = (g.H * g.W + (1 << 20) - 1) >> 20;   // 2^20 cells
-  if (g.rule.C > 2) return g.rule.r <= (m <= 1 ? (g.frame ? 9 : 12) : m < 16 ? 5 : m < 30 ? 7 : m < 128 ? 12 : 15);
+  if (g.rule.C > 2) return g.rule.r <= (m <= 1 ? (g.frame ? 9 : 12) : m < 16 ? 5 : m < 64 ? 7 : m < 128 ? 9 : 12);
   if (g.frame) return g.rule.r <= (m <= 1 ? 7 : m <= 16 ? 4 : 0);
   return g.rule.r <= (m <= 1 ? 16 : m <= 4 ? 9 : m <= 16 ? 4 : 0);
 }
 
 // Several steps of a two-state uint8 grid (us per step, tensor-core steps
 // last).  Reading and writing bits is worth most on large grids and with many
-// steps between the bytes at both ends; a wave of strips fits grids of 10 to 36
+// steps between the bytes at both ends; a wave of strips fits grids of 6 to 50
 // 2^20 cells badly, and a torus pays for a frame per launch:
-//   4096^2, n = 2 / 4 / 8   r = 4: 9.4 / 7.3 / 5.8 and 10.2; r = 7: 11.2 / 7.9 /
-//                           7.7 and 10.6; r = 10: 11.7 / 9.6 / 9.4 and 11.1;
-//                           r = 12: 12.0 / 11.5 / 11.3 and 11.1
-//   5792^2, n = 2 / 4 / 8   r = 8: 18.5 / 16.5 / 15.4 and 17.9; r = 16: 22.0 /
-//                           19.9 / 18.7 and 19.5
-//   7000^2, n = 2 / 3       r = 16: 27.8 / 26.0 and 26.1
-//   8192^2, n = 2 / 8       r = 4: 20.1 / 17.3 and 28.3; r = 16: 33.5 / 28.2 and 33.3
-//   16384^2, n = 2 / 8      r = 12: 92.6 / 75.5 and 106.4
-//   torus, n = 8            2048^2, r = 12: 9.0 and 7.5; 4096^2, r = 7 / 12: 10.9
-//                           / 14.6 and 13.0; 5792^2, r = 12: 17.9 and 19.6
+//   2896^2, n = 2 / 4 / 8   r = 10: 8.1 / 6.8 / 6.7 and 7.9; r = 12: 8.2 / 8.0 /
+//                           7.8 and 7.9
+//   4096^2, n = 2 / 4 / 8   r = 4: 9.4 / 7.3 / 5.8 and 9.9; r = 7: 11.2 / 7.7 /
+//                           7.5 and 9.9; r = 10: 11.7 / 9.5 / 9.3 and 9.9;
+//                           r = 12: 12.0 / 11.5 / 11.3 and 9.9
+//   5792^2, n = 2 / 4 / 8   r = 8: 18.5 / 16.3 / 15.3 and 16.7; r = 16: 22.0 /
+//                           19.9 / 18.7 and 19.0
+//   7000^2, n = 2 / 3 / 4   r = 12: 24.0 / 22.5 / 21.7 and 22.8; r = 16: 27.8 /
+//                           25.8 / 24.6 and 24.8
+//   8192^2, n = 2 / 3 / 8   r = 4: 20.1 / 18.8 / 17.3 and 27.2; r = 8: 29.2 / 27.0
+//                           / 24.0 and 28.2; r = 16: 33.5 / 31.3 / 28.3 and 32.1
+//   16384^2, n = 2 / 8      r = 12: 92.6 / 75.5 and 98.5
+//   torus, n = 8            2048^2, r = 12: 9.0 and 7.1; 4096^2, r = 7 / 12: 10.9
+//                           / 14.6 and 12.1; 5792^2, r = 12: 18.0 and 18.7;
+//                           7000^2, r = 11 / 15: 23.6 / 22.7 and 23.4
 bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps) {
   const int64_t m = (g.H * g.W + (1 << 20) - 1) >> 20;
   const int r = g.rule.r;
-  if (g.frame) return r <= 7 || (m >= 30 && n_steps >= (m >= 64 ? 2 : r == 16 ? 8 : 3));
-  if (r <= 7) return m <= 4 || m > 16 || n_steps >= (r == 7 ? 4 : r >= 5 ? 3 : 2);
-  if (m <= 10 || m > 50) return true;
+  if (g.frame) return r <= 7 || (m >= 30 && n_steps >= (m < 64 ? 8 : r == 8 || r >= 14 ? 3 : 2));
+  if (r <= 7) return m <= 4 || m > 24 || n_steps >= (r == 7 ? 4 : r >= 5 ? 3 : 2);
+  if (m <= (r <= 10 ? 10 : 6)) return true;
   if (m <= 24) return r <= 10 && n_steps >= 4;
-  return n_steps >= (m <= 36 ? (r == 16 ? 8 : 4) : (r == 16 ? 3 : 2));
+  if (m <= 36) return n_steps >= (r == 16 ? 8 : 4);
+  return n_steps >= (m <= 50 || r == 8 || r == 16 ? 3 : 2);
 }
 
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
