@@ -461,7 +461,8 @@ __device__ __forceinline__ bool pass2_f16(int DT, int r) { return DT == 0 || 2 *
 // the band has 2r + 1 ones, so the offset is a constant that the rule's bounds
 // take up.  16384^2, us a step: r = 8 .. 15 106.3 against 116.8 with H in f16
 // (r = 12: 256^2 4.8 against 5.1, 2048^2 6.0 against 6.8, 8192^2 31.0 against
-// 33.7).  Only the one-instance kernel without a re-encoded window has it: a
+// 33.7); with the range test and the epilogue warps of now 98.5, and r = 16,
+// in f16, 112.3.  Only the one-instance kernel without a re-encoded window has it: a
 // choice by radius inside a kernel cost r = 16 2%, and with a re-encoded
 // window the convert warps are what bounds the kernel and four conversions a
 // word cost more than the shorter pass 2 gives (r = 10, C = 16: 184.0 against

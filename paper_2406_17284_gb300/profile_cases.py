@@ -22,6 +22,8 @@ from . import build, cat, inputs
 CASES = {
     # name: (rule, Grid options, kernel name a profiler filters on)
     "fp8_r16": (inputs.scaled_rule(16), dict(kernel="tcgen05", dtype="fp8"), "ltl_tc_kernel"),
+    "fp8_r12": (inputs.scaled_rule(12), dict(kernel="tcgen05", dtype="fp8"), "ltl_tc_kernel"),
+    "c16_r10": (inputs.MULTISTATE_R10_C16, dict(kernel="tcgen05", dtype="fp8"), "ltl_tc_kernel"),
     "fp8_r4": (inputs.scaled_rule(4), dict(kernel="tcgen05", dtype="fp8"), "ltl_tc_kernel"),
     "fp16_r16": (inputs.scaled_rule(16), dict(kernel="tcgen05", dtype="fp16"), "ltl_tc_kernel"),
     "vn_r16": (inputs.vn_scaled_rule(16), dict(kernel="tcgen05", dtype="fp8"), "ltl_vn_kernel"),
@@ -31,8 +33,10 @@ CASES = {
     "big_r20": (inputs.scaled_rule(20), dict(kernel="tcgen05", dtype="fp8"), "ltl_big16_kernel"),
     "nib_c16": (inputs.MULTISTATE_R10_C16, dict(kernel="tcgen05", dtype="fp8", storage=cat.STORE_NIB4), "ltl_nib_kernel"),
     "fp4_r16": (inputs.scaled_rule(16), dict(kernel="tcgen05", dtype="fp4"), "ltl_fp4_kernel"),
-    "bitslice_r1": (inputs.scaled_rule(1), dict(kernel="bitslice", storage=cat.STORE_BIT1), "ltl_swar_kernel"),
-    "bitslice_r2": (inputs.scaled_rule(2), dict(kernel="bitslice", storage=cat.STORE_BIT1), "ltl_swar_kernel"),
+    "planes_bits_r2": (inputs.scaled_rule(2), dict(kernel="auto", dtype="auto", storage=cat.STORE_BIT1), "planes_kernel"),
+    "planes_bits_r16": (inputs.scaled_rule(16), dict(kernel="auto", dtype="auto", storage=cat.STORE_BIT1), "planes_kernel"),
+    "planes_nib_c16": (inputs.MULTISTATE_R10_C16, dict(kernel="auto", dtype="auto", storage=cat.STORE_NIB4), "planes_kernel"),
+    "planes_u8_c16": (inputs.MULTISTATE_R10_C16, dict(kernel="auto", dtype="auto"), "planes_kernel"),
     "runsum_r8": (inputs.scaled_rule(8), dict(kernel="runsum", dtype="auto"), "runsum_kernel"),
     "stencil_r1": (inputs.scaled_rule(1), dict(kernel="stencil", dtype="auto"), "smem_stencil_kernel"),
 }
