@@ -978,15 +978,15 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   // One pass over the instances (thousands, in no order in memory).
   bool all_tc = true;   // Moore, zero boundary, uint8 storage, no FP4: other instances step one by one
   // Several steps of grids whose options are all left to the library, on bit
-  // planes: from six steps and 2^25 cells on, or four and 2^27 (512 grids with
-  // sides up to 900 / 1400 / 2048, 54 / 102 / 179 million cells, us for 4 steps:
-  // tiles 165 / 260 / 408, planes 185 / 274 / 408; for 6: 242 / 385 / 607
-  // against 243 / 362 / 545; for 12: 472 / 761 / 1201 against 418 / 632 / 956).
+  // planes: from eight steps and 2^25 cells on, or six and 2^27 (512 grids with
+  // sides up to 900 / 1400 / 2048, 54 / 102 / 179 million cells, us for 6 steps:
+  // tiles 230 / 371 / 582, planes 243 / 362 / 545; for 8: 302 / 490 / 771 against
+  // 302 / 453 / 681; for 12: 448 / 730 / 1149 against 418 / 634 / 954).
   // A captured call keeps to the tiles, one launch per
   // step, since the planes need the radii side by side.
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   CAT_CUDA(cudaStreamIsCapturing(s, &cs));
-  bool packed = n_steps >= 4 && cs == cudaStreamCaptureStatusNone;
+  bool packed = n_steps >= 6 && cs == cudaStreamCaptureStatusNone;
   int64_t cells = 0;
   bool one_device = true, one_dtype = true, small = true;
   for (int32_t i = 0; i < count; ++i) {
@@ -999,7 +999,7 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
     one_dtype &= h->dtype == hs[0]->dtype;
     small &= h->H <= 128 * 32767 && h->W <= 128 * 32767;
   }
-  packed &= cells >= (n_steps >= 6 ? 1 << 25 : 1 << 27);
+  packed &= cells >= (n_steps >= 8 ? 1 << 25 : 1 << 27);
   std::unique_lock<std::mutex> lk(g_plan_mu);
   BatchPlan *pl = nullptr;
   for (BatchPlan *c : g_plans)

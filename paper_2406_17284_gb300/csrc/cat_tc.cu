@@ -579,14 +579,17 @@ __device__ __forceinline__ uint32_t rule4_binary_h(uint32_t s01, uint32_t s23, u
   return ~neg & 0x01010101u;
 }
 
-// The same where no count is above 961 (r <= 15): S is in a range iff
-// |S - middle| <= half its width, both exact in f16 as multiples of half the
-// scale below 2^11, and so is every difference (equality gives +0; an empty
-// range has half width -1/2).  Two operations a range and pair instead of
+// The same by another test: S is in a range iff |S - middle| <= half its width.
+// Where no count is above 961 (r <= 15) both are exact in f16 as multiples of
+// half the scale below 2^11, and so is every difference (equality gives +0; an
+// empty range has half width -1/2); larger counts come less a constant (512 for
+// r = 16, 1024 for counts up to 2025), which makes middles and half widths exact
+// again, and a difference that rounds is above every half width.  Two operations a range and pair instead of
 // three, so both ranges are tested for every cell and one logic operation
 // picks by the cell's byte: 16384^2, r = 7 / 12, 96.2
 // -> 94.2 and 106.6 -> 100.6 us a step; C = 16, r = 10, 171.5 -> 160.3; FP16 150.9
-// -> 146.8.
+// -> 146.8; r = 16 112.3 -> 110.0, FP4 r = 12 135.2 -> 130.5, 512 uneven grids,
+// 4 steps 407 -> 392.
 // (The fields of HalfRule hold middles, bl2 and sl2, and half widths then.)
 __device__ __forceinline__ HalfRule make_range_rule(const RuleDev &R, float scale, int offset) {
   const float top = (float)((2 * R.r + 1) * (2 * R.r + 1)), o = (float)offset;
@@ -899,7 +902,10 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   constexpr int EK = EW / 4, EC = 8 / EK;   // of a quarter; warp kq takes the 16-column chunks kq, kq + EK, ..
   using G = Geo<SW, WIDE, BIG>;
   using T = Tm<DT, SW, WIDE, BIG>;
-  constexpr bool kRange = R15 || SW;
+  // packed storage keeps the former test; where a count may exceed 961 (r = 16)
+  // it is taken less kCentre, which leaves half steps exact in f16
+  constexpr bool kRange = !BITS && !NIB;
+  constexpr int kCentre = kRange && !R15 && !SW ? 512 : 0;
   constexpr bool DEC = T::kDec;       // D1 and D2 in separate regions, pass 2 on e4m3 digits
   constexpr int KW = BIG ? 192 : kWin;   // window columns = pass-1 K = pass-2 K
   constexpr int KS = KW / 32;            // K-steps of one e4m3 band product
@@ -1397,7 +1403,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       if constexpr (WIDE) return make_float_rule(p.rule, kScale);
       else return make_int_rule(p.rule);
     }();
-    const HalfRule hr = make_half_rule(p.rule, kScale);
+    const HalfRule hr = make_range_rule(p.rule, kScale, 1024);   // HB: counts up to 2025, less 1024
     TileSeq<false, false, G::kTS> seq(p, first, n_my);
     for (int j = 0; ok && j < n_all; ++j, seq.next(p)) {
       const int reg = j % ND2, k = j % NR;
@@ -1437,13 +1443,14 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               // f16 pairs of cells (2i, 2i + 1): packed by pass 2, or converted
               // here (exact, S * 2^-9 < 4)
               auto pr = [&](int i) -> uint32_t {
-                if constexpr (HB == 2) return v[c][i];
-                else return h2_bits(__floats2half2_rn(__uint_as_float(v[c][2 * i]), __uint_as_float(v[c][2 * i + 1])));
+                const __half2 c1024 = __float2half2_rn(1024.0f * kScale);
+                if constexpr (HB == 2) return h2_bits(__hsub2(as_h2(v[c][i]), c1024));
+                else return h2_bits(__hsub2(__floats2half2_rn(__uint_as_float(v[c][2 * i]), __uint_as_float(v[c][2 * i + 1])), c1024));
               };
-              ov.x = rule4_binary_h(pr(0), pr(1), cv.x, hr);
-              ov.y = rule4_binary_h(pr(2), pr(3), cv.y, hr);
-              ov.z = rule4_binary_h(pr(4), pr(5), cv.z, hr);
-              ov.w = rule4_binary_h(pr(6), pr(7), cv.w, hr);
+              ov.x = rule4_range_h(pr(0), pr(1), cv.x, hr);
+              ov.y = rule4_range_h(pr(2), pr(3), cv.y, hr);
+              ov.z = rule4_range_h(pr(4), pr(5), cv.z, hr);
+              ov.w = rule4_range_h(pr(6), pr(7), cv.w, hr);
             }
             *cell = ov;
           } else {   // box counts
@@ -1481,7 +1488,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     bool ok = true;
     auto offset_of = [](const RuleDev &R) { return OF ? 16 * (2 * R.r + 1) : 0; };
     auto make_rule = [&](const RuleDev &R) {
-      if constexpr (kRange) return make_range_rule(R, kScale, offset_of(R));
+      if constexpr (kRange) return make_range_rule(R, kScale, offset_of(R) + kCentre);
       else return make_half_rule(R, kScale);
     };
     HalfRule hr = make_rule(BATCH ? RuleDev{} : p.rule);
@@ -1508,6 +1515,9 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
       if (!(ok = warp_wait(&bars->c_full[k], (j / NR) & 1, bars, p.timeout_ns))) break;
       uint8_t *ring = smem + L::kRing + k * L::kRingBytes;
       {
+        auto count = [](uint32_t s2) {   // as the rule's middles take it
+          return kCentre ? h2_bits(__hsub2(as_h2(s2), __float2half2_rn(kCentre * kScale))) : s2;
+        };
         const bool sums_mode = !BATCH && p.sums != nullptr;
         if (BITS && !sums_mode) {
           // 16 cells of a chunk are 16 bits of the row (lowest x lowest);
@@ -1553,7 +1563,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             const uint4 cv = *cell;
             uint4 ov;
             auto next = [&](int i, uint32_t cells) {
-              if constexpr (kRange) return rule4_range_h(v[c][i], v[c][i + 1], cells, hr);
+              if constexpr (kRange) return rule4_range_h(count(v[c][i]), count(v[c][i + 1]), cells, hr);
               else return rule4_binary_h(v[c][i], v[c][i + 1], cells, hr);
             };
             ov = make_uint4(next(0, cv.x), next(2, cv.y), next(4, cv.z), next(6, cv.w));
@@ -1569,15 +1579,15 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               const uint4 cv = *cell;
               uint4 ov;
               if (R.C <= 128) {
-                ov.x = rule4_multistate_small_h<kRange>(v[c][0], v[c][1], cv.x, hr, Kc);
-                ov.y = rule4_multistate_small_h<kRange>(v[c][2], v[c][3], cv.y, hr, Kc);
-                ov.z = rule4_multistate_small_h<kRange>(v[c][4], v[c][5], cv.z, hr, Kc);
-                ov.w = rule4_multistate_small_h<kRange>(v[c][6], v[c][7], cv.w, hr, Kc);
+                ov.x = rule4_multistate_small_h<kRange>(count(v[c][0]), count(v[c][1]), cv.x, hr, Kc);
+                ov.y = rule4_multistate_small_h<kRange>(count(v[c][2]), count(v[c][3]), cv.y, hr, Kc);
+                ov.z = rule4_multistate_small_h<kRange>(count(v[c][4]), count(v[c][5]), cv.z, hr, Kc);
+                ov.w = rule4_multistate_small_h<kRange>(count(v[c][6]), count(v[c][7]), cv.w, hr, Kc);
               } else {
-                ov.x = rule4_multistate_h<kRange>(v[c][0], v[c][1], cv.x, hr, Cb);
-                ov.y = rule4_multistate_h<kRange>(v[c][2], v[c][3], cv.y, hr, Cb);
-                ov.z = rule4_multistate_h<kRange>(v[c][4], v[c][5], cv.z, hr, Cb);
-                ov.w = rule4_multistate_h<kRange>(v[c][6], v[c][7], cv.w, hr, Cb);
+                ov.x = rule4_multistate_h<kRange>(count(v[c][0]), count(v[c][1]), cv.x, hr, Cb);
+                ov.y = rule4_multistate_h<kRange>(count(v[c][2]), count(v[c][3]), cv.y, hr, Cb);
+                ov.z = rule4_multistate_h<kRange>(count(v[c][4]), count(v[c][5]), cv.z, hr, Cb);
+                ov.w = rule4_multistate_h<kRange>(count(v[c][6]), count(v[c][7]), cv.w, hr, Cb);
               }
               *cell = ov;
             }
@@ -1592,10 +1602,10 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
               uint4 *cell = reinterpret_cast<uint4 *>(ring + off_c[c]);
               const uint4 cv = *cell;
               uint4 ov;
-              ov.x = rule4_multistate_h<kRange>(v[c][0], v[c][1], cv.x, hr, Cb);
-              ov.y = rule4_multistate_h<kRange>(v[c][2], v[c][3], cv.y, hr, Cb);
-              ov.z = rule4_multistate_h<kRange>(v[c][4], v[c][5], cv.z, hr, Cb);
-              ov.w = rule4_multistate_h<kRange>(v[c][6], v[c][7], cv.w, hr, Cb);
+              ov.x = rule4_multistate_h<kRange>(count(v[c][0]), count(v[c][1]), cv.x, hr, Cb);
+              ov.y = rule4_multistate_h<kRange>(count(v[c][2]), count(v[c][3]), cv.y, hr, Cb);
+              ov.z = rule4_multistate_h<kRange>(count(v[c][4]), count(v[c][5]), cv.z, hr, Cb);
+              ov.w = rule4_multistate_h<kRange>(count(v[c][6]), count(v[c][7]), cv.w, hr, Cb);
               *cell = ov;
             }
           }
