@@ -212,11 +212,16 @@ cat::PlanesGrid planes_grid(const cat_instance *h, int in) {
                          h->dev.id, h->dev.sms};
 }
 
+// The bit-plane kernels multiply a row by a pitch of 32 bits (planes::row_ptr);
+// a caller's buffers may have a longer one, which the tensor maps of the other
+// kernels take.
+bool planes_pitch(const cat_instance *h) { return h->pitch <= (int64_t)UINT32_MAX; }
+
 // Options left to the library: the bit-plane kernel steps the grids on which
 // it is the faster one (the configuration that cat_get_options reports serves
 // the others, box sums and the bounded-wait test).
 bool use_planes(const cat_instance *h) {
-  return h->auto_choice && h->inject == 0 && cat::planes_preferred(planes_grid(h, 0));
+  return h->auto_choice && h->inject == 0 && planes_pitch(h) && cat::planes_preferred(planes_grid(h, 0));
 }
 
 // The first steps of n_steps from buffer `in` into the other one; *taken: how many.
@@ -238,7 +243,7 @@ int launch_planes(cat_instance *h, int in, int64_t n_steps, int64_t *taken, cuda
 // outside the grid's rows are not touched).
 bool packed_steps_possible(const cat_instance *h, int64_t n_steps) {
   return n_steps >= 2 && h->auto_choice && h->inject == 0 && h->storage == CAT_STORE_U8 && h->rule.C == 2 &&
-         h->rule.nbhd == 'M' && h->rule.r <= 16 && h->W >= 64;
+         h->rule.nbhd == 'M' && h->rule.r <= 16 && h->W >= 64 && planes_pitch(h);
 }
 
 bool use_packed_steps(const cat_instance *h, int64_t n_steps) {

@@ -171,7 +171,7 @@ cudaError_t swar_sums_launch(const uint8_t *in, int64_t pitch, int64_t H, int64_
 struct PlanesGrid {
   const uint8_t *in;   // row 0 of the input and output: grid cell 0 for uint8, cell -frame for packed rows
   uint8_t *out;
-  int64_t pitch, H, W; // (one pitch for both)
+  int64_t pitch, H, W; // (one pitch for both, below 2^32)
   int32_t storage_in, storage_out;   // the same, or uint8 and one bit (C = 2)
   int32_t frame;       // ghost frame of a periodic grid (16 cells, filled), else 0
   RuleDev rule;

@@ -20,7 +20,8 @@ planes::Kernel find(const PlanesGrid &g, int *kind) {
   const int r = g.rule.r;
   const bool from_u8 = g.storage_in == CAT_STORE_U8, to_u8 = g.storage_out == CAT_STORE_U8;
   *kind = from_u8 && to_u8 ? (g.rule.C > 2 ? 1 : 0) : from_u8 ? 2 : to_u8 ? 3 : g.storage_in == CAT_STORE_BIT1 ? 4 : 5;
-  if (g.rule.nbhd != 0 || r < 1 || r > planes::kMaxR || g.rule.C > 16) return planes::Kernel{};
+  if (g.rule.nbhd != 0 || r < 1 || r > planes::kMaxR || g.rule.C > 16 || g.pitch > (int64_t)UINT32_MAX)
+    return planes::Kernel{};
   if (*kind >= 2 && *kind <= 4 && g.rule.C != 2) return planes::Kernel{};
   switch (*kind) {
     case 0: return planes::kernel_u8(r);
@@ -244,7 +245,8 @@ cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaSt
   t.p.rows = plan.rows;
   t.p.strips = (int32_t)((g.H + plan.rows - 1) / plan.rows);
   const int64_t smem = tile_smem(g, plan);
-  if (!k.fn || plan.steps > max_tile_steps(g.rule.r) || smem > kMaxSmem) return cudaErrorInvalidValue;
+  if (!k.fn || plan.steps > max_tile_steps(g.rule.r) || smem > kMaxSmem || g.pitch > (int64_t)UINT32_MAX)
+    return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
   if (e == cudaSuccess)   // (as the streaming kernels ask for: launches of both follow each other)
     e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);

@@ -92,3 +92,30 @@ def test_rejections(cat):
         assert e.value.code == cat.CAT_ERR_UNSUPPORTED
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("n", [1, 5])
+def test_pitch_above_four_gib(cat, n):
+    """Rows more than 2^32 bytes apart, with every option left to the library."""
+    import torch
+    H, W, pitch = 3, 200, (1 << 32) + 4096
+    size = (H - 1) * pitch + 4096
+    if torch.cuda.mem_get_info()[0] < 3 * size:
+        pytest.skip("not enough device memory")
+    rule = inputs.scaled_rule(4)
+    grid = inputs.bernoulli(H, W, 0.5, 17)
+    a = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    b = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    rows = [torch.as_strided(t, (H, W), (pitch, 1)) for t in (a, b)]
+    rows[0].copy_(torch.from_numpy(grid))
+    g = cat.Grid(H, W, rule, kernel="auto", dtype="auto")
+    try:
+        cat.cat_bind(g.handle, a.data_ptr(), b.data_ptr(), pitch)
+        g.step(n)
+        torch.cuda.synchronize()
+        assert g.status() == cat.CAT_OK
+    finally:
+        g.close()
+    assert np.array_equal(rows[n & 1].cpu().numpy(), oracle.step(grid, orule(rule), n_steps=n))
+    for t in (a, b):    # nothing between the rows
+        assert not bool(t[4096:pitch].any()) and not bool(t[pitch + 4096:2 * pitch].any())

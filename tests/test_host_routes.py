@@ -1,0 +1,85 @@
+"""Which launches a call makes, on the CPU: the library's host code (cat_api.cu,
+cat_tune.cu) linked with a CUDA runtime and launchers that keep a record
+(tests/host/fake_cuda.cpp), under which bit planes are preferred wherever the
+host code asks about them."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2406_17284_gb300 import build, cat, inputs
+
+CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(build._nvcc())), "include")
+
+
+class Host:
+    """The C ABI on the fake runtime."""
+
+    def __init__(self, lib):
+        self.lib = lib
+
+    def __getattr__(self, name):
+        def call(*args):
+            rc = getattr(self.lib, name)(*[ctypes.c_int64(a) if isinstance(a, int) else a for a in args])
+            assert rc == cat.CAT_OK, (name, rc, self.lib.cat_last_error())
+        return call
+
+    def rc(self, name, *args):
+        return getattr(self.lib, name)(*[ctypes.c_int64(a) if isinstance(a, int) else a for a in args])
+
+    def grid(self, H, W, r, C=2, storage=0, boundary=0):
+        h = ctypes.c_void_p()
+        rule = cat.make_rule(**inputs.scaled_rule(r, C=C))
+        self.cat_create_ex(H, W, ctypes.byref(rule), boundary, storage, ctypes.byref(h))
+        return h
+
+    def log(self):
+        out = ctypes.create_string_buffer(1 << 16)
+        assert self.lib.fake_log(out, len(out)) >= 0
+        return out.value.decode().split("\n")[:-1]
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "libcat_host.so")
+    src = [os.path.join(build.CSRC, f) for f in ("cat_api.cu", "cat_tune.cu")]
+    src.append(os.path.join(os.path.dirname(os.path.abspath(__file__)), "host", "fake_cuda.cpp"))
+    cmd = ["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-fvisibility=hidden", "-I", CUDA_INCLUDE, "-I", build.CSRC,
+           "-x", "c++", *src, "-o", so]
+    subprocess.run(cmd, check=True)
+    return ctypes.CDLL(so)
+
+
+@pytest.fixture
+def host(lib):
+    h = Host(lib)
+    lib.cat_last_error.restype = ctypes.c_char_p
+    yield h
+    lib.fake_fail(None)
+    lib.fake_capturing(0)
+    h.log()
+
+
+# Buffers that no launch touches here: only their addresses and pitch matter.
+A, B = 1 << 44, 1 << 45
+
+
+@pytest.mark.parametrize("pitch,route", [((1 << 32) - 16, "planes u8 to u8"), (1 << 32, "tensor cores"),
+                                         ((1 << 32) + 4096, "tensor cores")])
+def test_pitches_that_the_bit_planes_take(host, pitch, route):
+    """The bit-plane kernels multiply a row by a pitch of 32 bits; longer ones,
+    which cat_bind accepts, go to the tensor cores, in every way to step."""
+    h = host.grid(3, 200, 4)
+    host.cat_bind(h, A, B, pitch)
+    host.cat_step(h, 1, None)
+    assert host.log() == [route]
+    host.cat_step(h, 4, None)
+    assert all((x == "tensor cores") == (route == "tensor cores") for x in host.log())
+    host.cat_destroy(h)
+    if route == "tensor cores":
+        large = host.grid(8192, 8192, 4)   # enough cells for a batch to step on bit planes
+        host.cat_bind(large, A, B, pitch)
+        host.cat_batch_step((ctypes.c_void_p * 1)(large), 1, 8, None)
+        assert "batch planes" not in host.log()
+        host.cat_destroy(large)
