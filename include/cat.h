@@ -326,7 +326,10 @@ CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
 /* Advances the instance by n_steps >= 0 synchronous LTL steps on `stream`:
  * the host loop of Sec. IV-C (Alg. 1), one launch reading buffer A and
  * writing buffer B, then the two swap (with steps_per_launch = k > 1, k steps
- * per launch, the swap inside it).  The buffer that does not hold the state
+ * per launch, the swap inside it).  However the steps are split into launches,
+ * the state is afterwards in the buffer that held it before when n_steps is
+ * even, so a captured call of an even number of steps can be replayed.  The
+ * buffer that does not hold the state
  * afterwards has no defined contents.  Each step computes the band products of
  * Sec. IV (Eqs. 1-2) and the rule of Sec. V-A for every cell.  Errors:
  * INVALID_ARG (NULL, n_steps < 0), CUDA (launch failure); device-side

@@ -224,12 +224,12 @@ bool use_planes(const cat_instance *h) {
   return h->auto_choice && h->inject == 0 && planes_pitch(h) && cat::planes_preferred(planes_grid(h, 0));
 }
 
-// The first steps of n_steps from buffer `in` into the other one; *taken: how many.
-int launch_planes(cat_instance *h, int in, int64_t n_steps, int64_t *taken, cudaStream_t s) {
+// n_steps steps from buffer `in` into the other one, in one launch (more than
+// one step where planes_launches said so).
+int launch_planes(cat_instance *h, int in, int64_t n_steps, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   const cat::PlanesGrid g = planes_grid(h, in);
-  const cat::TilePlan plan = cat::planes_tile_plan(g, n_steps);
-  *taken = plan.steps > 0 ? plan.steps : 1;
+  const cat::TilePlan plan = cat::planes_tile_steps(g, n_steps);
   if (h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, false, s);
   if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
@@ -301,10 +301,7 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
 // cooperative launch of the tcgen05 Moore kernel (zero boundary).
 int launch_step(cat_instance *h, int in, int32_t *sums, int64_t sums_ld, cudaStream_t s, int n_steps = 1) {
   cudaError_t e;
-  if (!sums && n_steps == 1 && use_planes(h)) {
-    int64_t taken;
-    return launch_planes(h, in, 1, &taken, s);
-  }
+  if (!sums && n_steps == 1 && use_planes(h)) return launch_planes(h, in, 1, s);
   if (h->kernel == CAT_KERNEL_TCGEN05) {
     if (h->ghost) {  // periodic: refresh the input's ghost frame first
       e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, true, s);
@@ -954,15 +951,20 @@ int cat_step(cat_handle_t h, int64_t n_steps, void *stream) {
     if (rc == CAT_OK) h->cur ^= (int)(n_steps & 1);
     return rc;
   }
-  for (int64_t t = 0; t < n_steps;) {
-    if (h->storage == CAT_STORE_BIT1 && use_planes(h)) {   // library-owned buffers: the state moves with every launch
-      int64_t taken;
-      const int rc = launch_planes(h, h->cur, n_steps - t, &taken, (cudaStream_t)stream);
+  if (h->storage == CAT_STORE_BIT1 && n_steps > 0 && use_planes(h)) {
+    // the state moves with every launch, and as many times as n_steps steps
+    // would move it, odd or even: a captured call of an even number of steps
+    // ends in the buffer that its replay reads
+    for (int64_t left = n_steps, launches = cat::planes_launches(planes_grid(h, h->cur), n_steps); launches > 0; --launches) {
+      const int64_t k = (left + launches - 1) / launches;
+      const int rc = launch_planes(h, h->cur, k, (cudaStream_t)stream);
       if (rc) return rc;
       h->cur ^= 1;
-      t += taken;
-      continue;
+      left -= k;
     }
+    return CAT_OK;
+  }
+  for (int64_t t = 0; t < n_steps;) {
     const int m = (int)std::min<int64_t>(h->steps_per_launch, n_steps - t);
     int rc = launch_step(h, h->cur, nullptr, 0, (cudaStream_t)stream, m);
     if (rc) return rc;

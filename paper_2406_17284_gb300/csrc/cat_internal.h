@@ -190,6 +190,10 @@ struct TilePlan {
   int32_t steps, rows;   // steps per launch, output rows per strip
 };
 TilePlan planes_tile_plan(const PlanesGrid &g, int64_t n_left);
+TilePlan planes_tile_steps(const PlanesGrid &g, int64_t steps);   // for a launch of just these steps
+// Launches for n_steps >= 1 steps whose number is odd or even as n_steps is, of
+// equally many steps but for the remainder (the first ones take one more).
+int64_t planes_launches(const PlanesGrid &g, int64_t n_steps);
 TilePlan planes_tile_fixed(const PlanesGrid &g, int steps);
 cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaStream_t s);
 // Two-state uint8 grids of any sizes, radii (<= 16) and rules, advanced several

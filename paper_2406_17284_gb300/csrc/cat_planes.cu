@@ -215,17 +215,32 @@ cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
 // 2.7 / 4.4 / 6.1; 4096^2: 5.4 / 7.5 / 10.5 / 12.8 -> 3.1 / 5.9 / 9.3 / 12.5).
 // A single step pays only where the streaming kernel's first 2r rows weigh
 // more than two barriers (r >= 8).
-TilePlan planes_tile_plan(const PlanesGrid &g, int64_t n_left) {
+static int64_t fewest_launches(int r, int64_t n_steps) {
+  const int most = std::min({8, std::max(1, 20 / r), max_tile_steps(r)});
+  return (n_steps + most - 1) / most;
+}
+
+TilePlan planes_tile_steps(const PlanesGrid &g, int64_t steps) {
   const TilePlan none{0, 0};
   const int r = g.rule.r;
-  if (g.rule.nbhd != 0 || r > planes::kMaxR || g.rule.C != 2 || g.storage_in == CAT_STORE_NIB4 || g.frame || n_left < 1)
+  if (g.rule.nbhd != 0 || r > planes::kMaxR || g.rule.C != 2 || g.storage_in == CAT_STORE_NIB4 || g.frame || steps < 1 ||
+      steps > max_tile_steps(r))
     return none;
-  const int most = std::min({8, std::max(1, 20 / r), max_tile_steps(r)});
-  const int64_t launches = (n_left + most - 1) / most;
-  const int steps = (int)((n_left + launches - 1) / launches);
   if (steps == 1 && r < 8) return none;
-  const TilePlan t{steps, one_wave_rows(g)};
+  const TilePlan t{(int32_t)steps, one_wave_rows(g)};
   return t.rows > 0 && tile_smem(g, t) <= kMaxSmem ? t : none;
+}
+
+TilePlan planes_tile_plan(const PlanesGrid &g, int64_t n_left) {
+  if (n_left < 1 || g.rule.r > planes::kMaxR) return TilePlan{0, 0};
+  const int64_t launches = fewest_launches(g.rule.r, n_left);
+  return planes_tile_steps(g, (n_left + launches - 1) / launches);
+}
+
+int64_t planes_launches(const PlanesGrid &g, int64_t n_steps) {
+  int64_t launches = fewest_launches(g.rule.r, n_steps);
+  launches += (launches ^ n_steps) & 1;   // (at most n_steps)
+  return planes_tile_steps(g, (n_steps + launches - 1) / launches).steps > 0 ? launches : n_steps;
 }
 
 // k steps per launch as asked for, on any grid: several waves of strips where

@@ -137,6 +137,8 @@ bool planes_preferred(const PlanesGrid &g) { return g.rule.nbhd == 0 && g.rule.r
 bool planes_steps_preferred(const PlanesGrid &, int64_t) { return true; }
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t) { return launched("planes " + storages(g)); }
 TilePlan planes_tile_plan(const PlanesGrid &, int64_t) { return TilePlan{0, 0}; }
+TilePlan planes_tile_steps(const PlanesGrid &, int64_t) { return TilePlan{0, 0}; }
+int64_t planes_launches(const PlanesGrid &, int64_t n_steps) { return n_steps; }
 TilePlan planes_tile_fixed(const PlanesGrid &, int steps) { return TilePlan{steps, 64}; }
 cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &, cudaStream_t) { return launched("tile " + storages(g)); }
 struct PlanesBatch {};

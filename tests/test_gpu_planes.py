@@ -193,3 +193,34 @@ def test_packed_batch_of_uneven_grids(cat):
     finally:
         for g in grids + [big, ref]:
             g.close()
+
+
+@pytest.mark.parametrize("storage,H,W,r,n", [(1, 300, 700, 1, 2), (1, 300, 700, 1, 8), (1, 130, 2000, 1, 100),
+                                             (1, 300, 700, 4, 4), (1, 300, 700, 10, 2), (1, 50, 90, 16, 4),
+                                             (0, 300, 700, 1, 8), (0, 300, 700, 10, 6), (0, 130, 1031, 4, 2),
+                                             (2, 200, 333, 3, 2)])
+def test_captured_steps_with_the_options_left(cat, storage, H, W, r, n):
+    """An even number of steps of a default grid, captured into a graph in one
+    call and replayed three times, then a plain call of an odd number."""
+    import torch
+    rule = inputs.scaled_rule(r, M=1, C=5 if storage == 2 else 2)
+    host = board(H, W, rule["C"], 3 * r + n)
+    g = cat.Grid(H, W, rule, kernel="auto", dtype="auto", storage=storage)
+    try:
+        g.set_state(host)
+        at = cat.cat_state_ptr(g.handle)[0]
+        s = torch.cuda.Stream()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            g.step(n, s)
+        assert cat.cat_state_ptr(g.handle)[0] == at
+        for _ in range(3):
+            graph.replay()
+        torch.cuda.synchronize()
+        want = oracle.step(host, oracle.Rule(**rule), n_steps=3 * n)
+        assert np.array_equal(g.get_state(), want)
+        g.step(3)
+        assert cat.cat_state_ptr(g.handle)[0] != at
+        assert np.array_equal(g.get_state(), oracle.step(want, oracle.Rule(**rule), n_steps=3))
+    finally:
+        g.close()
