@@ -316,9 +316,9 @@ CAT_API int cat_state_ptr(cat_handle_t h, void **dptr, int64_t *pitch);
  * is taken from a as it is (no copy); after a step the state is in b, then a
  * again, as cat_state_ptr reports.  The instance's own buffers are freed; the
  * library never frees bound ones (cat_destroy leaves them to the caller, who
- * must keep them alive while the instance uses them).  Of the two buffers,
- * the one that does not hold the state is the library's to work in.
- * Synchronises the device.  Zero boundary and uint8 storage only (UNSUPPORTED otherwise, and
+ * must keep them alive while the instance uses them).  After n >= 1 steps in
+ * one call the other buffer holds the generation before the state, as after n
+ * single steps.  Synchronises the device.  Zero boundary and uint8 storage only (UNSUPPORTED otherwise, and
  * for a later change to one-bit storage).  Errors: INVALID_ARG, UNSUPPORTED,
  * CUDA.                                                                     */
 CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
@@ -329,8 +329,8 @@ CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
  * per launch, the swap inside it).  However the steps are split into launches,
  * the state is afterwards in the buffer that held it before when n_steps is
  * even, so a captured call of an even number of steps can be replayed.  The
- * buffer that does not hold the state
- * afterwards has no defined contents.  Each step computes the band products of
+ * buffer that does not hold the state afterwards has no defined contents,
+ * unless it is a caller's (cat_bind).  Each step computes the band products of
  * Sec. IV (Eqs. 1-2) and the rule of Sec. V-A for every cell.  Errors:
  * INVALID_ARG (NULL, n_steps < 0), CUDA (launch failure); device-side
  * timeouts are reported by cat_status.                                     */
@@ -343,7 +343,7 @@ CAT_API int cat_step(cat_handle_t h, int64_t n_steps, void *stream);
  * persistent launch over a flat tile work-list of all instances, and when
  * `stream` is not capturing the n_steps launches are replayed from a CUDA
  * graph cached for this handle list (with every instance's options left to the
- * library, and n_steps >= 8 with 2^25 cells or more or n_steps >= 6 with 2^27,
+ * library, on buffers of its own, and n_steps >= 8 with 2^25 cells or more or n_steps >= 6 with 2^27,
  * that graph packs the two-state grids, steps them on bit planes and unpacks them); otherwise every instance is stepped by
  * its own launches, one step at a time.  Errors: INVALID_ARG (NULL or
  * repeated handles, instances on different devices, mixed dtypes in a

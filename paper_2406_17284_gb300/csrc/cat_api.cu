@@ -946,10 +946,15 @@ int cat_state_ptr(cat_handle_t h, void **dptr, int64_t *pitch) {
 int cat_step(cat_handle_t h, int64_t n_steps, void *stream) {
   if (!h) return fail(CAT_ERR_INVALID_ARG, "handle is NULL");
   if (n_steps < 0) return fail(CAT_ERR_INVALID_ARG, "n_steps < 0");
-  if (use_packed_steps(h, n_steps)) {
-    const int rc = launch_packed_steps(h, n_steps, (cudaStream_t)stream);
-    if (rc == CAT_OK) h->cur ^= (int)(n_steps & 1);
-    return rc;
+  // a caller's other buffer holds the generation before the last, as after steps
+  // one by one: the last step goes from bytes to bytes
+  int64_t packed = h->owns_buffers ? n_steps : n_steps - 1;
+  if (use_packed_steps(h, packed)) {
+    const int rc = launch_packed_steps(h, packed, (cudaStream_t)stream);
+    if (rc) return rc;
+    h->cur ^= (int)(packed & 1);
+  } else {
+    packed = 0;
   }
   if (h->storage == CAT_STORE_BIT1 && n_steps > 0 && use_planes(h)) {
     // the state moves with every launch, and as many times as n_steps steps
@@ -964,7 +969,7 @@ int cat_step(cat_handle_t h, int64_t n_steps, void *stream) {
     }
     return CAT_OK;
   }
-  for (int64_t t = 0; t < n_steps;) {
+  for (int64_t t = packed; t < n_steps;) {
     const int m = (int)std::min<int64_t>(h->steps_per_launch, n_steps - t);
     int rc = launch_step(h, h->cur, nullptr, 0, (cudaStream_t)stream, m);
     if (rc) return rc;
@@ -1000,7 +1005,7 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
     const cat_instance *h = hs[i];
     all_tc &= h->kernel == CAT_KERNEL_TCGEN05 && h->ghost == 0 && h->storage == CAT_STORE_U8 &&
               h->rule.nbhd == 'M' && !wide_tile(h) && h->dtype != CAT_DTYPE_FP4_E2M1;
-    packed &= packed_steps_possible(h, n_steps);
+    packed &= packed_steps_possible(h, n_steps) && h->owns_buffers;   // (see cat_step: the generation before)
     cells += h->H * h->W;
     one_device &= h->dev.id == hs[0]->dev.id;
     one_dtype &= h->dtype == hs[0]->dtype;

@@ -119,3 +119,34 @@ def test_pitch_above_four_gib(cat, n):
     assert np.array_equal(rows[n & 1].cpu().numpy(), oracle.step(grid, orule(rule), n_steps=n))
     for t in (a, b):    # nothing between the rows
         assert not bool(t[4096:pitch].any()) and not bool(t[pitch + 4096:2 * pitch].any())
+
+
+@pytest.mark.parametrize("H,W,pitch,r,n", [(130, 1024, 1024, 4, 2), (130, 1024, 1024, 4, 3), (70, 97, 112, 1, 9),
+                                           (300, 517, 544, 12, 4), (2600, 2700, 2704, 2, 8)])
+def test_the_other_buffer_holds_the_generation_before(cat, H, W, pitch, r, n):
+    """A caller's two buffers after several steps in one call, every option left
+    to the library: the state, and the generation before it (cat_step and
+    cat_batch_step)."""
+    import torch
+    rule = inputs.scaled_rule(r)
+    grid = inputs.bernoulli(H, W, 0.5, H + n)
+    before = oracle.step(grid, orule(rule), n_steps=n - 1)
+    after = oracle.step(before, orule(rule))
+    for batch in (False, True):
+        a = torch.zeros((H, pitch), dtype=torch.uint8, device="cuda")
+        b = torch.zeros((H, pitch), dtype=torch.uint8, device="cuda")
+        a[:, :W] = torch.from_numpy(grid).cuda()
+        g = cat.Grid(H, W, rule, kernel="auto", dtype="auto")
+        try:
+            cat.cat_bind(g.handle, a.data_ptr(), b.data_ptr(), pitch)
+            if batch:
+                cat.cat_batch_step([g.handle], n)
+            else:
+                g.step(n)
+            torch.cuda.synchronize()
+            state, other = (b, a) if n & 1 else (a, b)
+            assert cat.cat_state_ptr(g.handle)[0] == state.data_ptr()
+        finally:
+            g.close()
+        assert np.array_equal(state[:, :W].cpu().numpy(), after), batch
+        assert np.array_equal(other[:, :W].cpu().numpy(), before), batch

@@ -83,3 +83,20 @@ def test_pitches_that_the_bit_planes_take(host, pitch, route):
         host.cat_batch_step((ctypes.c_void_p * 1)(large), 1, 8, None)
         assert "batch planes" not in host.log()
         host.cat_destroy(large)
+
+
+@pytest.mark.parametrize("bound", [False, True])
+def test_steps_of_a_callers_buffers_end_from_bytes_to_bytes(host, bound):
+    """Several steps keep the states between as bits; on a caller's buffers the
+    last one reads bytes, so that the other buffer holds the generation before.
+    A batch does so only on buffers of the library's own."""
+    h = host.grid(8192, 8192, 4)
+    if bound:
+        host.cat_bind(h, A, B, 8192)
+    host.cat_step(h, 4, None)
+    last = "planes u8 to u8" if bound else "planes bit1 to u8"
+    assert host.log() == ["planes u8 to bit1", "planes bit1 to bit1", *(["planes bit1 to u8"] if bound else
+                                                                        ["planes bit1 to bit1"]), last]
+    host.cat_batch_step((ctypes.c_void_p * 1)(h), 1, 8, None)
+    assert ("batch tiles" in host.log()) == bound
+    host.cat_destroy(h)
