@@ -318,7 +318,10 @@ CAT_API int cat_state_ptr(cat_handle_t h, void **dptr, int64_t *pitch);
  * library never frees bound ones (cat_destroy leaves them to the caller, who
  * must keep them alive while the instance uses them).  After n >= 1 steps in
  * one call the other buffer holds the generation before the state, as after n
- * single steps.  Synchronises the device.  Zero boundary and uint8 storage only (UNSUPPORTED otherwise, and
+ * single steps.  Rows are stored in units of 16 bytes: the bytes from W up to
+ * the next multiple of 16 of a row may be written (by the TCGEN05 kernels and
+ * by cat_batch_step, whatever was there) and are never read as cells; no other
+ * byte past W is touched.  Synchronises the device.  Zero boundary and uint8 storage only (UNSUPPORTED otherwise, and
  * for a later change to one-bit storage).  Errors: INVALID_ARG, UNSUPPORTED,
  * CUDA.                                                                     */
 CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);

@@ -611,7 +611,8 @@ __device__ __forceinline__ void batch_step(const BatchParams &b, const BatchGrid
   p.H = __ldg(&g->H);
   p.W = __ldg(&g->W);
   // the last step's row goes on to the end of its last 16 cells, like the
-  // tensor-core kernel's stores (the first step's input ends at W)
+  // tensor-core kernels' stores, which cover whole 16-byte units: the bytes there
+  // are the same on both routes of a batch (the first step's input ends at W)
   p.written = b.step == b.steps - 1 ? (p.W + 15) & ~15 : p.W;
   p.seg = __ldg(&g->seg);
   p.rows = __ldg(&g->rows);

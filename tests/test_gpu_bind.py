@@ -150,3 +150,35 @@ def test_the_other_buffer_holds_the_generation_before(cat, H, W, pitch, r, n):
             g.close()
         assert np.array_equal(state[:, :W].cpu().numpy(), after), batch
         assert np.array_equal(other[:, :W].cpu().numpy(), before), batch
+
+
+@pytest.mark.parametrize("kernel,dtype,r,tile", [("tcgen05", "fp8", 4, 0), ("tcgen05", "fp8", 9, 0), ("tcgen05", "fp16", 9, 0),
+                                                 ("tcgen05", "fp4", 9, 0), ("tcgen05", "fp8", 24, 0),
+                                                 ("tcgen05", "fp8", 24, 96), ("mma_sync", "fp16", 4, 0),
+                                                 ("stencil", "auto", 4, 0), ("runsum", "auto", 4, 0), ("auto", "auto", 4, 0),
+                                                 ("auto", "auto", 9, 0)])
+def test_no_byte_past_a_rows_last_unit_is_touched(cat, kernel, dtype, r, tile):
+    """A pitch above W, births everywhere: the bytes from W to the next multiple
+    of 16 are the library's, those beyond stay, by cat_step and cat_batch_step."""
+    import torch
+    H, W, pitch, unit = 150, 101, 144, 112
+    rule = dict(inputs.scaled_rule(r), b1=0, b2=(2 * r + 1) ** 2)
+    grid = inputs.bernoulli(H, W, 0.5, r)
+    for batch in (False, True):
+        a = torch.full((H, pitch), 255, dtype=torch.uint8, device="cuda")
+        b = torch.full((H, pitch), 254, dtype=torch.uint8, device="cuda")
+        a[:, :W] = torch.from_numpy(grid).cuda()
+        g = cat.Grid(H, W, rule, kernel=kernel, dtype=dtype, tile=tile)
+        try:
+            cat.cat_bind(g.handle, a.data_ptr(), b.data_ptr(), pitch)
+            for n in (1, 2):
+                if batch:
+                    cat.cat_batch_step([g.handle], n)
+                else:
+                    g.step(n)
+            torch.cuda.synchronize()
+            assert g.status() == cat.CAT_OK
+        finally:
+            g.close()
+        assert np.array_equal(b[:, :W].cpu().numpy(), oracle.step(grid, orule(rule), n_steps=3)), batch
+        assert bool((a[:, unit:] == 255).all()) and bool((b[:, unit:] == 254).all()), batch
