@@ -750,7 +750,9 @@ int cat_create_ex(int64_t H, int64_t W, const cat_rule_t *rule, int32_t boundary
   return CAT_OK;
 }
 
-int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t storage, int32_t steps_per_launch) {
+// cached: CAT_KERNEL_AUTO takes the autotuner's choice from CAT_AUTOTUNE_CACHE.
+static int set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t storage, int32_t steps_per_launch,
+                       bool cached) {
   if (!h) return fail(CAT_ERR_INVALID_ARG, "handle is NULL");
   if (kernel < CAT_KERNEL_AUTO || kernel > CAT_KERNEL_RUNSUM) return fail(CAT_ERR_INVALID_ARG, "unknown kernel %d", kernel);
   if (dtype < CAT_DTYPE_AUTO || dtype > CAT_DTYPE_FP4_E2M1) return fail(CAT_ERR_INVALID_ARG, "unknown dtype %d", dtype);
@@ -764,7 +766,7 @@ int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t stora
   // AUTO: the autotuner's cached choice when CAT_AUTOTUNE_CACHE names a file
   // holding one for this instance (with the storage asked for), else a fixed rule
   int32_t tuned_tile = -1, tuned_window = 0;
-  if (kernel == CAT_KERNEL_AUTO && storage == h->storage) {
+  if (cached && kernel == CAT_KERNEL_AUTO && storage == h->storage) {
     cat::InstanceInfo f{};
     cat::host_instance_info(h, &f);
     int32_t k = 0, d = 0, t = 0, w = 0, spl = 0;
@@ -868,6 +870,10 @@ int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t stora
     cat_set_tile(h, tuned_tile, tuned_tile, tuned_window);   // a stale entry keeps the radius's own tile
   }
   return CAT_OK;
+}
+
+int cat_set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t storage, int32_t steps_per_launch) {
+  return set_options(h, kernel, dtype, storage, steps_per_launch, true);
 }
 
 int cat_get_options(cat_handle_t h, int32_t *kernel, int32_t *dtype, int32_t *storage, int32_t *steps_per_launch,
@@ -1170,3 +1176,10 @@ int cat_destroy(cat_handle_t h) {
 }
 
 }  // extern "C"
+
+namespace cat {
+int host_leave_options(cat_handle_t h) {
+  const int rc = cat_set_tile(h, 0, 0, 0);
+  return rc ? rc : set_options(h, CAT_KERNEL_AUTO, CAT_DTYPE_AUTO, h->storage, 1, false);
+}
+}  // namespace cat

@@ -119,6 +119,8 @@ struct InstanceInfo {
   bool left;   // options left to the library
 };
 int host_instance_info(cat_handle_t h, InstanceInfo *out);
+// Leaves every option to the library, whatever CAT_AUTOTUNE_CACHE holds.
+int host_leave_options(cat_handle_t h);
 // The autotuner's cached choice for an instance from the JSON-lines file named
 // by the environment variable CAT_AUTOTUNE_CACHE (cat_tune.cu); false when
 // the variable is unset or the file holds no entry for the instance.

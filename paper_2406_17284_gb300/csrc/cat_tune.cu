@@ -82,8 +82,8 @@ void cache_write(const char *path, const std::string &key, const Cand &c, double
 // Sets every option of `h` to candidate c; false (options left unspecified)
 // when the instance cannot run it.
 bool apply(cat_handle_t h, const InstanceInfo &f, const Cand &c) {
+  if (c.left) return host_leave_options(h) == CAT_OK;
   if (cat_set_tile(h, 0, 0, 0) != CAT_OK) return false;
-  if (c.left) return cat_set_options(h, CAT_KERNEL_AUTO, CAT_DTYPE_AUTO, f.storage, 1) == CAT_OK;
   if (cat_set_options(h, c.kernel, c.dtype, f.storage, c.spl) != CAT_OK) return false;
   return cat_set_tile(h, c.tile, c.tile, c.window) == CAT_OK;
 }
@@ -160,7 +160,8 @@ extern "C" CAT_API int cat_autotune(cat_handle_t h, int32_t n_steps, const char 
   for (const Cand &c : cat::candidates(f)) {
     if (!cat::apply(h, f, c)) continue;
     const int64_t steps = (n_steps + c.spl - 1) / c.spl * c.spl;
-    if (cat_set_state(h, saved, f.W, 1, stream) || cat_step(h, c.spl, stream) || cudaEventRecord(a, s) ||
+    // (untimed first: the launches of the timed call; the library may take others for one step)
+    if (cat_set_state(h, saved, f.W, 1, stream) || cat_step(h, c.left ? steps : c.spl, stream) || cudaEventRecord(a, s) ||
         cat_step(h, steps, stream) || cudaEventRecord(b, s) || cudaEventSynchronize(b))
       continue;
     float ms = 0;

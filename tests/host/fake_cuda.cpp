@@ -5,8 +5,8 @@
 // fake_log     the launches so far, one per line, and forgets them
 // fake_fail    launches named so fail from now on (NULL: none)
 // fake_capturing  what cudaStreamIsCapturing returns as its error
-// Device memory is host memory; a tensor-core launch takes ten times as long as
-// any other (cudaEventElapsedTime).
+// Device memory is host memory; a step on tensor cores takes ten times as long
+// as a launch on bit planes (cudaEventElapsedTime).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -111,7 +111,9 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return launched("gr
 }
 
 namespace cat {
-cudaError_t tc_launch(const TcParams &, int, bool, bool, bool, int, cudaStream_t) { return launched("tensor cores", 10); }
+cudaError_t tc_launch(const TcParams &p, int, bool, bool, bool, int, cudaStream_t) {
+  return launched("tensor cores", 10.0f * (float)p.n_steps);
+}
 cudaError_t vn_launch(const TcParams &, int, cudaStream_t) { return launched("tensor cores", 10); }
 cudaError_t wide_launch(const TcParams &, int, cudaStream_t) { return launched("tensor cores", 10); }
 cudaError_t big_launch(const TcParams &, int, cudaStream_t) { return launched("tensor cores", 10); }

@@ -3,6 +3,7 @@ cat_tune.cu) linked with a CUDA runtime and launchers that keep a record
 (tests/host/fake_cuda.cpp), under which bit planes are preferred wherever the
 host code asks about them."""
 import ctypes
+import json
 import os
 import subprocess
 
@@ -33,6 +34,11 @@ class Host:
         rule = cat.make_rule(**inputs.scaled_rule(r, C=C))
         self.cat_create_ex(H, W, ctypes.byref(rule), boundary, storage, ctypes.byref(h))
         return h
+
+    def options(self, h):
+        v = [ctypes.c_int32() for _ in range(6)]
+        self.cat_get_options(h, *[ctypes.byref(x) for x in v])
+        return dict(zip(("kernel", "dtype", "storage", "steps_per_launch", "tile", "window"), (x.value for x in v)))
 
     def log(self):
         out = ctypes.create_string_buffer(1 << 16)
@@ -99,4 +105,30 @@ def test_steps_of_a_callers_buffers_end_from_bytes_to_bytes(host, bound):
                                                                         ["planes bit1 to bit1"]), last]
     host.cat_batch_step((ctypes.c_void_p * 1)(h), 1, 8, None)
     assert ("batch tiles" in host.log()) == bound
+    host.cat_destroy(h)
+
+
+def cache_line(H, W, r, **choice):
+    key = f"H={H} W={W} r={r} C=2 nbhd=M boundary=0 storage=0 gpu=fake/152"
+    return json.dumps({"key": key, **choice, "cell_updates_per_s": 1.0}) + "\n"
+
+
+FP16_TILES = dict(kernel=cat.KERNEL_TCGEN05, dtype=cat.DTYPE_FP16, tile=128, window=160, steps_per_launch=1)
+
+
+def test_the_autotuner_times_what_the_library_would_choose(host, tmp_path, monkeypatch):
+    """Tuning again while CAT_AUTOTUNE_CACHE names an older, explicit choice:
+    the candidate that leaves the options to the library is timed as that."""
+    old, new = tmp_path / "old.jsonl", tmp_path / "new.jsonl"
+    old.write_text(cache_line(64, 96, 4, **FP16_TILES))
+    h = host.grid(64, 96, 4)
+    monkeypatch.setenv("CAT_AUTOTUNE_CACHE", str(old))
+    host.cat_autotune(h, 8, str(new).encode(), cat.CAT_TUNE_REMEASURE, None)
+    line = json.loads(new.read_text())
+    assert line["left"] == 1 and line["dtype"] == cat.DTYPE_FP8_E4M3
+    assert line["cell_updates_per_s"] == pytest.approx(64 * 96 * 8 / 8e-3)   # eight launches of a millisecond
+    assert host.options(h)["dtype"] == cat.DTYPE_FP8_E4M3
+    host.log()
+    host.cat_step(h, 1, None)
+    assert host.log() == ["planes u8 to u8"]
     host.cat_destroy(h)
