@@ -770,8 +770,14 @@ static int set_options(cat_handle_t h, int32_t kernel, int32_t dtype, int32_t st
     cat::InstanceInfo f{};
     cat::host_instance_info(h, &f);
     int32_t k = 0, d = 0, t = 0, w = 0, spl = 0;
-    if (cat::tune_cache_lookup_env(f, &k, &d, &t, &w, &spl) && k >= CAT_KERNEL_TCGEN05 && k <= CAT_KERNEL_RUNSUM &&
-        d >= CAT_DTYPE_AUTO && d <= CAT_DTYPE_FP4_E2M1 && spl >= 1) {
+    bool left = false;
+    if (cat::tune_cache_lookup_env(f, &k, &d, &t, &w, &spl, &left) && left) {   // the library's own choice was the fastest
+      auto_choice = true;
+      dtype = CAT_DTYPE_AUTO;
+      steps_per_launch = 1;
+      tuned_tile = 0;
+    } else if (k >= CAT_KERNEL_TCGEN05 && k <= CAT_KERNEL_RUNSUM &&
+               d >= CAT_DTYPE_AUTO && d <= CAT_DTYPE_FP4_E2M1 && spl >= 1) {
       auto_choice = false;
       kernel = k;
       dtype = d;

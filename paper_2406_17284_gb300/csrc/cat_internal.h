@@ -123,9 +123,10 @@ int host_instance_info(cat_handle_t h, InstanceInfo *out);
 int host_leave_options(cat_handle_t h);
 // The autotuner's cached choice for an instance from the JSON-lines file named
 // by the environment variable CAT_AUTOTUNE_CACHE (cat_tune.cu); false when
-// the variable is unset or the file holds no entry for the instance.
+// the variable is unset or the file holds no entry for the instance.  *left:
+// every option left to the library was the fastest.
 bool tune_cache_lookup_env(const InstanceInfo &info, int32_t *kernel, int32_t *dtype, int32_t *tile,
-                           int32_t *window, int32_t *spl);
+                           int32_t *window, int32_t *spl, bool *left);
 
 // Host helpers defined in cat_api.cu (error message of the calling thread,
 // rule checks, TMA descriptor encoding of a uint8 grid).

@@ -117,10 +117,11 @@ int cuda_err(cudaError_t e, const char *what) {
 }  // namespace
 
 bool tune_cache_lookup_env(const InstanceInfo &info, int32_t *kernel, int32_t *dtype, int32_t *tile, int32_t *window,
-                           int32_t *spl) {
+                           int32_t *spl, bool *left) {
   const char *path = getenv("CAT_AUTOTUNE_CACHE");
   Cand c{};
-  if (!path || !*path || !cache_read(path, cache_key(info), &c, nullptr) || c.left) return false;
+  if (!path || !*path || !cache_read(path, cache_key(info), &c, nullptr)) return false;
+  *left = c.left;
   *kernel = c.kernel;
   *dtype = c.dtype;
   *tile = c.tile;

@@ -132,3 +132,22 @@ def test_the_autotuner_times_what_the_library_would_choose(host, tmp_path, monke
     host.cat_step(h, 1, None)
     assert host.log() == ["planes u8 to u8"]
     host.cat_destroy(h)
+
+
+@pytest.mark.parametrize("left", [False, True])
+def test_auto_takes_the_cached_choice(host, tmp_path, monkeypatch, left):
+    """CAT_KERNEL_AUTO takes the choice that CAT_AUTOTUNE_CACHE names in place of
+    the other arguments, also when that is to leave every option to the library."""
+    cache = tmp_path / "tune.jsonl"
+    default = dict(FP16_TILES, dtype=cat.DTYPE_FP8_E4M3, window=144)
+    cache.write_text(cache_line(64, 96, 4, **FP16_TILES))
+    if left:
+        cache.write_text(cache.read_text() + cache_line(64, 96, 4, **default).replace("}", ', "left": 1}'))
+    h = host.grid(64, 96, 4)
+    host.cat_set_tile(h, 128, 128, 160)
+    monkeypatch.setenv("CAT_AUTOTUNE_CACHE", str(cache))
+    host.cat_set_options(h, cat.KERNEL_AUTO, cat.DTYPE_FP16, cat.STORE_U8, 4)
+    assert host.options(h) == dict(default if left else FP16_TILES, storage=cat.STORE_U8)
+    host.cat_step(h, 1, None)
+    assert host.log() == ["planes u8 to u8" if left else "tensor cores"]
+    host.cat_destroy(h)
