@@ -335,8 +335,9 @@ CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
  * buffer that does not hold the state afterwards has no defined contents,
  * unless it is a caller's (cat_bind).  Each step computes the band products of
  * Sec. IV (Eqs. 1-2) and the rule of Sec. V-A for every cell.  Errors:
- * INVALID_ARG (NULL, n_steps < 0), CUDA (launch failure); device-side
- * timeouts are reported by cat_status.                                     */
+ * INVALID_ARG (NULL, n_steps < 0), CUDA (launch failure: the state is then that
+ * after the steps launched; what several steps need is loaded before the
+ * first); device-side timeouts are reported by cat_status.                                     */
 CAT_API int cat_step(cat_handle_t h, int64_t n_steps, void *stream);
 
 /* Advances `count` independent instances by n_steps each.  The instances may

@@ -253,7 +253,9 @@ bool use_packed_steps(const cat_instance *h, int64_t n_steps) {
 // Byte offset of a row's second row of bits.
 int64_t packed_second(const cat_instance *h) { return round_up((h->W + 2 * h->ghost + 31) / 32 * 4, 16); }
 
-int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
+// launch = false: only prepares each launch, so that one that cannot be made is
+// found before the first one writes bits over states.
+int packed_steps(cat_instance *h, int64_t n_steps, bool launch, cudaStream_t s) {
   const int64_t second = packed_second(h);
   // row 0 of a buffer's bits (on a torus they start at the frame's first cell)
   auto bits = [&](int b, int64_t off) { return h->buf[b] + h->ghost * h->pitch + off; };
@@ -278,7 +280,7 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
       k = plan.steps > 0 ? plan.steps : 1;
     }
     cudaError_t e = cudaSuccess;
-    if (h->ghost)
+    if (h->ghost && launch)
       e = t == 0 ? cat::ghost_fill_launch(h->buf[h->cur], h->pitch, h->H, h->W, h->ghost, false, s)
                  : cat::ghost_bits_launch(bits(at, off), h->pitch, h->H, h->W, s);
     if (t + k == n_steps) {
@@ -289,11 +291,21 @@ int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
       at = 1 - last;
       g.out = bits(at, off);
     }
-    if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
+    if (e == cudaSuccess)
+      e = !launch          ? cat::planes_prepare(g, plan)
+          : plan.steps > 0 ? cat::planes_tile_launch(g, plan, s)
+                           : cat::planes_launch(g, s);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     t += k;
   }
   return CAT_OK;
+}
+
+int launch_packed_steps(cat_instance *h, int64_t n_steps, cudaStream_t s) {
+  const cudaError_t e = h->ghost ? cat::ghost_prepare(h->dev.id) : cudaSuccess;
+  if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+  const int rc = packed_steps(h, n_steps, false, s);
+  return rc ? rc : packed_steps(h, n_steps, true, s);
 }
 
 // n_steps steps of instance h from buffer `in` (into buffer 1 - in after an

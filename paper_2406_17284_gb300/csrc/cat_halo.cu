@@ -10,6 +10,7 @@
 // + 2GH cells: 1.05 M cells for a 16384^2 grid, against 268 M in the grid.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "cat_internal.h"
@@ -147,6 +148,18 @@ __global__ void ghost_bits_kernel(uint32_t *base, int64_t pitch_words, int H, in
 }
 
 }  // namespace
+
+cudaError_t ghost_prepare(int device) {
+  static std::atomic<uint32_t> loaded{0};   // by device
+  const uint32_t bit = device >= 0 && device < 32 ? 1u << device : 0u;
+  if (loaded.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, ghost_fill_kernel);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ghost_frame_kernel);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ghost_bits_kernel);
+  if (e == cudaSuccess) loaded.fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
 
 cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W, cudaStream_t s) {
   const int words = (int)((W + 32 + 31) / 32), threads = 256;

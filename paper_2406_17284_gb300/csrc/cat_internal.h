@@ -159,6 +159,8 @@ cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W
 // The same for a one-bit grid whose rows start at cell -16 (G = 16; W >= 64);
 // row0: row 0 of the grid.
 cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W, cudaStream_t s);
+// Loads the kernels of both (see planes_prepare).
+cudaError_t ghost_prepare(int device);
 
 // Paper-style fragment kernels (cat_mma.cu).  dt: FP16 or INT8.
 cudaError_t mma_launch(const SimpleParams &p, int dt, cudaStream_t s);
@@ -199,6 +201,9 @@ TilePlan planes_tile_steps(const PlanesGrid &g, int64_t steps);   // for a launc
 int64_t planes_launches(const PlanesGrid &g, int64_t n_steps);
 TilePlan planes_tile_fixed(const PlanesGrid &g, int steps);
 cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaStream_t s);
+// What a launch of planes_tile_launch (planes_launch where plan.steps = 0) needs
+// before it, so that what can fail does so with nothing queued.
+cudaError_t planes_prepare(const PlanesGrid &g, const TilePlan &plan);
 // Two-state uint8 grids of any sizes, radii (<= 16) and rules, advanced several
 // steps per call on states packed to bits.  `buf` holds the states in buf[cur]; after n steps they are in
 // buf[cur ^ (n & 1)].

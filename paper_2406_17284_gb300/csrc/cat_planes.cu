@@ -188,6 +188,36 @@ bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps) {
   return n_steps >= (m <= 50 || r == 8 || r == 16 ? 3 : 2);
 }
 
+namespace {
+
+// The tile kernel's shared memory and carveout (the latter as the streaming
+// kernels ask for: launches of both follow each other), once per device.
+cudaError_t tile_attributes(const planes::TileKernel &k, const PlanesGrid &g) {
+  static std::atomic<bool> set[16][planes::kMaxR + 1];
+  std::atomic<bool> *slot = g.device >= 0 && g.device < 16 ? &set[g.device][g.rule.r] : nullptr;
+  if (slot && slot->load(std::memory_order_relaxed)) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess && slot) slot->store(true, std::memory_order_relaxed);
+  return e;
+}
+
+}  // namespace
+
+cudaError_t planes_prepare(const PlanesGrid &g, const TilePlan &plan) {
+  if (plan.steps > 0) {
+    const planes::TileKernel k = planes::tile_kernel(g.rule.r);
+    if (!k.fn || plan.steps > max_tile_steps(g.rule.r) || tile_smem(g, plan) > kMaxSmem || g.pitch > (int64_t)UINT32_MAX)
+      return cudaErrorInvalidValue;
+    return tile_attributes(k, g);
+  }
+  int kind;
+  Resident resident;
+  const planes::Kernel k = find(g, &kind);
+  return k.fn ? resident_warps(k, kind, g.rule.r, g, &resident) : cudaErrorInvalidValue;
+}
+
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
   int kind;
   Resident resident;
@@ -259,15 +289,10 @@ cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &plan, cudaSt
   t.out_u8 = g.storage_out == CAT_STORE_U8;
   t.p.rows = plan.rows;
   t.p.strips = (int32_t)((g.H + plan.rows - 1) / plan.rows);
-  const int64_t smem = tile_smem(g, plan);
-  if (!k.fn || plan.steps > max_tile_steps(g.rule.r) || smem > kMaxSmem || g.pitch > (int64_t)UINT32_MAX)
-    return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-  if (e == cudaSuccess)   // (as the streaming kernels ask for: launches of both follow each other)
-    e = cudaFuncSetAttribute(k.fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  const cudaError_t e = planes_prepare(g, plan);
   if (e != cudaSuccess) return e;
   const int64_t blocks = ((int64_t)t.p.strips * t.p.seg + planes::kOut - 1) / planes::kOut;
-  return launch(k.fn, t, blocks, 32 * planes::kTileWarps, (int)smem, s);
+  return launch(k.fn, t, blocks, 32 * planes::kTileWarps, (int)tile_smem(g, plan), s);
 }
 
 struct PlanesBatch {

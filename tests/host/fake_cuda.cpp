@@ -143,6 +143,10 @@ TilePlan planes_tile_steps(const PlanesGrid &, int64_t) { return TilePlan{0, 0};
 int64_t planes_launches(const PlanesGrid &, int64_t n_steps) { return n_steps; }
 TilePlan planes_tile_fixed(const PlanesGrid &, int steps) { return TilePlan{steps, 64}; }
 cudaError_t planes_tile_launch(const PlanesGrid &g, const TilePlan &, cudaStream_t) { return launched("tile " + storages(g)); }
+cudaError_t planes_prepare(const PlanesGrid &g, const TilePlan &) {
+  return "planes " + storages(g) == g_fail ? cudaErrorMemoryAllocation : cudaSuccess;
+}
+cudaError_t ghost_prepare(int) { return g_fail == "bit frame" ? cudaErrorMemoryAllocation : cudaSuccess; }
 struct PlanesBatch {};
 cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &, int, PlanesBatch **out) { *out = new PlanesBatch; return cudaSuccess; }
 cudaError_t planes_batch_update(PlanesBatch *, const std::vector<PlanesBatchItem> &) { return cudaSuccess; }

@@ -151,3 +151,23 @@ def test_auto_takes_the_cached_choice(host, tmp_path, monkeypatch, left):
     host.cat_step(h, 1, None)
     assert host.log() == ["planes u8 to u8" if left else "tensor cores"]
     host.cat_destroy(h)
+
+
+@pytest.mark.parametrize("boundary,fails", [(0, "planes u8 to bit1"), (0, "planes bit1 to bit1"), (0, "planes bit1 to u8"),
+                                            (1, "bit frame"), (1, "planes bit1 to u8")])
+def test_steps_that_cannot_all_be_launched_leave_the_state(host, boundary, fails):
+    """Several steps write bits over states, also in the buffer that holds the
+    state: a kernel that cannot be loaded is found before the first launch."""
+    h = host.grid(64, 96, 4, boundary=boundary)
+    at, pitch = ctypes.c_void_p(), ctypes.c_int64()
+    host.cat_state_ptr(h, ctypes.byref(at), ctypes.byref(pitch))
+    host.lib.fake_fail(fails.encode())
+    assert host.rc("cat_step", h, 5, None) == cat.CAT_ERR_CUDA
+    assert host.log() == []
+    now = ctypes.c_void_p()
+    host.cat_state_ptr(h, ctypes.byref(now), ctypes.byref(pitch))
+    assert now.value == at.value
+    host.lib.fake_fail(None)
+    host.cat_step(h, 5, None)
+    assert host.log()[-1] == "planes bit1 to u8"
+    host.cat_destroy(h)
