@@ -1020,9 +1020,7 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   // 302 / 453 / 681; for 12: 448 / 730 / 1149 against 418 / 634 / 954).
   // A captured call keeps to the tiles, one launch per
   // step, since the planes need the radii side by side.
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  CAT_CUDA(cudaStreamIsCapturing(s, &cs));
-  bool packed = n_steps >= 6 && cs == cudaStreamCaptureStatusNone;
+  bool packed = n_steps >= 6;
   int64_t cells = 0;
   bool one_device = true, one_dtype = true, small = true;
   for (int32_t i = 0; i < count; ++i) {
@@ -1070,6 +1068,9 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
       }
     return CAT_OK;
   }
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CAT_CUDA(cudaStreamIsCapturing(s, &cs));
+  packed &= cs == cudaStreamCaptureStatusNone;
   int rc;
   if (!pl) {
     if ((rc = build_plan(hs, count, &pl))) return rc;

@@ -171,3 +171,18 @@ def test_steps_that_cannot_all_be_launched_leave_the_state(host, boundary, fails
     host.cat_step(h, 5, None)
     assert host.log()[-1] == "planes bit1 to u8"
     host.cat_destroy(h)
+
+
+def test_a_batch_asks_for_the_capture_only_where_it_matters(host):
+    """The legacy stream has no capture status while another stream is captured
+    (cudaErrorStreamCaptureImplicit): calls that launch nothing, or nothing that a
+    capture changes, do not ask for it."""
+    u8, bits = host.grid(64, 96, 4), host.grid(64, 96, 4, storage=cat.STORE_BIT1)
+    host.lib.fake_capturing(906)
+    host.cat_batch_step((ctypes.c_void_p * 1)(u8), 1, 0, None)
+    host.cat_batch_step((ctypes.c_void_p * 1)(bits), 1, 2, None)
+    assert host.rc("cat_batch_step", (ctypes.c_void_p * 2)(u8, u8), 2, 2, None) == cat.CAT_ERR_INVALID_ARG
+    assert host.rc("cat_batch_step", (ctypes.c_void_p * 1)(u8), 1, 2, None) == cat.CAT_ERR_CUDA
+    host.lib.fake_capturing(0)
+    host.cat_destroy(u8)
+    host.cat_destroy(bits)
