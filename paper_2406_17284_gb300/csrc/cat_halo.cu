@@ -80,15 +80,19 @@ __global__ void ghost_fill_kernel(uint8_t *base, int64_t pitch, int H, int W, in
 // remainder for each (above) took longer than the step itself where W % 16 is
 // not 0, and whole chunks shifted into place in registers hardly less
 // (4600^2, r = 5, tensor-core steps back to back: 64 and 31 us a step; so
-// 14.8, and 13.1 with no frame to refresh).  Chunks of 16 cells to a thread
-// where W % 16 is 0 are no better (8192^2, r = 5 / 12 / 16: 36.0 / 34.4 / 38.5
-// against 33.1 / 33.5 / 35.4).
+// 14.8, and 13.1 with no frame to refresh).
+// CHUNKS: a thread takes 16 cells of the sides (W % 16 = 0, so both ends are
+// aligned).  Tall grids need it, whose sides are the work: r = 12, a thread per
+// cell / per chunk, 16384 x 64 8.0 / 7.1 us a step, 65536 x 64 17.8 / 12.0,
+// 1048576 x 64 206 / 103, 131072 x 256 34.5 / 22.3; others gain nothing (8192 x
+// 1024 9.9 / 9.9, 16384 x 4096 34.2 / 33.7 and at r = 5 33.2 / 33.8).
 // early: the next kernel may start its set-up beside the previous one's end.
 // The tensor-core step gains by that (256^2: 5.6 against 6.4), the bit-plane
 // steps, whose blocks only wait, lose (2048^2, r = 12, two steps: 10.1 against 9.1).
 __device__ __forceinline__ int frame_at(int f, int n) { return f < 16 ? f : n + f; }
 __device__ __forceinline__ int frame_from(int f, int n) { return f < 16 ? n + f : f; }
 
+template <bool CHUNKS>
 __global__ void ghost_frame_kernel(uint8_t *base, int64_t pitch, int H, int W, unsigned row_blocks, bool early) {
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -102,11 +106,14 @@ __global__ void ghost_frame_kernel(uint8_t *base, int64_t pitch, int H, int W, u
     if (k < chunks) reinterpret_cast<uint4 *>(dst)[k] = reinterpret_cast<const uint4 *>(src)[k];
     else dst[15 * (int64_t)chunks + k] = src[15 * (int64_t)chunks + k];
   } else {                         // the frame's cells beside the grid's rows, and the corners
-    const int64_t i = (int64_t)(blockIdx.x - row_blocks) * blockDim.x + threadIdx.x, q = i >> 5;
+    const int64_t i = (int64_t)(blockIdx.x - row_blocks) * blockDim.x + threadIdx.x, q = CHUNKS ? i >> 1 : i >> 5;
     if (q >= H + 32) return;
-    const int f = (int)(i & 31);
+    const int f = CHUNKS ? 16 * (int)(i & 1) : (int)(i & 31);
     const int64_t to = q < H ? q + 16 : frame_at((int)(q - H), H), from = q < H ? q + 16 : frame_from((int)(q - H), H);
-    base[to * pitch + frame_at(f, W)] = base[from * pitch + frame_from(f, W)];
+    uint8_t *const dst = base + to * pitch + frame_at(f, W);
+    const uint8_t *const src = base + from * pitch + frame_from(f, W);
+    if (CHUNKS) *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+    else *dst = *src;
   }
 }
 
@@ -155,7 +162,8 @@ cudaError_t ghost_prepare(int device) {
   if (loaded.load(std::memory_order_relaxed) & bit) return cudaSuccess;
   cudaFuncAttributes a;
   cudaError_t e = cudaFuncGetAttributes(&a, ghost_fill_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ghost_frame_kernel);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ghost_frame_kernel<false>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ghost_frame_kernel<true>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ghost_bits_kernel);
   if (e == cudaSuccess) loaded.fetch_or(bit, std::memory_order_relaxed);
   return e;
@@ -182,9 +190,9 @@ cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W
 // dependent on it.
 cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, bool early, cudaStream_t s) {
   const int threads = 256;
-  const bool small = H < 16 || W < 16 || G != 16;
+  const bool small = H < 16 || W < 16 || G != 16, chunks = W % 16 == 0 && H >= 16384 && H >= 8 * W;
   const int64_t rows = (32 * (W / 16 + W % 16) + threads - 1) / threads;
-  const int64_t sides = ((H + 32) * 32 + threads - 1) / threads;
+  const int64_t sides = ((H + 32) * (chunks ? 2 : 32) + threads - 1) / threads;
   const int64_t n = 2 * (int64_t)G * ((W + 15) / 16) + 2 * H + 4 * (int64_t)G * G;
   const int64_t want = (n + threads - 1) / threads;
   cudaLaunchConfig_t cfg = {};
@@ -197,7 +205,7 @@ cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (small) return cudaLaunchKernelEx(&cfg, ghost_fill_kernel, base, pitch, (int)H, (int)W, G);
-  return cudaLaunchKernelEx(&cfg, ghost_frame_kernel, base, pitch, (int)H, (int)W,
+  return cudaLaunchKernelEx(&cfg, chunks ? ghost_frame_kernel<true> : ghost_frame_kernel<false>, base, pitch, (int)H, (int)W,
                             (unsigned)rows, early);
 }
 

@@ -37,3 +37,19 @@ def test_frame_of_every_width(cat, kernel, dtype, r, H):
             assert np.array_equal(g.get_state(), oracle.step(grid, oracle.Rule(**rule), boundary=1, n_steps=2)), W
         finally:
             g.close()
+
+
+@pytest.mark.parametrize("kernel,dtype,r,n", [("tcgen05", "fp8", 16, 2), ("auto", "auto", 4, 1), ("auto", "auto", 4, 3)])
+@pytest.mark.parametrize("H", [16383, 16384])
+def test_frame_of_tall_grids(cat, kernel, dtype, r, n, H):
+    """Sides in chunks of 16 cells from 16384 rows on, where W is a multiple of 16."""
+    rule = inputs.scaled_rule(r, M=1)
+    for W in (16, 48, 64, 65):
+        grid = inputs.bernoulli(H, W, 0.5, H + W)
+        g = cat.Grid(H, W, rule, kernel=kernel, dtype=dtype, boundary=1)
+        try:
+            g.set_state(grid)
+            g.step(n)
+            assert np.array_equal(g.get_state(), oracle.step(grid, oracle.Rule(**rule), boundary=1, n_steps=n)), W
+        finally:
+            g.close()
