@@ -72,7 +72,7 @@ __global__ void ghost_fill_kernel(uint8_t *base, int64_t pitch, int H, int W, in
   }
 }
 
-// The same for H, W >= 16, which is nearly every grid, in as few instructions
+// The same for H, W >= 16 and below 2^19 rows, which is nearly every grid, in as few instructions
 // as that takes, a thread per cell: frame position f of 32 (0 .. 15 before the
 // grid, 16 .. 31 after it) is framed coordinate f or N + f and wraps to N + f
 // or f.  The step kernel leaves none of these instructions in an SM's cache,
@@ -85,7 +85,10 @@ __global__ void ghost_fill_kernel(uint8_t *base, int64_t pitch, int H, int W, in
 // aligned).  Tall grids need it, whose sides are the work: r = 12, a thread per
 // cell / per chunk, 16384 x 64 8.0 / 7.1 us a step, 65536 x 64 17.8 / 12.0,
 // 1048576 x 64 206 / 103, 131072 x 256 34.5 / 22.3; others gain nothing (8192 x
-// 1024 9.9 / 9.9, 16384 x 4096 34.2 / 33.7 and at r = 5 33.2 / 33.8).
+// 1024 9.9 / 9.9, 16384 x 4096 34.2 / 33.7 and at r = 5 33.2 / 33.8).  From 2^19
+// rows on the loop above is as fast or, where the grid is about as large as the
+// L2, faster (r = 4, loop / chunks: 524288 x 128 53.7 / 53.1, 700000 x 128 73.9 /
+// 79.6, 819200 x 128 87 / 97, 1638400 x 128 191.8 / 190.3).
 // early: the next kernel may start its set-up beside the previous one's end.
 // The tensor-core step gains by that (256^2: 5.6 against 6.4), the bit-plane
 // steps, whose blocks only wait, lose (2048^2, r = 12, two steps: 10.1 against 9.1).
@@ -190,13 +193,14 @@ cudaError_t ghost_bits_launch(uint8_t *row0, int64_t pitch, int64_t H, int64_t W
 // dependent on it.
 cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W, int G, bool early, cudaStream_t s) {
   const int threads = 256;
-  const bool small = H < 16 || W < 16 || G != 16, chunks = W % 16 == 0 && H >= 16384 && H >= 8 * W;
+  const bool chunks = W % 16 == 0 && H >= 16384 && H >= 8 * W;
+  const bool loop = H < 16 || W < 16 || G != 16 || (chunks && H >= 1 << 19);
   const int64_t rows = (32 * (W / 16 + W % 16) + threads - 1) / threads;
   const int64_t sides = ((H + 32) * (chunks ? 2 : 32) + threads - 1) / threads;
   const int64_t n = 2 * (int64_t)G * ((W + 15) / 16) + 2 * H + 4 * (int64_t)G * G;
   const int64_t want = (n + threads - 1) / threads;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(!small ? rows + sides : want < 4096 ? want : 4096));
+  cfg.gridDim = dim3((unsigned)(!loop ? rows + sides : want < 4096 ? want : 4096));
   cfg.blockDim = dim3(threads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -204,7 +208,7 @@ cudaError_t ghost_fill_launch(uint8_t *base, int64_t pitch, int64_t H, int64_t W
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (small) return cudaLaunchKernelEx(&cfg, ghost_fill_kernel, base, pitch, (int)H, (int)W, G);
+  if (loop) return cudaLaunchKernelEx(&cfg, ghost_fill_kernel, base, pitch, (int)H, (int)W, G);
   return cudaLaunchKernelEx(&cfg, chunks ? ghost_frame_kernel<true> : ghost_frame_kernel<false>, base, pitch, (int)H, (int)W,
                             (unsigned)rows, early);
 }

@@ -122,6 +122,21 @@ int32_t one_wave_rows(const PlanesGrid &g) {
   return strips < 1 ? 0 : (int32_t)std::min<int64_t>(((g.H + strips - 1) / strips + 7) / 8 * 8, 1 << 20);
 }
 
+int64_t words_of(const PlanesGrid &g) { return (g.W + 2 * g.frame + 31) / 32 + 1; }   // of a row, the zero word too
+
+// A grid in units of 2^20 cells, as a warp of 30 words counts them: a narrow
+// grid's zero word and half empty last word take their share (a grid of 1024
+// columns or more is its own cells).
+int64_t mega_cells(const PlanesGrid &g) {
+  return (g.H * std::max(g.W, 30 * words_of(g)) + (1 << 20) - 1) >> 20;
+}
+
+// The words pad a row by 7% more than the tiles' columns do, or it fills three
+// words and most of one tile.
+bool padded(const PlanesGrid &g) {
+  return 100 * 32 * words_of(g) > 107 * ((g.W + 127) / 128 * 128) || (g.W > 80 && g.W <= 96);
+}
+
 int64_t tile_smem(const PlanesGrid &g, const TilePlan &t) {
   const planes::TileKernel k = planes::tile_kernel(g.rule.r);
   return (int64_t)k.row_bytes * (t.rows + 2 * t.steps * g.rule.r) + k.block_bytes;
@@ -152,10 +167,16 @@ bool planes_preferred(const PlanesGrid &g) {
   int kind;
   if (!find(g, &kind).fn) return false;
   if (g.storage_in != CAT_STORE_U8) return true;
-  const int64_t m = (g.H * g.W + (1 << 20) - 1) >> 20;   // 2^20 cells
-  if (g.rule.C > 2) return g.rule.r <= (m <= 1 ? (g.frame ? 9 : 12) : m < 16 ? 5 : m < 64 ? 7 : m < 128 ? 9 : 12);
-  if (g.frame) return g.rule.r <= (m <= 1 ? 7 : m <= 16 ? 4 : 0);
-  return g.rule.r <= (m <= 1 ? 16 : m <= 4 ? 9 : m <= 16 ? 4 : 0);
+  const int64_t m = mega_cells(g);
+  const bool narrow = padded(g), odd = g.W % 16 != 0;
+  const int r = g.rule.r;
+  if (g.rule.C > 2) {
+    if (narrow && m >= 16)
+      return r <= (g.frame ? (m < 64 ? (g.W <= 128 ? 3 : 5) : g.W <= 256 ? 0 : 5) : m < 64 ? 5 : g.W <= 128 && odd ? 0 : 7);
+    return r <= (m <= 1 ? (g.frame ? 9 : 12) : m < 16 ? 5 : m < 64 ? 7 : m < 128 ? 9 : 12);
+  }
+  if (g.frame) return r <= (m <= 1 ? 7 : m <= 16 ? (narrow ? 2 : 4) : 0);
+  return r <= (m <= 1 ? 16 : m <= 4 ? 9 : m <= 16 ? (narrow && odd ? 2 : 4) : 0);
 }
 
 // Several steps of a two-state uint8 grid (us per step, tensor-core steps
@@ -178,8 +199,17 @@ bool planes_preferred(const PlanesGrid &g) {
 //                           / 14.6 and 12.1; 5792^2, r = 12: 18.0 and 18.7;
 //                           7000^2, r = 11 / 15: 23.6 / 22.7 and 23.4
 bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps) {
-  const int64_t m = (g.H * g.W + (1 << 20) - 1) >> 20;
+  const int64_t m = mega_cells(g);
+  const bool odd = g.W % 16 != 0;
   const int r = g.rule.r;
+  if (padded(g) && g.frame) {
+    if (m > 4 && m <= 36 && r > 4) return false;
+    if (m > 12 && g.W <= 128) return false;
+    if (m > 36) return r <= 7 || n_steps >= 8;
+  } else if (padded(g) && m > 24) {
+    if (g.W <= 96) return n_steps >= (m > 64 && odd ? 8 : 4);
+    return n_steps >= 8 && (g.W > 128 || (r <= 4 && m <= 64));
+  }
   if (g.frame) return r <= 7 || (m >= 30 && n_steps >= (m < 64 ? 8 : r == 8 || r >= 14 ? 3 : 2));
   if (r <= 7) return m <= 4 || m > 24 || n_steps >= (r == 7 ? 4 : r >= 5 ? 3 : 2);
   if (m <= (r <= 10 ? 10 : 6)) return true;

@@ -40,9 +40,10 @@ def test_frame_of_every_width(cat, kernel, dtype, r, H):
 
 
 @pytest.mark.parametrize("kernel,dtype,r,n", [("tcgen05", "fp8", 16, 2), ("auto", "auto", 4, 1), ("auto", "auto", 4, 3)])
-@pytest.mark.parametrize("H", [16383, 16384])
+@pytest.mark.parametrize("H", [16383, 16384, 1 << 19])
 def test_frame_of_tall_grids(cat, kernel, dtype, r, n, H):
-    """Sides in chunks of 16 cells from 16384 rows on, where W is a multiple of 16."""
+    """Sides in chunks of 16 cells from 16384 rows on, where W is a multiple of 16,
+    and by the looping kernel from 2^19."""
     rule = inputs.scaled_rule(r, M=1)
     for W in (16, 48, 64, 65):
         grid = inputs.bernoulli(H, W, 0.5, H + W)
