@@ -163,6 +163,12 @@ int64_t tile_smem(const PlanesGrid &g, const TilePlan &t) {
 //                         The frame that a torus refreshes first costs a short
 //                         step more: 1024^2, r = 7 / 9: 5.5 / 5.8 against 5.7;
 //                         2048^2, r = 4 / 6: 6.4 / 7.5 against 7.1
+// Narrow grids: where the words pad a row more than the tiles do, the tiles keep
+// what they do faster (C = 16: 1048576 x 100, r = 4 / 9: 101 / 113 against 81 / 83;
+// 932067 x 225, r = 9: 170 against 145; torus 1638400 x 128, r = 2 / 5: 258 / 268
+// against 202; two states 37282 x 225, r = 4: 10.7 against 8.9).  Up to 64 columns it is the other way round, three words
+// against a tile of which half is outside the grid (C = 16: 1092266 x 48, r = 10 /
+// 16: 63 / 75 against 109; 32768 x 48, r = 16: 12.6 against 9.6).
 bool planes_preferred(const PlanesGrid &g) {
   int kind;
   if (!find(g, &kind).fn) return false;
@@ -171,6 +177,7 @@ bool planes_preferred(const PlanesGrid &g) {
   const bool narrow = padded(g), odd = g.W % 16 != 0;
   const int r = g.rule.r;
   if (g.rule.C > 2) {
+    if (!g.frame && g.W <= 64 && m >= 24) return true;
     if (narrow && m >= 16)
       return r <= (g.frame ? (m < 64 ? (g.W <= 128 ? 3 : 5) : g.W <= 256 ? 0 : 5) : m < 64 ? 5 : g.W <= 128 && odd ? 0 : 7);
     return r <= (m <= 1 ? (g.frame ? 9 : 12) : m < 16 ? 5 : m < 64 ? 7 : m < 128 ? 9 : 12);
@@ -195,6 +202,11 @@ bool planes_preferred(const PlanesGrid &g) {
 //   8192^2, n = 2 / 3 / 8   r = 4: 20.1 / 18.8 / 17.3 and 27.2; r = 8: 29.2 / 27.0
 //                           / 24.0 and 28.2; r = 16: 33.5 / 31.3 / 28.3 and 32.1
 //   16384^2, n = 2 / 8      r = 12: 92.6 / 75.5 and 98.5
+//   narrow, n = 2 / 3 / 8   1048576 x 100, r = 4: 75.8 / 71.2 / 53.0 and 60.0;
+//                           1638400 x 128, r = 7: 105 / 106 / 95 and 73; 873813 x
+//                           96, r = 3: 48.0 / 47.5 / .. and 41.8 (n = 5: 40.7); 362539
+//                           x 376, r = 16: .. / 69.2 / .. and 59.9; torus 65536 x
+//                           96, r = 7: .. / 15.3 / 16.1 and 12.3
 //   torus, n = 8            2048^2, r = 12: 9.0 and 7.1; 4096^2, r = 7 / 12: 10.9
 //                           / 14.6 and 12.1; 5792^2, r = 12: 18.0 and 18.7;
 //                           7000^2, r = 11 / 15: 23.6 / 22.7 and 23.4

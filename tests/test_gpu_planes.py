@@ -224,3 +224,24 @@ def test_captured_steps_with_the_options_left(cat, storage, H, W, r, n):
         assert np.array_equal(g.get_state(), oracle.step(want, oracle.Rule(**rule), n_steps=3))
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("H,W", [(450000, 33), (840000, 16), (450000, 64), (450000, 65), (300000, 90), (300000, 120)])
+@pytest.mark.parametrize("r", [3, 13, 16])
+def test_tall_grids(cat, H, W, r):
+    """Narrow and tall: where the choice between bit planes and tensor cores
+    depends on the words of a row, both give the same states."""
+    import torch
+    for C, boundary, n in ((16, 0, 2), (2, 0, 1), (2, 0, 8), (2, 1, 3)):
+        rule = inputs.scaled_rule(r, M=1, C=C)
+        host = board(H, W, C, W + r)
+        a = cat.Grid(H, W, rule, kernel="auto", dtype="auto", boundary=boundary)
+        b = cat.Grid(H, W, rule, kernel="tcgen05", dtype="fp8", boundary=boundary)
+        try:
+            for g in (a, b):
+                g.set_state(host)
+                g.step(n)
+            assert torch.equal(a.state_tensor(), b.state_tensor()), (C, boundary, n)
+        finally:
+            a.close()
+            b.close()
