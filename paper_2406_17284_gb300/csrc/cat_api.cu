@@ -224,6 +224,10 @@ bool use_planes(const cat_instance *h) {
   return h->auto_choice && h->inject == 0 && planes_pitch(h) && cat::planes_preferred(planes_grid(h, 0));
 }
 
+cudaError_t planes_step(const cat::PlanesGrid &g, cudaStream_t s) {
+  return cat::planes_few_rows(g) ? cat::swar_step_launch(g, s) : cat::planes_launch(g, s);
+}
+
 // n_steps steps from buffer `in` into the other one, in one launch (more than
 // one step where planes_launches said so).
 int launch_planes(cat_instance *h, int in, int64_t n_steps, cudaStream_t s) {
@@ -231,7 +235,7 @@ int launch_planes(cat_instance *h, int in, int64_t n_steps, cudaStream_t s) {
   const cat::PlanesGrid g = planes_grid(h, in);
   const cat::TilePlan plan = cat::planes_tile_steps(g, n_steps);
   if (h->ghost) e = cat::ghost_fill_launch(h->buf[in], h->pitch, h->H, h->W, h->ghost, false, s);
-  if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : cat::planes_launch(g, s);
+  if (e == cudaSuccess) e = plan.steps > 0 ? cat::planes_tile_launch(g, plan, s) : planes_step(g, s);
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return CAT_OK;
 }
@@ -382,7 +386,7 @@ int launch_step(cat_instance *h, int in, int32_t *sums, int64_t sums_ld, cudaStr
     else if (h->kernel == CAT_KERNEL_BITSLICE && n_steps > 1)   // temporal blocking: n_steps in one launch
       e = cat::planes_tile_launch(planes_grid(h, in), cat::planes_tile_fixed(planes_grid(h, in), n_steps), s);
     else if (h->kernel == CAT_KERNEL_BITSLICE)
-      e = cat::planes_launch(planes_grid(h, in), s);
+      e = planes_step(planes_grid(h, in), s);
     else if (h->kernel == CAT_KERNEL_RUNSUM)
       e = cat::runsum_launch(p, s);
     else

@@ -172,6 +172,9 @@ cudaError_t runsum_launch(const SimpleParams &p, cudaStream_t s);
 // holds packed rows at `pitch` bytes (a multiple of 4).
 cudaError_t swar_sums_launch(const uint8_t *in, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule, int32_t *sums,
                              int64_t sums_ld, cudaStream_t s);
+struct PlanesGrid;
+// One step of a one-bit grid in the same way, r <= 5: where planes_few_rows.
+cudaError_t swar_step_launch(const PlanesGrid &g, cudaStream_t s);
 // Box sums in bit planes on CUDA cores (cat_planes.cuh): one step of a grid.
 struct PlanesGrid {
   const uint8_t *in;   // row 0 of the input and output: grid cell 0 for uint8, cell -frame for packed rows
@@ -188,6 +191,8 @@ bool planes_preferred(const PlanesGrid &g);
 // states between them kept as bits.
 bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps);
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s);
+// A one-bit grid of so few and so wide rows that swar_step_launch is faster.
+bool planes_few_rows(const PlanesGrid &g);
 // Several steps per launch on tiles in shared memory (cat_planes_tile.cuh; two
 // states): the split for a launch with n_left steps to go; steps = 0 where
 // planes_launch, step by step, is faster.

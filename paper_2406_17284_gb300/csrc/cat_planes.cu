@@ -10,6 +10,26 @@
 #include "cat_planes_tile.cuh"
 
 namespace cat {
+namespace planes {
+
+// A bound K of the rule as the words of a carry chain (at_least), K clamped to
+// [0, 2^planes): no count reaches 2^planes - 1 (an odd square is 1 mod 8), so
+// K = 2^planes - 1 means never.
+static void set_bound(uint32_t *k, int64_t K, int planes) {
+  const int64_t top = (int64_t(1) << planes) - 1;
+  const uint32_t c = ~(uint32_t)(K < 0 ? 0 : K > top ? top : K);
+  for (int i = 0; i < planes; ++i) k[i] = 0u - ((c >> i) & 1u);
+}
+
+void set_bounds(uint32_t (*bound)[kMaxS], const RuleDev &rule, int planes) {
+  set_bound(bound[kSurviveLo], rule.s_lo, planes);
+  set_bound(bound[kSurviveHi], (int64_t)rule.s_lo + rule.s_w + 1, planes);
+  set_bound(bound[kBirthLo], rule.b_lo, planes);
+  set_bound(bound[kBirthHi], (int64_t)rule.b_lo + rule.b_w + 1, planes);
+}
+
+}  // namespace planes
+
 namespace {
 
 constexpr int kMaxSmem = 232448;   // of one block
@@ -65,15 +85,6 @@ cudaError_t resident_warps(const planes::Kernel &k, int kind, int r, const Plane
   return cudaSuccess;
 }
 
-// A bound K of the rule as the words of a carry chain (planes::at_least), K
-// clamped to [0, 2^planes): no count reaches 2^planes - 1 (an odd square is 1
-// mod 8), so K = 2^planes - 1 means never.
-void set_bound(uint32_t *k, int64_t K, int planes) {
-  const int64_t top = (int64_t(1) << planes) - 1;
-  const uint32_t c = ~(uint32_t)(K < 0 ? 0 : K > top ? top : K);
-  for (int i = 0; i < planes; ++i) k[i] = 0u - ((c >> i) & 1u);
-}
-
 planes::Params make_params(const PlanesGrid &g, int planes) {
   planes::Params p;
   p.in = g.in;
@@ -86,10 +97,7 @@ planes::Params make_params(const PlanesGrid &g, int planes) {
   p.rows = p.strips = 0;
   p.last = (uint32_t)(g.rule.C - 1) * 0x11111111u;
   p.two = g.rule.C > 2 ? 0x11111111u : 0u;
-  set_bound(p.bound[planes::kSurviveLo], g.rule.s_lo, planes);
-  set_bound(p.bound[planes::kSurviveHi], (int64_t)g.rule.s_lo + g.rule.s_w + 1, planes);
-  set_bound(p.bound[planes::kBirthLo], g.rule.b_lo, planes);
-  set_bound(p.bound[planes::kBirthHi], (int64_t)g.rule.b_lo + g.rule.b_w + 1, planes);
+  planes::set_bounds(p.bound, g.rule, planes);
   return p;
 }
 
@@ -260,6 +268,16 @@ cudaError_t planes_prepare(const PlanesGrid &g, const TilePlan &plan) {
   return k.fn ? resident_warps(k, kind, g.rule.r, g, &resident) : cudaErrorInvalidValue;
 }
 
+// A one-bit grid of a row or a few, too wide for one wave of warps: a warp here
+// sums 2r rows and steps four (or eight) for those it writes, and a word to a
+// thread with the rows in registers is the faster way (us a step, this / that: 1 x
+// 2^20, r = 2: 3.2 / 2.0; 1 x 100 * 2^20, r = 1 / 2 / 5: 111 / 29, 111 / 46, 190 /
+// 167; 5 x 100 * 2^20, r = 2 / 3: 157 / 136, 166 / 192; 2 x 100 * 2^20, r = 3 / 5: 111 /
+// 108, 191 / 217).
+bool planes_few_rows(const PlanesGrid &g) {
+  return g.storage_in == CAT_STORE_BIT1 && g.W >= 1 << 19 && g.H <= 5 && g.rule.r <= (g.H == 1 ? 5 : g.H == 2 ? 4 : 2);
+}
+
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t s) {
   int kind;
   Resident resident;
@@ -399,11 +417,7 @@ cudaError_t planes_batch_create(const std::vector<PlanesBatchItem> &items, int s
     g.second = q.second;
     g.r = q.rule.r;
     of_radius[g.r].push_back((int32_t)i);
-    const int planes = planes::kernel_bit1(q.rule.r).planes;
-    set_bound(g.bound[planes::kSurviveLo], q.rule.s_lo, planes);
-    set_bound(g.bound[planes::kSurviveHi], (int64_t)q.rule.s_lo + q.rule.s_w + 1, planes);
-    set_bound(g.bound[planes::kBirthLo], q.rule.b_lo, planes);
-    set_bound(g.bound[planes::kBirthHi], (int64_t)q.rule.b_lo + q.rule.b_w + 1, planes);
+    planes::set_bounds(g.bound, q.rule, planes::kernel_bit1(q.rule.r).planes);
   }
   std::vector<planes::BatchBlock> blocks;
   std::vector<size_t> first;

@@ -235,6 +235,8 @@ __device__ __forceinline__ void ring_store(uint8_t *s, int tid, const uint32_t (
 constexpr int kMaxS = bits_for((2 * kMaxR + 1) * (2 * kMaxR + 1));
 enum { kSurviveLo, kSurviveHi, kBirthLo, kBirthHi };   // in range: >= lo and not >= hi
 
+void set_bounds(uint32_t (*bound)[kMaxS], const RuleDev &rule, int planes);
+
 struct Params {
   const uint8_t *in;   // row 0: cell 0 of the grid for uint8, cell -frame for packed rows
   uint8_t *out;

@@ -1,6 +1,6 @@
 // Box counts of a one-bit grid by bit-sliced (SWAR) adders, radii 1..5: the
-// verification path of the bit-sliced kernel choice (its steps run on
-// cat_planes.cuh).
+// verification path of the bit-sliced kernel choice, and its step on grids of a
+// few very wide rows (the other steps run on cat_planes.cuh).
 //
 // Every 32-bit word of a packed row holds 32 cells, and the counts of all 32
 // are computed at once as bit planes (bit b of every cell's count in one
@@ -20,7 +20,7 @@
 
 #include <cstdint>
 
-#include "cat_internal.h"
+#include "cat_planes.cuh"
 
 namespace cat {
 namespace {
@@ -56,11 +56,13 @@ struct SwarParams {
   const uint32_t *in;
   int64_t pitch_words;   // 32-bit words between rows
   int32_t H, W, words;   // rows, cells per row, words holding them
-  int32_t *sums;
+  int32_t *sums;         // counts, or next states
   int64_t sums_ld;
+  uint32_t *out;
+  uint32_t bound[4][planes::kMaxS];
 };
 
-template <int R>
+template <int R, bool STEP>
 __global__ void __launch_bounds__(kBlock) ltl_swar_kernel(const SwarParams p) {
   constexpr int NH = Bits<R>::kH, NS = Bits<R>::kS, WIN = 2 * R + 1;
   const int lane = threadIdx.x & 31;
@@ -75,6 +77,10 @@ __global__ void __launch_bounds__(kBlock) ltl_swar_kernel(const SwarParams p) {
   const bool nc_ok = nc >= 0 && nc < p.words;
   const uint32_t nmask = nc == p.words - 1 ? last_mask : ~0u;
   const uint32_t *in_c = p.in + (col ? wi : 0), *in_n = p.in + (nc_ok ? nc : 0);
+  if (STEP) {   // (ordinary loads: the launch may start before the grid that it reads is written)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
 
   // horizontal sums of row y for this thread's 32 cells (every lane takes part)
   auto hsum = [&](int y, uint32_t (&h)[NH]) {
@@ -118,6 +124,13 @@ __global__ void __launch_bounds__(kBlock) ltl_swar_kernel(const SwarParams p) {
 #pragma unroll
       for (int k = 1; k < WIN; ++k) bs_add<NS, NH>(S, hs[k]);
       if (!col) continue;
+      if (STEP) {
+        const uint32_t c = in_c[(int64_t)y * p.pitch_words];
+        const uint32_t keep = planes::at_least<NS>(S, p.bound[planes::kSurviveLo]) & ~planes::at_least<NS>(S, p.bound[planes::kSurviveHi]);
+        const uint32_t born = planes::at_least<NS>(S, p.bound[planes::kBirthLo]) & ~planes::at_least<NS>(S, p.bound[planes::kBirthHi]);
+        p.out[(int64_t)y * p.pitch_words + wi] = ((c & keep) | (~c & born)) & mask;
+        continue;
+      }
       int32_t *row = p.sums + (int64_t)y * p.sums_ld;
       for (int t = 0; t < 32 && 32 * wi + t < p.W; ++t) {
         int v = 0;
@@ -129,31 +142,63 @@ __global__ void __launch_bounds__(kBlock) ltl_swar_kernel(const SwarParams p) {
   }
 }
 
-}  // namespace
+typedef void (*SwarKernel)(SwarParams);
+template <bool STEP>
+SwarKernel swar_kernel(int r) {
+  switch (r) {
+    case 1: return ltl_swar_kernel<1, STEP>;
+    case 2: return ltl_swar_kernel<2, STEP>;
+    case 3: return ltl_swar_kernel<3, STEP>;
+    case 4: return ltl_swar_kernel<4, STEP>;
+    case 5: return ltl_swar_kernel<5, STEP>;
+    default: return nullptr;
+  }
+}
 
-cudaError_t swar_sums_launch(const uint8_t *in, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule, int32_t *sums,
-                             int64_t sums_ld, cudaStream_t s) {
-  SwarParams p;
+SwarParams swar_params(const uint8_t *in, int64_t pitch, int64_t H, int64_t W) {
+  SwarParams p{};
   p.in = reinterpret_cast<const uint32_t *>(in);
   p.pitch_words = pitch / 4;
   p.H = (int32_t)H;
   p.W = (int32_t)W;
   p.words = (int32_t)((W + 31) / 32);
+  return p;
+}
+
+dim3 swar_grid(const SwarParams &p) {
+  const int64_t strips = ((int64_t)p.H + kRows - 1) / kRows;
+  return dim3((unsigned)((p.words + kBlock - 1) / kBlock), (unsigned)(strips < 65535 ? strips : 65535));
+}
+
+}  // namespace
+
+cudaError_t swar_sums_launch(const uint8_t *in, int64_t pitch, int64_t H, int64_t W, const RuleDev &rule, int32_t *sums,
+                             int64_t sums_ld, cudaStream_t s) {
+  const SwarKernel kern = swar_kernel<false>(rule.r);
+  if (!kern) return cudaErrorInvalidValue;
+  SwarParams p = swar_params(in, pitch, H, W);
   p.sums = sums;
   p.sums_ld = sums_ld;
-  const int64_t strips = (H + kRows - 1) / kRows;
-  const dim3 grid((unsigned)((p.words + kBlock - 1) / kBlock), (unsigned)(strips < 65535 ? strips : 65535));
-  void (*kern)(SwarParams) = nullptr;
-  switch (rule.r) {
-    case 1: kern = ltl_swar_kernel<1>; break;
-    case 2: kern = ltl_swar_kernel<2>; break;
-    case 3: kern = ltl_swar_kernel<3>; break;
-    case 4: kern = ltl_swar_kernel<4>; break;
-    case 5: kern = ltl_swar_kernel<5>; break;
-    default: return cudaErrorInvalidValue;
-  }
-  kern<<<grid, kBlock, 0, s>>>(p);
+  kern<<<swar_grid(p), kBlock, 0, s>>>(p);
   return cudaGetLastError();
+}
+
+cudaError_t swar_step_launch(const PlanesGrid &g, cudaStream_t s) {
+  const SwarKernel kern = swar_kernel<true>(g.rule.r);
+  if (!kern) return cudaErrorInvalidValue;
+  SwarParams p = swar_params(g.in, g.pitch, g.H, g.W);
+  p.out = reinterpret_cast<uint32_t *>(g.out);
+  planes::set_bounds(p.bound, g.rule, planes::bits_for((2 * g.rule.r + 1) * (2 * g.rule.r + 1)));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = swar_grid(p);
+  cfg.blockDim = dim3(kBlock);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
 }  // namespace cat

@@ -137,6 +137,8 @@ cudaError_t unpack_nib_launch(const uint8_t *, int64_t, uint8_t *, int64_t, int6
 // bit planes: preferred wherever they are asked about, one step per launch
 bool planes_preferred(const PlanesGrid &g) { return g.rule.nbhd == 0 && g.rule.r <= 16; }
 bool planes_steps_preferred(const PlanesGrid &, int64_t) { return true; }
+bool planes_few_rows(const PlanesGrid &) { return false; }
+cudaError_t swar_step_launch(const PlanesGrid &, cudaStream_t) { return launched("one-bit step"); }
 cudaError_t planes_launch(const PlanesGrid &g, cudaStream_t) { return launched("planes " + storages(g)); }
 TilePlan planes_tile_plan(const PlanesGrid &, int64_t) { return TilePlan{0, 0}; }
 TilePlan planes_tile_steps(const PlanesGrid &, int64_t) { return TilePlan{0, 0}; }

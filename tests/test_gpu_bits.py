@@ -277,3 +277,24 @@ def test_ragged_6600x1001_two_steps(cat):
     grid = _grid(H, W, 0.4, 66)
     want = oracle.step(grid, orule(rule), n_steps=2)
     assert_same(run_bits(cat, grid, rule, 2), want, "6600x1001")
+
+
+@pytest.mark.parametrize("H,r", [(1, 1), (1, 5), (1, 6), (2, 4), (2, 5), (5, 2), (5, 3), (6, 1)])
+@pytest.mark.parametrize("kernel", ["auto", "bitslice"])
+def test_a_few_very_wide_rows(cat, H, r, kernel):
+    """From 2^19 columns on, grids of a row or a few take a kernel of their own."""
+    if kernel == "bitslice" and r > 5:
+        pytest.skip("the bit-sliced kernel choice serves r <= 5")
+    for W in ((1 << 19) - 1, 1 << 19, (1 << 19) + 43):
+        rule = rule_dict(r, M=r & 1)
+        grid = inputs.bernoulli(H, W, 0.5, H + r)
+        g = cat.Grid(H, W, rule, kernel=kernel, dtype="auto", storage=cat.STORE_BIT1)
+        try:
+            g.set_state(grid)
+            g.step(3)
+            assert g.status() == cat.CAT_OK
+            assert_same(g.get_state(), oracle.step(grid, orule(rule), n_steps=3), f"{H} x {W}")
+            row = g.state_tensor().cpu().numpy()
+            assert np.array_equal(np.unpackbits(row, axis=1, bitorder="little")[:, W:].any(), False)
+        finally:
+            g.close()
