@@ -347,8 +347,9 @@ CAT_API int cat_step(cat_handle_t h, int64_t n_steps, void *stream);
  * persistent launch over a flat tile work-list of all instances, and when
  * `stream` is not capturing the n_steps launches are replayed from a CUDA
  * graph cached for this handle list (with every instance's options left to the
- * library, on buffers of its own, and n_steps >= 8 with 2^25 cells or more or n_steps >= 6 with 2^27,
- * that graph packs the two-state grids, steps them on bit planes and unpacks them); otherwise every instance is stepped by
+ * library, on buffers of its own, n_steps >= 8 with 2^25 cells or more or
+ * n_steps >= 6 with 2^27, and grids of r >= 10 in the minority, that graph packs
+ * the two-state grids, steps them on bit planes and unpacks them); otherwise every instance is stepped by
  * its own launches, one step at a time.  Errors: INVALID_ARG (NULL or
  * repeated handles, instances on different devices, mixed dtypes in a
  * batched launch), UNSUPPORTED (a batched instance above 4194176 cells per

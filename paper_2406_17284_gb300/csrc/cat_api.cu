@@ -1019,25 +1019,36 @@ int cat_batch_step(const cat_handle_t *hs, int32_t count, int64_t n_steps, void 
   bool all_tc = true;   // Moore, zero boundary, uint8 storage, no FP4: other instances step one by one
   // Several steps of grids whose options are all left to the library, on bit
   // planes: from eight steps and 2^25 cells on, or six and 2^27 (512 grids with
-  // sides up to 900 / 1400 / 2048, 54 / 102 / 179 million cells, us for 6 steps:
-  // tiles 230 / 371 / 582, planes 243 / 362 / 545; for 8: 302 / 490 / 771 against
-  // 302 / 453 / 681; for 12: 448 / 730 / 1149 against 418 / 634 / 954).
+  // sides up to 2048 and one radius, us a step, n = 8: r = 1 / 5 / 9: 173 / 202 / 232
+  // against the tiles' 229 / 229 / 245; for 6: 184 / 213 / 243; 64 grids of 1024^2,
+  // r = 3, n = 8: 19 against 30).  From r = 10 on the tiles are faster (r = 10 / 16,
+  // n = 16: 309 / 331 against 245), so grids of those radii may make up a quarter of
+  // the cells, or half from twelve steps on (r = 1 .. 16, n = 6 / 8 / 16: 254 / 243 /
+  // 225 against 246; r = 6 and 16: 276 / 261 / 243 against 244); nor may the words
+  // pad the grids by a tenth more than the tiles do (40 grids of 20000 x 128, n = 8:
+  // 62 against 57).
   // A captured call keeps to the tiles, one launch per
   // step, since the planes need the radii side by side.
   bool packed = n_steps >= 6;
-  int64_t cells = 0;
+  int64_t cells = 0, wide = 0, by_words = 0, by_tiles = 0;   // wide: of r >= 10
   bool one_device = true, one_dtype = true, small = true;
   for (int32_t i = 0; i < count; ++i) {
     const cat_instance *h = hs[i];
     all_tc &= h->kernel == CAT_KERNEL_TCGEN05 && h->ghost == 0 && h->storage == CAT_STORE_U8 &&
               h->rule.nbhd == 'M' && !wide_tile(h) && h->dtype != CAT_DTYPE_FP4_E2M1;
     packed &= packed_steps_possible(h, n_steps) && h->owns_buffers;   // (see cat_step: the generation before)
-    cells += h->H * h->W;
+    if (packed) {
+      cells += h->H * h->W;
+      if (h->rule.r >= 10) wide += h->H * h->W;
+      by_words += h->H * 30 * ((h->W + 31) / 32 + 1);
+      by_tiles += round_up(h->H, 128) * round_up(h->W, 128);
+    }
     one_device &= h->dev.id == hs[0]->dev.id;
     one_dtype &= h->dtype == hs[0]->dtype;
     small &= h->H <= 128 * 32767 && h->W <= 128 * 32767;
   }
-  packed &= cells >= (n_steps >= 8 ? 1 << 25 : 1 << 27);
+  packed &= cells >= (n_steps >= 8 ? 1 << 25 : 1 << 27) && wide <= cells / (n_steps >= 12 ? 2 : 4) &&
+            10 * by_words <= 11 * by_tiles;
   std::unique_lock<std::mutex> lk(g_plan_mu);
   BatchPlan *pl = nullptr;
   for (BatchPlan *c : g_plans)

@@ -186,3 +186,24 @@ def test_a_batch_asks_for_the_capture_only_where_it_matters(host):
     host.lib.fake_capturing(0)
     host.cat_destroy(u8)
     host.cat_destroy(bits)
+
+
+@pytest.mark.parametrize("radii,n,planes", [((9, 9, 9, 9), 8, True), ((4, 4, 4, 10), 8, True), ((4, 4, 10, 10), 8, False),
+                                            ((4, 4, 10, 10), 12, True), ((4, 10, 10, 10), 16, False), ((4,) * 4, 7, False)])
+def test_batches_of_large_radii_keep_to_the_tiles(host, radii, n, planes):
+    """The bit planes of a batch gain up to r = 9; larger radii may make up a
+    quarter of the cells, or half of them from twelve steps on."""
+    grids = [host.grid(3000, 3000, r) for r in radii]
+    host.cat_batch_step((ctypes.c_void_p * 4)(*grids), 4, n, None)
+    assert ("batch planes" in host.log()) == planes
+    for g in grids:
+        host.cat_destroy(g)
+
+
+@pytest.mark.parametrize("W,planes", [(128, False), (2048, True)])
+def test_batches_of_narrow_grids_keep_to_the_tiles(host, W, planes):
+    grids = [host.grid((1 << 24) // W, W, 4) for _ in range(2)]
+    host.cat_batch_step((ctypes.c_void_p * 2)(*grids), 2, 8, None)
+    assert ("batch planes" in host.log()) == planes
+    for g in grids:
+        host.cat_destroy(g)
