@@ -245,3 +245,59 @@ def test_tall_grids(cat, H, W, r):
         finally:
             a.close()
             b.close()
+
+
+def test_foreign_kernels_between_default_steps(cat):
+    """Kernels without the early-launch trigger on both sides of every call: they
+    read the state just stepped and rewrite parts of it, in place, on one stream
+    with grids of other storages, each stepped in turn."""
+    import torch
+    H, W, pitch = 600, 700, 720
+    rule = inputs.scaled_rule(4)
+    grid = board(H, W, 2, 31)
+    a = torch.zeros((H, pitch), dtype=torch.uint8, device="cuda")
+    b = torch.zeros((H, pitch), dtype=torch.uint8, device="cuda")
+    a[:, :W] = torch.from_numpy(grid).cuda()
+    bound = cat.Grid(H, W, rule, kernel="auto", dtype="auto")
+    cat.cat_bind(bound.handle, a.data_ptr(), b.data_ptr(), pitch)
+    others = []
+    for r, C, storage, boundary in ((2, 2, 1, 0), (9, 2, 1, 0), (1, 2, 0, 0), (5, 5, 2, 0), (3, 16, 0, 0), (4, 2, 0, 1)):
+        rr, host = inputs.scaled_rule(r, C=C), board(300 + 7 * r, 401, C, r)
+        g = cat.Grid(*host.shape, rr, kernel="auto", dtype="auto", storage=storage, boundary=boundary)
+        g.set_state(host)
+        others.append([g, oracle.Rule(**rr), host, boundary])
+    try:
+        cur, other, want = a, b, grid
+        for k, n in enumerate((1, 2, 5, 1, 4)):
+            bound.step(n)
+            if n & 1:
+                cur, other = other, cur
+            snap, want = cur[:, :W].clone(), oracle.step(want, oracle.Rule(**rule), n_steps=n)
+            cur[50 + 40 * k:90 + 40 * k, :W] ^= 1
+            cur[:, 9 * k:9 * k + 20] = 0
+            for o in others:
+                o[0].step(n)
+                o[2] = oracle.step(o[2], o[1], boundary=o[3], n_steps=n)
+                if o[0].storage == 0:    # the first row dies, by a torch kernel
+                    o[0].state_tensor()[0] = 0
+                    o[2] = o[2].copy()
+                    o[2][0] = 0
+            assert np.array_equal(snap.cpu().numpy(), want), k
+            want = want.copy()
+            want[50 + 40 * k:90 + 40 * k] ^= 1
+            want[:, 9 * k:9 * k + 20] = 0
+        for g, rr, host, boundary in others:
+            assert np.array_equal(g.get_state(), host), (rr, boundary)
+    finally:
+        for g in [bound] + [o[0] for o in others]:
+            g.close()
+
+
+@pytest.mark.parametrize("r,n", [(10, 4), (10, 8), (3, 6), (2, 32), (1, 32)])
+def test_tiles_of_as_many_steps_as_they_take(cat, r, n):
+    """The most steps per launch: two at r = 10, after which 30 of the 32 cells of
+    a neighbouring word are stale."""
+    for H, W in [(40, 33), (200, 961), (90, 1031)]:
+        check(cat, H, W, inputs.scaled_rule(r, M=1), 1, steps=n)
+        if W >= 64:
+            check(cat, H, W, inputs.scaled_rule(r, M=1), 0, steps=n + 1)
