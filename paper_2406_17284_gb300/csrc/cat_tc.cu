@@ -872,7 +872,7 @@ __device__ __forceinline__ int32_t *tile_err(const TcParams &p, int first, int j
 }
 
 template <int DT, bool ENC, bool BATCH, bool SW, bool BITS, bool MS, bool WIDE = false, bool NIB = false,
-          bool FP4 = false, bool BIG = false, int HB = 0, bool R15 = false>
+          bool FP4 = false, bool BIG = false, bool HB = false, bool R15 = false>
 __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   constexpr bool OF = R15 && DT == 1 && !ENC;   // the offset pass 2
   static_assert(!MS || !BATCH, "several steps per launch serve single instances");
@@ -886,9 +886,8 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
   static_assert(!BIG || (DT == 1 && !ENC && !BATCH && !SW && !BITS && !MS && !WIDE && !NIB && !FP4),
                 "the big window serves single two-state instances on FP8 operands, one step per launch");
   // HB (big window, r <= 22, every count <= 45^2 = 2025 exact in f16): the
-  // epilogue tests f16 pairs, converted from the f32 accumulator (1) or
-  // accumulated in f16 by pass 2 (2); 0: the f32 test
-  static_assert(HB == 0 || BIG, "f16 pairs serve the big window");
+  // epilogue tests f16 pairs, accumulated in f16 by pass 2
+  static_assert(!HB || BIG, "f16 pairs serve the big window");
   // R15 (r <= 15): the epilogue tests ranges by middle and half width, and
   // without a re-encoded window (r >= 8 then) pass 2 takes H - 16
   static_assert(!R15 || (!BATCH && !SW && !BITS && !WIDE && !NIB && !FP4 && !BIG),
@@ -1166,7 +1165,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     // tile's own D1 region.
     if (lane == 0) {
       // the wide tile: N = 96 and f32 accumulators (counts up to 4225)
-      const uint32_t idesc2 = ((WIDE || BIG) && HB != 2) ? idesc_f32acc(128, G::kTS) : idesc_f16acc(128, kTile);
+      const uint32_t idesc2 = ((WIDE || BIG) && !HB) ? idesc_f32acc(128, G::kTS) : idesc_f16acc(128, kTile);
       const uint32_t band16 = tmem + T::kBand16, band8 = tmem + T::kBand8P2;
       const uint32_t band_hi = tmem + T::kBand8x16;   // wide tile: the band of 16s for the second digit
       const OpDesc hop0 = op_descs(s_base + L::kH);
@@ -1399,23 +1398,23 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
     constexpr int nch = G::kTS / 16 / EK;
     static_assert(nch * EK * 16 == G::kTS, "the warps of a quarter take the same number of chunks");
     bool ok = true;
-    const auto ir = [&] {
+    const auto range = [&] {
       if constexpr (WIDE) return make_float_rule(p.rule, kScale);
+      else if constexpr (HB) return make_range_rule(p.rule, kScale, 1024);   // counts up to 2025, less 1024
       else return make_int_rule(p.rule);
     }();
-    const HalfRule hr = make_range_rule(p.rule, kScale, 1024);   // HB: counts up to 2025, less 1024
     TileSeq<false, false, G::kTS> seq(p, first, n_my);
     for (int j = 0; ok && j < n_all; ++j, seq.next(p)) {
       const int reg = j % ND2, k = j % NR;
       const Tile t = seq.get(p);
       if (!(ok = warp_wait(&bars->d2_full[reg], (j / ND2) & 1, bars, p.timeout_ns))) break;
       tc_fence_after();
-      uint32_t v[nch][HB == 2 ? 8 : 16];               // S * scale as f32, or f16 pairs (HB 2)
+      uint32_t v[nch][HB ? 8 : 16];                    // S * scale as f32, or f16 pairs (HB)
       if (rows) {
         const uint32_t treg = tmem + lane_addr + T::kD2Base + reg * T::kD2Cols;
 #pragma unroll
         for (int c = 0; c < nch; ++c) {
-          if constexpr (HB == 2) tmem_ld16_pack16(treg + 16 * (kq + EK * c), v[c]);
+          if constexpr (HB) tmem_ld16_pack16(treg + 16 * (kq + EK * c), v[c]);
           else tmem_ld16(treg + 16 * (kq + EK * c), v[c]);
         }
         tmem_wait_ld();
@@ -1433,24 +1432,20 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             uint4 *cell = reinterpret_cast<uint4 *>(ring + (BIG ? y * 128 + (((cc ^ y) & 7) << 4) : y * G::kTS + 16 * cc));
             const uint4 cv = *cell;
             uint4 ov;
-            if constexpr (HB == 0) {
+            if constexpr (!HB) {
               auto next = [&](int i, uint32_t cells) {
-                if constexpr (WIDE) return rule4_range_f(v[c] + i, cells, ir);
-                else return rule4_binary_i(v[c] + i, cells, ir);
+                if constexpr (WIDE) return rule4_range_f(v[c] + i, cells, range);
+                else return rule4_binary_i(v[c] + i, cells, range);
               };
               ov = make_uint4(next(0, cv.x), next(4, cv.y), next(8, cv.z), next(12, cv.w));
             } else {
-              // f16 pairs of cells (2i, 2i + 1): packed by pass 2, or converted
-              // here (exact, S * 2^-9 < 4)
-              auto pr = [&](int i) -> uint32_t {
-                const __half2 c1024 = __float2half2_rn(1024.0f * kScale);
-                if constexpr (HB == 2) return h2_bits(__hsub2(as_h2(v[c][i]), c1024));
-                else return h2_bits(__hsub2(__floats2half2_rn(__uint_as_float(v[c][2 * i]), __uint_as_float(v[c][2 * i + 1])), c1024));
+              auto pr = [&](int i) -> uint32_t {   // cells (2i, 2i + 1)
+                return h2_bits(__hsub2(as_h2(v[c][i]), __float2half2_rn(1024.0f * kScale)));
               };
-              ov.x = rule4_range_h(pr(0), pr(1), cv.x, hr);
-              ov.y = rule4_range_h(pr(2), pr(3), cv.y, hr);
-              ov.z = rule4_range_h(pr(4), pr(5), cv.z, hr);
-              ov.w = rule4_range_h(pr(6), pr(7), cv.w, hr);
+              ov.x = rule4_range_h(pr(0), pr(1), cv.x, range);
+              ov.y = rule4_range_h(pr(2), pr(3), cv.y, range);
+              ov.z = rule4_range_h(pr(4), pr(5), cv.z, range);
+              ov.w = rule4_range_h(pr(6), pr(7), cv.w, range);
             }
             *cell = ov;
           } else {   // box counts
@@ -1459,7 +1454,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             for (int i = 0; i < 16; ++i) {
               const int gx = t.x0 + 16 * cc + i;
               float sv;
-              if constexpr (HB == 2) sv = (i & 1) ? half_hi(v[c][i >> 1]) : half_lo(v[c][i >> 1]);
+              if constexpr (HB) sv = (i & 1) ? half_hi(v[c][i >> 1]) : half_lo(v[c][i >> 1]);
               else sv = __uint_as_float(v[c][i]);
               if (gy < t.H && gx < t.W) p.sums[(int64_t)gy * p.sums_ld + gx] = __float2int_rn(sv * (1.0f / kScale));
             }
@@ -1563,8 +1558,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
             const uint4 cv = *cell;
             uint4 ov;
             auto next = [&](int i, uint32_t cells) {
-              if constexpr (kRange) return rule4_range_h(count(v[c][i]), count(v[c][i + 1]), cells, hr);
-              else return rule4_binary_h(v[c][i], v[c][i + 1], cells, hr);
+              return rule4_range_h(count(v[c][i]), count(v[c][i + 1]), cells, hr);
             };
             ov = make_uint4(next(0, cv.x), next(2, cv.y), next(4, cv.z), next(6, cv.w));
             *cell = ov;
@@ -1641,7 +1635,7 @@ __device__ __forceinline__ void ltl_tc_body(const TcParams &p) {
 
 template <int DT, bool ENC, bool BATCH, bool SW, bool R15>
 __global__ void __launch_bounds__(kThreads, 1) ltl_tc_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<DT, ENC, BATCH, SW, false, false, false, false, false, false, 0, R15>(p);
+  ltl_tc_body<DT, ENC, BATCH, SW, false, false, false, false, false, false, false, R15>(p);
 }
 
 // One bit per cell: the same body under its own name, so that a profiler can
@@ -1682,14 +1676,14 @@ __global__ void __launch_bounds__(threads_with(kEpiWarpsMore), 1) ltl_big_kernel
 // accumulates in f16 and the epilogue tests f16 pairs (measured 7% faster
 // than the f32 test, 2% faster than converting the f32 accumulator).
 __global__ void __launch_bounds__(threads_with(kEpiWarpsMore), 1) ltl_big16_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<1, false, false, false, false, false, false, false, false, true, 2>(p);
+  ltl_tc_body<1, false, false, false, false, false, false, false, false, true, true>(p);
 }
 
 // Several steps of a single instance in one cooperative launch (separate
 // instantiations, so that the one-step kernels carry none of it).
 template <int DT, bool ENC, bool SW, bool BITS, bool R15>
 __global__ void __launch_bounds__(kThreads, 1) ltl_tc_multi_kernel(const __grid_constant__ TcParams p) {
-  ltl_tc_body<DT, ENC, false, SW, BITS, true, false, false, false, false, 0, R15>(p);
+  ltl_tc_body<DT, ENC, false, SW, BITS, true, false, false, false, false, false, R15>(p);
 }
 
 // ---------------------------------------------------------------------------
