@@ -21,11 +21,12 @@
 // All additions are exact, so the next states are those of every other kernel
 // (Sec. IV, Eqs. 1-2 define the same count as two band products).
 //
-// What bounds it: the integer pipe (ncu, one bit per cell, 32768^2, r = 16: ALU
-// 82%, DRAM 9%; four bits, r = 10: ALU 69%).  32768^2 one-bit steps: r = 2
-// 224 -> 148 us, r = 16 594 -> 320 us; 24576^2, C = 16, r = 10: four bits 436
-// -> 297 us, one byte 398 -> 355 us (before: the tensor-core kernels, and at
-// r <= 5 a bit-sliced kernel that added the 2r + 1 cells and rows one by one).
+// What bounds it: the integer pipe (ncu, 16384^2: one bit per cell, r = 2 / 16:
+// ALU 78% / 83%, DRAM 10% / 5%; C = 16, r = 10: four bits 81%, one byte 74%).
+// 32768^2 one-bit steps: r = 2 224 -> 148 us, r = 16 594 -> 327 us; 24576^2,
+// C = 16, r = 10: four bits 435 -> 269 us, one byte 398 -> 333 us (before: the
+// tensor-core kernels, and at r <= 5 a bit-sliced kernel that added the 2r + 1
+// cells and rows one by one).
 //
 // Lanes are laid over a virtual row of words: the row strips of the grid side
 // by side, each followed by one zero word (the dead cells beyond its right
@@ -570,7 +571,8 @@ __global__ void __launch_bounds__(32, Cfg<R, MS>::kWarps) planes_kernel(const __
 // state that is still needed (as one grid's steps are): the bytes are packed,
 // stepped and unpacked by separate launches, since the small grids' few warps
 // do not keep enough bytes in flight to step from them (512 uneven grids, 4
-// steps: 465 us with the first and last step on bytes, 310 us so).
+// steps: 465 us with the first and last step on bytes, 371 us so; the tiles, which
+// serve so short calls, 351).
 struct BatchGrid {
   uint8_t *buf[2];
   int64_t pitch;
