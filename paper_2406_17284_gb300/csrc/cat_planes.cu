@@ -214,7 +214,8 @@ bool planes_preferred(const PlanesGrid &g) {
 //                           1638400 x 128, r = 7: 105 / 106 / 95 and 73; 873813 x
 //                           96, r = 3: 48.0 / 47.5 / .. and 41.8 (n = 5: 40.7); 362539
 //                           x 376, r = 16: .. / 69.2 / .. and 59.9; torus 65536 x
-//                           96, r = 7: .. / 15.3 / 16.1 and 12.3
+//                           96, r = 7: .. / 15.3 / 16.1 and 12.3; torus 384362 x
+//                           320, r = 13: 99 / .. / .. and 90
 //   torus, n = 8            2048^2, r = 12: 9.0 and 7.1; 4096^2, r = 7 / 12: 10.9
 //                           / 14.6 and 12.1; 5792^2, r = 12: 18.0 and 18.7;
 //                           7000^2, r = 11 / 15: 23.6 / 22.7 and 23.4
@@ -225,12 +226,12 @@ bool planes_steps_preferred(const PlanesGrid &g, int64_t n_steps) {
   if (padded(g) && g.frame) {
     if (m > 4 && m <= 36 && r > 4) return false;
     if (m > 12 && g.W <= 128) return false;
-    if (m > 36) return r <= 7 || n_steps >= 8;
+    if (m > 36) return r <= 4 || n_steps >= 8;
   } else if (padded(g) && m > 24) {
     if (g.W <= 96) return n_steps >= (m > 64 && odd ? 8 : 4);
     return n_steps >= 8 && (g.W > 128 || (r <= 4 && m <= 64));
   }
-  if (g.frame) return r <= 7 || (m >= 30 && n_steps >= (m < 64 ? 8 : r == 8 || r >= 14 ? 3 : 2));
+  if (g.frame) return r <= 7 || (m >= 30 && n_steps >= (m < 64 ? 8 : r == 8 || r >= (g.W < 512 ? 10 : 14) ? 3 : 2));
   if (r <= 7) return m <= 4 || m > 24 || n_steps >= (r == 7 ? 4 : r >= 5 ? 3 : 2);
   if (m <= (r <= 10 ? 10 : 6)) return true;
   if (m <= 24) return r <= 10 && n_steps >= 4;
