@@ -7,7 +7,10 @@ One bench step = one LTL step of each of the 16 grids (16 kernel launches,
 16 x 2^28 cell updates).  The grids (256 MiB each) exceed the 129 MB L2, so no
 flush is needed between launches.
 
-Prints ONE JSON line (metric cell-updates/s).  `--impl reference` times the
+Prints ONE JSON line (metric cell-updates/s), short enough for the last 1500
+characters of the output to hold it; every other figure (rates per radius and
+kernel, the other workloads, their rooflines) goes to stderr as one JSON line
+{"detail": ...}.  `--impl reference` times the
 CPU oracle (the paper has no code to run) on a bounded sample of the same
 workload.
 """
@@ -55,6 +58,22 @@ def parse():
     ap.add_argument("--no-wide", action="store_true", help="skip the r > 16 measurement")
     ap.add_argument("--no-fp4", action="store_true", help="skip the FP4 / FP8 precision measurement")
     return ap.parse_args()
+
+
+CONTRACT = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches", "e2e", "clocks", "cpu_baseline", "roofline")
+BRIEF = {"roofline": ("bound", "achieved", "peak", "unit", "frac", "kernel"),
+         "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+         "cpu_baseline": ("value", "unit", "cores", "kind", "sample")}
+
+
+def headline(line):
+    """What the benchmark prints of all that it measured (see the module's docstring)."""
+    out = {k: line[k] for k in CONTRACT if k in line}
+    for k, keys in BRIEF.items():
+        if out.get(k):
+            out[k] = {q: out[k][q] for q in keys if q in out[k]}
+    return out
 
 
 def job_rate(ms_total_local, cells_per_step_per_rank, steps, world, dist=None, device="cpu"):
@@ -873,7 +892,8 @@ def run_cat(args, rank, world, local):
             "cpu_baseline": cpu,
             "clocks": clk.summary(),
         }
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"detail": line}), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
