@@ -331,7 +331,8 @@ CAT_API int cat_bind(cat_handle_t h, uint8_t *a, uint8_t *b, int64_t pitch);
  * writing buffer B, then the two swap (with steps_per_launch = k > 1, k steps
  * per launch, the swap inside it).  However the steps are split into launches,
  * the state is afterwards in the buffer that held it before when n_steps is
- * even, so a captured call of an even number of steps can be replayed.  The
+ * even, so a captured call of an even number of steps can be replayed (but
+ * BITSLICE with several steps per launch moves it once per launch).  The
  * buffer that does not hold the state afterwards has no defined contents,
  * unless it is a caller's (cat_bind).  Each step computes the band products of
  * Sec. IV (Eqs. 1-2) and the rule of Sec. V-A for every cell.  Errors:
